@@ -20,6 +20,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "passes.cuh"
 
 namespace lru {
 
@@ -35,173 +36,178 @@ __device__ __forceinline__ const T* opvec(const DevOperand& O, const DevLayout& 
     return reinterpret_cast<const T*>(O.dense) + (L.vo(w) * O.slots + (long long)a * n);
 }
 
-// One CTA per walker.  ws: 2 * kk * n_w scalars per walker (Y, then Z).
-template <typename T, bool PF, bool DELAYED>
-__global__ void __launch_bounds__(AT) k_backward(DevLayout L, DevState<T> S, DevOperand Vop, const T* C, const T* g,
-                                                  T* ws, T* gU, T* gV, T* gA, T* gC) {
-    __shared__ T sR[AMAXKK * AMAXKK];
-    __shared__ int siv[AMAXKK];
-    __shared__ T sVP[AMAXKK * 64];
-    const int w = blockIdx.x;
+// gC = skew part of -[C^{-1} (M^{-1} - C) C^{-1}]^T / 2 of walker w (C = -J when
+// C is null), by one thread; sR: M^{-1}.
+template <typename T>
+__device__ void backward_core(const T* Cw, int m, const T* sR, T gw, T* gCw) {
+    T Cm[AMAXKK * AMAXKK], Ci[AMAXKK * AMAXKK], T1[AMAXKK * AMAXKK];
+    for (int a = 0; a < m; ++a)
+        for (int b = 0; b < m; ++b) {
+            double v = (b == a + m / 2) ? -1.0 : ((a == b + m / 2) ? 1.0 : 0.0);   // -J
+            Cm[a * AMAXKK + b] = Cw ? Cw[a * m + b] : make_real<T>(v);
+        }
+    // C^{-1} by Gauss-Jordan on a copy (small, m <= 16)
+    for (int a = 0; a < m; ++a)
+        for (int b = 0; b < m; ++b) Ci[a * AMAXKK + b] = Cm[a * AMAXKK + b];
+    {
+        int swp[AMAXKK];
+        for (int k = 0; k < m; ++k) {
+            int p = k;
+            double best = (double)s_abs2(Ci[k * AMAXKK + k]);
+            for (int i = k + 1; i < m; ++i)
+                if ((double)s_abs2(Ci[i * AMAXKK + k]) > best) { best = (double)s_abs2(Ci[i * AMAXKK + k]); p = i; }
+            swp[k] = p;
+            if (p != k)
+                for (int j = 0; j < m; ++j) {
+                    T t = Ci[k * AMAXKK + j]; Ci[k * AMAXKK + j] = Ci[p * AMAXKK + j]; Ci[p * AMAXKK + j] = t;
+                }
+            T ip = s_recip(Ci[k * AMAXKK + k]);
+            Ci[k * AMAXKK + k] = make_real<T>(1.0);
+            for (int j = 0; j < m; ++j) Ci[k * AMAXKK + j] = Ci[k * AMAXKK + j] * ip;
+            for (int i = 0; i < m; ++i) {
+                if (i == k) continue;
+                T f = Ci[i * AMAXKK + k];
+                Ci[i * AMAXKK + k] = s_zero(T());
+                for (int j = 0; j < m; ++j) Ci[i * AMAXKK + j] = s_fms(f, Ci[k * AMAXKK + j], Ci[i * AMAXKK + j]);
+            }
+        }
+        for (int k = m - 1; k >= 0; --k)
+            if (swp[k] != k)
+                for (int i = 0; i < m; ++i) {
+                    T t = Ci[i * AMAXKK + k]; Ci[i * AMAXKK + k] = Ci[i * AMAXKK + swp[k]]; Ci[i * AMAXKK + swp[k]] = t;
+                }
+    }
+    // T1 = (M^{-1} - C) C^{-1}; then G = C^{-1} T1
+    for (int a = 0; a < m; ++a)
+        for (int b = 0; b < m; ++b) {
+            T s = s_zero(T());
+            for (int c = 0; c < m; ++c) s = s_fma(sR[a * AMAXKK + c] - Cm[a * AMAXKK + c], Ci[c * AMAXKK + b], s);
+            T1[a * AMAXKK + b] = s;
+        }
+    for (int a = 0; a < m; ++a)
+        for (int b = 0; b < m; ++b) {
+            // unconstrained gradient entry (a, b) = -[C^{-1} T1]_{b a} / 2
+            T sba = s_zero(T()), sab = s_zero(T());
+            for (int c = 0; c < m; ++c) {
+                sba = s_fma(Ci[b * AMAXKK + c], T1[c * AMAXKK + a], sba);
+                sab = s_fma(Ci[a * AMAXKK + c], T1[c * AMAXKK + b], sab);
+            }
+            // skew part: (G_ab - G_ba) / 2 with G_ab = -sba / 2, G_ba = -sab / 2
+            T v = s_half(s_half(sab - sba));
+            gCw[a * m + b] = gw * s_conj(v);
+        }
+}
+
+template <typename T>
+struct BackSmem {
+    YSmem<T> y;                  // det: Y of the item's columns, then its rows of the outer product
+    T R[AMAXKK * AMAXKK];
+    T VP[AMAXKK * 64];
+    T out[AMAXKK][YC];           // the item's rows, conjugated: R^{-1} Y (det) or X M^{-1} (pf)
+    int iv[AMAXKK];
+};
+
+// One CTA per work item (walker, columns [l0, l1) of A^{-1}), in blocks of YC.
+// The gradient of A is the outer product of two rank-kk factors, n^2 outputs
+// that nothing but the store should bound: a thread keeps the kk values of its
+// column j in registers and walks the block's rows, whose factors are in
+// shared memory, so the stores are coalesced and every factor is read once per
+// block.
+//   det: T = R^{-1} Y;  gU = g conj(T), gV = g conj(X R^{-1}),
+//        gA[i][j] = -g conj(sum_a X_a[j] T[a][i])
+//   pf : Z = X M^{-1};  gB = g conj(Z), gA[i][j] = -g conj(sum_b Z[i][b] X_b[j]) / 2
+template <typename T, bool PF, bool DELAYED, int KBM>
+__global__ void __launch_bounds__(AT, 2) k_backward(DevLayout L, DevState<T> S, DevOperand Vop, const T* C, const T* g,
+                                                     T* gU, T* gV, T* gA, T* gC, const int4* items) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    BackSmem<T>& sm = *reinterpret_cast<BackSmem<T>*>(dsm);
+    const int4 it = items[blockIdx.x];
+    const int w = it.x;
+    if (!LRU_DEBUG_OK(w >= 0 && w < L.W, S.err)) return;
     const int n = L.nw(w), kk = L.kv(w);
+    if (!LRU_DEBUG_OK(it.y >= 0 && it.y <= it.z && it.z <= n, S.err)) return;
     const long long vo = L.vo(w);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int slots = L.kk;
     T* gUw = gU ? gU + vo * slots : nullptr;
     T* gVw = gV ? gV + vo * slots : nullptr;
     T* gAw = gA ? gA + L.mo(w) : nullptr;
+    const int rows = it.z - it.y;
     if (S.pst[w] != 0) {
         // no pending proposal with a valid core: zero gradient
-        for (long long e = threadIdx.x; e < (long long)kk * n; e += AT) {
-            if (gUw) gUw[e] = s_zero(T());
-            if (gVw) gVw[e] = s_zero(T());
+        for (int e = threadIdx.x; e < kk * rows; e += AT) {
+            const int a = e / rows, j = it.y + e - a * rows;
+            if (gUw) gUw[(long long)a * n + j] = s_zero(T());
+            if (gVw) gVw[(long long)a * n + j] = s_zero(T());
         }
         if (gAw)
-            for (long long e = threadIdx.x; e < (long long)n * n; e += AT) gAw[e] = s_zero(T());
-        if (gC && threadIdx.x < kk * kk) gC[(long long)w * L.kk * L.kk + threadIdx.x] = s_zero(T());
+            for (long long e = threadIdx.x; e < (long long)rows * n; e += AT) gAw[(long long)it.y * n + e] = s_zero(T());
+        if (gC && it.y == 0 && threadIdx.x < kk * kk) gC[(long long)w * L.kk * L.kk + threadIdx.x] = s_zero(T());
         return;
     }
     const T gw = g[w];
     const T* X = S.X + vo * L.kk;             // kk vectors of n: X[a*n + j] = (A^{-1} U)_{j a}
-    T* Y = ws + vo * 2 * slots;               // kk x n
-    T* Z = Y + (long long)slots * n;          // n x kk, Z[j*kk + b]
-    for (int e = threadIdx.x; e < AMAXKK * AMAXKK; e += AT) sR[e] = S.Rinv[(long long)w * AMAXKK * AMAXKK + e];
+    for (int e = threadIdx.x; e < kk * kk; e += AT) {
+        const int a = e / kk, b = e - a * kk;
+        sm.R[a * AMAXKK + b] = S.Rinv[(long long)w * AMAXKK * AMAXKK + a * AMAXKK + b];
+    }
     if (threadIdx.x < kk)
-        siv[threadIdx.x] = ((Vop.mask >> threadIdx.x) & 1u) ? Vop.idx[(long long)w * Vop.slots + threadIdx.x] : -1;
+        sm.iv[threadIdx.x] = ((Vop.mask >> threadIdx.x) & 1u) ? Vop.idx[(long long)w * Vop.slots + threadIdx.x] : -1;
     const int cu = DELAYED ? S.tau[w] * kk : 0;
     if constexpr (DELAYED && !PF)
         for (int e = threadIdx.x; e < kk * cu; e += AT) {
-            const int b = e / cu, c = e % cu;
-            sVP[b * 64 + c] = S.VP[(long long)w * AMAXKK * L.Kc + b * L.Kc + c];
+            const int b = e / cu, c = e - b * cu;
+            sm.VP[b * 64 + c] = S.VP[(long long)w * AMAXKK * L.Kc + b * L.Kc + c];
         }
     __syncthreads();
+    if (PF && gC && it.y == 0 && threadIdx.x == 0)
+        backward_core<T>(C ? C + (long long)w * L.kk * L.kk : nullptr, kk, sm.R, gw, gC + (long long)w * L.kk * L.kk);
 
-    // Z = X R^{-1} (n x kk)
-    for (int j = threadIdx.x; j < n; j += AT)
-        for (int b = 0; b < kk; ++b) {
-            T z = s_zero(T());
-            for (int a = 0; a < kk; ++a) z = s_fma(X[(long long)a * n + j], sR[a * AMAXKK + b], z);
-            Z[(long long)j * kk + b] = z;
+    for (int l0 = it.y; l0 < it.z; l0 += YC) {
+        const int nc = min(YC, it.z - l0);
+        if constexpr (!PF) {
+            if (gUw || gAw) {
+                const T* Vw = Vop.dense ? opvec<T>(Vop, L, w, 0, n) : nullptr;
+                dense_y_cols<T, KBM>(S.G + L.mo(w), n, l0, nc, Vw, sm.iv, kk, sm.y);
+                if (cu > 0) slot_correct_y<T>(S.Q + vo * L.Kc, L.Kc, cu, l0, nc, sm.VP, kk, sm.y);
+            }
         }
-
-    if constexpr (!PF) {
-        // Y = V A^{-1}: one warp per column l of A^{-1} (a contiguous chunk)
-        const T* Gw = S.G + L.mo(w);
-        for (int l = wid; l < n; l += AT / 32) {
-            const T* col = Gw + (long long)l * n;
+        // this block's rows of the left factor, and the operand gradients
+        for (int e = threadIdx.x; e < kk * nc; e += AT) {
+            const int a = e / nc, c = e - a * nc, j = l0 + c;
+            T t = s_zero(T()), z = s_zero(T());
             for (int b = 0; b < kk; ++b) {
-                T y;
-                if (siv[b] >= 0) {
-                    y = col[siv[b]];
-                } else {
-                    const T* vb = opvec<T>(Vop, L, w, b, n);
-                    T part = s_zero(T());
-                    for (int j = lane; j < n; j += 32) part = s_fma(vb[j], col[j], part);
-                    y = warp_sum(part);
+                if constexpr (!PF) {
+                    if (gUw || gAw) t = s_fma(sm.R[a * AMAXKK + b], sm.y.y[b][c], t);
                 }
-                if constexpr (DELAYED) {
-                    const T* qrow = S.Q + (vo + l) * L.Kc;
-                    for (int c = 0; c < cu; ++c) y = s_fms(sVP[b * 64 + c], qrow[c], y);
-                }
-                if (lane == 0) Y[(long long)b * n + l] = y;
+                z = s_fma(X[(long long)b * n + j], sm.R[b * AMAXKK + a], z);
+            }
+            sm.out[a][c] = s_conj(PF ? z : t);
+            if (PF) {
+                if (gUw) gUw[(long long)a * n + j] = gw * s_conj(z);
+            } else {
+                if (gUw) gUw[(long long)a * n + j] = gw * s_conj(t);
+                if (gVw) gVw[(long long)a * n + j] = gw * s_conj(z);
             }
         }
-    }
-    __syncthreads();
-
-    if constexpr (!PF) {
-        // gU[a][j] = g conj((R^{-1} Y)_{a j}),  gV[b][j] = g conj(Z[j][b])
-        for (int j = threadIdx.x; j < n; j += AT)
-            for (int a = 0; a < kk; ++a) {
-                if (gUw) {
+        __syncthreads();
+        if (gAw) {
+            const T gs = PF ? s_half(s_neg(gw)) : s_neg(gw);
+            for (int j = threadIdx.x; j < n; j += AT) {
+                T x[KBM];   // the cotangent goes into the n kk factors, not the n^2 outputs
+#pragma unroll
+                for (int b = 0; b < KBM; ++b) x[b] = b < kk ? gs * s_conj(X[(long long)b * n + j]) : s_zero(T());
+#pragma unroll 4
+                for (int c = 0; c < nc; ++c) {
                     T s = s_zero(T());
-                    for (int b = 0; b < kk; ++b) s = s_fma(sR[a * AMAXKK + b], Y[(long long)b * n + j], s);
-                    gUw[(long long)a * n + j] = gw * s_conj(s);
+#pragma unroll
+                    for (int b = 0; b < KBM; ++b)
+                        if (b < kk) s = s_fma(x[b], sm.out[b][c], s);
+                    for (int b = KBM; b < kk; ++b) s = s_fma(gs * s_conj(X[(long long)b * n + j]), sm.out[b][c], s);
+                    gAw[(long long)(l0 + c) * n + j] = s;
                 }
-                if (gVw) gVw[(long long)a * n + j] = gw * s_conj(Z[(long long)j * kk + a]);
             }
-        // gA[i][j] = -g conj(sum_b Z[j][b] Y[b][i])  (row-major)
-        if (gAw)
-            for (long long e = threadIdx.x; e < (long long)n * n; e += AT) {
-                const int i = (int)(e / n), j = (int)(e % n);
-                T s = s_zero(T());
-                for (int b = 0; b < kk; ++b) s = s_fma(Z[(long long)j * kk + b], Y[(long long)b * n + i], s);
-                gAw[e] = s_neg(gw * s_conj(s));
-            }
-    } else {
-        // gB[b][j] = g conj(Z[j][b]) with Z = X M^{-1}
-        if (gUw)
-            for (int j = threadIdx.x; j < n; j += AT)
-                for (int b = 0; b < kk; ++b) gUw[(long long)b * n + j] = gw * s_conj(Z[(long long)j * kk + b]);
-        // gA[i][j] = g conj((X M^{-1} X^T)_{j i} / 2) = -g conj(sum_b Z[i][b] X_b[j]) / 2
-        if (gAw)
-            for (long long e = threadIdx.x; e < (long long)n * n; e += AT) {
-                const int i = (int)(e / n), j = (int)(e % n);
-                T s = s_zero(T());
-                for (int b = 0; b < kk; ++b) s = s_fma(Z[(long long)i * kk + b], X[(long long)b * n + j], s);
-                gAw[e] = s_neg(s_half(gw * s_conj(s)));
-            }
-        // gC = skew part of -[C^{-1} (M^{-1} - C) C^{-1}]^T / 2 (C = -J when C is null)
-        if (gC && threadIdx.x == 0) {
-            T Cm[AMAXKK * AMAXKK], Ci[AMAXKK * AMAXKK], T1[AMAXKK * AMAXKK];
-            const int m = kk;
-            for (int a = 0; a < m; ++a)
-                for (int b = 0; b < m; ++b) {
-                    double v = (b == a + m / 2) ? -1.0 : ((a == b + m / 2) ? 1.0 : 0.0);   // -J
-                    Cm[a * AMAXKK + b] = C ? C[(long long)w * L.kk * L.kk + a * m + b] : make_real<T>(v);
-                }
-            // C^{-1} by Gauss-Jordan on a copy (small, m <= 16)
-            for (int a = 0; a < m; ++a)
-                for (int b = 0; b < m; ++b) Ci[a * AMAXKK + b] = Cm[a * AMAXKK + b];
-            {
-                int swp[AMAXKK];
-                for (int k = 0; k < m; ++k) {
-                    int p = k;
-                    double best = (double)s_abs2(Ci[k * AMAXKK + k]);
-                    for (int i = k + 1; i < m; ++i)
-                        if ((double)s_abs2(Ci[i * AMAXKK + k]) > best) { best = (double)s_abs2(Ci[i * AMAXKK + k]); p = i; }
-                    swp[k] = p;
-                    if (p != k)
-                        for (int j = 0; j < m; ++j) {
-                            T t = Ci[k * AMAXKK + j]; Ci[k * AMAXKK + j] = Ci[p * AMAXKK + j]; Ci[p * AMAXKK + j] = t;
-                        }
-                    T ip = s_recip(Ci[k * AMAXKK + k]);
-                    Ci[k * AMAXKK + k] = make_real<T>(1.0);
-                    for (int j = 0; j < m; ++j) Ci[k * AMAXKK + j] = Ci[k * AMAXKK + j] * ip;
-                    for (int i = 0; i < m; ++i) {
-                        if (i == k) continue;
-                        T f = Ci[i * AMAXKK + k];
-                        Ci[i * AMAXKK + k] = s_zero(T());
-                        for (int j = 0; j < m; ++j) Ci[i * AMAXKK + j] = s_fms(f, Ci[k * AMAXKK + j], Ci[i * AMAXKK + j]);
-                    }
-                }
-                for (int k = m - 1; k >= 0; --k)
-                    if (swp[k] != k)
-                        for (int i = 0; i < m; ++i) {
-                            T t = Ci[i * AMAXKK + k]; Ci[i * AMAXKK + k] = Ci[i * AMAXKK + swp[k]]; Ci[i * AMAXKK + swp[k]] = t;
-                        }
-            }
-            // T1 = (M^{-1} - C) C^{-1}; then G = C^{-1} T1
-            for (int a = 0; a < m; ++a)
-                for (int b = 0; b < m; ++b) {
-                    T s = s_zero(T());
-                    for (int c = 0; c < m; ++c) s = s_fma(sR[a * AMAXKK + c] - Cm[a * AMAXKK + c], Ci[c * AMAXKK + b], s);
-                    T1[a * AMAXKK + b] = s;
-                }
-            T* gCw = gC + (long long)w * L.kk * L.kk;
-            for (int a = 0; a < m; ++a)
-                for (int b = 0; b < m; ++b) {
-                    // unconstrained gradient entry (a, b) = -[C^{-1} T1]_{b a} / 2
-                    T sba = s_zero(T()), sab = s_zero(T());
-                    for (int c = 0; c < m; ++c) {
-                        sba = s_fma(Ci[b * AMAXKK + c], T1[c * AMAXKK + a], sba);
-                        sab = s_fma(Ci[a * AMAXKK + c], T1[c * AMAXKK + b], sab);
-                    }
-                    // skew part: (G_ab - G_ba) / 2 with G_ab = -sba / 2, G_ba = -sab / 2
-                    T v = s_half(s_half(sab - sba));
-                    gCw[a * m + b] = gw * s_conj(v);
-                }
         }
+        __syncthreads();
     }
 }
 
@@ -267,13 +273,26 @@ __global__ void k_scatter_rows(DevLayout L, const T* gA, const int* rows, int m,
     }
 }
 
+template <typename T, int KBM>
+static void launch_backward_k(bool pf, bool delayed, const DevLayout& L, const DevState<T>& S, const DevOperand& V,
+                              const T* C, const T* g, T* gU, T* gV, T* gA, T* gC, const int4* items, int nitems,
+                              cudaStream_t st) {
+    auto kern = pf ? (delayed ? k_backward<T, true, true, KBM> : k_backward<T, true, false, KBM>)
+                   : (delayed ? k_backward<T, false, true, KBM> : k_backward<T, false, false, KBM>);
+    const int dyn = (int)sizeof(BackSmem<T>);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    kern<<<nitems, AT, dyn, st>>>(L, S, V, C, g, gU, gV, gA, gC, items);
+}
+
 template <typename T>
 void launch_backward(bool pf, bool delayed, const DevLayout& L, const DevState<T>& S, const DevOperand& V,
-                     const T* C, const T* g, T* ws, T* gU, T* gV, T* gA, T* gC, cudaStream_t st) {
-    if (!pf && !delayed) k_backward<T, false, false><<<L.W, AT, 0, st>>>(L, S, V, C, g, ws, gU, gV, gA, gC);
-    if (!pf && delayed) k_backward<T, false, true><<<L.W, AT, 0, st>>>(L, S, V, C, g, ws, gU, gV, gA, gC);
-    if (pf && !delayed) k_backward<T, true, false><<<L.W, AT, 0, st>>>(L, S, V, C, g, ws, gU, gV, gA, gC);
-    if (pf && delayed) k_backward<T, true, true><<<L.W, AT, 0, st>>>(L, S, V, C, g, ws, gU, gV, gA, gC);
+                     const T* C, const T* g, T* gU, T* gV, T* gA, T* gC, const int* items, int nitems,
+                     cudaStream_t st) {
+    const int4* it = reinterpret_cast<const int4*>(items);
+    if (L.kk == 1) launch_backward_k<T, 1>(pf, delayed, L, S, V, C, g, gU, gV, gA, gC, it, nitems, st);
+    else if (L.kk == 2) launch_backward_k<T, 2>(pf, delayed, L, S, V, C, g, gU, gV, gA, gC, it, nitems, st);
+    else if (L.kk <= 4) launch_backward_k<T, 4>(pf, delayed, L, S, V, C, g, gU, gV, gA, gC, it, nitems, st);
+    else launch_backward_k<T, kb_max<T>()>(pf, delayed, L, S, V, C, g, gU, gV, gA, gC, it, nitems, st);
 }
 
 template <typename T>
@@ -341,7 +360,7 @@ void launch_slog_grad(int W, int n, bool pf, const T* Ginv, const double* g_l, c
     template void launch_slog_grad<T>(int, int, bool, const T*, const double*, const T*, const T*, T*,        \
                                       cudaStream_t);                                                          \
     template void launch_backward<T>(bool, bool, const DevLayout&, const DevState<T>&, const DevOperand&,     \
-                                     const T*, const T*, T*, T*, T*, T*, T*, cudaStream_t);                   \
+                                     const T*, const T*, T*, T*, T*, T*, const int*, int, cudaStream_t);       \
     template void launch_backward_logvalue<T>(bool, bool, const DevLayout&, const DevState<T>&, const T*, T*, \
                                               cudaStream_t);                                                  \
     template void launch_log_ratio<T>(int, const T*, T*, cudaStream_t);                                       \

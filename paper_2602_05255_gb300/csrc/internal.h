@@ -52,7 +52,6 @@ struct DevState {
     T* ratio;      // W
     int* pst;      // W proposal status
     T* VP;         // det delayed: V P (MAXKK x Kc per walker)
-    T* QtU;        // delayed, dense U columns: Q^T U (Kc x MAXKK per walker)
     int* err;      // sticky device error word
 };
 
@@ -61,12 +60,17 @@ struct DevOperand {
     const int* idx;
     unsigned mask;   // bit a: slot a is one-hot
     int slots;       // vector slots per walker in the buffers (kmax)
-    int pre = -1;    // dense slot whose A^{-1} u_a a separate pass has already written to X (-1: none)
 };
+
+// rows of X per work item of the persistent step (XT in passes.cuh)
+constexpr int STEP_X_ROWS = 64;
 
 // Control block of the persistent fused step (see k_step).
 struct StepCtl {
     int* counter;             // work-queue head, zeroed before each launch
+    int* x_done;              // W counters of finished X tiles (zeroed)
+    const int2* x_items;      // X tiles (walker, row block), largest walkers first
+    int n_x_items;            // 0: every column of U is one-hot
     int* prop_done;           // W flags, zeroed before each launch
     int* items_done;          // W counters, zeroed before each launch
     int* fin;                 // W flags: the walker's propose, accept and commit are done (zeroed)
@@ -192,7 +196,8 @@ void launch_slogdet(int W, int n, const T* A, T* ws, int nws, double* logabs, T*
 // ---- adjoint (adjoint.cu) ----
 template <typename T>
 void launch_backward(bool pf, bool delayed, const DevLayout& L, const DevState<T>& S, const DevOperand& V,
-                     const T* C, const T* g, T* ws, T* gU, T* gV, T* gA, T* gC, cudaStream_t st);
+                     const T* C, const T* g, T* gU, T* gV, T* gA, T* gC, const int* items, int nitems,
+                     cudaStream_t st);
 template <typename T>
 void launch_backward_logvalue(bool pf, bool delayed, const DevLayout& L, const DevState<T>& S, const T* g, T* gA,
                               cudaStream_t st);

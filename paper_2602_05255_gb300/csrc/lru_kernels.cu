@@ -9,6 +9,7 @@
 #include "internal.h"
 #include "small_core.cuh"
 #include "df.cuh"
+#include "passes.cuh"
 
 #include <cuda_bf16.h>
 
@@ -58,26 +59,6 @@ __device__ __forceinline__ void store_split(const DevState<T>& S, int PQ, long l
 template <typename T>
 __device__ __forceinline__ const T* vec_ptr(const DevOperand& O, const DevLayout& L, int w, int a, int n) {
     return reinterpret_cast<const T*>(O.dense) + (L.vo(w) * O.slots + (long long)a * n);
-}
-
-// Thread-block reduction of NV values per thread into out[0..NV) (smem red has
-// >= 8*NV entries).  All threads must call it.
-template <typename T, int NV>
-__device__ void block_reduce_vec(T (&v)[NV], T* red, T* out) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NV; ++q) v[q] = warp_sum(v[q]);
-    __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < NV; ++q) red[wid * NV + q] = v[q];
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        T s = s_zero(T());
-        for (int q = 0; q < PT / 32; ++q) s = s + red[q * NV + threadIdx.x];
-        out[threadIdx.x] = s;
-    }
-    __syncthreads();
 }
 
 // The (walker, tile) work of a flush, enumerated without atomics: every CTA
@@ -140,6 +121,11 @@ __device__ __forceinline__ int flush_scan(const DevLayout& L, const DevState<T>&
     return min(FLUSH_SCAN, L.W - w0);
 }
 
+template <typename T>
+size_t propose_smem(int Kc, bool delayed) {
+    return delayed ? sizeof(SlotSmem<T>) + (size_t)Kc * MAXKK * sizeof(T) : 0;
+}
+
 // ---------------------------------------------------------------------------
 // propose: X = A^{-1} U (delayed: A_0^{-1} U -/+ P (Q^T U)), core, small solve
 // det: Sec. 2.1 Eq. det_R, delayed Sec. 2.3 (R_tau, a_tau equations)
@@ -154,11 +140,12 @@ template <typename T, bool PF, bool DELAYED, bool SKEWM = DELAYED>
 __device__ void propose_walker(const int w, const DevLayout L, const DevState<T> S, const DevOperand U,
                                const DevOperand V, const T* C, T* ratio_out, int* st_out) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
-    T* s_qtu = reinterpret_cast<T*>(dyn_smem);  // Kc x MAXKK (delayed only)
+    // delayed only: the scratch of the slot products, then Q^T U (Kc x MAXKK)
+    SlotSmem<T>& s_slot = *reinterpret_cast<SlotSmem<T>*>(dyn_smem);
+    T* s_qtu = reinterpret_cast<T*>(dyn_smem + sizeof(SlotSmem<T>));
     __shared__ T s_core[MAXKK * MAXKK];
     __shared__ T s_inv[MAXKK * MAXKK];
     __shared__ T s_cinv[MAXKK * MAXKK];
-    __shared__ T s_red[8 * 16];
     __shared__ int s_iu[MAXKK], s_iv[MAXKK];
     __shared__ int s_bad;
     __shared__ T s_pfc;
@@ -227,21 +214,26 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
         return;
     }
 
-    // ---- delayed: Q^T U (cu x kk), the (b_t^T U) / (a_t^T B) factors ----
-    // one-hot columns read row i of Q; dense columns were reduced by k_qtu_dense
+    int dlu[MAXKK], ndu = 0, dlv[MAXKK], ndv = 0;   // dense slots of U and of V
+    for (int a = 0; a < kk; ++a) {
+        if (s_iu[a] < 0) dlu[ndu++] = a;
+        if (s_iv[a] < 0) dlv[ndv++] = a;
+    }
+
+    // ---- delayed: Q^T U (cu x kk), the (b_t^T U) / (a_t^T B) factors: one-hot
+    //      columns read row i of Q ----
     if constexpr (DELAYED) {
-        for (int a = 0; a < kk; ++a) {
-            if (s_iu[a] >= 0) {
+        for (int a = 0; a < kk; ++a)
+            if (s_iu[a] >= 0)
                 for (int c = tid; c < cu; c += PT) s_qtu[c * MAXKK + a] = S.Q[(vo + s_iu[a]) * Kc + c];
-            } else {
-                for (int c = tid; c < cu; c += PT) s_qtu[c * MAXKK + a] = S.QtU[((long long)w * Kc + c) * MAXKK + a];
-            }
-        }
+        if (ndu > 0)
+            slot_dot<T, false>(S.Q + vo * Kc, Kc, cu, n, vec_ptr<T>(U, L, w, 0, n), dlu, ndu, s_slot,
+                               [&](int c, int a, T v) { s_qtu[c * MAXKK + a] = v; });
         __syncthreads();
     }
 
-    // ---- X = A^{-1} U ----
-    // one-hot columns: a contiguous chunk copy; dense columns: axpy over chunks
+    // ---- X = A^{-1} U: one-hot columns are a contiguous chunk copy; the dense
+    //      ones are there already (dense_x_rows, or a double-float pass) ----
     for (int a = 0; a < kk; ++a) {
         T* Xa = X + (long long)a * n;
         if (s_iu[a] >= 0) {
@@ -249,71 +241,20 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
             for (int j = tid; j < n; j += PT) Xa[j] = col[j];
         }
     }
-    {
-        // dense columns, four at a time
-        int dl[MAXKK], nd = 0;
-        for (int a = 0; a < kk; ++a)
-            if (s_iu[a] < 0 && a != U.pre) dl[nd++] = a;
-        if (nd == 1) {
-            // one dense column (the Pfaffian row-and-column move, a rank-1
-            // dense update): each thread walks the columns for its rows with
-            // the loads of eight columns in flight, one accumulator per row
-            // (the same FMA order as the grouped loop below)
-            const T* u0 = vec_ptr<T>(U, L, w, dl[0], n);
-            T* Xa = X + (long long)dl[0] * n;
-            for (int j = tid; j < n; j += PT) {
-                T acc = s_zero(T());
-#pragma unroll 8
-                for (int l = 0; l < n; ++l) acc = s_fma(G[(long long)l * n + j], u0[l], acc);
-                Xa[j] = acc;
-            }
-            nd = 0;
-        }
-        for (int g0 = 0; g0 < nd; g0 += 4) {
-            const int ng = min(4, nd - g0);
-            T acc[4][JPT];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int m = 0; m < JPT; ++m) acc[q][m] = s_zero(T());
-            const T* up[4];
-            for (int q = 0; q < 4; ++q) up[q] = vec_ptr<T>(U, L, w, dl[g0 + min(q, ng - 1)], n);
-            for (int l = 0; l < n; ++l) {
-                const T* col = G + (long long)l * n;
-                T ul[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) ul[q] = up[q][l];
-#pragma unroll
-                for (int m = 0; m < JPT; ++m) {
-                    const int j = tid + m * PT;
-                    if (j < n) {
-                        T g = col[j];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) acc[q][m] = s_fma(g, ul[q], acc[q][m]);
-                    }
-                }
-            }
-            for (int q = 0; q < ng; ++q) {
-                T* Xa = X + (long long)dl[g0 + q] * n;
-#pragma unroll
-                for (int m = 0; m < JPT; ++m) {
-                    const int j = tid + m * PT;
-                    if (j < n) Xa[j] = acc[q][m];
-                }
-            }
-        }
-    }
     __syncthreads();
 
     if constexpr (DELAYED) {
         // X -= P (Q^T U) (det)   or   X += P (Q^T B) (pf)
-        for (int j = tid; j < n; j += PT) {
-            const T* prow = S.P + (vo + j) * Kc;
-            for (int a = 0; a < kk; ++a) {
-                T s = s_zero(T());
-                for (int c = 0; c < cu; ++c) s = s_fma(prow[c], s_qtu[c * MAXKK + a], s);
-                T* Xa = X + (long long)a * n;
-                Xa[j] = PF ? (Xa[j] + s) : (Xa[j] - s);
+        for (int a = 0; a < kk; a += 4) {
+            T* Xa = X + (long long)a * n;
+            const T *P = S.P + vo * Kc, *q = s_qtu + a;
+            if (kk - a > 2) {
+                if (kk - a > 3) slot_correct<T, 4>(P, Kc, cu, n, q, PF, Xa);
+                else slot_correct<T, 3>(P, Kc, cu, n, q, PF, Xa);
+            } else if (kk - a == 2) {
+                slot_correct<T, 2>(P, Kc, cu, n, q, PF, Xa);
+            } else {
+                slot_correct<T, 1>(P, Kc, cu, n, q, PF, Xa);
             }
         }
         __syncthreads();
@@ -332,40 +273,49 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
         }
     }
 
-    // ---- core: R = I + V X (det) or M = C^{-1} + B^T X (pf) ----
-    for (int p = wid; p < kk * kk; p += PT / 32) {
-        const int b = p / kk, a = p % kk;
-        const T* Xa = X + (long long)a * n;
-        T s;
+    // ---- core: R = I + V X (det) or M = C^{-1} + B^T X (pf); a warp takes one
+    //      row of V against up to four columns of X ----
+    const int na4 = (kk + 3) / 4;
+    for (int p = wid; p < kk * na4; p += PT / 32) {
+        const int b = p / na4, a0 = (p - b * na4) * 4, na = min(4, kk - a0);
+        const T* Xa = X + (long long)a0 * n;
+        T s[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[q] = s_zero(T());
+        const int q = spread_index<4>();   // the column this lane holds after the sum
         if (s_iv[b] >= 0) {
-            s = Xa[s_iv[b]];
+            if (q < na) s[0] = Xa[(long long)q * n + s_iv[b]];
         } else {
             const T* vb = vec_ptr<T>(Vop, L, w, b, n);
-            T part = s_zero(T());
-            for (int j = lane; j < n; j += 32) part = s_fma(vb[j], Xa[j], part);
-            s = warp_sum(part);
+            if (na == 1) {
+                for (int j = lane; j < n; j += 32) s[0] = s_fma(vb[j], Xa[j], s[0]);
+                s[0] = warp_sum(s[0]);
+            } else {
+                for (int j = lane; j < n; j += 32) {
+                    const T v = vb[j];
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+                        if (a < na) s[a] = s_fma(v, Xa[(long long)a * n + j], s[a]);
+                }
+                warp_sum_spread<4>(s);
+            }
         }
-        if (lane == 0) {
+        if (spread_owner<4>() && q < na) {
+            const int a = a0 + q;
             T base = PF ? s_cinv[b * MAXKK + a] : make_real<T>(b == a ? 1.0 : 0.0);
-            s_core[b * MAXKK + a] = base + s;
+            s_core[b * MAXKK + a] = base + s[0];
         }
     }
     // ---- det delayed: V P (kk x cu) for the accept's correction ----
     if constexpr (DELAYED && !PF) {
         T* VP = S.VP + (long long)w * MAXKK * Kc;
-        for (int p = wid; p < kk * cu; p += PT / 32) {
-            const int b = p / cu, c = p % cu;
-            T s;
-            if (s_iv[b] >= 0) {
-                s = S.P[(vo + s_iv[b]) * Kc + c];
-            } else {
-                const T* vb = vec_ptr<T>(Vop, L, w, b, n);
-                T part = s_zero(T());
-                for (int j = lane; j < n; j += 32) part = s_fma(vb[j], S.P[(vo + j) * Kc + c], part);
-                s = warp_sum(part);
-            }
-            if (lane == 0) VP[b * Kc + c] = s;
+        for (int e = tid; e < kk * cu; e += PT) {
+            const int b = e / cu, c = e - b * cu;
+            if (s_iv[b] >= 0) VP[b * Kc + c] = S.P[(vo + s_iv[b]) * Kc + c];
         }
+        if (ndv > 0)
+            slot_dot<T, true>(S.P + vo * Kc, Kc, cu, n, vec_ptr<T>(Vop, L, w, 0, n), dlv, ndv, s_slot,
+                              [&](int c, int b, T v) { VP[b * Kc + c] = v; });
     }
     __syncthreads();
 
@@ -443,109 +393,95 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
     }
 }
 
-// X_a = A^{-1} u_a for the one dense column a of a proposal (the Pfaffian
-// row-and-column move B = [x, e_i], a rank-1 dense update), before the
-// propose kernel, which then skips that column.  One CTA per walker; thread t
-// owns rows t + PT r (r < NR) and walks the columns of A^{-1} (contiguous in
-// the rows, so every load is coalesced) with two independent accumulators per
-// row (the column range split in halves) and few registers, so that many
-// CTAs per SM hide the load latency.  DF (real FP64 only): the products in
-// double-float arithmetic on the FP32 pipe (integer-split elements against
-// the split u), so the pass is bound by HBM instead of the FP64 pipe.
-template <typename T, int NR, bool DF>
-__global__ void __launch_bounds__(PT, 4) k_dense_column(DevLayout L, DevState<T> S, DevOperand U, int a) {
-    __shared__ T su[2048];
-    __shared__ float2 suf[DF ? 2048 : 1];
-    const int w = blockIdx.x;
-    const int n = L.nw(w);
-    const T* u = vec_ptr<T>(U, L, w, a, n);
-    for (int l = threadIdx.x; l < n; l += PT) {
-        su[l] = u[l];
-        if constexpr (DF) {
-            float h, lo;
-            split_d((double)u[l], h, lo);
-            suf[l] = make_float2(h, lo);
-        }
-    }
-    __syncthreads();
-    const T* G = S.G + L.mo(w);
-    T* Xa = S.X + L.vo(w) * L.kk + (long long)a * n;
-    const int h = n / 2;
-    if constexpr (DF) {
-        float ah0[NR], al0[NR], ah1[NR], al1[NR];
-#pragma unroll
-        for (int r = 0; r < NR; ++r) ah0[r] = al0[r] = ah1[r] = al1[r] = 0.f;
-#pragma unroll 4
-        for (int l = 0; l < h; ++l) {
-            const double* c0 = reinterpret_cast<const double*>(G) + (long long)l * n;
-            const double* c1 = reinterpret_cast<const double*>(G) + (long long)(l + h) * n;
-            const float2 u0 = suf[l], u1 = suf[l + h];
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int j = threadIdx.x + PT * r;
-                if (j < n) {
-                    float gh, gl;
-                    split_d(c0[j], gh, gl);
-                    df_fma(ah0[r], al0[r], u0.x, u0.y, gh, gl);
-                    split_d(c1[j], gh, gl);
-                    df_fma(ah1[r], al1[r], u1.x, u1.y, gh, gl);
-                }
-            }
-        }
-        if (n & 1) {
-            const double* c = reinterpret_cast<const double*>(G) + (long long)(n - 1) * n;
-            const float2 ul = suf[n - 1];
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int j = threadIdx.x + PT * r;
-                if (j < n) {
-                    float gh, gl;
-                    split_d(c[j], gh, gl);
-                    df_fma(ah0[r], al0[r], ul.x, ul.y, gh, gl);
-                }
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            const int j = threadIdx.x + PT * r;
-            df_add(ah0[r], al0[r], ah1[r], al1[r]);
-            if (j < n) reinterpret_cast<double*>(Xa)[j] = df_to_double(ah0[r], al0[r]);
+// X = A^{-1} U for the dense columns of a proposal, before the propose kernel:
+// one CTA (ordered dtypes: one warp) per walker and XT rows.
+template <typename T, int KBM>
+__global__ void __launch_bounds__(PT) k_dense_x(DevLayout L, DevState<T> S, DevOperand U) {
+    if constexpr (ordered<T>()) {
+        // a warp per tile; for a single dense column a pair of warps
+        constexpr int TPC = PT / 32 / (KBM == 1 ? 2 : 1);
+        const int nt = (L.n_max + XT - 1) / XT, wid = threadIdx.x >> 5;
+        const long long task = (long long)blockIdx.x * TPC + wid % TPC;
+        const int w = (int)min(task / nt, (long long)L.W - 1), j0 = (int)(task % nt) * XT, n = L.nw(w);
+        const bool active = task < (long long)L.W * nt && j0 < n;
+        const T *G = S.G + L.mo(w), *u = vec_ptr<T>(U, L, w, 0, n);
+        T* X = S.X + L.vo(w) * L.kk;
+        if constexpr (KBM == 1) {
+            __shared__ T s_half[TPC][2 * 32];
+            int a = 0;
+            while ((U.mask >> a) & 1u) ++a;
+            dense_x_halves<T>(G, n, j0, u, a, wid / TPC, active && a < L.kv(w), X, s_half[wid % TPC]);
+        } else if (active) {
+            dense_x_rows_warp<T, KBM>(G, n, j0, u, U.mask, L.kv(w), X);
         }
         return;
-    } else {
-        T acc0[NR], acc1[NR];
+    }
+    __shared__ XSmem<T> sm;
+    const int w = blockIdx.x, n = L.nw(w), j0 = blockIdx.y * XT;
+    if (j0 >= n) return;
+    const long long vo = L.vo(w);
+    dense_x_rows<T, KBM>(S.G + L.mo(w), n, j0, vec_ptr<T>(U, L, w, 0, n), U.mask, L.kv(w), S.X + vo * L.kk, sm);
+}
+
+// X_a = A^{-1} u_a for the one dense column a of a proposal with the products
+// in double-float arithmetic on the FP32 pipe (integer-split elements against
+// the split u), so that the pass is bound by HBM instead of the FP64 pipe.
+// One CTA per walker; thread t owns rows t + PT r (r < NR) and walks the
+// columns of A^{-1} (contiguous in the rows, so every load is coalesced) with
+// two independent accumulators per row (the column range split in halves).
+template <int NR>
+__global__ void __launch_bounds__(PT, 4) k_dense_column_df(DevLayout L, DevState<double> S, DevOperand U, int a) {
+    __shared__ float2 suf[2048];
+    const int w = blockIdx.x;
+    const int n = L.nw(w);
+    const double* u = vec_ptr<double>(U, L, w, a, n);
+    for (int l = threadIdx.x; l < n; l += PT) {
+        float h, lo;
+        split_d(u[l], h, lo);
+        suf[l] = make_float2(h, lo);
+    }
+    __syncthreads();
+    const double* G = S.G + L.mo(w);
+    double* Xa = S.X + L.vo(w) * L.kk + (long long)a * n;
+    const int h = n / 2;
+    float ah0[NR], al0[NR], ah1[NR], al1[NR];
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            acc0[r] = s_zero(T());
-            acc1[r] = s_zero(T());
-        }
+    for (int r = 0; r < NR; ++r) ah0[r] = al0[r] = ah1[r] = al1[r] = 0.f;
 #pragma unroll 4
-        for (int l = 0; l < h; ++l) {
-            const T* c0 = G + (long long)l * n;
-            const T* c1 = G + (long long)(l + h) * n;
-            const T u0 = su[l], u1 = su[l + h];
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int j = threadIdx.x + PT * r;
-                if (j < n) {
-                    acc0[r] = s_fma(c0[j], u0, acc0[r]);
-                    acc1[r] = s_fma(c1[j], u1, acc1[r]);
-                }
-            }
-        }
-        if (n & 1) {
-            const T* c = G + (long long)(n - 1) * n;
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int j = threadIdx.x + PT * r;
-                if (j < n) acc0[r] = s_fma(c[j], su[n - 1], acc0[r]);
-            }
-        }
+    for (int l = 0; l < h; ++l) {
+        const double* c0 = G + (long long)l * n;
+        const double* c1 = G + (long long)(l + h) * n;
+        const float2 u0 = suf[l], u1 = suf[l + h];
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const int j = threadIdx.x + PT * r;
-            if (j < n) Xa[j] = acc0[r] + acc1[r];
+            if (j < n) {
+                float gh, gl;
+                split_d(c0[j], gh, gl);
+                df_fma(ah0[r], al0[r], u0.x, u0.y, gh, gl);
+                split_d(c1[j], gh, gl);
+                df_fma(ah1[r], al1[r], u1.x, u1.y, gh, gl);
+            }
         }
+    }
+    if (n & 1) {
+        const double* c = G + (long long)(n - 1) * n;
+        const float2 ul = suf[n - 1];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int j = threadIdx.x + PT * r;
+            if (j < n) {
+                float gh, gl;
+                split_d(c[j], gh, gl);
+                df_fma(ah0[r], al0[r], ul.x, ul.y, gh, gl);
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int j = threadIdx.x + PT * r;
+        df_add(ah0[r], al0[r], ah1[r], al1[r]);
+        if (j < n) Xa[j] = df_to_double(ah0[r], al0[r]);
     }
 }
 
@@ -636,36 +572,6 @@ __global__ void __launch_bounds__(PT) k_propose(DevLayout L, DevState<T> S, DevO
     propose_walker<T, PF, DELAYED, PF>(blockIdx.x, L, S, U, V, C, ratio_out, st_out);
 }
 
-// Q^T U for the dense U columns of the delayed propose, one CTA per walker
-// and column: QtU[w][c][a] = sum_j Q[j][c] u_a[j].  Runs before k_propose.
-template <typename T>
-__global__ void __launch_bounds__(PT) k_qtu_dense(DevLayout L, DevState<T> S, DevOperand U) {
-    __shared__ T s_red[8 * 16];
-    __shared__ T s_out[16];
-    const int w = blockIdx.x, a = blockIdx.y;
-    const int n = L.nw(w), kk = L.kv(w);
-    if (a >= kk || ((U.mask >> a) & 1u)) return;
-    const int Kc = L.Kc, cu = S.tau[w] * kk;
-    const long long vo = L.vo(w);
-    const T* u = vec_ptr<T>(U, L, w, a, n);
-    for (int c0 = 0; c0 < cu; c0 += 16) {
-        T part[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) part[q] = s_zero(T());
-        for (int j = threadIdx.x; j < n; j += PT) {
-            const T* qrow = S.Q + (vo + j) * Kc + c0;
-            T uj = u[j];
-#pragma unroll
-            for (int q = 0; q < 16; ++q)
-                if (c0 + q < cu) part[q] = s_fma(qrow[q], uj, part[q]);
-        }
-        block_reduce_vec<T, 16>(part, s_red, s_out);
-        if (threadIdx.x < 16 && c0 + threadIdx.x < cu)
-            S.QtU[((long long)w * Kc + c0 + threadIdx.x) * MAXKK + a] = s_out[threadIdx.x];
-        __syncthreads();
-    }
-}
-
 // ---------------------------------------------------------------------------
 // accept pass: one warp per chunk l (column l of A^{-1})
 //   y_b = V_b . chunk_l (dense) or chunk_l[i_b] (one-hot)      [= (V A^{-1})_{bl}]
@@ -673,7 +579,7 @@ __global__ void __launch_bounds__(PT) k_qtu_dense(DevLayout L, DevState<T> S, De
 //            generic Woodbury A^{-1} - X M^{-1} (B^T A^{-1}))
 //   delayed: y -= (V P) Q[l,:]^T ; Q[l, tau] = (R^{-1} y)^T     (b_tau equation)
 // ---------------------------------------------------------------------------
-template <typename T, bool DELAYED, int NPL, int KKS>
+template <typename T, int NPL, int KKS>
 __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> S, const DevOperand V,
                             const uint8_t* mask) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
@@ -693,9 +599,6 @@ __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> 
     const bool use_smem = it.w != 0;
     __shared__ T sR[MAXKK * MAXKK];
     __shared__ int siv[MAXKK];
-    __shared__ T sVP[MAXKK * 64];
-    const int Kc = L.Kc;
-    const int cu = DELAYED ? S.tau[w] * kk : 0;
 
     const T* Xg = S.X + vo * L.kk;
     const T* sX = Xg;
@@ -712,11 +615,6 @@ __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> 
     }
     if (threadIdx.x < kk) siv[threadIdx.x] = ((V.mask >> threadIdx.x) & 1u) ? V.idx[(long long)w * V.slots + threadIdx.x] : -1;
     for (int e = threadIdx.x; e < MAXKK * MAXKK; e += PT) sR[e] = S.Rinv[(long long)w * MAXKK * MAXKK + e];
-    if constexpr (DELAYED)
-        for (int e = threadIdx.x; e < kk * cu; e += PT) {
-            const int b = e / cu, c = e % cu;
-            sVP[b * 64 + c] = S.VP[(long long)w * MAXKK * Kc + b * Kc + c];
-        }
     __syncthreads();
 
     T* Gw = S.G + L.mo(w);
@@ -743,13 +641,6 @@ __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> 
                 }
                 y[b] = warp_sum(part);
             }
-            if constexpr (DELAYED) {
-                // lanes split the slot sum (c = lane, lane + 32) and reduce
-                const T* qrow = S.Q + (vo + l) * Kc;
-                T corr = s_zero(T());
-                for (int c = lane; c < cu; c += 32) corr = s_fma(sVP[b * 64 + c], qrow[c], corr);
-                y[b] = y[b] - warp_sum(corr);
-            }
         }
         T z[KKS > 0 ? KKS : MAXKK];
 #pragma unroll
@@ -759,37 +650,80 @@ __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> 
             for (int b = 0; b < (KKS > 0 ? KKS : kk); ++b) s = s_fma(sR[a * MAXKK + b], y[b], s);
             z[a] = s;
         }
-        if constexpr (!DELAYED) {
 #pragma unroll
-            for (int m = 0; m < NPL; ++m) {
-                const int j = lane + 32 * m;
-                if (j < n) {
-                    T d = v[m];
+        for (int m = 0; m < NPL; ++m) {
+            const int j = lane + 32 * m;
+            if (j < n) {
+                T d = v[m];
 #pragma unroll
-                    for (int a = 0; a < (KKS > 0 ? KKS : kk); ++a) d = s_fms(sX[(size_t)a * n + j], z[a], d);
-                    col[j] = d;
-                }
-            }
-        } else {
-            if (lane < kk) {
-                T zz = z[0];
-#pragma unroll
-                for (int a = 1; a < (KKS > 0 ? KKS : kk); ++a)
-                    if (a == lane) zz = z[a];
-                const long long off = (vo + l) * Kc + cu + lane;
-                S.Q[off] = zz;
-                if constexpr (!traits<T>::is_complex && sizeof(T) == 8) {
-                    if (S.P32h) store_split(S, 1, (vo + l) * L.Kc32 + cu + lane, (double)zz);
-                }
+                for (int a = 0; a < (KKS > 0 ? KKS : kk); ++a) d = s_fms(sX[(size_t)a * n + j], z[a], d);
+                col[j] = d;
             }
         }
     }
 }
 
-template <typename T, bool DELAYED, int NPL, int KKS>
+template <typename T, int NPL, int KKS>
 __global__ void __launch_bounds__(PT, 2) k_accept(DevLayout L, DevState<T> S, DevOperand V, const uint8_t* mask,
                                                    const int4* items) {
-    accept_item<T, DELAYED, NPL, KKS>(items[blockIdx.x], L, S, V, mask);
+    accept_item<T, NPL, KKS>(items[blockIdx.x], L, S, V, mask);
+}
+
+// The delayed accept of rank k for the columns of one work item: y = V A_0^{-1}
+// of the columns (dense_y_cols), less the slots' part, times R^{-1}.
+template <typename T>
+struct DelayedSmem {
+    YSmem<T> y;
+    T R[MAXKK * MAXKK];
+    T VP[MAXKK * 64];
+    int iv[MAXKK];
+};
+
+template <typename T, int KBM>
+__device__ void accept_delayed_item(const int4 it, const DevLayout L, const DevState<T> S, const DevOperand V,
+                                    const uint8_t* mask) {
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    DelayedSmem<T>& sm = *reinterpret_cast<DelayedSmem<T>*>(dyn_smem);
+    const int w = it.x;
+    if (!LRU_DEBUG_OK(w >= 0 && w < L.W, S.err)) return;
+    if (mask && !mask[w]) return;
+    if (S.pst[w] != 0) return;
+    const int n = L.nw(w), kk = L.kv(w);
+    if (!LRU_DEBUG_OK(it.y >= 0 && it.y <= it.z && it.z <= n, S.err)) return;
+    const long long vo = L.vo(w);
+    const int Kc = L.Kc, cu = S.tau[w] * kk;
+    if (threadIdx.x < kk) sm.iv[threadIdx.x] = ((V.mask >> threadIdx.x) & 1u) ? V.idx[(long long)w * V.slots + threadIdx.x] : -1;
+    for (int e = threadIdx.x; e < kk * kk; e += PT) {
+        const int a = e / kk, b = e - a * kk;
+        sm.R[a * MAXKK + b] = S.Rinv[(long long)w * MAXKK * MAXKK + a * MAXKK + b];
+    }
+    for (int e = threadIdx.x; e < kk * cu; e += PT) {
+        const int b = e / cu, c = e - b * cu;
+        sm.VP[b * 64 + c] = S.VP[(long long)w * MAXKK * Kc + b * Kc + c];
+    }
+    __syncthreads();
+    const T* Gw = S.G + L.mo(w);
+    const T* Vw = (V.dense != nullptr) ? vec_ptr<T>(V, L, w, 0, n) : nullptr;
+    for (int l0 = it.y; l0 < it.z; l0 += YC) {
+        const int nc = min(YC, it.z - l0);
+        dense_y_cols<T, KBM>(Gw, n, l0, nc, Vw, sm.iv, kk, sm.y);
+        if (cu > 0) slot_correct_y<T>(S.Q + vo * Kc, Kc, cu, l0, nc, sm.VP, kk, sm.y);
+        for (int e = threadIdx.x; e < kk * nc; e += PT) {
+            const int c = e / kk, a = e - c * kk;
+            T z = s_zero(T());
+            for (int b = 0; b < kk; ++b) z = s_fma(sm.R[a * MAXKK + b], sm.y.y[b][c], z);
+            S.Q[(vo + l0 + c) * Kc + cu + a] = z;
+            if constexpr (!traits<T>::is_complex && sizeof(T) == 8) {
+                if (S.P32h) store_split(S, 1, (vo + l0 + c) * L.Kc32 + cu + a, (double)z);
+            }
+        }
+    }
+}
+
+template <typename T, int KBM>
+__global__ void __launch_bounds__(PT, 2) k_accept_delayed_cols(DevLayout L, DevState<T> S, DevOperand V,
+                                                                const uint8_t* mask, const int4* items) {
+    accept_delayed_item<T, KBM>(items[blockIdx.x], L, S, V, mask);
 }
 
 // Plain Pfaffian accept in skew form (Eq. pf_inv with (A^{-1})^T = -A^{-1}):
@@ -1421,14 +1355,16 @@ constexpr long long STEP_WAIT_POLLS = 1ll << 24;   // >= 1 s of polling
 // ---------------------------------------------------------------------------
 // Persistent fused step for walkers of uneven n and k: one launch of a fixed
 // grid that pulls work from a device queue,
-//   items [0, W)                  : propose walker order[i] (largest n^2 k
-//                                   first), then the accept decision (mask,
-//                                   or Metropolis |r|^2 >= u)
-//   items [W, W + nacc)           : accept items (walker, chunk range),
+//   nx items                      : X = A^{-1} U of the dense columns, XT rows of
+//                                   a walker each (largest walkers first)
+//   W items                       : the rest of the propose of walker order[i]
+//                                   (largest n^2 k first), then the accept
+//                                   decision (mask, or Metropolis |r|^2 >= u)
+//   nacc items                    : accept items (walker, chunk range),
 //                                   largest first; the last one of a walker
 //                                   commits log|value|, the sign (and, in the
 //                                   delayed form, tau += 1)
-//   items [W + nacc, + nflush)    : delayed form only: flush strips (walker,
+//   nflush items                  : delayed form only: flush strips (walker,
 //                                   32 columns of A_0^{-1}); a strip waits for
 //                                   its walker's commit and, if tau reached K,
 //                                   folds the slots in (Eq. delayed_Ainv /
@@ -1451,84 +1387,94 @@ __device__ __forceinline__ void commit_walker(const DevState<T>& S, int w, bool 
     S.pst[w] = 4;
 }
 
-// Q^T u_a of the dense columns a of U (the (b_t^T U) / (B^T a_t) factors of
-// the delayed propose) for walker w, by the whole CTA (k_qtu_dense in one block)
-template <typename T>
-__device__ void qtu_block(int w, const DevLayout& L, const DevState<T>& S, const DevOperand& U) {
-    __shared__ T s_red[8 * 16];
-    __shared__ T s_out[16];
-    const int n = L.nw(w), kk = L.kv(w);
-    const int Kc = L.Kc, cu = S.tau[w] * kk;
-    const long long vo = L.vo(w);
-    for (int a = 0; a < kk; ++a) {
-        if ((U.mask >> a) & 1u) continue;
-        const T* u = vec_ptr<T>(U, L, w, a, n);
-        for (int c0 = 0; c0 < cu; c0 += 16) {
-            T part[16];
-#pragma unroll
-            for (int q = 0; q < 16; ++q) part[q] = s_zero(T());
-            for (int j = threadIdx.x; j < n; j += PT) {
-                const T* qrow = S.Q + (vo + j) * Kc + c0;
-                const T uj = u[j];
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    if (c0 + q < cu) part[q] = s_fma(qrow[q], uj, part[q]);
-            }
-            block_reduce_vec<T, 16>(part, s_red, s_out);
-            if (threadIdx.x < 16 && c0 + threadIdx.x < cu)
-                S.QtU[((long long)w * Kc + c0 + threadIdx.x) * MAXKK + a] = s_out[threadIdx.x];
-            __syncthreads();
-        }
-    }
-    __syncthreads();
-}
-
 constexpr int STEP_FLUSH_CH = 16;   // slot columns per chunk of a flush tile inside the step
 template <typename T>
 constexpr size_t step_flush_smem() {
     return (size_t)(2 * 32 * (STEP_FLUSH_CH + 1) + 32 * 33) * sizeof(T);
 }
 
-template <typename T, bool PF, bool DEL, int NPL, int KKS>
-__global__ void __launch_bounds__(PT) k_step(DevLayout L, DevState<T> S, DevOperand U, DevOperand V, const T* C,
-                                              T* ratio_out, int* st_out, StepCtl ctl) {
+template <typename T, bool PF, bool DEL, int NPL, int KKS, int KBM>
+__global__ void __launch_bounds__(PT, 2) k_step(DevLayout L, DevState<T> S, DevOperand U, DevOperand V, const T* C,
+                                                 T* ratio_out, int* st_out, StepCtl ctl) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     __shared__ int s_item, s_ok, s_tau;
+    const int nx = ordered<T>() ? (ctl.n_x_items + PT / 32 - 1) / (PT / 32) : ctl.n_x_items;
     const int nacc = (ctl.do_accept && !(PF && DEL)) ? ctl.nacc : 0;
     const int nfl = (ctl.do_accept && DEL) ? ctl.nflush : 0;
-    const int total = L.W + nacc + nfl;
+    const int total = nx + L.W + nacc + nfl;
+    if (threadIdx.x == 0) s_item = atomicAdd(ctl.counter, 1);
     for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(ctl.counter, 1);
         __syncthreads();
-        const int item = s_item;
+        int item = s_item;
         __syncthreads();
         if (item >= total) break;
-        if (item < L.W) {
-            const int w = ctl.order[item];
-            if (!LRU_DEBUG_OK(w >= 0 && w < L.W, S.err)) continue;
-            if constexpr (DEL) qtu_block<T>(w, L, S, U);
-            propose_walker<T, PF, DEL, DEL>(w, L, S, U, V, C, ratio_out, st_out);
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                bool acc = ctl.do_accept && S.pst[w] == 0;
-                if (acc && ctl.mask) acc = ctl.mask[w] != 0;
-                if (acc && ctl.u) acc = (double)s_abs2(S.ratio[w]) >= ctl.u[w];
-                ctl.acc[w] = acc ? 1 : 0;
-                if (PF && DEL) {
-                    // the slots are already written: commit here
-                    if (acc) commit_walker(S, w, true);
-                    __threadfence();
-                    st_release_gpu(&ctl.fin[w], 1);
+        // the next item is drawn while this one is worked on; a CTA works its
+        // items in the order drawn, so the waits below still end
+        int next = 0;
+        if (threadIdx.x == 0) next = atomicAdd(ctl.counter, 1);
+        if (item < nx) {
+            if constexpr (ordered<T>()) {
+                // a warp per X tile
+                const int t = item * (PT / 32) + ((int)threadIdx.x >> 5);
+                if (t < ctl.n_x_items) {
+                    const int2 xi = ctl.x_items[t];
+                    const int w = xi.x, n = L.nw(w);
+                    dense_x_rows_warp<T, KBM>(S.G + L.mo(w), n, XT * xi.y, vec_ptr<T>(U, L, w, 0, n), U.mask,
+                                                     L.kv(w), S.X + L.vo(w) * L.kk);
+                    __syncwarp();
+                    if ((threadIdx.x & 31) == 0) {
+                        __threadfence();
+                        atomicAdd(&ctl.x_done[w], 1);
+                    }
                 }
-                __threadfence();
-                st_release_gpu(&ctl.prop_done[w], 1);
+            } else {
+                const int2 xi = ctl.x_items[item];
+                const int w = xi.x, n = L.nw(w);
+                if (LRU_DEBUG_OK(w >= 0 && w < L.W && xi.y >= 0 && XT * xi.y < n, S.err)) {
+                    dense_x_rows<T, KBM>(S.G + L.mo(w), n, XT * xi.y, vec_ptr<T>(U, L, w, 0, n), U.mask, L.kv(w),
+                                         S.X + L.vo(w) * L.kk, *reinterpret_cast<XSmem<T>*>(dyn_smem));
+                    __syncthreads();
+                    if (threadIdx.x == 0) {
+                        __threadfence();
+                        atomicAdd(&ctl.x_done[w], 1);
+                    }
+                }
             }
-        } else if (item < L.W + nacc) {
-            const int4 it = ctl.acc_items[item - L.W];
+        } else if ((item -= nx) < L.W) {
+            const int w = ctl.order[item];
+            if (LRU_DEBUG_OK(w >= 0 && w < L.W, S.err)) {
+                if (threadIdx.x == 0)
+                    s_ok = (nx == 0 || bounded_acquire_wait(&ctl.x_done[w], (L.nw(w) + XT - 1) / XT, STEP_WAIT_POLLS,
+                                                            S.err)) ? 1 : 0;
+                __syncthreads();
+                if (s_ok) {
+                    propose_walker<T, PF, DEL, DEL>(w, L, S, U, V, C, ratio_out, st_out);
+                    __syncthreads();
+                    if (threadIdx.x == 0) {
+                        bool acc = ctl.do_accept && S.pst[w] == 0;
+                        if (acc && ctl.mask) acc = ctl.mask[w] != 0;
+                        if (acc && ctl.u) acc = (double)s_abs2(S.ratio[w]) >= ctl.u[w];
+                        ctl.acc[w] = acc ? 1 : 0;
+                        if (PF && DEL) {
+                            // the slots are already written: commit here
+                            if (acc) commit_walker(S, w, true);
+                            __threadfence();
+                            st_release_gpu(&ctl.fin[w], 1);
+                        }
+                        __threadfence();
+                        st_release_gpu(&ctl.prop_done[w], 1);
+                    }
+                }
+            }
+        } else if ((item -= L.W) < nacc) {
+            const int4 it = ctl.acc_items[item];
             const int w = it.x;
             if (threadIdx.x == 0) s_ok = bounded_acquire_wait(&ctl.prop_done[w], 1, STEP_WAIT_POLLS, S.err) ? 1 : 0;
             __syncthreads();
-            if (s_ok && ctl.acc[w]) accept_item<T, DEL, NPL, KKS>(it, L, S, V, nullptr);
+            if (s_ok && ctl.acc[w]) {
+                if constexpr (DEL) accept_delayed_item<T, KBM>(it, L, S, V, nullptr);
+                else accept_item<T, NPL, KKS>(it, L, S, V, nullptr);
+            }
             __syncthreads();
             if (threadIdx.x == 0 && s_ok) {
                 __threadfence();
@@ -1540,31 +1486,33 @@ __global__ void __launch_bounds__(PT) k_step(DevLayout L, DevState<T> S, DevOper
                 }
             }
         } else {
-            const int2 fi = ctl.flush_items[item - L.W - nacc];
+            const int2 fi = ctl.flush_items[item - nacc];
             const int w = fi.x, tL = fi.y;
-            if (!LRU_DEBUG_OK(w >= 0 && w < L.W && tL >= 0 && 32 * tL < L.nw(w), S.err)) continue;
-            if (threadIdx.x == 0) {
-                s_ok = bounded_acquire_wait(&ctl.fin[w], 1, STEP_WAIT_POLLS, S.err) ? 1 : 0;
-                s_tau = s_ok ? *(volatile const int*)&S.tau[w] : 0;
-            }
-            __syncthreads();
-            const int tau = s_tau;
-            if (s_ok && tau >= L.K) {
-                T* sP = reinterpret_cast<T*>(dyn_smem);
-                T* sQ = sP + 32 * (STEP_FLUSH_CH + 1);
-                T* sT = sQ + 32 * (STEP_FLUSH_CH + 1);
-                const int nt = (L.nw(w) + 31) / 32;
-                const int tJ_end = PF ? tL + 1 : nt;
-                for (int tJ = 0; tJ < tJ_end; ++tJ)
-                    flush_native_tile<T, PF, STEP_FLUSH_CH>(L, S, w, tau, tJ, tL, sP, sQ, sT);
-            }
-            __syncthreads();
-            if (threadIdx.x == 0 && s_ok) {
-                __threadfence();
-                const int done = atomicAdd(&ctl.flush_done[w], 1) + 1;
-                if (done == ctl.nflush_w[w] && tau >= L.K) S.tau[w] = 0;
+            if (LRU_DEBUG_OK(w >= 0 && w < L.W && tL >= 0 && 32 * tL < L.nw(w), S.err)) {
+                if (threadIdx.x == 0) {
+                    s_ok = bounded_acquire_wait(&ctl.fin[w], 1, STEP_WAIT_POLLS, S.err) ? 1 : 0;
+                    s_tau = s_ok ? *(volatile const int*)&S.tau[w] : 0;
+                }
+                __syncthreads();
+                const int tau = s_tau;
+                if (s_ok && tau >= L.K) {
+                    T* sP = reinterpret_cast<T*>(dyn_smem);
+                    T* sQ = sP + 32 * (STEP_FLUSH_CH + 1);
+                    T* sT = sQ + 32 * (STEP_FLUSH_CH + 1);
+                    const int nt = (L.nw(w) + 31) / 32;
+                    const int tJ_end = PF ? tL + 1 : nt;
+                    for (int tJ = 0; tJ < tJ_end; ++tJ)
+                        flush_native_tile<T, PF, STEP_FLUSH_CH>(L, S, w, tau, tJ, tL, sP, sQ, sT);
+                }
+                __syncthreads();
+                if (threadIdx.x == 0 && s_ok) {
+                    __threadfence();
+                    const int done = atomicAdd(&ctl.flush_done[w], 1) + 1;
+                    if (done == ctl.nflush_w[w] && tau >= L.K) S.tau[w] = 0;
+                }
             }
         }
+        if (threadIdx.x == 0) s_item = next;
     }
 }
 
@@ -1575,30 +1523,39 @@ void launch_step(bool pf, bool delayed, const DevLayout& L, const DevState<T>& S
     const int nmax = L.n_max;
     int npl = 1;
     while (32 * npl < nmax) npl *= 2;
-    size_t dyn = (size_t)2 * L.kk * nmax * sizeof(T);
-    if (dyn > 160 * 1024) dyn = 0;   // accept items then carry use_smem = 0
-    if (delayed) {
-        dyn = std::max(dyn, (size_t)L.Kc * MAXKK * sizeof(T));   // Q^T U in the propose
-        dyn = std::max(dyn, step_flush_smem<T>());
-    }
     const bool rank1 = L.kk == 1 && L.kvec == nullptr;
-#define LRU_STEP_K(PFV, DELV, N)                                                                          \
+    size_t dyn = sizeof(XSmem<T>);
+#define LRU_STEP_GO(...)                                                                                  \
     {                                                                                                     \
-        auto k = rank1 ? k_step<T, PFV, DELV, N, 1> : k_step<T, PFV, DELV, N, 0>;                         \
+        auto k = __VA_ARGS__;                                                                             \
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);                 \
         k<<<grid, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out, ctl);                                  \
     }
+    if (delayed) {
+        dyn = std::max(dyn, propose_smem<T>(L.Kc, true));
+        dyn = std::max(dyn, step_flush_smem<T>());
+        dyn = std::max(dyn, sizeof(DelayedSmem<T>));
+        if (pf) {
+            if (L.kk <= 2) LRU_STEP_GO(k_step<T, true, true, 1, 0, 2>)
+            else LRU_STEP_GO(k_step<T, true, true, 1, 0, kb_max<T>()>)
+        } else {
+            if (L.kk == 1) LRU_STEP_GO(k_step<T, false, true, 1, 0, 1>)
+            else LRU_STEP_GO(k_step<T, false, true, 1, 0, kb_max<T>()>)
+        }
+        return;
+    }
+    size_t acc = (size_t)2 * L.kk * nmax * sizeof(T);
+    if (acc > 160 * 1024) acc = 0;   // accept items then carry use_smem = 0
+    dyn = std::max(dyn, acc);
 #define LRU_STEP(N)                                                                                       \
     case N:                                                                                               \
-        if (pf) {                                                                                         \
-            if (delayed) LRU_STEP_K(true, true, N) else LRU_STEP_K(true, false, N)                        \
-        } else {                                                                                          \
-            if (delayed) LRU_STEP_K(false, true, N) else LRU_STEP_K(false, false, N)                      \
-        }                                                                                                 \
+        if (pf) LRU_STEP_GO(k_step<T, true, false, N, 0, kb_max<T>()>)                                              \
+        else if (rank1) LRU_STEP_GO(k_step<T, false, false, N, 1, 1>)                                     \
+        else LRU_STEP_GO(k_step<T, false, false, N, 0, kb_max<T>()>)                                                \
         break;
     switch (npl) { LRU_STEP(1) LRU_STEP(2) LRU_STEP(4) LRU_STEP(8) LRU_STEP(16) LRU_STEP(32) LRU_STEP(64) default: break; }
 #undef LRU_STEP
-#undef LRU_STEP_K
+#undef LRU_STEP_GO
 }
 #endif  // !LRU_NO_STEP
 
@@ -1802,22 +1759,20 @@ __global__ void k_commit_moves(int W, int n, int k, int* occ, const int* slot, c
 // ---------------------------------------------------------------------------
 template <typename T>
 void launch_propose(bool pf, bool delayed, bool df, const DevLayout& L, const DevState<T>& S,
-                    const DevOperand& U_in, const DevOperand& V, const T* C, T* ratio_out, int* st_out,
+                    const DevOperand& U, const DevOperand& V, const T* C, T* ratio_out, int* st_out,
                     cudaStream_t st) {
-    const size_t dyn = delayed ? (size_t)L.Kc * MAXKK * sizeof(T) : 0;
+    const size_t dyn = propose_smem<T>(L.Kc, delayed);
     const unsigned all = (L.kk >= 32) ? 0xffffffffu : ((1u << L.kk) - 1u);
-    DevOperand U = U_in;
-    if (delayed && (U.mask & all) != all)
-        k_qtu_dense<T><<<dim3(L.W, L.kk), PT, 0, st>>>(L, S, U);
-    // exactly one dense column: its pass over A^{-1} runs as its own kernel
+    // the dense columns' pass over A^{-1} runs as its own kernel
     const unsigned dense = ~U.mask & all;
-    if (dense != 0 && (dense & (dense - 1)) == 0) {
-        int a = 0;
-        while (!((dense >> a) & 1u)) ++a;
-        const int nr = (L.n_max + PT - 1) / PT;
-        bool launched = false;
-        if constexpr (std::is_same<T, double>::value) {
-            if (df && pf && L.n_uni > 0 && (L.n_uni % 2) == 0 && L.n_uni <= 2048) {
+    const bool one = dense != 0 && (dense & (dense - 1)) == 0;
+    bool launched = dense == 0;
+    if constexpr (std::is_same<T, double>::value) {
+        if (df && one) {
+            int a = 0;
+            while (!((dense >> a) & 1u)) ++a;
+            const int nr = (L.n_max + PT - 1) / PT;
+            if (pf && L.n_uni > 0 && (L.n_uni % 2) == 0 && L.n_uni <= 2048) {
                 // Pfaffian: A^{-1} is exactly skew, so X = -(u^T A^{-1})^T streams
                 // contiguous rows, one warp each
                 dim3 grid(L.W, (L.n_max + DF_CPB - 1) / DF_CPB);
@@ -1828,22 +1783,23 @@ void launch_propose(bool pf, bool delayed, bool df, const DevLayout& L, const De
                     LRU_PF_WDF(4) LRU_PF_WDF(8) LRU_PF_WDF(16) LRU_PF_WDF(32) default: break;
                 }
 #undef LRU_PF_WDF
-                launched = true;
-            } else if (df) {
-                if (nr <= 1) k_dense_column<T, 1, true><<<L.W, PT, 0, st>>>(L, S, U, a);
-                else if (nr <= 2) k_dense_column<T, 2, true><<<L.W, PT, 0, st>>>(L, S, U, a);
-                else if (nr <= 4) k_dense_column<T, 4, true><<<L.W, PT, 0, st>>>(L, S, U, a);
-                else k_dense_column<T, 8, true><<<L.W, PT, 0, st>>>(L, S, U, a);
-                launched = true;
+            } else {
+                if (nr <= 1) k_dense_column_df<1><<<L.W, PT, 0, st>>>(L, S, U, a);
+                else if (nr <= 2) k_dense_column_df<2><<<L.W, PT, 0, st>>>(L, S, U, a);
+                else if (nr <= 4) k_dense_column_df<4><<<L.W, PT, 0, st>>>(L, S, U, a);
+                else k_dense_column_df<8><<<L.W, PT, 0, st>>>(L, S, U, a);
             }
+            launched = true;
         }
-        if (!launched) {
-            if (nr <= 1) k_dense_column<T, 1, false><<<L.W, PT, 0, st>>>(L, S, U, a);
-            else if (nr <= 2) k_dense_column<T, 2, false><<<L.W, PT, 0, st>>>(L, S, U, a);
-            else if (nr <= 4) k_dense_column<T, 4, false><<<L.W, PT, 0, st>>>(L, S, U, a);
-            else k_dense_column<T, 8, false><<<L.W, PT, 0, st>>>(L, S, U, a);
-        }
-        U.pre = a;
+    }
+    if (!launched) {
+        const int nt = (L.n_max + XT - 1) / XT;
+        const int nd = __builtin_popcount(dense), tpc = nd == 1 ? PT / 64 : PT / 32;
+        const dim3 grid = ordered<T>() ? dim3((unsigned)(((long long)L.W * nt + tpc - 1) / tpc)) : dim3(L.W, nt);
+        if (nd == 1) k_dense_x<T, 1><<<grid, PT, 0, st>>>(L, S, U);
+        else if (nd == 2) k_dense_x<T, 2><<<grid, PT, 0, st>>>(L, S, U);
+        else if (nd <= 4) k_dense_x<T, 4><<<grid, PT, 0, st>>>(L, S, U);
+        else k_dense_x<T, kb_max<T>()><<<grid, PT, 0, st>>>(L, S, U);
     }
     if (!pf && !delayed) k_propose<T, false, false><<<L.W, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out);
     if (!pf && delayed) {
@@ -1857,21 +1813,16 @@ void launch_propose(bool pf, bool delayed, bool df, const DevLayout& L, const De
     }
 }
 
-template <typename T, bool DELAYED>
-static void accept_npl(int npl, const DevLayout& L, const DevState<T>& S, const DevOperand& V,
-                       const uint8_t* mask, const int* items, int nitems, size_t dyn, cudaStream_t st) {
-    const int4* it = reinterpret_cast<const int4*>(items);
+template <typename T>
+static void accept_plain(int npl, const DevLayout& L, const DevState<T>& S, const DevOperand& V, const uint8_t* mask,
+                         const int4* it, int nitems, size_t dyn, cudaStream_t st) {
     const bool rank1 = L.kk == 1 && L.kvec == nullptr;
 #define LRU_ACC(N)                                                                                          \
-    case N:                                                                                                 \
-        if (rank1) {                                                                                        \
-            cudaFuncSetAttribute(k_accept<T, DELAYED, N, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); \
-            k_accept<T, DELAYED, N, 1><<<nitems, PT, dyn, st>>>(L, S, V, mask, it);                          \
-        } else {                                                                                            \
-            cudaFuncSetAttribute(k_accept<T, DELAYED, N, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn); \
-            k_accept<T, DELAYED, N, 0><<<nitems, PT, dyn, st>>>(L, S, V, mask, it);                          \
-        }                                                                                                   \
-        break;
+    case N: {                                                                                               \
+        auto k = rank1 ? k_accept<T, N, 1> : k_accept<T, N, 0>;                                             \
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);                     \
+        k<<<nitems, PT, dyn, st>>>(L, S, V, mask, it);                                                      \
+    } break;
     switch (npl) {
         LRU_ACC(1) LRU_ACC(2) LRU_ACC(4) LRU_ACC(8) LRU_ACC(16) LRU_ACC(32) LRU_ACC(64)
         default: break;
@@ -1927,8 +1878,17 @@ void launch_accept(bool pf, bool delayed, bool df, const DevLayout& L, const Dev
             done = true;
         }
         if (!done) {
-            if (delayed) accept_npl<T, true>(npl, L, S, V, mask, items, nitems, dyn, st);
-            else accept_npl<T, false>(npl, L, S, V, mask, items, nitems, dyn, st);
+            const int4* it = reinterpret_cast<const int4*>(items);
+            if (!delayed) {
+                accept_plain<T>(npl, L, S, V, mask, it, nitems, dyn, st);
+            } else {
+                auto kern = L.kk == 1 ? k_accept_delayed_cols<T, 1>
+                                      : (L.kk == 2 ? k_accept_delayed_cols<T, 2>
+                                                   : (L.kk <= 4 ? k_accept_delayed_cols<T, 4> : k_accept_delayed_cols<T, kb_max<T>()>));
+                const int ds = (int)sizeof(DelayedSmem<T>);
+                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ds);
+                kern<<<nitems, PT, ds, st>>>(L, S, V, mask, it);
+            }
         }
     }
     k_commit<T><<<(L.W + 255) / 256, 256, 0, st>>>(L, S, mask, delayed);

@@ -74,10 +74,12 @@ struct lru_ctx {
     int* d_order = nullptr;
     int* d_sitems = nullptr;
     int* d_nacc_w = nullptr;
-    int* d_ctl = nullptr;        // counter, prop_done[W], items_done[W], fin[W], flush_done[W]
+    int* d_ctl = nullptr;        // counter, prop_done[W], items_done[W], fin[W], flush_done[W], x_done[W]
     int* d_fitems = nullptr;     // delayed: flush strips (walker, 32-column block)
     int* d_nflush_w = nullptr;
     int nflush = 0;
+    int* d_xitems = nullptr;     // X tiles of the dense columns (walker, row block)
+    int nx = 0;
     uint8_t* d_acc = nullptr;
     int* d_never = nullptr;      // a flag no kernel writes (bounded-wait self-test)
     bool items_smem = true;
@@ -86,7 +88,7 @@ struct lru_ctx {
     int* tau = nullptr;
     double* logabs = nullptr;
     void* sgn = nullptr;
-    void *X = nullptr, *Rinv = nullptr, *ratio = nullptr, *VP = nullptr, *QtU = nullptr;
+    void *X = nullptr, *Rinv = nullptr, *ratio = nullptr, *VP = nullptr;
     int* pst = nullptr;
     int* err = nullptr;
     // refresh workspace (allocated on first use)
@@ -107,8 +109,6 @@ struct lru_ctx {
     void* ozM = nullptr;         // fresh inverses when the drift is asked for
     size_t ozM_bytes = 0;
     bool oz_ok = false;          // the tensor-core refresh applies to this handle
-    // adjoint workspace (allocated on first use)
-    void* bws = nullptr;
     int n_sm = 148;
     // debug build: offsets of the guard zones between the regions of the allocation
     std::vector<size_t> canaries;
@@ -148,7 +148,6 @@ struct lru_ctx {
         S.ratio = (T*)ratio;
         S.pst = pst;
         S.VP = (T*)VP;
-        S.QtU = (T*)QtU;
         S.err = err;
         return S;
     }
@@ -352,6 +351,14 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
             nflush_w[w] = nt;
         }
     h->nflush = (int)fitems.size() / 2;
+    // X tiles of the persistent step, largest walkers first
+    std::vector<int> xitems;
+    for (int w : order)
+        for (int t = 0; t * STEP_X_ROWS < h->n_h[w]; ++t) {
+            xitems.push_back(w);
+            xitems.push_back(t);
+        }
+    h->nx = (int)xitems.size() / 2;
 
     // one allocation: persistent state first, then scratch and metadata
     const bool tc = delayed && cfg->flush != LRU_FLUSH_NATIVE && cfg->flush != LRU_FLUSH_DF &&
@@ -383,7 +390,6 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
     const size_t oRatio = take((size_t)h->W * sz);
     const size_t oPst = take((size_t)h->W * sizeof(int));
     const size_t oVP = delayed ? take((size_t)h->W * MAXKK * h->Kc * sz) : 0;
-    const size_t oQtU = delayed ? take((size_t)h->W * h->Kc * MAXKK * sz) : 0;
     const size_t oErr = take(sizeof(int));
     const size_t oN = take((size_t)h->W * sizeof(int));
     const size_t oMoff = take((size_t)h->W * sizeof(long long));
@@ -393,7 +399,8 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
     const size_t oOrder = take((size_t)h->W * sizeof(int));
     const size_t oSItems = take(sitems.size() * sizeof(int));
     const size_t oNacc = take((size_t)h->W * sizeof(int));
-    const size_t oCtl = take((size_t)(1 + 4 * h->W) * sizeof(int));
+    const size_t oCtl = take((size_t)(1 + 5 * h->W) * sizeof(int));
+    const size_t oXit = take(xitems.size() * sizeof(int));
     const size_t oFit = take(std::max<size_t>(fitems.size(), 2) * sizeof(int));
     const size_t oNfl = take((size_t)h->W * sizeof(int));
     const size_t oAcc = take((size_t)h->W);
@@ -421,7 +428,7 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
     h->Rinv = b + oRinv;
     h->ratio = b + oRatio;
     h->pst = (int*)(b + oPst);
-    if (delayed) { h->VP = b + oVP; h->QtU = b + oQtU; }
+    if (delayed) h->VP = b + oVP;
     h->err = (int*)(b + oErr);
     h->d_n = (int*)(b + oN);
     h->d_moff = (long long*)(b + oMoff);
@@ -432,6 +439,7 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
     h->d_sitems = (int*)(b + oSItems);
     h->d_nacc_w = (int*)(b + oNacc);
     h->d_ctl = (int*)(b + oCtl);
+    h->d_xitems = (int*)(b + oXit);
     h->d_fitems = (int*)(b + oFit);
     h->d_nflush_w = (int*)(b + oNfl);
     h->d_acc = (uint8_t*)(b + oAcc);
@@ -445,6 +453,7 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
         cudaMemcpy(h->d_items, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_order, order.data(), h->W * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_sitems, sitems.data(), sitems.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(h->d_xitems, xitems.data(), xitems.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_nacc_w, nacc_w.data(), h->W * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         (!fitems.empty() &&
          cudaMemcpy(h->d_fitems, fitems.data(), fitems.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) ||
@@ -472,7 +481,6 @@ lru_status lru_destroy(lru_handle h) {
     else cudaDeviceSynchronize();
     cudaFree(h->base);
     if (h->ws) cudaFree(h->ws);
-    if (h->bws) cudaFree(h->bws);
     if (h->ozw) cudaFree(h->ozw);
     if (h->ozM) cudaFree(h->ozM);
     for (auto& v : h->prof_ev)
@@ -597,14 +605,6 @@ lru_status lru_refresh_from_scratch(lru_handle h, const void* A, const uint8_t* 
     return do_init(h, A, mask, drift, nullptr, nullptr, true);
 }
 
-// 1 if exactly one slot of the operand is dense (launch_propose then runs that
-// column's pass over A^{-1} as its own kernel), else 0
-static int one_dense_column(unsigned onehot_mask, int kk) {
-    const unsigned all = (kk >= 32) ? 0xffffffffu : ((1u << kk) - 1u);
-    const unsigned dense = ~onehot_mask & all;
-    return (dense != 0 && (dense & (dense - 1)) == 0) ? 1 : 0;
-}
-
 static bool operand_ok(const lru_operand* o, int kk) {
     if (!o) return false;
     const unsigned all = (kk >= 32) ? 0xffffffffu : ((1u << kk) - 1u);
@@ -624,7 +624,7 @@ lru_status lru_propose_det(lru_handle h, const lru_operand* U, const lru_operand
     DevOperand dV{V->dense, V->idx, V->onehot_mask, h->kk};
     DevLayout L = h->layout();
     const unsigned all = (1u << h->kk) - 1u;
-    h->launches += 1 + ((h->delayed && (dU.mask & all) != all) ? 1 : 0) + one_dense_column(dU.mask, h->kk);
+    h->launches += 1 + ((dU.mask & all) != all ? 1 : 0);
     prof_begin(h, LRU_PROF_PROPOSE);
     LRU_DISPATCH(h, {
         launch_propose<T>(false, h->delayed, h->df, L, h->state<T>(), dU, dV, nullptr, (T*)ratio, st, h->stream);
@@ -646,7 +646,7 @@ lru_status lru_propose_pf(lru_handle h, const lru_operand* B, const void* C, voi
     DevOperand dB{B->dense, B->idx, B->onehot_mask, h->kk};
     DevLayout L = h->layout();
     const unsigned all = (1u << h->kk) - 1u;
-    h->launches += 1 + ((h->delayed && (dB.mask & all) != all) ? 1 : 0) + one_dense_column(dB.mask, h->kk);
+    h->launches += 1 + ((dB.mask & all) != all ? 1 : 0);
     prof_begin(h, LRU_PROF_PROPOSE);
     LRU_DISPATCH(h, {
         launch_propose<T>(true, h->delayed, h->df, L, h->state<T>(), dB, dB, (const T*)C, (T*)ratio, st, h->stream);
@@ -676,6 +676,9 @@ lru_status lru_step_persistent(lru_handle h, const lru_operand* U, const lru_ope
     ctl.items_done = h->d_ctl + 1 + h->W;
     ctl.fin = h->d_ctl + 1 + 2 * h->W;
     ctl.flush_done = h->d_ctl + 1 + 3 * h->W;
+    ctl.x_done = h->d_ctl + 1 + 4 * h->W;
+    ctl.x_items = reinterpret_cast<const int2*>(h->d_xitems);
+    ctl.n_x_items = (~dU.mask & ((1u << h->kk) - 1u)) != 0 ? h->nx : 0;
     ctl.acc = acc_out ? acc_out : h->d_acc;
     ctl.order = h->d_order;
     ctl.acc_items = reinterpret_cast<const int4*>(h->d_sitems);
@@ -687,7 +690,7 @@ lru_status lru_step_persistent(lru_handle h, const lru_operand* U, const lru_ope
     ctl.do_accept = accept != 0;
     ctl.mask = mask;
     ctl.u = u;
-    CK(cudaMemsetAsync(h->d_ctl, 0, (size_t)(1 + 4 * h->W) * sizeof(int), h->stream));
+    CK(cudaMemsetAsync(h->d_ctl, 0, (size_t)(1 + 5 * h->W) * sizeof(int), h->stream));
     DevLayout L = h->layout();
     h->launches += 1;
     prof_begin(h, LRU_PROF_PROPOSE);
@@ -938,18 +941,11 @@ static lru_status do_backward(lru_handle h, bool pf, const void* g, void* gU, vo
     if (h->pf != pf) return LRU_ERR_STATE;
     if (!h->has_prop) return LRU_ERR_STATE;
     CK(cudaSetDevice(h->device));
-    if (!h->bws) {
-        if (cudaMalloc(&h->bws, (size_t)2 * h->sum_n * h->kk * dtype_size(h->dtype)) != cudaSuccess) {
-            cudaGetLastError();
-            h->bws = nullptr;
-            return LRU_ERR_NOMEM;
-        }
-    }
     DevLayout L = h->layout();
     h->launches += 1;
     LRU_DISPATCH(h, {
-        launch_backward<T>(pf, h->delayed, L, h->state<T>(), h->lastV, (const T*)h->lastC, (const T*)g, (T*)h->bws,
-                           (T*)gU, (T*)gV, (T*)gA, (T*)gC, h->stream);
+        launch_backward<T>(pf, h->delayed, L, h->state<T>(), h->lastV, (const T*)h->lastC, (const T*)g, (T*)gU,
+                           (T*)gV, (T*)gA, (T*)gC, h->d_items, h->nitems, h->stream);
     });
     return cuda_check();
 }
