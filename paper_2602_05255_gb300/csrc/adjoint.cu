@@ -326,7 +326,7 @@ void launch_scatter_rows(const DevLayout& L, const T* gA, const int* rows, int m
 // inverses, Ginv[w][l n + j] = (A_w^{-1})_{jl}, so (A^{-H})_{ij} is
 // conj(Ginv[w][i n + j]).
 template <typename T>
-__global__ void k_slog_grad(int W, int n, bool pf, const T* Ginv, const double* g_l, const T* g_s, const T* sign,
+__global__ void k_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_t* compact, const double* g_l, const T* g_s, const T* sign,
                             T* gA) {
     const long long nn = (long long)n * n, total = nn * W;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
@@ -334,7 +334,8 @@ __global__ void k_slog_grad(int W, int n, bool pf, const T* Ginv, const double* 
         const int w = (int)(e / nn);
         const long long r = e - (long long)w * nn;
         const int i = (int)(r / n), j = (int)(r - (long long)i * n);
-        const T* G = Ginv + (long long)w * nn;
+        const T* G = Ginv + (long long)w * nr * nr;
+        const int ld = compact && compact[w] ? n : nr;
         T c = make_real<T>(g_l ? g_l[w] : 0.0);
         if constexpr (traits<T>::is_complex) {
             if (g_s) {
@@ -342,22 +343,22 @@ __global__ void k_slog_grad(int W, int n, bool pf, const T* Ginv, const double* 
                 c.im = -q.im;
             }
         }
-        T v = G[(long long)i * n + j];
-        if (pf) v = s_half(s_half(v - G[(long long)j * n + i]));   // (1/2) of the skew part
+        T v = G[(long long)i * ld + j];
+        if (pf) v = s_half(s_half(v - G[(long long)j * ld + i]));   // (1/2) of the skew part
         gA[e] = c * s_conj(v);
     }
 }
 
 template <typename T>
-void launch_slog_grad(int W, int n, bool pf, const T* Ginv, const double* g_l, const T* g_s, const T* sign, T* gA,
+void launch_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_t* compact, const double* g_l, const T* g_s, const T* sign, T* gA,
                       cudaStream_t st) {
     const long long total = (long long)n * n * W;
     const int grid = (int)std::min<long long>((total + 255) / 256, 152 * 16);
-    k_slog_grad<T><<<grid, 256, 0, st>>>(W, n, pf, Ginv, g_l, g_s, sign, gA);
+    k_slog_grad<T><<<grid, 256, 0, st>>>(W, n, nr, pf, Ginv, compact, g_l, g_s, sign, gA);
 }
 
 #define LRU_INST_A(T)                                                                                        \
-    template void launch_slog_grad<T>(int, int, bool, const T*, const double*, const T*, const T*, T*,        \
+    template void launch_slog_grad<T>(int, int, int, bool, const T*, const uint8_t*, const double*, const T*, const T*, T*,        \
                                       cudaStream_t);                                                          \
     template void launch_backward<T>(bool, bool, const DevLayout&, const DevState<T>&, const DevOperand&,     \
                                      const T*, const T*, T*, T*, T*, T*, const int*, int, cudaStream_t);       \

@@ -125,41 +125,60 @@ void launch_zero_split_tail(const DevLayout& L, const DevState<T>& S, const uint
 constexpr int OZ_B = 64;   // panel width = inner dimension of each trailing update
 constexpr int OZ_S = 7;    // BF16 slices per operand (8 bits each: 56 bits)
 struct OzWork {
-    double* M;        // W x n x n row-major working matrix (M = A^T, inverted in place)
-    int* perm;        // W x n pivot rows
-    double* logacc;   // W running log|det|
-    double* sgnacc;   // W running sign
+    double* M;        // W x nr x nc row-major working matrix (M = A^T, inverted in place)
+    int* perm;        // W x nr pivot rows
     int* sing;        // W zero-pivot flags
-    uint16_t* Sb;     // W x OZ_S x n x OZ_B  BF16 slices of the columns of S (panel rows of M)
-    uint16_t* Pb;     // W x OZ_S x n x OZ_B  BF16 slices of the rows of (panel - E)
-    int* eS;          // W x n  power-of-two exponents of the S columns
-    int* eP;          // W x n  power-of-two exponents of the panel rows
-    uint8_t* go;      // W      walkers that flush now (split-product flush)
+    uint16_t* Sb;     // W x OZ_S x nc x OZ_B  BF16 slices of the columns of S (panel rows of M)
+    uint16_t* Pb;     // W x OZ_S x nr x OZ_B  BF16 slices of the rows of (panel - E)
+    int* eS;          // W x nc power-of-two exponents of the S columns
+    int* eP;          // W x nr power-of-two exponents of the panel rows
+    uint8_t* go;      // W      walkers that flush now (split-product flush), or that this form inverts
+    uint8_t* odd;     // W      walkers whose matrix is left to the FP64 form (see k_oz_sort)
     int* cs;          // W x 64 exponent shifts of the slot columns (split-product flush)
-    double* piv;      // W x n  pivots of the register panel kernel (log|det| and sign at the end)
+    double* piv;      // W x nr scalars: pivots (log|det| and sign at the end)
+    int* rmax;        // W x nr largest biased exponent of each row of M
 };
 // columns a split-product update writes: [c_lo, c_hi) minus [s_lo, s_hi), in
-// the 128-column tiles jt_lo .. jt_hi - 1
+// the 128-column tiles jt_lo .. jt_hi - 1 (doubles), rows from tile it_lo on
 struct OzCols {
-    int c_lo, c_hi, s_lo, s_hi, jt_lo, jt_hi;
+    int c_lo, c_hi, s_lo, s_hi, jt_lo, jt_hi, it_lo;
 };
-size_t oz_work_bytes(int W, int n);
-void oz_work_carve(OzWork& Z, void* base, int W, int n);
-void launch_oz_load(int W, int n, const double* A, double* M, const uint8_t* mask, cudaStream_t st);
-void launch_oz_panel(int W, int w0, int n, int k0, const OzWork& Z, const uint8_t* mask, cudaStream_t st);
-// one 16-column sub-panel (n <= 1024): elimination and its row exchanges on the
+// rows of the working matrix of an n x n inverse: n padded by the identity
+int oz_rows(int n);
+// The sizes eliminated on padded copies.  Against the FP64 form (one CTA per
+// walker), refresh of 1 / 1024 F64 walkers on GB300: n = 64 0.35 / 1.1 ms against
+// 0.52 / 2.5, n = 72 (padded to 128) 0.72 / 3.1 against 0.73 / 4.0; between 64 and
+// 72 the padding costs a single walker more than the products gain, and below 56
+// a padded panel does.
+constexpr bool oz_padded(int n) { return n >= 72 || (n >= 56 && n <= 64); }
+// bytes of the workspace of W walkers of nr rows (cx = 2: complex), and its parts when Z is given
+size_t oz_work_layout(OzWork* Z, void* base, int W, int nr, int cx, bool with_M);
+// M[w] = A[w]^T (or A[w]) with an identity in rows and columns n .. nr - 1
+template <typename T>
+void launch_oz_load(int W, int n, int nr, const T* A, bool transpose, bool sort, const OzWork& Z, const uint8_t* mask,
+                    cudaStream_t st);
+// sorts the loaded walkers with mask[w] into Z.go and Z.odd
+void launch_oz_sort(int W, int n, int nr, const OzWork& Z, const uint8_t* mask, cudaStream_t st);
+// one sub-panel of the panel at column k0: elimination and its row exchanges on the
 // other panel columns; the last one of a panel also exchanges the outside columns
-// the tensor-core refresh eliminates its panels in FP64 sub-panels (pivots
-// recorded per row, log|det| summed at the end) up to this n
-constexpr int OZ_SUBPANEL_MAX_N = 2048;
-// width of the FP64 sub-panels of the tensor-core refresh for this n (16, or 8
-// above n = 1024, where a thread holds four rows)
-int oz_subpanel_width(int n);
-bool launch_oz_subpanel(int W, int n, int k0, int sp, const OzWork& Z, const uint8_t* mask, cudaStream_t st);
-void launch_oz_finish(int W, int n, const OzWork& Z, const DevState<double>& S, const uint8_t* mask, bool delayed,
-                      bool reset_tau, cudaStream_t st);
-void launch_oz_drift_store(int W, int n, const DevLayout& L, const DevState<double>& S, const double* M,
-                           const uint8_t* mask, double* drift, bool delayed, cudaStream_t st);
+template <typename T> int oz_subpanel_width(int nr);
+template <typename T>
+void launch_oz_subpanel(int W, int nr, int k0, int sp, bool lu, const OzWork& Z, const uint8_t* mask, cudaStream_t st);
+template <typename T>
+bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, int* err, cudaStream_t st,
+                  void (*hook)(void*, int, int), void* hctx);
+// permute: the row exchanges undone as a column permutation of M's rows 0 .. n - 1;
+// then log|det|, sign (and status, tau := 0, where given)
+template <typename T>
+void launch_oz_finish(int W, int n, int nr, bool permute, const OzWork& Z, const uint8_t* mask, double* logabs, T* sgn,
+                      int* pst, int* tau, cudaStream_t st);
+// M := (M - M^T) / 2 exactly skew, n x n of rows of nr
+template <typename T>
+void launch_oz_skew(int W, int n, int nr, double* M, const uint8_t* mask, cudaStream_t st);
+// the state of walkers w0 .. := the inverses in M (rows of nr), with the drift of the tracked ones when asked for
+template <typename T>
+void launch_oz_store(int W, int w0, int n, int nr, const DevLayout& L, const DevState<T>& S, const OzWork& Z,
+                     const uint8_t* mask, double* drift, bool delayed, bool pf, cudaStream_t st);
 // delayed flush A_0^{-1} += sgnQ * P Q^T (determinant: -1, Pfaffian: +1) as the
 // same exact split product (uniform n, n % 128 == 0, Kc <= 64); walkers with
 // tau >= K, or force && tau > 0 (their go flags stay set for launch_skew_project)
@@ -170,7 +189,7 @@ bool launch_flush_split(int W, int n, int K, int Kc, int kk, const double* P, co
 void launch_skew_project(int W, int n, double* G, const uint8_t* go, cudaStream_t st);
 // hook(ctx, class, begin) brackets the panel (class 4) and update (class 5) launches
 bool launch_refresh_oz(int W, int n, const double* A, const OzWork& Z, const DevState<double>& S,
-                       const uint8_t* mask, bool delayed, bool reset_tau, int* err, cudaStream_t st,
+                       const uint8_t* mask, bool delayed, bool in_state, int* err, cudaStream_t st,
                        void (*hook)(void*, int, int), void* hctx);
 void launch_wait_selftest(const int* flag, long long iters, int* err, cudaStream_t st);
 void launch_commit_moves(int W, int n, int k, int* occ, const int* slot, const int* newrow, const uint8_t* mask,
@@ -191,7 +210,11 @@ template <typename T>
 void launch_slogpf(const DevLayout& L, const T* A, const uint8_t* mask, T* ws, int nws, double* logabs, T* sgn,
                    cudaStream_t st);
 template <typename T>
-void launch_slogdet(int W, int n, const T* A, T* ws, int nws, double* logabs, T* sgn, cudaStream_t st);
+void launch_slogdet(int W, int n, const T* A, T* ws, int nws, double* logabs, T* sgn, const uint8_t* mask,
+                    cudaStream_t st);
+// M (slots of nr^2 scalars) of the masked walkers := the Gauss-Jordan inverse of A^T as n rows of n
+template <typename T>
+void launch_gj_compact(int W, int n, int nr, const T* A, T* M, const uint8_t* mask, cudaStream_t st);
 
 // ---- adjoint (adjoint.cu) ----
 template <typename T>
@@ -204,8 +227,9 @@ void launch_backward_logvalue(bool pf, bool delayed, const DevLayout& L, const D
 template <typename T>
 void launch_log_ratio(int W, const T* ratio, T* out, cudaStream_t st);
 // gradient of (sign, log|det|) or (phase, log|pf|) from the column-major inverses
+// (slots of nr^2 scalars, rows of nr; of n where compact[w])
 template <typename T>
-void launch_slog_grad(int W, int n, bool pf, const T* Ginv, const double* g_l, const T* g_s, const T* sign, T* gA,
+void launch_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_t* compact, const double* g_l, const T* g_s, const T* sign, T* gA,
                       cudaStream_t st);
 template <typename T>
 void launch_scatter_rows(const DevLayout& L, const T* gA, const int* rows, int m, T* gPhi, int* err, cudaStream_t st);

@@ -108,7 +108,9 @@ struct lru_ctx {
     size_t oz_bytes = 0;
     void* ozM = nullptr;         // fresh inverses when the drift is asked for
     size_t ozM_bytes = 0;
-    bool oz_ok = false;          // the tensor-core refresh applies to this handle
+    bool oz_ok = false;          // the tensor-core refresh applies to this handle, in place
+    void* ozg = nullptr;         // workspace of the same refresh through padded copies (other F64 / C128 handles)
+    size_t ozg_bytes = 0;
     int n_sm = 148;
     // debug build: offsets of the guard zones between the regions of the allocation
     std::vector<size_t> canaries;
@@ -483,6 +485,7 @@ lru_status lru_destroy(lru_handle h) {
     if (h->ws) cudaFree(h->ws);
     if (h->ozw) cudaFree(h->ozw);
     if (h->ozM) cudaFree(h->ozM);
+    if (h->ozg) cudaFree(h->ozg);
     for (auto& v : h->prof_ev)
         for (auto& e : v) { cudaEventDestroy(e.first); cudaEventDestroy(e.second); }
     cudaGetLastError();
@@ -500,7 +503,7 @@ lru_status lru_set_stream(lru_handle h, void* stream) {
 lru_status lru_device_bytes(lru_handle h, size_t* bytes) {
     LRU_RANGE();
     if (!h || !bytes) return LRU_ERR_ARG;
-    *bytes = h->bytes + (h->ws ? (size_t)h->nws * h->n_max * h->n_max * dtype_size(h->dtype) : 0) + h->oz_bytes + h->ozM_bytes;
+    *bytes = h->bytes + (h->ws ? (size_t)h->nws * h->n_max * h->n_max * dtype_size(h->dtype) : 0) + h->oz_bytes + h->ozM_bytes + h->ozg_bytes;
     return LRU_OK;
 }
 
@@ -512,7 +515,7 @@ static void oz_prof_hook(void* p, int cls, int begin) {
 
 static lru_status ensure_oz(lru_ctx* h) {
     if (h->ozw) return LRU_OK;
-    const size_t b = oz_work_bytes(h->W, h->n_uni);
+    const size_t b = oz_work_layout(nullptr, nullptr, h->W, h->n_uni, 1, false);
     if (cudaMalloc(&h->ozw, b) != cudaSuccess) {
         cudaGetLastError();
         h->ozw = nullptr;
@@ -521,6 +524,76 @@ static lru_status ensure_oz(lru_ctx* h) {
     h->oz_bytes = b;
     return LRU_OK;
 }
+
+// ---- the tensor-core elimination on padded copies ------------------------------
+// Matrices that are not F64 determinants of n % 128 == 0 (Pfaffians, complex,
+// other n, the standalone calls) are eliminated in a copy of oz_rows(n) rows,
+// a chunk of walkers at a time in a bounded workspace.
+
+constexpr size_t OZ_CHUNK_BYTES = size_t(3) << 30;
+
+static int oz_chunk(int64_t W, int n, int cx) {
+    const int nr = oz_rows(n);
+    const size_t per = oz_work_layout(nullptr, nullptr, 64, nr, cx, true) / 64;
+    int64_t c = std::min<int64_t>({W, 65535, std::max<int64_t>(1, (int64_t)(OZ_CHUNK_BYTES / per)),
+                                   ((1ll << 31) - 1) / ((int64_t)OZ_S * nr * cx)});
+    if (c < W && c > 152) c -= c % 152;   // whole waves of the kernels that take a CTA per walker
+    return (int)c;
+}
+
+// the workspace of a handle's padded refresh: the chunk, then a byte per walker
+// (matrices left to the FP64 form).  Not available: false, and the FP64 form runs
+// (out of memory, or a first use inside a stream capture, where nothing may be
+// allocated).
+static bool ensure_ozg(lru_ctx* h, int cx) {
+    if (h->ozg) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    const int chunk = oz_chunk(h->W, h->n_uni, cx);
+    const size_t b = oz_work_layout(nullptr, nullptr, chunk, oz_rows(h->n_uni), cx, true) + (size_t)h->W;
+    if (cudaMalloc(&h->ozg, b) != cudaSuccess) {
+        cudaGetLastError();
+        h->ozg = nullptr;
+        return false;
+    }
+    h->ozg_bytes = b;
+    return true;
+}
+
+// inverse (and for determinants log|det|, sign) of the masked walkers into the state
+extern "C++" {
+template <typename T>
+static bool refresh_padded(lru_ctx* h, const T* A, const uint8_t* mask, double* drift) {
+    constexpr int cx = traits<T>::is_complex ? 2 : 1;
+    if (!ensure_ozg(h, cx)) return false;
+    const int n = h->n_uni, nr = oz_rows(n), chunk = oz_chunk(h->W, n, cx);
+    OzWork Z;
+    const size_t zb = oz_work_layout(&Z, h->ozg, chunk, nr, cx, true);
+    uint8_t* odd = (uint8_t*)h->ozg + zb;
+    const DevLayout L = h->layout();
+    DevState<T> S = h->state<T>();
+    for (int w0 = 0; w0 < h->W; w0 += chunk) {
+        const int Wc = std::min(chunk, h->W - w0);
+        const uint8_t* m = mask ? mask + w0 : nullptr;
+        Z.odd = odd + w0;
+        launch_oz_load<T>(Wc, n, nr, A + (size_t)w0 * n * n, true, true, Z, m, h->stream);
+        launch_oz_sort(Wc, n, nr, Z, m, h->stream);
+        if (!oz_eliminate<T>(Wc, nr, Z, Z.go, false, h->err, h->stream, h->prof_on ? oz_prof_hook : nullptr, h))
+            return false;   // tensor maps unavailable: nothing has been written to the state
+        launch_oz_finish<T>(Wc, n, nr, true, Z, Z.go, h->pf ? nullptr : S.logabs + w0, h->pf ? nullptr : S.sgn + w0,
+                            S.pst + w0, nullptr, h->stream);
+        if (h->pf) launch_oz_skew<T>(Wc, n, nr, Z.M, Z.go, h->stream);
+        launch_oz_store<T>(Wc, w0, n, nr, L, S, Z, Z.go, drift, h->delayed, h->pf, h->stream);
+    }
+    // the FP64 form for the walkers sorted out (usually none: every CTA leaves at once)
+    launch_refresh<T>(h->pf, h->delayed, L, S, A, odd, drift ? (T*)Z.M : nullptr, chunk, drift, !h->pf, h->stream);
+    h->launches += ((h->W + chunk - 1) / chunk) * (4 + 4 * (nr / OZ_B) * cx) + 1;
+    return true;
+}
+}  // extern "C++"
 
 static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, double* drift, double* logabs_out,
                           void* sign_out, bool with_ws) {
@@ -541,14 +614,15 @@ static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, doub
             h->ozM_bytes = b;
         }
         OzWork Z{};
-        oz_work_carve(Z, h->ozw, h->W, h->n_uni);
+        oz_work_layout(&Z, h->ozw, h->W, h->n_uni, 1, false);
         Z.M = drift ? (double*)h->ozM : (double*)h->G;
         DevState<double> S = h->state<double>();
         prof_begin(h, LRU_PROF_REFRESH);
         bool ok = launch_refresh_oz(h->W, h->n_uni, (const double*)A, Z, S, mask, h->delayed, !drift, h->err,
                                     h->stream, h->prof_on ? oz_prof_hook : nullptr, h);
         if (ok && drift)
-            launch_oz_drift_store(h->W, h->n_uni, h->layout(), S, Z.M, mask, drift, h->delayed, h->stream);
+            launch_oz_store<double>(h->W, 0, h->n_uni, h->n_uni, h->layout(), S, Z, mask, drift, h->delayed, false,
+                                    h->stream);
         prof_end(h, LRU_PROF_REFRESH);
         if (ok) {
             h->launches += 2 + 4 * (h->n_uni / OZ_B);
@@ -562,17 +636,23 @@ static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, doub
         }
         cudaGetLastError();   // tensor maps unavailable: the FP64 form below
     }
-    if (with_ws || h->pf) {
+    prof_begin(h, LRU_PROF_REFRESH);
+    bool done = false;
+    if (!h->oz_ok && oz_padded(h->n_uni) && h->cfg.refresh != LRU_REFRESH_FP64) {
+        if (h->dtype == LRU_F64) done = refresh_padded<double>(h, (const double*)A, mask, drift);
+        else if (h->dtype == LRU_C128) done = refresh_padded<c128>(h, (const c128*)A, mask, drift);
+    }
+    if ((with_ws && !done) || h->pf) {
         lru_status s = ensure_ws(h);
-        if (s != LRU_OK) return s;
+        if (s != LRU_OK) { prof_end(h, LRU_PROF_REFRESH); return s; }
     }
     DevLayout L = h->layout();
-    prof_begin(h, LRU_PROF_REFRESH);
-    h->launches += h->pf ? 2 : 1;
+    h->launches += (done ? 0 : 1) + (h->pf ? 1 : 0);
     LRU_DISPATCH(h, {
         DevState<T> S = h->state<T>();
-        launch_refresh<T>(h->pf, h->delayed, L, S, (const T*)A, mask, with_ws ? (T*)h->ws : nullptr, h->nws,
-                          drift, !h->pf, h->stream);
+        if (!done)
+            launch_refresh<T>(h->pf, h->delayed, L, S, (const T*)A, mask, with_ws ? (T*)h->ws : nullptr, h->nws,
+                              drift, !h->pf, h->stream);
         if (h->pf) launch_slogpf<T>(L, (const T*)A, mask, (T*)h->ws, h->nws, S.logabs, S.sgn, h->stream);
     });
     prof_end(h, LRU_PROF_REFRESH);
@@ -715,7 +795,7 @@ static lru_status do_flush(lru_handle h, const uint8_t* force) {
         lru_status s = ensure_oz(h);
         if (s != LRU_OK) { prof_end(h, LRU_PROF_FLUSH); return s; }
         OzWork Z{};
-        oz_work_carve(Z, h->ozw, h->W, h->n_uni);
+        oz_work_layout(&Z, h->ozw, h->W, h->n_uni, 1, false);
         Z.M = (double*)h->G;
         h->launches += 4;   // flush flags, column balance, two slicings, GEMM (+ finish counted above)
         // determinant: A_0^{-1} -= P Q^T (Eq. delayed_Ainv); Pfaffian: A_0^{-1} += P Q^T
@@ -1013,11 +1093,75 @@ lru_status lru_launch_count(lru_handle h, int64_t* count) {
     return LRU_OK;
 }
 
+extern "C++" {
+// log|det| and sign of a batch, the elimination on the tensor cores (lu: the
+// inverse is not formed).  false: no workspace, nothing done.
+template <typename T>
+static bool slogdet_padded(int W, int n, const T* A, double* logabs, T* sign, cudaStream_t st) {
+    constexpr int cx = traits<T>::is_complex ? 2 : 1;
+    const int nr = oz_rows(n), chunk = oz_chunk(W, n, cx);
+    void* ws = nullptr;
+    if (cudaMallocAsync(&ws, oz_work_layout(nullptr, nullptr, chunk, nr, cx, true), st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    OzWork Z;
+    oz_work_layout(&Z, ws, chunk, nr, cx, true);
+    bool ok = true;
+    for (int w0 = 0; ok && w0 < W; w0 += chunk) {
+        const int Wc = std::min(chunk, W - w0);
+        const T* Aw = A + (size_t)w0 * n * n;
+        launch_oz_load<T>(Wc, n, nr, Aw, false, true, Z, nullptr, st);
+        launch_oz_sort(Wc, n, nr, Z, nullptr, st);
+        ok = oz_eliminate<T>(Wc, nr, Z, Z.go, true, nullptr, st, nullptr, nullptr);
+        if (!ok) break;
+        launch_oz_finish<T>(Wc, n, nr, false, Z, Z.go, logabs + w0, sign + w0, nullptr, nullptr, st);
+        launch_slogdet<T>(Wc, n, Aw, (T*)Z.M, Wc, logabs + w0, sign + w0, Z.odd, st);
+    }
+    cudaFreeAsync(ws, st);
+    return ok;
+}
+
+// gradient of (sign, log|det|) or (phase, log|pf|), the inverses formed chunk by chunk on the tensor cores
+template <typename T>
+static bool slog_backward_padded(bool pf, int W, int n, const T* A, const double* g_l, const T* g_s, const T* sign,
+                                 T* gA, cudaStream_t st) {
+    constexpr int cx = traits<T>::is_complex ? 2 : 1;
+    const int nr = oz_rows(n), chunk = oz_chunk(W, n, cx);
+    void* ws = nullptr;
+    if (cudaMallocAsync(&ws, oz_work_layout(nullptr, nullptr, chunk, nr, cx, true), st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    OzWork Z;
+    oz_work_layout(&Z, ws, chunk, nr, cx, true);
+    bool ok = true;
+    for (int w0 = 0; ok && w0 < W; w0 += chunk) {
+        const int Wc = std::min(chunk, W - w0);
+        const T* Aw = A + (size_t)w0 * n * n;
+        launch_oz_load<T>(Wc, n, nr, Aw, true, true, Z, nullptr, st);
+        launch_oz_sort(Wc, n, nr, Z, nullptr, st);
+        ok = oz_eliminate<T>(Wc, nr, Z, Z.go, false, nullptr, st, nullptr, nullptr);
+        if (!ok) break;
+        launch_oz_finish<T>(Wc, n, nr, true, Z, Z.go, nullptr, (T*)nullptr, nullptr, nullptr, st);
+        launch_gj_compact<T>(Wc, n, nr, Aw, (T*)Z.M, Z.odd, st);
+        launch_slog_grad<T>(Wc, n, nr, pf, (const T*)Z.M, Z.odd, g_l ? g_l + w0 : nullptr, g_s ? g_s + w0 : nullptr,
+                            sign ? sign + w0 : nullptr, gA + (size_t)w0 * n * n, st);
+    }
+    cudaFreeAsync(ws, st);
+    return ok;
+}
+}  // extern "C++"
+
 static lru_status batched_dense(bool pf, int32_t dtype, int64_t W, int32_t n, const void* A, double* logabs,
                                 void* sign, void* stream) {
     if (W < 1 || W > (int64_t)INT32_MAX || n < 1 || n > MAXN || !A || !logabs || !sign || dtype_size(dtype) == 0)
         return LRU_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
+    if (!pf && oz_padded(n) &&
+        ((dtype == LRU_F64 && slogdet_padded<double>((int)W, n, (const double*)A, logabs, (double*)sign, st)) ||
+         (dtype == LRU_C128 && slogdet_padded<c128>((int)W, n, (const c128*)A, logabs, (c128*)sign, st))))
+        return cuda_check();
     int dev = 0, nsm = 148;
     CK(cudaGetDevice(&dev));
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); nsm = 148; }
@@ -1033,7 +1177,7 @@ static lru_status batched_dense(bool pf, int32_t dtype, int64_t W, int32_t n, co
     lru_ctx* h = &tmp;
     LRU_DISPATCH(h, {
         if (pf) launch_slogpf<T>(L, (const T*)A, nullptr, (T*)ws, nws, logabs, (T*)sign, st);
-        else launch_slogdet<T>((int)W, n, (const T*)A, (T*)ws, nws, logabs, (T*)sign, st);
+        else launch_slogdet<T>((int)W, n, (const T*)A, (T*)ws, nws, logabs, (T*)sign, nullptr, st);
     });
     lru_status s = cuda_check();
     cudaFreeAsync(ws, st);
@@ -1052,6 +1196,12 @@ static lru_status slog_backward(bool pf, int32_t dtype, int64_t W, int32_t n, co
     if (pf && (n & 1)) return LRU_ERR_ARG;
     if (g_sign && !sign) return LRU_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
+    if (oz_padded(n) &&
+        ((dtype == LRU_F64 && slog_backward_padded<double>(pf, (int)W, n, (const double*)A, g_logabs,
+                                                           (const double*)g_sign, (const double*)sign, (double*)gA, st)) ||
+         (dtype == LRU_C128 && slog_backward_padded<c128>(pf, (int)W, n, (const c128*)A, g_logabs, (const c128*)g_sign,
+                                                          (const c128*)sign, (c128*)gA, st))))
+        return cuda_check();
     int dev = 0, nsm = 148;
     CK(cudaGetDevice(&dev));
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); nsm = 148; }
@@ -1078,7 +1228,7 @@ static lru_status slog_backward(bool pf, int32_t dtype, int64_t W, int32_t n, co
         S.G = (T*)Ginv;
         S.pst = pst;
         launch_refresh<T>(false, false, L, S, (const T*)A, nullptr, (T*)ws, nws, nullptr, false, st);
-        launch_slog_grad<T>((int)W, n, pf, (const T*)Ginv, g_logabs, (const T*)g_sign, (const T*)sign, (T*)gA, st);
+        launch_slog_grad<T>((int)W, n, n, pf, (const T*)Ginv, nullptr, g_logabs, (const T*)g_sign, (const T*)sign, (T*)gA, st);
     });
     lru_status s = cuda_check();
     cudaFreeAsync(buf, st);

@@ -404,7 +404,8 @@ __global__ void __launch_bounds__(RT) k_slogpf(DevLayout L, const T* A, const ui
 
 // standalone slogdet (GJ on a workspace copy)
 template <typename T>
-__global__ void __launch_bounds__(RT) k_slogdet(int W, int n, const T* A, T* ws, double* logabs, T* sgn) {
+__global__ void __launch_bounds__(RT) k_slogdet(int W, int n, const T* A, T* ws, double* logabs, T* sgn,
+                                                 const uint8_t* mask) {
     extern __shared__ __align__(16) unsigned char dsm[];
     GJSmem<T>& sm = *reinterpret_cast<GJSmem<T>*>(dsm);
     __shared__ int perm[2048];
@@ -412,6 +413,7 @@ __global__ void __launch_bounds__(RT) k_slogdet(int W, int n, const T* A, T* ws,
     __shared__ T s_s;
     __shared__ int s_sing;
     for (int w = blockIdx.x; w < W; w += gridDim.x) {
+        if (mask && !mask[w]) continue;
         T* M = ws + (long long)blockIdx.x * n * n;
         const T* Aw = A + (long long)w * n * n;
         for (long long e = threadIdx.x; e < (long long)n * n; e += RT) M[e] = Aw[e];
@@ -443,101 +445,140 @@ void launch_slogpf(const DevLayout& L, const T* A, const uint8_t* mask, T* ws, i
 }
 
 template <typename T>
-void launch_slogdet(int W, int n, const T* A, T* ws, int nws, double* logabs, T* sgn, cudaStream_t st) {
+void launch_slogdet(int W, int n, const T* A, T* ws, int nws, double* logabs, T* sgn, const uint8_t* mask,
+                    cudaStream_t st) {
     const int dyn = (int)sizeof(GJSmem<T>);
     cudaFuncSetAttribute(k_slogdet<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    k_slogdet<T><<<nws, RT, dyn, st>>>(W, n, A, ws, logabs, sgn);
+    k_slogdet<T><<<nws, RT, dyn, st>>>(W, n, A, ws, logabs, sgn, mask);
 }
+
+template <typename T>
+__global__ void __launch_bounds__(RT) k_gj_compact(int n, int nr, const T* A, T* M, const uint8_t* mask) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    GJSmem<T>& sm = *reinterpret_cast<GJSmem<T>*>(dsm);
+    __shared__ int perm[2048];
+    __shared__ double s_l;
+    __shared__ T s_s;
+    __shared__ int s_sing;
+    const int w = blockIdx.x;
+    if (!mask[w]) return;
+    T* Mw = M + (long long)w * nr * nr;
+    load_transposed(Mw, A + (long long)w * n * n, n, sm.tile);
+    __syncthreads();
+    gj_invert(Mw, n, perm, &s_l, &s_s, &s_sing, sm);
+}
+
+template <typename T>
+void launch_gj_compact(int W, int n, int nr, const T* A, T* M, const uint8_t* mask, cudaStream_t st) {
+    const int dyn = (int)sizeof(GJSmem<T>);
+    cudaFuncSetAttribute(k_gj_compact<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    k_gj_compact<T><<<W, RT, dyn, st>>>(n, nr, A, M, mask);
+}
+
 
 // ---------------------------------------------------------------------------
 // FP64 parts of the tensor-core refresh (the GEMM is in refresh_oz.cu)
 // ---------------------------------------------------------------------------
 
-// M[w] = A[w]^T through 32 x 32 tiles; grid (n/32, n/32, W), block 32 x 8
-__global__ void k_oz_load(int n, const double* A, double* M, const uint8_t* mask) {
-    __shared__ double tile[32][33];
+// largest biased exponent of a scalar's parts (0x7ff: not finite)
+__device__ __forceinline__ int bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ int bexp(c128 x) { return max(bexp(x.re), bexp(x.im)); }
+
+// M[w] = A[w]^T (or A[w]) through 32 x 32 tiles, the identity in the padding,
+// and (sort) the largest exponent of every row of M in Z.rmax (zeroed before);
+// grid (nr/32, nr/32, W), block 32 x 8
+template <typename T>
+__global__ void k_oz_load(int n, int nr, const T* A, bool transpose, bool sort, OzWork Z, const uint8_t* mask) {
+    __shared__ T tile[32][33];
     const int w = blockIdx.z;
     if (mask && !mask[w]) return;
-    const long long off = (long long)w * n * n;
-    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32, tx = threadIdx.x;
-    for (int q = threadIdx.y; q < 32; q += 8) tile[q][tx] = A[off + (long long)(r0 + q) * n + c0 + tx];
-    __syncthreads();
-    for (int q = threadIdx.y; q < 32; q += 8) M[off + (long long)(c0 + q) * n + r0 + tx] = tile[tx][q];
-}
-
-// Panel [k0, k0 + OZ_B) of walker w: Gauss-Jordan elimination of its columns
-// over all rows (updates confined to the panel), then its row exchanges
-// applied, in pivot order, to every column outside the panel.  log|pivot|
-// and the sign carry over between panels in Z.logacc / Z.sgnacc / Z.sing.
-__global__ void __launch_bounds__(RT) k_oz_panel(int n, int k0, int w0, OzWork Z, const uint8_t* mask) {
-    extern __shared__ __align__(16) unsigned char dsm[];
-    GJSmem<double>& sm = *reinterpret_cast<GJSmem<double>*>(dsm);
-    __shared__ double s_log, s_sgn;
-    __shared__ int s_sing;
-    const int w = w0 + blockIdx.x;
-    if (mask && !mask[w]) return;
-    double* M = Z.M + (long long)w * n * n;
-    int* perm = Z.perm + (long long)w * n;
-    if (threadIdx.x == 0) {
-        s_log = k0 ? Z.logacc[w] : 0.0;
-        s_sgn = k0 ? Z.sgnacc[w] : 1.0;
-        s_sing = k0 ? Z.sing[w] : 0;
-    }
-    __syncthreads();
-    gj_columns<double>(M, n, k0, k0 + OZ_B, k0, k0 + OZ_B, perm, s_log, s_sgn, s_sing, sm);
-    __syncthreads();
-    for (int j = threadIdx.x; j < n; j += RT) {
-        if (j >= k0 && j < k0 + OZ_B) continue;
-        for (int kc = 0; kc < OZ_B; ++kc) {
-            const int k = k0 + kc, p = perm[k];
-            if (p != k) {
-                const double a = M[(long long)k * n + j];
-                M[(long long)k * n + j] = M[(long long)p * n + j];
-                M[(long long)p * n + j] = a;
-            }
+    const T* Aw = A + (long long)w * n * n;
+    T* M = reinterpret_cast<T*>(Z.M) + (long long)w * nr * nr;
+    const int tx = threadIdx.x, r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;   // of M
+    if (transpose) {
+        for (int q = threadIdx.y; q < 32; q += 8) {
+            const int r = c0 + q, c = r0 + tx;   // of A
+            if (r < n && c < n) tile[tx][q] = Aw[(long long)r * n + c];
         }
+        __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        Z.logacc[w] = s_log;
-        Z.sgnacc[w] = s_sgn;
-        Z.sing[w] = s_sing;
+    for (int q = threadIdx.y; q < 32; q += 8) {
+        const int r = r0 + q, c = c0 + tx;
+        T v = make_real<T>(r == c ? 1.0 : 0.0);
+        const bool in = r < n && c < n;
+        if (in) v = transpose ? tile[q][tx] : Aw[(long long)r * n + c];
+        M[(long long)r * nr + c] = v;
+        if (!sort) continue;
+        const int e = __reduce_max_sync(0xffffffffu, in ? bexp(v) : 0);
+        if (tx == 0 && e > 0) atomicMax(&Z.rmax[(long long)w * nr + r], e);
     }
 }
 
-// One SW-column sub-panel of panel [k0, k0 + OZ_B) with the rows in registers
-// (SW = 16 for n <= 1024, 8 up to n = 2048): thread t owns rows t + q * blockDim
-// (q < RPT, blockDim = n / RPT).  The sub-panel is eliminated in registers (pivot by a block reduction,
+// Which of the loaded walkers the split products take (go) and which are left
+// to the FP64 form (odd): those with an entry that is not finite, with rows of
+// very different size (a panel row's digits share one scale, so rows 2^s apart
+// cost s bits) or with entries so large or small that a product of scales could
+// leave the exponent range.  One warp per walker.
+__global__ void k_oz_sort(int W, int n, int nr, OzWork Z, const uint8_t* mask) {
+    const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (w >= W) return;
+    int hi = 0, lo = 0x7ff;
+    for (int r = threadIdx.x & 31; r < n; r += 32) {
+        const int e = Z.rmax[(long long)w * nr + r];
+        hi = max(hi, e);
+        lo = min(lo, e);
+    }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    if ((threadIdx.x & 31) == 0) {
+        const bool on = !mask || mask[w], fit = hi - lo <= 6 && hi < 1023 + 200 && hi > 1023 - 200;
+        Z.go[w] = on && fit;
+        Z.odd[w] = on && !fit;
+    }
+}
+
+// One SW-column sub-panel of panel [k0, k0 + PB) (PB = 64 real or 32 complex
+// columns) with the rows in registers (SW = 16 for nr <= 1024, 8 up to 2048;
+// complex half of that): thread t owns rows t + q * blockDim (q < RPT,
+// blockDim = nr / RPT); lu: only the rows from k0 on.  The sub-panel is eliminated in registers (pivot by a block reduction,
 // row swaps through shared memory) and its transform columns written back;
 // its row exchanges are then applied to the other panel columns, whose update
 // by the transform is a split product on the tensor cores (refresh_oz.cu).
 // The last sub-panel of a panel also applies the panel's exchanges, in pivot
 // order, to the columns outside it.  Pivots go to Z.piv (log|det| and the
 // sign are summed at the end).
-template <int RPT, int SW>
-__global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int sp, OzWork Z, const uint8_t* mask) {
-    static_assert(SW % 2 == 0 && OZ_B % SW == 0, "sub-panel width");
-    __shared__ double s_rowk[SW], s_bufA[SW], s_bufB[SW];
+template <typename T, int RPT, int SW>
+__global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int sp, bool lu, OzWork Z,
+                                                              const uint8_t* mask) {
+    constexpr int CX = traits<T>::is_complex ? 2 : 1, PB = OZ_B / CX;
+    static_assert(SW * CX % 2 == 0 && PB % SW == 0, "sub-panel width");
+    __shared__ T s_rowk[SW], s_bufA[SW], s_bufB[SW];
     __shared__ unsigned long long s_wk[16];
     __shared__ int s_wi[16];
     __shared__ int s_sing;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
     const int w = blockIdx.x;
     if (mask && !mask[w]) return;
-    double* M = Z.M + (long long)w * n * n;
+    T* M = reinterpret_cast<T*>(Z.M) + (long long)w * n * n;
+    T* pivots = reinterpret_cast<T*>(Z.piv) + (long long)w * n;
+    const int i_lo = lu ? k0 : 0;
     int* perm = Z.perm + (long long)w * n;
     if (tid == 0) s_sing = (k0 || sp) ? Z.sing[w] : 0;
     __syncthreads();
     {
         const int ks = k0 + SW * sp;
-        double v[RPT][SW];
+        constexpr int VL = 2 / CX;   // scalars per 16-byte load
+        struct alignas(16) Pair { T e[VL]; };
+        T v[RPT][SW];
 #pragma unroll
         for (int q = 0; q < RPT; ++q) {
-            const double2* src = reinterpret_cast<const double2*>(M + (long long)(tid + q * nt) * n + ks);
+            const Pair* src = reinterpret_cast<const Pair*>(M + (long long)(tid + q * nt) * n + ks);
+            if (tid + q * nt < i_lo) continue;
 #pragma unroll
-            for (int c = 0; c < SW / 2; ++c) {
-                const double2 x = src[c];
-                v[q][2 * c] = x.x;
-                v[q][2 * c + 1] = x.y;
+            for (int c = 0; c < SW / VL; ++c) {
+                const Pair x = src[c];
+#pragma unroll
+                for (int e = 0; e < VL; ++e) v[q][VL * c + e] = x.e[e];
             }
         }
 #pragma unroll
@@ -554,9 +595,13 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
 #pragma unroll
             for (int q = 0; q < RPT; ++q) {
                 const int r = tid + q * nt;
-                unsigned long long a = (unsigned long long)__double_as_longlong(v[q][kc]) & 0x7FFFFFFFFFFFFFFFull;
+                if (r < k) continue;
+                double mag;
+                if constexpr (CX == 1) mag = v[q][kc];
+                else mag = s_abs2(v[q][kc]);
+                unsigned long long a = (unsigned long long)__double_as_longlong(mag) & 0x7FFFFFFFFFFFFFFFull;
                 if (a > 0x7FF0000000000000ull) a = 0ull;
-                if (r >= k && (bi < 0 || a > bk)) { bk = a; bi = r; }
+                if (bi < 0 || a > bk) { bk = a; bi = r; }
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -575,7 +620,7 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
             }
             const int p = bi;
             if (bk == 0ull || p < 0) {
-                if (tid == 0) { perm[k] = k; s_sing = 1; Z.piv[(long long)w * n + k] = 0.0; }
+                if (tid == 0) { perm[k] = k; s_sing = 1; pivots[k] = s_zero(T()); }
                 __syncthreads();   // every thread has read s_wk before the next pivot writes it
                 continue;
             }
@@ -595,9 +640,10 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
             // ---- scale the pivot row: 16 threads, one element each; the pivot
             //      is recorded (log|det| and the sign are summed at the end) ----
             if (tid < SW) {
-                const double piv = s_bufA[kc];
-                s_rowk[tid] = (tid == kc ? 1.0 : s_bufA[tid]) / piv;
-                if (tid == 0) Z.piv[(long long)w * n + k] = piv;
+                const T piv = s_bufA[kc], x = tid == kc ? make_real<T>(1.0) : s_bufA[tid];
+                if constexpr (CX == 1) s_rowk[tid] = x / piv;
+                else s_rowk[tid] = x * s_recip(piv);
+                if (tid == 0) pivots[k] = piv;
             }
             __syncthreads();
             // ---- exchange: row k becomes the scaled pivot row, row p the old row k ----
@@ -614,28 +660,34 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
 #pragma unroll
             for (int q = 0; q < RPT; ++q) {
                 const int r = tid + q * nt;
-                if (r != k) {
-                    const double f = v[q][kc];
+                if (r != k && r >= i_lo) {
+                    const T f = v[q][kc];
 #pragma unroll
-                    for (int c = 0; c < SW; ++c) v[q][c] = fma(-f, s_rowk[c], c == kc ? 0.0 : v[q][c]);
+                    for (int c = 0; c < SW; ++c) v[q][c] = s_fms(f, s_rowk[c], c == kc ? s_zero(T()) : v[q][c]);
                 }
             }
         }
         // ---- the sub-panel's transform columns back to M ----
 #pragma unroll
         for (int q = 0; q < RPT; ++q) {
-            double2* dst = reinterpret_cast<double2*>(M + (long long)(tid + q * nt) * n + ks);
+            Pair* dst = reinterpret_cast<Pair*>(M + (long long)(tid + q * nt) * n + ks);
+            if (tid + q * nt < i_lo) continue;
 #pragma unroll
-            for (int c = 0; c < SW / 2; ++c) dst[c] = make_double2(v[q][2 * c], v[q][2 * c + 1]);
+            for (int c = 0; c < SW / VL; ++c) {
+                Pair x;
+#pragma unroll
+                for (int e = 0; e < VL; ++e) x.e[e] = v[q][VL * c + e];
+                dst[c] = x;
+            }
         }
         __syncthreads();
         // ---- this sub-panel's exchanges on the other panel columns ----
-        for (int t = tid; t < OZ_B - SW; t += nt) {
+        for (int t = tid; t < PB - SW; t += nt) {
             const int col = k0 + t + (t >= SW * sp ? SW : 0);
             for (int kc = 0; kc < SW; ++kc) {
                 const int kk = ks + kc, p = perm[kk];
                 if (p != kk) {
-                    const double a = M[(long long)kk * n + col];
+                    const T a = M[(long long)kk * n + col];
                     M[(long long)kk * n + col] = M[(long long)p * n + col];
                     M[(long long)p * n + col] = a;
                 }
@@ -648,16 +700,16 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
     // is built once in shared memory; then every 32-column tile of those rows
     // is gathered into shared memory (independent, coalesced loads) and
     // written back permuted, instead of 64 dependent swaps per column.
-    if (sp == OZ_B / SW - 1) {
+    if (sp == PB / SW - 1) {
         __shared__ int s_src[2048];            // n <= 2048 for this kernel
-        __shared__ int s_from[2 * OZ_B], s_to[2 * OZ_B];
+        __shared__ int s_from[2 * PB], s_to[2 * PB];
         __shared__ int s_cnt;
-        __shared__ double s_xb[2 * OZ_B][33];
+        __shared__ T s_xb[2 * PB][33];
         for (int r = tid; r < n; r += nt) s_src[r] = r;
         if (tid == 0) s_cnt = 0;
         __syncthreads();
         if (tid == 0)
-            for (int kc = 0; kc < OZ_B; ++kc) {
+            for (int kc = 0; kc < PB; ++kc) {
                 const int k = k0 + kc, p = perm[k];
                 const int a = s_src[k];
                 s_src[k] = s_src[p];
@@ -666,21 +718,21 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
         __syncthreads();
         for (int r = tid; r < n; r += nt)
             if (s_src[r] != r) {
-                const int e = atomicAdd(&s_cnt, 1);   // at most 2 * OZ_B rows move
+                const int e = atomicAdd(&s_cnt, 1);   // at most 2 * PB rows move
                 s_to[e] = r;
                 s_from[e] = s_src[r];
             }
         __syncthreads();
         const int cnt = s_cnt;
-        for (int j0 = 0; j0 < n && cnt > 0; j0 += 32) {
-            if (j0 >= k0 && j0 < k0 + OZ_B) continue;   // the panel's own columns (64-aligned)
+        for (int j0 = lu ? k0 + PB : 0; j0 < n && cnt > 0; j0 += 32) {
+            if (j0 >= k0 && j0 < k0 + PB) continue;   // the panel's own columns (PB is a multiple of 32)
             // eight independent loads per thread in flight before any store
             for (int e0 = tid; e0 < cnt * 32; e0 += 8 * nt) {
-                double x[8];
+                T x[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int e = e0 + u * nt;
-                    x[u] = e < cnt * 32 ? M[(long long)s_from[e >> 5] * n + j0 + (e & 31)] : 0.0;
+                    x[u] = e < cnt * 32 ? M[(long long)s_from[e >> 5] * n + j0 + (e & 31)] : s_zero(T());
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -703,145 +755,204 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
 // the inverse (idx composes the swaps, last first: M'[i][c] = M[i][idx[c]]),
 // four rows at a time through shared memory; then log|det|, sign and the
 // fresh-state flags.
-__global__ void __launch_bounds__(RT) k_oz_finish(int n, OzWork Z, DevState<double> S, const uint8_t* mask,
-                                                  bool delayed, bool reset_tau) {
+template <typename T>
+__global__ void __launch_bounds__(RT) k_oz_finish(int n, int nr, bool permute, OzWork Z, const uint8_t* mask,
+                                                  double* logabs, T* sgn, int* pst, int* tau) {
     extern __shared__ __align__(16) unsigned char dsm[];
-    double* buf = reinterpret_cast<double*>(dsm);
+    T* buf = reinterpret_cast<T*>(dsm);
     int* idx = reinterpret_cast<int*>(buf + 4 * n);
+    __shared__ double s_sum[32];
+    __shared__ T s_unit_part[RT];
     const int w = blockIdx.x;
     if (mask && !mask[w]) return;
-    const int* perm = Z.perm + (long long)w * n;
-    for (int c = threadIdx.x; c < n; c += RT) idx[c] = c;
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int k = n - 1; k >= 0; --k) {
-            const int p = perm[k];
-            if (p != k) { const int t = idx[k]; idx[k] = idx[p]; idx[p] = t; }
-        }
-    __syncthreads();
-    double* M = Z.M + (long long)w * n * n;
-    for (int i0 = 0; i0 < n; i0 += 4) {
-        const int rows = min(4, n - i0);
-        for (int e = threadIdx.x; e < rows * n; e += RT) buf[e] = M[(long long)i0 * n + e];
+    const int* perm = Z.perm + (long long)w * nr;
+    if (permute) {
+        for (int c = threadIdx.x; c < n; c += RT) idx[c] = c;
         __syncthreads();
-        for (int e = threadIdx.x; e < rows * n; e += RT) {
-            const int r = e / n, c = e % n;
-            M[(long long)(i0 + r) * n + c] = buf[r * n + idx[c]];
-        }
+        if (threadIdx.x == 0)
+            for (int k = n - 1; k >= 0; --k) {
+                const int p = perm[k];
+                if (p != k) { const int t = idx[k]; idx[k] = idx[p]; idx[p] = t; }
+            }
         __syncthreads();
+        T* M = reinterpret_cast<T*>(Z.M) + (long long)w * nr * nr;
+        for (int i0 = 0; i0 < n; i0 += 4) {
+            const int rows = min(4, n - i0);
+            for (int r = 0; r < rows; ++r)
+                for (int c = threadIdx.x; c < n; c += RT) buf[r * n + c] = M[(long long)(i0 + r) * nr + c];
+            __syncthreads();
+            for (int r = 0; r < rows; ++r)
+                for (int c = threadIdx.x; c < n; c += RT) M[(long long)(i0 + r) * nr + c] = buf[r * n + idx[c]];
+            __syncthreads();
+        }
     }
+    // log|det| = sum log|pivot|, sign = prod of the pivots' signs * (-1)^(row exchanges)
+    const T* pv = reinterpret_cast<const T*>(Z.piv) + (long long)w * nr;
     double la = 0.0;
-    int neg = 0;
-    const bool piv_rec = n <= OZ_SUBPANEL_MAX_N;   // the sub-panel path records the pivots
-    if (piv_rec) {
-        // log|det| = sum log|pivot|, sign = prod sign(pivot) * (-1)^(row exchanges)
-        const double* pv = Z.piv + (long long)w * n;
-        for (int k = threadIdx.x; k < n; k += RT) {
-            const double x = pv[k];
-            la += log(fabs(x));
-            neg += (x < 0.0) + (perm[k] != k);
-        }
-        la = block_sum(la, buf);
+    T u = make_real<T>(1.0);
+    for (int k = threadIdx.x; k < n; k += RT) {
+        la += log(s_absd(pv[k]));
+        u = u * s_unit(pv[k]);
+        if (perm[k] != k) u = s_neg(u);
     }
-    __shared__ int s_neg;
-    if (threadIdx.x == 0) s_neg = 0;
+    la = block_sum(la, s_sum);
+    s_unit_part[threadIdx.x] = u;
     __syncthreads();
-    if (neg & 1) atomicXor(&s_neg, 1);
-    __syncthreads();
+    for (int h = RT / 2; h > 0; h /= 2) {
+        if (threadIdx.x < h) s_unit_part[threadIdx.x] = s_unit_part[threadIdx.x] * s_unit_part[threadIdx.x + h];
+        __syncthreads();
+    }
     if (threadIdx.x == 0) {
         const int sing = Z.sing[w];
-        const double lg = piv_rec ? la : Z.logacc[w];
-        const double sg = piv_rec ? (s_neg ? -1.0 : 1.0) : Z.sgnacc[w];
-        S.logabs[w] = sing ? -INFINITY : lg;
-        S.sgn[w] = sing ? 0.0 : s_renorm(sg);
-        if (delayed && reset_tau) S.tau[w] = 0;
-        S.pst[w] = sing ? 1 : 5;
+        if (logabs) logabs[w] = sing ? -INFINITY : la;
+        if (sgn) sgn[w] = sing ? s_zero(T()) : s_renorm(s_unit_part[0]);
+        if (tau) tau[w] = 0;
+        if (pst) pst[w] = sing ? 1 : 5;
     }
 }
 
-// Drift of the tracked inverse against the fresh one in M (relative
-// Frobenius norm; the delayed form's pending slots are applied on the fly,
-// A^{-1} = A_0^{-1} - P Q^T), then M replaces the state and tau is reset.
-__global__ void __launch_bounds__(RT) k_oz_drift_store(int n, DevLayout L, DevState<double> S, const double* M,
-                                                       const uint8_t* mask, double* drift, bool delayed) {
+// M := (M - M^T) / 2, exactly skew, by 32 x 32 tiles (tJ <= tL); block 32 x 8
+template <typename T>
+__global__ void k_oz_skew(int n, int nr, T* M, const uint8_t* mask) {
+    __shared__ T a[32][33], b[32][33];
+    const int w = blockIdx.z;
+    if ((mask && !mask[w]) || blockIdx.y > blockIdx.x) return;
+    T* Mw = M + (long long)w * nr * nr;
+    const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32, tx = threadIdx.x;
+    for (int q = threadIdx.y; q < 32; q += 8) {
+        if (i0 + q < n && j0 + tx < n) a[q][tx] = Mw[(long long)(i0 + q) * nr + j0 + tx];
+        if (j0 + q < n && i0 + tx < n) b[q][tx] = Mw[(long long)(j0 + q) * nr + i0 + tx];
+    }
+    __syncthreads();
+    for (int q = threadIdx.y; q < 32; q += 8) {
+        // rows i < j get the half difference, rows j > i its exact negative
+        if (i0 + q < n && j0 + tx < n && i0 + q < j0 + tx)
+            Mw[(long long)(i0 + q) * nr + j0 + tx] = s_half(a[q][tx] - b[tx][q]);
+        if (j0 + q < n && i0 + tx < n && i0 + tx <= j0 + q)
+            Mw[(long long)(j0 + q) * nr + i0 + tx] =
+                i0 + tx == j0 + q ? s_zero(T()) : s_neg(s_half(a[tx][q] - b[q][tx]));
+    }
+}
+
+// The fresh inverses in M (rows of nr) become the state of walkers w0 + blockIdx.x;
+// with drift, the relative Frobenius distance of the tracked inverse first (the
+// delayed form's pending slots applied on the fly, A^{-1} = A_0^{-1} -/+ P Q^T).
+// A warp per row, VR scalars per load, four loads of each stream in flight.
+// (The column permutation stays in k_oz_finish: folded in here, through shared
+// memory, the barriers between the rows cost 16 ms at 512 walkers, n = 1024,
+// against 1.7 ms for its own pass.)
+constexpr int ST = 1024;
+template <typename T, int VR>
+__global__ void __launch_bounds__(ST) k_oz_store(int w0, int n, int nr, DevLayout L, DevState<T> S, OzWork Z,
+                                                 const uint8_t* mask, double* drift, bool delayed, bool pf) {
+    struct alignas(VR * sizeof(T)) V { T e[VR]; };
     __shared__ double s_red[32];
-    const int w = blockIdx.x;
-    if (mask && !mask[w]) return;
-    const long long off = (long long)w * n * n;
+    const int w = w0 + blockIdx.x;
+    if (mask && !mask[blockIdx.x]) return;
+    T* G = S.G + (long long)w * n * n;
+    const T* Mw = reinterpret_cast<const T*>(Z.M) + (long long)blockIdx.x * nr * nr;
     const long long vo = (long long)w * n;
-    const int cu = delayed ? S.tau[w] * L.kk : 0;
+    const int cu = delayed ? S.tau[w] * L.kk : 0, lane = threadIdx.x & 31;
     double num = 0.0, den = 0.0;
-    for (long long e = threadIdx.x; e < (long long)n * n; e += RT) {
-        const int l = (int)(e / n), j = (int)(e % n);   // storage [l * n + j] = (A^{-1})_{jl}
-        double tr = S.G[off + e];
-        if (cu) {
-            const double* pr = S.P + (vo + j) * L.Kc;
-            const double* qr = S.Q + (vo + l) * L.Kc;
-            double sm = 0.0;
-            for (int c = 0; c < cu; ++c) sm = fma(pr[c], qr[c], sm);
-            tr -= sm;
+    for (int l = threadIdx.x >> 5; l < n; l += ST / 32) {
+        const T* mrow = Mw + (long long)l * nr;   // [l][j] = (A^{-1})_{jl}
+        T* grow = G + (long long)l * n;
+#pragma unroll 4
+        for (int j = lane * VR; j < n; j += 32 * VR) {
+            const V f = *reinterpret_cast<const V*>(mrow + j);
+            if (drift) {
+                V tr = *reinterpret_cast<const V*>(grow + j);
+#pragma unroll
+                for (int r = 0; r < VR; ++r) {
+                    if (cu) {
+                        const T *pr = S.P + (vo + j + r) * L.Kc, *qr = S.Q + (vo + l) * L.Kc;
+                        T sum = s_zero(T());
+                        for (int c = 0; c < cu; ++c) sum = s_fma(pr[c], qr[c], sum);
+                        tr.e[r] = pf ? tr.e[r] + sum : tr.e[r] - sum;
+                    }
+                    num += (double)s_abs2(tr.e[r] - f.e[r]);
+                    den += (double)s_abs2(f.e[r]);
+                }
+            }
+            *reinterpret_cast<V*>(grow + j) = f;
         }
-        const double f = M[off + e];
-        num += (tr - f) * (tr - f);
-        den += f * f;
-        S.G[off + e] = f;
     }
-    num = block_sum(num, s_red);
-    den = block_sum(den, s_red);
-    if (threadIdx.x == 0) {
-        if (drift) drift[w] = den > 0 ? sqrt(num / den) : 0.0;
-        if (delayed) S.tau[w] = 0;
+    if (drift) {
+        num = block_sum(num, s_red);
+        den = block_sum(den, s_red);
+        if (threadIdx.x == 0) drift[w] = den > 0 ? sqrt(num / den) : 0.0;
     }
+    if (delayed && threadIdx.x == 0) S.tau[w] = 0;
 }
 
-void launch_oz_drift_store(int W, int n, const DevLayout& L, const DevState<double>& S, const double* M,
-                           const uint8_t* mask, double* drift, bool delayed, cudaStream_t st) {
-    k_oz_drift_store<<<W, RT, 0, st>>>(n, L, S, M, mask, drift, delayed);
+template <typename T>
+void launch_oz_load(int W, int n, int nr, const T* A, bool transpose, bool sort, const OzWork& Z, const uint8_t* mask,
+                    cudaStream_t st) {
+    if (sort) cudaMemsetAsync(Z.rmax, 0, (size_t)W * nr * sizeof(int), st);
+    k_oz_load<T><<<dim3(nr / 32, nr / 32, W), dim3(32, 8), 0, st>>>(n, nr, A, transpose, sort, Z, mask);
 }
 
-void launch_oz_load(int W, int n, const double* A, double* M, const uint8_t* mask, cudaStream_t st) {
-    k_oz_load<<<dim3(n / 32, n / 32, W), dim3(32, 8), 0, st>>>(n, A, M, mask);
+void launch_oz_sort(int W, int n, int nr, const OzWork& Z, const uint8_t* mask, cudaStream_t st) {
+    k_oz_sort<<<(W + 7) / 8, 256, 0, st>>>(W, n, nr, Z, mask);
 }
 
-int oz_subpanel_width(int n) { return n <= 1024 ? 16 : 8; }
+template <typename T> int oz_subpanel_width(int nr) { return (nr <= 1024 ? 16 : 8) / (traits<T>::is_complex ? 2 : 1); }
 
-bool launch_oz_subpanel(int W, int n, int k0, int sp, const OzWork& Z, const uint8_t* mask, cudaStream_t st) {
-    if (n <= 512) {
-        k_oz_subpanel_rows<1, 16><<<W, n, 0, st>>>(n, k0, sp, Z, mask);
-        return true;
+template <typename T>
+void launch_oz_subpanel(int W, int nr, int k0, int sp, bool lu, const OzWork& Z, const uint8_t* mask, cudaStream_t st) {
+    constexpr int CX = traits<T>::is_complex ? 2 : 1;
+    if (nr <= 512) k_oz_subpanel_rows<T, 1, 16 / CX><<<W, nr, 0, st>>>(nr, k0, sp, lu, Z, mask);
+    else if (nr <= 1024) k_oz_subpanel_rows<T, 2, 16 / CX><<<W, nr / 2, 0, st>>>(nr, k0, sp, lu, Z, mask);
+    // four rows of half as many sub-panel columns per thread keep the registers
+    else k_oz_subpanel_rows<T, 4, 8 / CX><<<W, nr / 4, 0, st>>>(nr, k0, sp, lu, Z, mask);
+}
+
+template <typename T>
+void launch_oz_finish(int W, int n, int nr, bool permute, const OzWork& Z, const uint8_t* mask, double* logabs, T* sgn,
+                      int* pst, int* tau, cudaStream_t st) {
+    const int dyn = (int)(4 * n * sizeof(T) + n * sizeof(int));
+    cudaFuncSetAttribute(k_oz_finish<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    k_oz_finish<T><<<W, RT, dyn, st>>>(n, nr, permute, Z, mask, logabs, sgn, pst, tau);
+}
+
+template <typename T>
+void launch_oz_skew(int W, int n, int nr, double* M, const uint8_t* mask, cudaStream_t st) {
+    const int nt = (n + 31) / 32;
+    k_oz_skew<T><<<dim3(nt, nt, W), dim3(32, 8), 0, st>>>(n, nr, reinterpret_cast<T*>(M), mask);
+}
+
+template <typename T>
+void launch_oz_store(int W, int w0, int n, int nr, const DevLayout& L, const DevState<T>& S, const OzWork& Z,
+                     const uint8_t* mask, double* drift, bool delayed, bool pf, cudaStream_t st) {
+    if constexpr (!traits<T>::is_complex) {
+        if (n % 2 == 0) {   // rows of both matrices start on 16-byte boundaries
+            k_oz_store<T, 2><<<W, ST, 0, st>>>(w0, n, nr, L, S, Z, mask, drift, delayed, pf);
+            return;
+        }
     }
-    if (n <= 1024) {
-        k_oz_subpanel_rows<2, 16><<<W, n / 2, 0, st>>>(n, k0, sp, Z, mask);
-        return true;
-    }
-    if (n <= OZ_SUBPANEL_MAX_N && n % 4 == 0) {
-        // four rows of eight sub-panel columns per thread keep the registers
-        // of the 16-column form
-        k_oz_subpanel_rows<4, 8><<<W, n / 4, 0, st>>>(n, k0, sp, Z, mask);
-        return true;
-    }
-    return false;
+    k_oz_store<T, 1><<<W, ST, 0, st>>>(w0, n, nr, L, S, Z, mask, drift, delayed, pf);
 }
 
-void launch_oz_panel(int W, int w0, int n, int k0, const OzWork& Z, const uint8_t* mask, cudaStream_t st) {
-    const int dyn = (int)sizeof(GJSmem<double>);
-    cudaFuncSetAttribute(k_oz_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    k_oz_panel<<<W, RT, dyn, st>>>(n, k0, w0, Z, mask);
-}
-
-void launch_oz_finish(int W, int n, const OzWork& Z, const DevState<double>& S, const uint8_t* mask, bool delayed,
-                      bool reset_tau, cudaStream_t st) {
-    const int dyn = (int)(4 * n * sizeof(double) + n * sizeof(int));
-    cudaFuncSetAttribute(k_oz_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    k_oz_finish<<<W, RT, dyn, st>>>(n, Z, S, mask, delayed, reset_tau);
-}
+#define LRU_INST_OZ(T)                                                                                       \
+    template int oz_subpanel_width<T>(int);                                                                  \
+    template void launch_gj_compact<T>(int, int, int, const T*, T*, const uint8_t*, cudaStream_t);           \
+    template void launch_oz_load<T>(int, int, int, const T*, bool, bool, const OzWork&, const uint8_t*,       \
+                                    cudaStream_t);                                                           \
+    template void launch_oz_subpanel<T>(int, int, int, int, bool, const OzWork&, const uint8_t*, cudaStream_t);  \
+    template void launch_oz_finish<T>(int, int, int, bool, const OzWork&, const uint8_t*, double*, T*, int*,     \
+                                      int*, cudaStream_t);                                                   \
+    template void launch_oz_skew<T>(int, int, int, double*, const uint8_t*, cudaStream_t);                   \
+    template void launch_oz_store<T>(int, int, int, int, const DevLayout&, const DevState<T>&, const OzWork&, \
+                                     const uint8_t*, double*, bool, bool, cudaStream_t);
+LRU_INST_OZ(double)
+LRU_INST_OZ(c128)
 
 #define LRU_INST_R(T)                                                                                       \
     template void launch_refresh<T>(bool, bool, const DevLayout&, const DevState<T>&, const T*,            \
                                     const uint8_t*, T*, int, double*, bool, cudaStream_t);                 \
     template void launch_slogpf<T>(const DevLayout&, const T*, const uint8_t*, T*, int, double*, T*,       \
                                    cudaStream_t);                                                          \
-    template void launch_slogdet<T>(int, int, const T*, T*, int, double*, T*, cudaStream_t);
+    template void launch_slogdet<T>(int, int, const T*, T*, int, double*, T*, const uint8_t*, cudaStream_t);
 
 LRU_INST_R(double)
 LRU_INST_R(float)
@@ -923,10 +1034,10 @@ extern "C" lru_status lru_slogdet_batched_noalloc(int32_t dtype, int64_t W, int3
     slots = std::min<long long>(slots, std::min<long long>(W, 2LL * nsm));
     cudaStream_t st = (cudaStream_t)stream;
     switch (dtype) {
-        case LRU_F64: launch_slogdet<double>((int)W, n, (const double*)A, (double*)ws, (int)slots, logabs, (double*)sign, st); break;
-        case LRU_C128: launch_slogdet<c128>((int)W, n, (const c128*)A, (c128*)ws, (int)slots, logabs, (c128*)sign, st); break;
-        case LRU_F32: launch_slogdet<float>((int)W, n, (const float*)A, (float*)ws, (int)slots, logabs, (float*)sign, st); break;
-        case LRU_C64: launch_slogdet<c64>((int)W, n, (const c64*)A, (c64*)ws, (int)slots, logabs, (c64*)sign, st); break;
+        case LRU_F64: launch_slogdet<double>((int)W, n, (const double*)A, (double*)ws, (int)slots, logabs, (double*)sign, nullptr, st); break;
+        case LRU_C128: launch_slogdet<c128>((int)W, n, (const c128*)A, (c128*)ws, (int)slots, logabs, (c128*)sign, nullptr, st); break;
+        case LRU_F32: launch_slogdet<float>((int)W, n, (const float*)A, (float*)ws, (int)slots, logabs, (float*)sign, nullptr, st); break;
+        case LRU_C64: launch_slogdet<c64>((int)W, n, (const c64*)A, (c64*)ws, (int)slots, logabs, (c64*)sign, nullptr, st); break;
     }
     return cudaGetLastError() == cudaSuccess ? LRU_OK : LRU_ERR_CUDA;
 }

@@ -94,52 +94,56 @@ __device__ __forceinline__ void oz_digits(long long X, uint16_t (&h)[OZ_S]) {
     }
 }
 
-// Rows of (Pan - E): row i of walker w, the width (<= 64) columns c0 .. of M,
-// minus 1 at (c0 + c, c); columns past the width are zero.  One warp per row;
-// lane covers c = lane and lane + 32.  A width of at most 16 (a sub-panel)
-// feeds a single K-step of 16, which reads only the first 16 columns of each
-// slice row, so only those are written.
-__global__ void __launch_bounds__(256) k_oz_slice_P(int n, int c0, int width, int w0, OzWork Z,
+// A walker's working matrix M has nr rows of nc doubles: nc = nr for real
+// scalars and 2 nr for complex ones (CX = 2: re, im interleaved).  A complex
+// update sum_c p_c s_c is two real ones of the interleaved row (re p, im p):
+// against (re s, -im s) for the real part, (im s, re s) for the imaginary one.
+// So the panel rows are sliced as they lie, the S columns twice, and the same
+// 64-wide products serve 64 real or 32 complex panel columns.
+
+// Rows of (Pan - E) from row i_lo: the width (<= 64) doubles c0 .. of M's row i,
+// minus 1 at the diagonal; columns past the width are zero.  One warp per row;
+// lane covers c = lane and lane + 32.
+__global__ void __launch_bounds__(256) k_oz_slice_P(int nr, int nc, int cx, int i_lo, int c0, int width, OzWork Z,
                                                     const uint8_t* mask) {
-    const int w = w0 + blockIdx.y;
+    const int w = blockIdx.y;
     if (mask && !mask[w]) return;
     const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (i >= n) return;
-    const double* row = Z.M + (long long)w * n * n + (long long)i * n + c0;
+    const int i = i_lo + blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= nr) return;
+    const double* row = Z.M + (long long)w * nr * nc + (long long)i * nc + c0;
     double a = lane < width ? row[lane] : 0.0, b = lane + 32 < width ? row[lane + 32] : 0.0;
-    if (lane < width && i == c0 + lane) a -= 1.0;
-    if (lane + 32 < width && i == c0 + lane + 32) b -= 1.0;
+    if (lane < width && i * cx == c0 + lane) a -= 1.0;
+    if (lane + 32 < width && i * cx == c0 + lane + 32) b -= 1.0;
     const int mx = __reduce_max_sync(0xffffffffu, max(oz_bexp(a), oz_bexp(b)));
     const int E = mx > 0 ? mx - 1022 : 0;
     uint16_t ha[OZ_S], hb[OZ_S];
     oz_digits(oz_fixed(a, E), ha);
     oz_digits(oz_fixed(b, E), hb);
-    const bool full = width > 16;
 #pragma unroll
     for (int t = 0; t < OZ_S; ++t) {
-        uint16_t* dst = Z.Pb + (((long long)w * OZ_S + t) * n + i) * OZ_B;
-        if (full || lane < 16) dst[lane] = ha[t];
-        if (full) dst[lane + 32] = hb[t];
+        uint16_t* dst = Z.Pb + (((long long)w * OZ_S + t) * nr + i) * OZ_B;
+        dst[lane] = ha[t];
+        dst[lane + 32] = hb[t];
     }
-    if (lane == 0) Z.eP[(long long)w * n + i] = E;
+    if (lane == 0) Z.eP[(long long)w * nr + i] = E;
 }
 
-// The same rows for a sub-panel (width <= 16): half a warp per row, lane c of
-// the half covering column c, so no lane splits a zero.  Writes the first 16
-// entries of each slice row and the row's exponent, exactly as k_oz_slice_P.
-// n is a multiple of 16, so both halves of a warp always have a row.
-__global__ void __launch_bounds__(256) k_oz_slice_P16(int n, int c0, int width, int w0, OzWork Z,
+// The same rows for a sub-panel (16 doubles or fewer): half a warp per row, lane c
+// of the half covering column c, so no lane splits a zero.  Such a width feeds a
+// single K-step of 16, which reads only the first 16 columns of each slice row,
+// so only those are written.  nr - i_lo is a multiple of 16.
+__global__ void __launch_bounds__(256) k_oz_slice_P16(int nr, int nc, int cx, int i_lo, int c0, int width, OzWork Z,
                                                       const uint8_t* mask) {
-    const int w = w0 + blockIdx.y;
+    const int w = blockIdx.y;
     if (mask && !mask[w]) return;
     const int c = threadIdx.x & 15;
-    const int i = blockIdx.x * 16 + (threadIdx.x >> 4);
+    const int i = i_lo + blockIdx.x * 16 + (threadIdx.x >> 4);
     const unsigned hmask = 0xFFFFu << (threadIdx.x & 16);   // this half of the warp
-    const bool ok = i < n;
-    const double* row = Z.M + (long long)w * n * n + (long long)i * n + c0;
+    const bool ok = i < nr;
+    const double* row = Z.M + (long long)w * nr * nc + (long long)i * nc + c0;
     double a = (ok && c < width) ? row[c] : 0.0;
-    if (c < width && i == c0 + c) a -= 1.0;
+    if (c < width && i * cx == c0 + c) a -= 1.0;
     int mx = oz_bexp(a);
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(hmask, mx, o));
@@ -148,24 +152,32 @@ __global__ void __launch_bounds__(256) k_oz_slice_P16(int n, int c0, int width, 
     oz_digits(oz_fixed(a, E), ha);
     if (!ok) return;
 #pragma unroll
-    for (int t = 0; t < OZ_S; ++t) Z.Pb[(((long long)w * OZ_S + t) * n + i) * OZ_B + c] = ha[t];
-    if (c == 0) Z.eP[(long long)w * n + i] = E;
+    for (int t = 0; t < OZ_S; ++t) Z.Pb[(((long long)w * OZ_S + t) * nr + i) * OZ_B + c] = ha[t];
+    if (c == 0) Z.eP[(long long)w * nr + i] = E;
 }
 
-// Columns of S = the nr (<= 64) rows r0 .. of M, zero past nr: a 64 x 64
-// block per CTA (column blocks jb0, jb0 + 1, ..) through shared memory
-// (stored transposed), then one warp per column j.  As for the panel rows,
-// nr <= 16 writes only the first 16 entries of each slice row.
-__global__ void __launch_bounds__(256) k_oz_slice_S(int n, int r0, int nr, int jb0, int w0, OzWork Z,
+// Columns of S = the rows r0 .. r0 + rows - 1 of M (rows * CX <= 64), zero past
+// them: 64 doubles of each row per CTA (column blocks jb0, jb0 + 1, ..) through
+// shared memory (stored transposed), then one warp per real column j.  At most
+// 16 doubles write only the first 16 entries of each slice row.
+template <int CX>
+__global__ void __launch_bounds__(256) k_oz_slice_S(int nr, int nc, int r0, int rows, int jb0, OzWork Z,
                                                     const uint8_t* mask) {
     __shared__ double sT[64][65];   // sT[j][c] = S[c][j0 + j]
-    const int w = w0 + blockIdx.y;
+    const int w = blockIdx.y;
     if (mask && !mask[w]) return;
-    const int j0 = (jb0 + blockIdx.x) * 64;
-    const double* M = Z.M + (long long)w * n * n;
-    for (int e = threadIdx.x; e < 64 * 64; e += 256) {
+    const int j0 = (jb0 + blockIdx.x) * 64, width = rows * CX;
+    if (j0 >= nc) return;
+    const double* M = Z.M + (long long)w * nr * nc;
+    for (int e = threadIdx.x; e < 64 * 64 / CX; e += 256) {
         const int c = e >> 6, j = e & 63;
-        sT[j][c] = c < nr ? M[(long long)(r0 + c) * n + j0 + j] : 0.0;
+        const double v = c < rows ? M[(long long)(r0 + c) * nc + j0 + j] : 0.0;
+        if constexpr (CX == 1) {
+            sT[j][c] = v;
+        } else {
+            sT[j][2 * c] = v;                              // re: (re s, .); im: (im s, .)
+            sT[j ^ 1][2 * c + 1] = (j & 1) ? -v : v;       // (., -im s) and (., re s)
+        }
     }
     __syncthreads();
     const int lane = threadIdx.x & 31;
@@ -178,11 +190,11 @@ __global__ void __launch_bounds__(256) k_oz_slice_S(int n, int r0, int nr, int j
         oz_digits(oz_fixed(b, E), hb);
 #pragma unroll
         for (int t = 0; t < OZ_S; ++t) {
-            uint16_t* dst = Z.Sb + (((long long)w * OZ_S + t) * n + j0 + j) * OZ_B;
-            if (nr > 16 || lane < 16) dst[lane] = ha[t];
-            if (nr > 16) dst[lane + 32] = hb[t];
+            uint16_t* dst = Z.Sb + (((long long)w * OZ_S + t) * nc + j0 + j) * OZ_B;
+            if (width > 16 || lane < 16) dst[lane] = ha[t];
+            if (width > 16) dst[lane + 32] = hb[t];
         }
-        if (lane == 0) Z.eS[(long long)w * n + j0 + j] = E;
+        if (lane == 0) Z.eS[(long long)w * nc + j0 + j] = E;
     }
 }
 
@@ -220,7 +232,7 @@ constexpr int OZ_THREADS = 512;   // 16 warps: 4 per TMEM lane quarter, each 16 
 
 template <int NKS>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_oz_gemm(const __grid_constant__ OzMaps maps, int W, int w0, int n, OzCols cols, OzWork Z,
+    k_oz_gemm(const __grid_constant__ OzMaps maps, int W, int nr, int nc, OzCols cols, OzWork Z,
               const uint8_t* mask, int* err) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -248,19 +260,21 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const uint32_t tmem = s_tmem;
     const uint32_t mb_tma = smem_u32(&mbar[0]), mb_mma = smem_u32(&mbar[1]);
     const uint32_t bytes_a = (uint32_t)OZ_S * OZ_SLICE_A, bytes_b = (uint32_t)OZ_S * OZ_SLICE_B;
-    const int ntj = cols.jt_hi - cols.jt_lo, nti = n / OZ_TI;
+    const int ntj = cols.jt_hi - cols.jt_lo, nti = nr / OZ_TI;
     const long long units = (long long)W * ntj;
     uint32_t ph_tma = 0, ph_mma = 0;
     for (long long un = blockIdx.x; un < units && !s_abort; un += gridDim.x) {
-        const int w = w0 + (int)(un / ntj);
+        const int w = (int)(un / ntj);
         if (mask && !mask[w]) continue;
         const int j0 = (cols.jt_lo + (int)(un % ntj)) * OZ_TJ;
-        const int ys = (int)((long long)w * OZ_S * n);
+        // rows past the walker's last column (a 128-wide tile at nc % 128 == 64) are
+        // the next slice's or zero, and their products are not kept
+        const int ys = (int)((long long)w * OZ_S * nc), yp = (int)((long long)w * OZ_S * nr) + cols.it_lo * OZ_TI;
         if (tid == 0) {
             mbar_expect_tx(mb_tma, bytes_a + bytes_b);
             for (int t = 0; t < OZ_S; ++t) {
-                tma_load_2d(smem_u32(sA + t * OZ_SLICE_A), &maps.S, 0, ys + t * n + j0, mb_tma);
-                tma_load_2d(smem_u32(sB + t * OZ_SLICE_B), &maps.P, 0, ys + t * n, mb_tma);
+                tma_load_2d(smem_u32(sA + t * OZ_SLICE_A), &maps.S, 0, ys + t * nc + j0, mb_tma);
+                tma_load_2d(smem_u32(sB + t * OZ_SLICE_B), &maps.P, 0, yp + t * nr, mb_tma);
             }
         }
         // per thread of the epilogue: column j (TMEM lane) and its scale
@@ -268,10 +282,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const int j = j0 + 32 * quad + lane;
         const bool keep = j >= cols.c_lo && j < cols.c_hi && !(j >= cols.s_lo && j < cols.s_hi);
         const bool wact = __any_sync(0xffffffffu, keep);   // a warp with no column to write skips its epilogue
-        const int eSj = Z.eS[(long long)w * n + j];
-        double* Mw = Z.M + (long long)w * n * n;
-        const int* eP = Z.eP + (long long)w * n;
-        for (int it = 0; it < nti; ++it) {
+        const int eSj = j < nc ? Z.eS[(long long)w * nc + j] : 0;
+        double* Mw = Z.M + (long long)w * nr * nc;
+        const int* eP = Z.eP + (long long)w * nr;
+        for (int it = cols.it_lo; it < nti; ++it) {
             const int i0 = it * OZ_TI;
             if (tid == 0) {
                 if (!mbar_wait(mb_tma, ph_tma)) {
@@ -307,7 +321,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             // overlap the MMAs
             double m[16];
 #pragma unroll
-            for (int c = 0; c < 16; ++c) m[c] = keep ? Mw[(long long)(i0 + 16 * part + c) * n + j] : 0.0;
+            for (int c = 0; c < 16; ++c) m[c] = keep ? Mw[(long long)(i0 + 16 * part + c) * nc + j] : 0.0;
             __syncthreads();
             if (s_abort) break;
             if (!mbar_wait(mb_mma, ph_mma)) {
@@ -322,7 +336,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             if (tid == 0 && it + 1 < nti) {
                 mbar_expect_tx(mb_tma, bytes_b);
                 for (int t = 0; t < OZ_S; ++t)
-                    tma_load_2d(smem_u32(sB + t * OZ_SLICE_B), &maps.P, 0, ys + t * n + i0 + OZ_TI, mb_tma);
+                    tma_load_2d(smem_u32(sB + t * OZ_SLICE_B), &maps.P, 0, yp + t * nr + (it + 1 - cols.it_lo) * OZ_TI, mb_tma);
             }
             // ---- epilogue: warp q reads TMEM lanes 32 (q % 4) .. +31 (columns j),
             //      and rows i0 + 16 (q / 4) .. +15 in two chunks of 8 ----
@@ -347,7 +361,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                     const long long F = ((long long)(n2 * 256 + n3) << 32) + ((long long)(n4 * 256 + n5) << 16) +
                                         ((long long)n6 << 8) + tl;
                     const double d = oz_i64_to_double(F, eP[i0 + c0 + c] + eSj);
-                    if (keep) Mw[(long long)(i0 + c0 + c) * n + j] = m[8 * ch + c] + d;
+                    if (keep) Mw[(long long)(i0 + c0 + c) * nc + j] = m[8 * ch + c] + d;
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -440,39 +454,31 @@ __global__ void __launch_bounds__(256) k_oz_slice_rows(int W, int n, int ldx, in
 
 // ---- host side ----------------------------------------------------------------
 
-size_t oz_work_bytes(int W, int n) {
-    const size_t Wn = (size_t)W * n;
-    size_t b = 0;
-    auto take = [&](size_t x) { b += (x + 255) / 256 * 256; };
-    take(Wn * sizeof(int));                        // perm
-    take((size_t)W * sizeof(double));              // logacc
-    take((size_t)W * sizeof(double));              // sgnacc
-    take((size_t)W * sizeof(int));                 // sing
-    take(Wn * OZ_S * OZ_B * sizeof(uint16_t));     // Sb
-    take(Wn * OZ_S * OZ_B * sizeof(uint16_t));     // Pb
-    take(Wn * sizeof(int));                        // eS
-    take(Wn * sizeof(int));                        // eP
-    take((size_t)W);                               // go
-    take(Wn * sizeof(double));                     // piv
-    take((size_t)W * OZ_B * sizeof(int));          // cs
-    return b;
-}
+int oz_rows(int n) { return n <= 1024 ? (n + 63) / 64 * 64 : (n + 127) / 128 * 128; }
 
-void oz_work_carve(OzWork& Z, void* base, int W, int n) {
-    const size_t Wn = (size_t)W * n;
-    unsigned char* p = (unsigned char*)base;
-    auto take = [&](size_t x) { unsigned char* q = p; p += (x + 255) / 256 * 256; return q; };
-    Z.perm = (int*)take(Wn * sizeof(int));
-    Z.logacc = (double*)take((size_t)W * sizeof(double));
-    Z.sgnacc = (double*)take((size_t)W * sizeof(double));
-    Z.sing = (int*)take((size_t)W * sizeof(int));
-    Z.Sb = (uint16_t*)take(Wn * OZ_S * OZ_B * sizeof(uint16_t));
-    Z.Pb = (uint16_t*)take(Wn * OZ_S * OZ_B * sizeof(uint16_t));
-    Z.eS = (int*)take(Wn * sizeof(int));
-    Z.eP = (int*)take(Wn * sizeof(int));
-    Z.go = (uint8_t*)take((size_t)W);
-    Z.piv = (double*)take(Wn * sizeof(double));
-    Z.cs = (int*)take((size_t)W * OZ_B * sizeof(int));
+size_t oz_work_layout(OzWork* Z, void* base, int W, int nr, int cx, bool with_M) {
+    const size_t Wr = (size_t)W * nr, Wc = Wr * cx;
+    size_t off = 0;
+    auto take = [&](size_t x) {
+        unsigned char* q = base ? (unsigned char*)base + off : nullptr;
+        off += (x + 255) / 256 * 256;
+        return q;
+    };
+    OzWork z{};
+    z.perm = (int*)take(Wr * sizeof(int));
+    z.sing = (int*)take((size_t)W * sizeof(int));
+    z.Sb = (uint16_t*)take(Wc * OZ_S * OZ_B * sizeof(uint16_t));
+    z.Pb = (uint16_t*)take(Wr * OZ_S * OZ_B * sizeof(uint16_t));
+    z.eS = (int*)take(Wc * sizeof(int));
+    z.eP = (int*)take(Wr * sizeof(int));
+    z.go = (uint8_t*)take((size_t)W);
+    z.odd = (uint8_t*)take((size_t)W);
+    z.piv = (double*)take(Wc * sizeof(double));
+    z.cs = (int*)take((size_t)W * OZ_B * sizeof(int));
+    z.rmax = (int*)take(Wr * sizeof(int));
+    if (with_M) z.M = (double*)take(Wr * nr * cx * sizeof(double));
+    if (Z) *Z = z;
+    return off;
 }
 
 // rows x 64 BF16 matrix, box 64 x box_rows, SWIZZLE_128B
@@ -488,16 +494,19 @@ static bool oz_map(CUtensorMap* m, const void* base, long long rows, int box_row
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The whole refresh of the selected walkers: M = A^T (Z.M is the state's
-// A^{-1} storage), n / 64 panels, then the column permutation and log|det|.
-// Needs n % 128 == 0, 128 <= n <= 2048 and W <= 65535 (checked by the caller).
-bool launch_refresh_oz(int W, int n, const double* A, const OzWork& Z, const DevState<double>& S,
-                       const uint8_t* mask, bool delayed, bool reset_tau, int* err, cudaStream_t st,
-                       void (*hook)(void*, int, int), void* hctx) {
-    const long long rows = (long long)W * OZ_S * n;
-    if (rows >= (1ll << 31)) return false;
+// Gauss-Jordan elimination of the W matrices Z.M (nr rows, nr % 64 == 0 up to
+// 1024, % 128 above) of the walkers with mask[w] (NULL: all): the row exchanges
+// stay in Z.perm, the pivots in Z.piv.  lu: rows above a panel and columns left
+// of it are left alone (a third of the work), enough for the determinant.
+template <typename T>
+bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, int* err, cudaStream_t st,
+                  void (*hook)(void*, int, int), void* hctx) {
+    constexpr int CX = traits<T>::is_complex ? 2 : 1, PB = OZ_B / CX;
+    const int nc = nr * CX;
+    const long long rows = (long long)W * OZ_S * nc;
+    if (rows >= (1ll << 31) || W > 65535) return false;
     OzMaps maps;
-    if (!oz_map(&maps.S, Z.Sb, rows, OZ_TJ) || !oz_map(&maps.P, Z.Pb, rows, OZ_TI)) return false;
+    if (!oz_map(&maps.S, Z.Sb, rows, OZ_TJ) || !oz_map(&maps.P, Z.Pb, (long long)W * OZ_S * nr, OZ_TI)) return false;
     const size_t dyn = 1024 + (size_t)OZ_S * (OZ_SLICE_A + OZ_SLICE_B);
     if (cudaFuncSetAttribute(k_oz_gemm<OZ_B / 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) !=
             cudaSuccess ||
@@ -508,33 +517,50 @@ bool launch_refresh_oz(int W, int n, const double* A, const OzWork& Z, const Dev
     int dev = 0, nsm = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    launch_oz_load(W, n, A, Z.M, mask, st);
-    const int SW = oz_subpanel_width(n);   // sub-panel width
-    for (int k0 = 0; k0 < n; k0 += OZ_B) {
+    const int SW = oz_subpanel_width<T>(nr);   // sub-panel width
+    const int ntj = (nc + OZ_TJ - 1) / OZ_TJ;
+    for (int k0 = 0; k0 < nr; k0 += PB) {
         if (hook) hook(hctx, 4, 1);
-        if (n <= OZ_SUBPANEL_MAX_N) {
-            // sub-panels: FP64 elimination, then the update of the other panel
-            // columns as a one-K-step split product on the panel's 128-column tile
-            const int jt = k0 / OZ_TJ;
-            for (int sp = 0; sp < OZ_B / SW; ++sp) {
-                const int ks = k0 + SW * sp;
-                launch_oz_subpanel(W, n, k0, sp, Z, mask, st);
-                k_oz_slice_P16<<<dim3(n / 16, W), 256, 0, st>>>(n, ks, SW, 0, Z, mask);
-                k_oz_slice_S<<<dim3(OZ_TJ / 64, W), 256, 0, st>>>(n, ks, SW, jt * (OZ_TJ / 64), 0, Z, mask);
-                const OzCols inner{k0, k0 + OZ_B, ks, ks + SW, jt, jt + 1};
-                k_oz_gemm<1><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, 0, n, inner, Z, mask, err);
-            }
-        } else {
-            launch_oz_panel(W, 0, n, k0, Z, mask, st);
+        // sub-panels: FP64 elimination, then the update of the other panel
+        // columns as a one-K-step split product on the panel's 128-column tile
+        const int c0 = k0 * CX, jt = c0 / OZ_TJ;
+        const int it0 = lu ? k0 / OZ_TI : 0, i0 = it0 * OZ_TI;
+        for (int sp = 0; sp < PB / SW; ++sp) {
+            const int ks = k0 + SW * sp;
+            launch_oz_subpanel<T>(W, nr, k0, sp, lu, Z, mask, st);
+            k_oz_slice_P16<<<dim3((nr - i0) / 16, W), 256, 0, st>>>(nr, nc, CX, i0, ks * CX, SW * CX, Z, mask);
+            k_oz_slice_S<CX><<<dim3(1, W), 256, 0, st>>>(nr, nc, ks, SW, c0 / 64, Z, mask);
+            const OzCols inner{c0, c0 + OZ_B, ks * CX, (ks + SW) * CX, jt, jt + 1, it0};
+            k_oz_gemm<1><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, inner, Z, mask, err);
         }
         if (hook) { hook(hctx, 4, 0); hook(hctx, 5, 1); }
-        k_oz_slice_P<<<dim3(n / 8, W), 256, 0, st>>>(n, k0, OZ_B, 0, Z, mask);
-        k_oz_slice_S<<<dim3(n / 64, W), 256, 0, st>>>(n, k0, OZ_B, 0, 0, Z, mask);
-        const OzCols outer{0, n, k0, k0 + OZ_B, 0, n / OZ_TJ};
-        k_oz_gemm<OZ_B / 16><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, 0, n, outer, Z, mask, err);
+        const int kn = k0 + PB, itn = lu ? kn / OZ_TI : 0, in = itn * OZ_TI, cl = lu ? kn * CX : 0;
+        if (!lu || kn < nr) {
+            k_oz_slice_P<<<dim3((nr - in) / 8, W), 256, 0, st>>>(nr, nc, CX, in, c0, OZ_B, Z, mask);
+            k_oz_slice_S<CX><<<dim3((nc - cl) / 64, W), 256, 0, st>>>(nr, nc, k0, PB, cl / 64, Z, mask);
+            const OzCols outer{cl, nc, c0, c0 + OZ_B, cl / OZ_TJ, ntj, itn};
+            k_oz_gemm<OZ_B / 16><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, outer, Z, mask, err);
+        }
         if (hook) hook(hctx, 5, 0);
     }
-    launch_oz_finish(W, n, Z, S, mask, delayed, reset_tau, st);
+    return true;
+}
+
+template bool oz_eliminate<double>(int, int, const OzWork&, const uint8_t*, bool, int*, cudaStream_t,
+                                   void (*)(void*, int, int), void*);
+template bool oz_eliminate<c128>(int, int, const OzWork&, const uint8_t*, bool, int*, cudaStream_t,
+                                 void (*)(void*, int, int), void*);
+
+// The whole refresh of the selected walkers: M = A^T, n / 64 panels, then the
+// column permutation and log|det|.  in_state: Z.M is the state's A^{-1} storage
+// and tau is reset; otherwise launch_oz_store does both.
+// Needs n % 128 == 0, 128 <= n <= 2048 and W <= 65535 (checked by the caller).
+bool launch_refresh_oz(int W, int n, const double* A, const OzWork& Z, const DevState<double>& S,
+                       const uint8_t* mask, bool delayed, bool in_state, int* err, cudaStream_t st,
+                       void (*hook)(void*, int, int), void* hctx) {
+    launch_oz_load<double>(W, n, n, A, true, false, Z, mask, st);
+    if (!oz_eliminate<double>(W, n, Z, mask, false, err, st, hook, hctx)) return false;
+    launch_oz_finish<double>(W, n, n, true, Z, mask, S.logabs, S.sgn, S.pst, delayed && in_state ? S.tau : nullptr, st);
     return true;
 }
 
@@ -583,8 +609,8 @@ bool launch_flush_split(int W, int n, int K, int Kc, int kk, const double* P, co
         case 4: kern = k_oz_gemm<4>; break;
         default: break;
     }
-    const OzCols all{0, n, -1, -1, 0, n / OZ_TJ};
-    kern<<<nsm, OZ_THREADS, dyn, st>>>(maps, W, 0, n, all, Z, Z.go, err);
+    const OzCols all{0, n, -1, -1, 0, n / OZ_TJ, 0};
+    kern<<<nsm, OZ_THREADS, dyn, st>>>(maps, W, n, n, all, Z, Z.go, err);
     return true;
 }
 
