@@ -33,12 +33,11 @@
 //     the rounding of an FP64 update, at tensor-core speed.
 // The output tile is 128 columns j (TMEM lanes, so the FP64 read-modify-write
 // of row-major M is coalesced) x 64 rows i; TMA stages the 7 S slices of a
-// column block once (112 KiB) and the 7 Pan slices of each row tile (56 KiB)
-// behind the previous tile's epilogue (SWIZZLE_128B, no multicast); one
-// thread issues the 39 MMAs x 4 K-steps.  Every wait is bounded as in the
-// delayed flush.  (Two accumulator sets for an MMA / epilogue overlap do not
-// fit the 512 TMEM columns at 64 rows; at 32 rows the MMAs, whose operands
-// are re-read from shared memory per instruction, become the bound.)
+// column block once (112 KiB) and the 7 Pan slices of each row tile (two stages
+// of 56 KiB; SWIZZLE_128B, no multicast).  Every wait is bounded as in the
+// delayed flush.  (At 32 rows, where two full accumulator sets fit, the MMAs,
+// whose operands are re-read from shared memory per instruction, become the
+// bound.)
 #include <algorithm>
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -206,29 +205,108 @@ __device__ __forceinline__ void oz_mma(uint32_t dtmem, uint64_t a, uint64_t b, u
         : "memory");
 }
 
-// F * 2^(e - 56) as a double, rounded to nearest even, by integer operations
-// (normal results only: the refresh's scales stay far from the exponent limits)
-__device__ __forceinline__ double oz_i64_to_double(long long F, int e) {
-    if (F == 0) return 0.0;
-    const unsigned long long sgn = (unsigned long long)F & 0x8000000000000000ull;
-    unsigned long long a = sgn ? (unsigned long long)(-F) : (unsigned long long)F;
-    const int lz = __clzll((long long)a);
-    a <<= lz;                                   // leading one at bit 63
-    unsigned long long mant = a >> 11;          // 53 bits
-    const unsigned r = (unsigned)(a & 0x7FFull);
-    mant += (r > 0x400u || (r == 0x400u && (mant & 1ull))) ? 1ull : 0ull;
-    int ex = 1023 + 63 - lz + e - 56;
-    if (mant >> 53) { mant >>= 1; ++ex; }
-    return __longlong_as_double((long long)(sgn | ((unsigned long long)ex << 52) | (mant & 0xFFFFFFFFFFFFFull)));
+// Levels 2 .. 6 of one element are integers N_l 2^(-8l), |N_l| < 2^23 (a float holds
+// them exactly), and the tail (levels 7 .. 10) is rounded to a multiple of 2^-56:
+// their sum F in units of 2^-56, |F| < 2^62, exactly, as two words.  N_2, N_3
+// (|N| <= 2^22) and the tail come out of the mantissa of x * scale + 1.5 * 2^23
+// (a tail above 2^22 is rounded to 2 units); the others can exceed 2^22 and take
+// the conversion unit.
+__device__ __forceinline__ void oz_sum2(float a2, float a3, int& hi) {
+    constexpr float magic = 12582912.0f;
+    const int n2 = __float_as_int(__fmaf_rn(a2, 65536.0f, magic)), n3 = __float_as_int(__fmaf_rn(a3, 16777216.0f, magic));
+    hi = n2 * 256 + n3 - (int)(0x4B400000u * 257u);
+}
+__device__ __forceinline__ void oz_sum4(float a4, float a5, int& hi, uint32_t& lo) {
+    const int b = __float2int_rn(a4 * 4294967296.0f) * 256 + __float2int_rn(a5 * 1099511627776.0f);
+    lo = (uint32_t)b << 16;
+    hi += b >> 16;
+}
+__device__ __forceinline__ void oz_sum6(float a6, float tail, int& hi, uint32_t& lo) {
+    const int c = __float2int_rn(a6 * 281474976710656.0f) * 256 +
+                  (__float_as_int(__fmaf_rn(tail, 72057594037927936.0f, 12582912.0f)) - 0x4B400000);
+    const uint32_t l = lo + (uint32_t)c;
+    hi += (c >> 31) + (l < lo ? 1 : 0);
+    lo = l;
+}
+
+// F * 2^(e - 56) as a double, rounded to nearest (ties away), by integer operations
+// (normal results only: the scales stay far from the exponent limits).  The
+// mantissa with its leading one is added to the exponent field less one, so a
+// rounding that carries out of it needs no case of its own.
+__device__ __forceinline__ double oz_to_double(int hi, uint32_t lo, int e) {
+    const int s = hi >> 31;
+    const unsigned long long F = ((unsigned long long)(uint32_t)hi << 32) | lo;
+    const unsigned long long sx = ((unsigned long long)(uint32_t)s << 32) | (uint32_t)s;
+    const unsigned long long a = (F ^ sx) - sx;   // |F|
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a;
+    const int lz = __clz((int)(ah ? ah : al)) + (ah ? 0 : 32);
+    const unsigned long long v = a << (lz & 63);                 // leading one at bit 63
+    const unsigned long long mant = (v >> 11) + ((v >> 10) & 1ull);
+    const uint32_t rh = (uint32_t)(mant >> 32) + ((uint32_t)(1029 + e - lz) << 20);
+    const bool nz = a != 0;
+    return __hiloint2double(nz ? (int)(rh | ((uint32_t)s & 0x80000000u)) : 0, nz ? (int)(uint32_t)mant : 0);
 }
 
 // M[i][j] += 2^(E_i + E_j) sum_c Pan[i][c] S[c][j] as a split product, with
 // NKS K-steps of 16 (4 for a 64-column panel, 1 for a sub-panel or the K = 16
 // flush), written only for the columns cols selects.  Persistent CTAs take
 // (walker, 128-column block) units: the 7 S slices of the block are loaded
-// once, then the 64-row tiles i stream through; the Pan slices of tile i+1
-// are loaded (TMA) while the epilogue of tile i runs.
-constexpr int OZ_THREADS = 512;   // 16 warps: 4 per TMEM lane quarter, each 16 of the 64 rows i
+// once, then the 64-row tiles i stream through.
+//
+// Run one after the other, the MMAs of a tile (with the wait for its slices) took
+// 36 ms and its epilogue 32 ms of the 66 ms that the trailing updates of a refresh
+// of 512 walkers, n = 1024 cost.  So the roles are split over warps: one thread
+// loads (two stages of Pan slices), one issues MMAs, 16 warps run the epilogue of
+// tile T while the MMAs of tile T + 1 run.  Two sets of six accumulators do not fit
+// the 512 TMEM columns; but 29 of the 39 slice products go to two of the six
+// accumulators (level 6, and the levels 7 .. 10 together), and two sets of those
+// fit beside one of the levels 2 .. 5.  The MMA thread does these 29 first and only
+// then waits for the epilogue to have read levels 2 .. 5 of the tile before, which
+// it does at once, into 64-bit sums in registers: 66 -> 46 ms (the sub-panel
+// products 27 -> 20 ms, the K = 16 flush of 1024 walkers 5.7 -> 4.9 ms).  A full
+// overlap would end at the 36 ms of the MMAs.
+constexpr int OZ_EPI_WARPS = 16;  // 4 per TMEM lane quarter, each 16 of the 64 rows i
+constexpr int OZ_THREADS = 32 * (OZ_EPI_WARPS + 2);
+constexpr size_t OZ_GEMM_SMEM = 1024 + (size_t)OZ_S * (OZ_SLICE_A + 2 * OZ_SLICE_B);
+
+// accumulator g (level g + 2; 5: the tail) of tile T
+__device__ __forceinline__ uint32_t oz_acc(uint32_t tmem, int g, uint32_t T) {
+    return tmem + 64u * (g < 4 ? (uint32_t)g : 4u + 2u * (uint32_t)(g - 4) + (T & 1u));
+}
+
+// bounded wait that also ends when another role has given up
+__device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
+    for (int i = 0; i < (1 << 20); ++i) {
+        if (mbar_try(bar, parity)) return true;
+        if (i > 64) {
+            __nanosleep(256);
+            if (*abort) return false;
+        }
+    }
+    return false;
+}
+
+// the products of tile T for accumulators g_lo .. g_hi - 1
+template <int NKS, int G_LO, int G_HI>
+__device__ __forceinline__ void oz_issue(uint32_t tmem, uint32_t T, uint64_t a0, uint64_t b0) {
+    // fully unrolled: descriptor offsets and accumulate flags are compile-time, so
+    // the issuing thread streams back-to-back MMAs
+    uint32_t started = 0;   // bit g: accumulator g holds a partial sum
+#pragma unroll
+    for (int t = 0; t < OZ_S; ++t)
+#pragma unroll
+        for (int u = 0; u < OZ_S; ++u) {
+            const int g = t + u < OZ_GROUPS - 1 ? t + u : OZ_GROUPS - 1;   // level t+u+2: 2 .. 6, then 7..10
+            if (u + t > OZ_MAXLV || g < G_LO || g >= G_HI) continue;
+            const uint64_t a = a0 + (uint64_t)((t * OZ_SLICE_A) >> 4), b = b0 + (uint64_t)((u * OZ_SLICE_B) >> 4);
+#pragma unroll
+            for (int ks = 0; ks < NKS; ++ks) {
+                const uint64_t adv = (uint64_t)(ks * 32) >> 4;   // 16 BF16 along K per MMA
+                oz_mma(oz_acc(tmem, g, T), a + adv, b + adv, (started >> g) & 1u);
+                started |= 1u << g;
+            }
+        }
+}
 
 template <int NKS>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
@@ -238,10 +316,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* sA = sm;                               // OZ_S slices of S, 128 rows each
-    unsigned char* sB = sA + OZ_S * OZ_SLICE_A;           // OZ_S slices of Pan, 64 rows each
-    __shared__ __align__(8) unsigned long long mbar[2];
+    unsigned char* sB = sA + OZ_S * OZ_SLICE_A;           // two stages of OZ_S slices of Pan, 64 rows each
+    constexpr uint32_t STAGE = (uint32_t)OZ_S * OZ_SLICE_B;
+    __shared__ __align__(8) unsigned long long mbar[8];
     __shared__ uint32_t s_tmem;
-    __shared__ int s_abort;
+    __shared__ volatile int s_abort;
+    const uint32_t m_sfull = smem_u32(&mbar[0]);          // S slices of a unit have landed
+    const uint32_t m_pfull = smem_u32(&mbar[1]);          // [2] Pan slices of a tile have landed
+    const uint32_t m_pfree = smem_u32(&mbar[3]);          // [2] the MMAs of a stage's tile are done
+    const uint32_t m_full = smem_u32(&mbar[5]);           // the accumulators of a tile are complete
+    const uint32_t m_free = smem_u32(&mbar[6]);           // the epilogue warps have read them
+    const uint32_t m_drain = smem_u32(&mbar[7]);          // (giving up) MMAs in flight are done
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                      "r"(OZ_TMEM_COLS)
@@ -249,8 +334,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        mbar_init(smem_u32(&mbar[0]), 1);
-        mbar_init(smem_u32(&mbar[1]), 1);
+        for (int i = 0; i < 8; ++i) mbar_init(smem_u32(&mbar[i]), i == 6 ? OZ_EPI_WARPS : 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_abort = 0;
     }
@@ -258,116 +342,159 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s_tmem;
-    const uint32_t mb_tma = smem_u32(&mbar[0]), mb_mma = smem_u32(&mbar[1]);
-    const uint32_t bytes_a = (uint32_t)OZ_S * OZ_SLICE_A, bytes_b = (uint32_t)OZ_S * OZ_SLICE_B;
+    const uint32_t bytes_a = (uint32_t)OZ_S * OZ_SLICE_A, bytes_b = STAGE;
     const int ntj = cols.jt_hi - cols.jt_lo, nti = nr / OZ_TI;
     const long long units = (long long)W * ntj;
-    uint32_t ph_tma = 0, ph_mma = 0;
-    for (long long un = blockIdx.x; un < units && !s_abort; un += gridDim.x) {
-        const int w = (int)(un / ntj);
-        if (mask && !mask[w]) continue;
-        const int j0 = (cols.jt_lo + (int)(un % ntj)) * OZ_TJ;
-        // rows past the walker's last column (a 128-wide tile at nc % 128 == 64) are
-        // the next slice's or zero, and their products are not kept
-        const int ys = (int)((long long)w * OZ_S * nc), yp = (int)((long long)w * OZ_S * nr) + cols.it_lo * OZ_TI;
-        if (tid == 0) {
-            mbar_expect_tx(mb_tma, bytes_a + bytes_b);
-            for (int t = 0; t < OZ_S; ++t) {
-                tma_load_2d(smem_u32(sA + t * OZ_SLICE_A), &maps.S, 0, ys + t * nc + j0, mb_tma);
-                tma_load_2d(smem_u32(sB + t * OZ_SLICE_B), &maps.P, 0, yp + t * nr, mb_tma);
-            }
-        }
-        // per thread of the epilogue: column j (TMEM lane) and its scale
-        const int quad = warp & 3, part = warp >> 2;
-        const int j = j0 + 32 * quad + lane;
-        const bool keep = j >= cols.c_lo && j < cols.c_hi && !(j >= cols.s_lo && j < cols.s_hi);
-        const bool wact = __any_sync(0xffffffffu, keep);   // a warp with no column to write skips its epilogue
-        const int eSj = j < nc ? Z.eS[(long long)w * nc + j] : 0;
-        double* Mw = Z.M + (long long)w * nr * nc;
-        const int* eP = Z.eP + (long long)w * nr;
-        for (int it = cols.it_lo; it < nti; ++it) {
-            const int i0 = it * OZ_TI;
-            if (tid == 0) {
-                if (!mbar_wait(mb_tma, ph_tma)) {
-                    set_dev_error(err, DEV_ERR_TIMEOUT);
-                    s_abort = 1;
-                    mbar_wait(mb_tma, ph_tma);   // let copies in flight land before leaving
-                } else {
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    // fully unrolled: descriptors and accumulate flags are compile-time, so
-                    // the issuing thread streams back-to-back MMAs
-                    const uint64_t a0 = desc_sw128(smem_u32(sA)), b0 = desc_sw128(smem_u32(sB));
-                    uint32_t started = 0;   // bit g: accumulator g holds a partial sum
-#pragma unroll
+    uint32_t T = 0, U = 0;   // tiles and units done; every role walks the same ones
+    auto give_up = [&]() {
+        set_dev_error(err, DEV_ERR_TIMEOUT);
+        s_abort = 1;
+    };
+    if (warp == OZ_EPI_WARPS) {
+        // ---- loads; the other lanes prefetch the tile's M into L2, two tiles
+        //      ahead of the epilogue that reads it (registers for a second set of
+        //      M values, and shared memory for one, are not to be had) ----
+        bool ok = true;
+        for (long long un = blockIdx.x; un < units && ok; un += gridDim.x) {
+            const int w = (int)(un / ntj);
+            if (mask && !mask[w]) continue;
+            const int j0 = (cols.jt_lo + (int)(un % ntj)) * OZ_TJ;
+            const int p0 = max(j0, cols.c_lo), p1 = min(j0 + OZ_TJ, cols.c_hi);   // multiples of 64
+            const double* Mp = Z.M + (long long)w * nr * nc + p0;
+            // rows past the walker's last column (a 128-wide tile at nc % 128 == 64) are
+            // the next slice's or zero, and their products are not kept
+            const int ys = (int)((long long)w * OZ_S * nc) + j0;
+            const int yp = (int)((long long)w * OZ_S * nr);
+            if (lane == 0) {
+                if (T > 0) ok = oz_wait(m_pfree + 8 * ((T - 1) & 1), ((T - 1) >> 1) & 1, &s_abort);   // the last unit's MMAs
+                if (ok) {
+                    mbar_expect_tx(m_sfull, bytes_a);
                     for (int t = 0; t < OZ_S; ++t)
-#pragma unroll
-                        for (int u = 0; u < OZ_S; ++u) {
-                            if (u + t > OZ_MAXLV) continue;
-                            const int g = min(t + u, OZ_GROUPS - 1);   // level t+u+2: 2 .. 6, then 7..10
-                            const uint64_t a = a0 + (uint64_t)((t * OZ_SLICE_A) >> 4);
-                            const uint64_t b = b0 + (uint64_t)((u * OZ_SLICE_B) >> 4);
-#pragma unroll
-                            for (int ks = 0; ks < NKS; ++ks) {
-                                const uint64_t adv = (uint64_t)(ks * 32) >> 4;   // 16 BF16 along K per MMA
-                                oz_mma(tmem + 64u * g, a + adv, b + adv, (started >> g) & 1u);
-                                started |= 1u << g;
-                            }
-                        }
-                    mma_commit(mb_mma);
-                }
-                ph_tma ^= 1u;
-            }
-            // this thread's 16 values of M (rows i0 + 16 (q / 4) ..): the loads
-            // overlap the MMAs
-            double m[16];
-#pragma unroll
-            for (int c = 0; c < 16; ++c) m[c] = keep ? Mw[(long long)(i0 + 16 * part + c) * nc + j] : 0.0;
-            __syncthreads();
-            if (s_abort) break;
-            if (!mbar_wait(mb_mma, ph_mma)) {
-                set_dev_error(err, DEV_ERR_TIMEOUT);
-                s_abort = 1;
-            }
-            ph_mma ^= 1u;
-            __syncthreads();
-            if (s_abort) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // the MMAs have read the Pan slices: load the next tile's during the epilogue
-            if (tid == 0 && it + 1 < nti) {
-                mbar_expect_tx(mb_tma, bytes_b);
-                for (int t = 0; t < OZ_S; ++t)
-                    tma_load_2d(smem_u32(sB + t * OZ_SLICE_B), &maps.P, 0, yp + t * nr + (it + 1 - cols.it_lo) * OZ_TI, mb_tma);
-            }
-            // ---- epilogue: warp q reads TMEM lanes 32 (q % 4) .. +31 (columns j),
-            //      and rows i0 + 16 (q / 4) .. +15 in two chunks of 8 ----
-#pragma unroll
-            for (int ch = 0; ch < 2 && wact; ++ch) {
-                const int c0 = 16 * part + 8 * ch;
-                float acc[OZ_GROUPS][8];
-#pragma unroll
-                for (int g = 0; g < OZ_GROUPS; ++g)
-                    tmem_ld8(tmem + ((uint32_t)(32 * quad) << 16) + 64u * g + (uint32_t)c0, acc[g]);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    // levels 2..6 are integers N_l 2^(-8l), |N_l| < 2^23, recovered exactly;
-                    // levels 7..10 rounded to a multiple of 2^-56.  F = sum in units of 2^-56
-                    // (|F| < 2^62): exact; one rounding to double, one in the add.
-                    const int n2 = __float2int_rn(acc[0][c] * 65536.0f);
-                    const int n3 = __float2int_rn(acc[1][c] * 16777216.0f);
-                    const int n4 = __float2int_rn(acc[2][c] * 4294967296.0f);
-                    const int n5 = __float2int_rn(acc[3][c] * 1099511627776.0f);
-                    const int n6 = __float2int_rn(acc[4][c] * 281474976710656.0f);
-                    const int tl = __float2int_rn(acc[5][c] * 72057594037927936.0f);
-                    const long long F = ((long long)(n2 * 256 + n3) << 32) + ((long long)(n4 * 256 + n5) << 16) +
-                                        ((long long)n6 << 8) + tl;
-                    const double d = oz_i64_to_double(F, eP[i0 + c0 + c] + eSj);
-                    if (keep) Mw[(long long)(i0 + c0 + c) * nc + j] = m[8 * ch + c] + d;
+                        tma_load_2d(smem_u32(sA + t * OZ_SLICE_A), &maps.S, 0, ys + t * nc, m_sfull);
+                    ++U;
                 }
             }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncthreads();
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            for (int it = cols.it_lo; it < nti && ok; ++it) {
+                if (lane == 0) {
+                    const uint32_t st = T & 1;
+                    if (T >= 2) ok = oz_wait(m_pfree + 8 * st, ((T - 2) >> 1) & 1, &s_abort);
+                    if (ok) {
+                        mbar_expect_tx(m_pfull + 8 * st, bytes_b);
+                        for (int t = 0; t < OZ_S; ++t)
+                            tma_load_2d(smem_u32(sB + st * STAGE + t * OZ_SLICE_B), &maps.P, 0,
+                                        yp + t * nr + it * OZ_TI, m_pfull + 8 * st);
+                        ++T;
+                    }
+                }
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (ok && p1 > p0)
+                    for (int r = lane; r < OZ_TI; r += 32)
+                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
+                                         Mp + (long long)(it * OZ_TI + r) * nc),
+                                     "r"((uint32_t)(p1 - p0) * 8u)
+                                     : "memory");
+            }
         }
+        if (!ok) {
+            if (lane == 0) {
+                give_up();
+                // let copies in flight land before leaving
+                if (U > 0) mbar_wait(m_sfull, (U - 1) & 1);
+                if (T >= 1) mbar_wait(m_pfull + 8 * ((T - 1) & 1), ((T - 1) >> 1) & 1);
+                if (T >= 2) mbar_wait(m_pfull + 8 * (T & 1), ((T - 2) >> 1) & 1);
+            }
+        }
+    } else if (warp == OZ_EPI_WARPS + 1) {
+        // ---- MMAs ----
+        const uint64_t a0 = desc_sw128(smem_u32(sA));
+        bool ok = true;
+        for (long long un = blockIdx.x; un < units && ok && lane == 0; un += gridDim.x) {
+            if (mask && !mask[(int)(un / ntj)]) continue;
+            ok = oz_wait(m_sfull, U & 1, &s_abort);
+            ++U;
+            for (int it = cols.it_lo; it < nti && ok; ++it, ++T) {
+                const uint32_t st = T & 1;
+                ok = oz_wait(m_pfull + 8 * st, (T >> 1) & 1, &s_abort);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t b0 = desc_sw128(smem_u32(sB + st * STAGE));
+                oz_issue<NKS, 4, 6>(tmem, T, a0, b0);
+                if (T > 0) ok = oz_wait(m_free, (T - 1) & 1, &s_abort);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                oz_issue<NKS, 0, 4>(tmem, T, a0, b0);
+                mma_commit(m_pfree + 8 * st);
+                mma_commit(m_full);
+            }
+        }
+        if (!ok && lane == 0) {
+            give_up();
+            mma_commit(m_drain);
+            mbar_wait(m_drain, 0);
+        }
+    } else {
+        // ---- epilogue: warp q reads TMEM lanes 32 (q % 4) .. +31 (columns j) and
+        //      rows i0 + 16 (q / 4) .. +15 ----
+        const int quad = warp & 3, part = warp >> 2;
+        const uint32_t lanes = (uint32_t)(32 * quad) << 16;
+        bool ok = true;
+        for (long long un = blockIdx.x; un < units && ok; un += gridDim.x) {
+            const int w = (int)(un / ntj);
+            if (mask && !mask[w]) continue;
+            const int j = (cols.jt_lo + (int)(un % ntj)) * OZ_TJ + 32 * quad + lane;   // this thread's column
+            const bool keep = j >= cols.c_lo && j < cols.c_hi && !(j >= cols.s_lo && j < cols.s_hi);
+            const bool wact = __any_sync(0xffffffffu, keep);   // a warp with no column to write only keeps step
+            const int eSj = j < nc ? Z.eS[(long long)w * nc + j] : 0;
+            for (int it = cols.it_lo; it < nti; ++it, ++T) {
+                const int i0 = it * OZ_TI + 16 * part;
+                double* Mj = Z.M + (long long)w * nr * nc + (long long)i0 * nc + j;
+                const int* eP = Z.eP + (long long)w * nr + i0;
+                // this thread's 16 values of M: the loads overlap the MMAs
+                double m[16];
+#pragma unroll
+                for (int c = 0; c < 16; ++c) m[c] = keep ? Mj[(long long)c * nc] : 0.0;
+                ok = oz_wait(m_full, T & 1, &s_abort);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                // the six accumulators into one exact sum per element, then the
+                // accumulators are free
+                int fh[16];
+                uint32_t fl[16];
+                if (wact) {
+#pragma unroll
+                    for (int ch = 0; ch < 2; ++ch) {
+                        float x[8], y[8];
+                        const uint32_t c0 = (uint32_t)(16 * part + 8 * ch);
+                        tmem_ld8(oz_acc(tmem, 0, T) + lanes + c0, x);
+                        tmem_ld8(oz_acc(tmem, 1, T) + lanes + c0, y);
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) oz_sum2(x[c], y[c], fh[8 * ch + c]);
+                        tmem_ld8(oz_acc(tmem, 2, T) + lanes + c0, x);
+                        tmem_ld8(oz_acc(tmem, 3, T) + lanes + c0, y);
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) oz_sum4(x[c], y[c], fh[8 * ch + c], fl[8 * ch + c]);
+                        tmem_ld8(oz_acc(tmem, 4, T) + lanes + c0, x);
+                        tmem_ld8(oz_acc(tmem, 5, T) + lanes + c0, y);
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) oz_sum6(x[c], y[c], fh[8 * ch + c], fl[8 * ch + c]);
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(m_free);
+                if (wact) {
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        const double d = oz_to_double(fh[c], fl[c], eP[c] + eSj);
+                        if (keep) Mj[(long long)c * nc] = m[c] + d;
+                    }
+                }
+            }
+        }
+        if (!ok && lane == 0) give_up();
     }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_TMEM_COLS)
@@ -507,7 +634,7 @@ bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, 
     if (rows >= (1ll << 31) || W > 65535) return false;
     OzMaps maps;
     if (!oz_map(&maps.S, Z.Sb, rows, OZ_TJ) || !oz_map(&maps.P, Z.Pb, (long long)W * OZ_S * nr, OZ_TI)) return false;
-    const size_t dyn = 1024 + (size_t)OZ_S * (OZ_SLICE_A + OZ_SLICE_B);
+    const size_t dyn = OZ_GEMM_SMEM;
     if (cudaFuncSetAttribute(k_oz_gemm<OZ_B / 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) !=
             cudaSuccess ||
         cudaFuncSetAttribute(k_oz_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
@@ -560,7 +687,8 @@ bool launch_refresh_oz(int W, int n, const double* A, const OzWork& Z, const Dev
                        void (*hook)(void*, int, int), void* hctx) {
     launch_oz_load<double>(W, n, n, A, true, false, Z, mask, st);
     if (!oz_eliminate<double>(W, n, Z, mask, false, err, st, hook, hctx)) return false;
-    launch_oz_finish<double>(W, n, n, true, Z, mask, S.logabs, S.sgn, S.pst, delayed && in_state ? S.tau : nullptr, st);
+    launch_oz_finish<double>(W, n, n, true, Z, mask, S.logabs, S.sgn, S.pst,
+                             delayed && in_state ? S.tau : nullptr, st);
     return true;
 }
 
@@ -582,7 +710,7 @@ bool launch_flush_split(int W, int n, int K, int Kc, int kk, const double* P, co
         cached[1] = Z.Pb;
         cached_rows = rows;
     }
-    const size_t dyn = 1024 + (size_t)OZ_S * (OZ_SLICE_A + OZ_SLICE_B);
+    const size_t dyn = OZ_GEMM_SMEM;
     static thread_local bool attr = false;
     if (!attr) {
         bool ok = true;
