@@ -134,14 +134,14 @@ struct OzWork {
     int* eP;          // W x nr power-of-two exponents of the panel rows
     uint8_t* go;      // W      walkers that flush now (split-product flush), or that this form inverts
     uint8_t* odd;     // W      walkers whose matrix is left to the FP64 form (see k_oz_sort)
-    int* cs;          // W x 64 exponent shifts of the slot columns (split-product flush)
     double* piv;      // W x nr scalars: pivots (log|det| and sign at the end)
     int* rmax;        // W x nr largest biased exponent of each row of M
 };
 // columns a split-product update writes: [c_lo, c_hi) minus [s_lo, s_hi), in
-// the 128-column tiles jt_lo .. jt_hi - 1 (doubles), rows from tile it_lo on
+// the 128-column tiles jt_lo .. jt_hi - 1 (doubles), rows from tile it_lo on; a
+// walker's M is rows x ld (the padded sizes of the slices, or the state's own)
 struct OzCols {
-    int c_lo, c_hi, s_lo, s_hi, jt_lo, jt_hi, it_lo;
+    int c_lo, c_hi, s_lo, s_hi, jt_lo, jt_hi, it_lo, rows, ld;
 };
 // rows of the working matrix of an n x n inverse: n padded by the identity
 int oz_rows(int n);
@@ -180,13 +180,16 @@ template <typename T>
 void launch_oz_store(int W, int w0, int n, int nr, const DevLayout& L, const DevState<T>& S, const OzWork& Z,
                      const uint8_t* mask, double* drift, bool delayed, bool pf, cudaStream_t st);
 // delayed flush A_0^{-1} += sgnQ * P Q^T (determinant: -1, Pfaffian: +1) as the
-// same exact split product (uniform n, n % 128 == 0, Kc <= 64); walkers with
-// tau >= K, or force && tau > 0 (their go flags stay set for launch_skew_project)
-bool launch_flush_split(int W, int n, int K, int Kc, int kk, const double* P, const double* Q, double sgnQ,
-                        const int* tau, const uint8_t* force, const OzWork& Z, int* err, cudaStream_t st);
-// A_0^{-1} of the walkers with go[w] set: the lower triangle := the exact
-// negative of the upper, diagonal 0 (after the Pfaffian split-product flush; n % 32 == 0)
-void launch_skew_project(int W, int n, double* G, const uint8_t* go, cudaStream_t st);
+// same exact split product (uniform n, K kk <= 64 doubles a row; Z of oz_flush_rows(n)
+// rows, Z.M the state); walkers with tau >= K, or force && tau > 0
+constexpr int oz_flush_rows(int n) { return (n + 63) / 64 * 64; }
+template <typename T>
+bool launch_flush_split(int W, int n, int K, int kk, const T* P, const T* Q, double sgnQ, const int* tau,
+                        const uint8_t* force, const OzWork& Z, int* err, cudaStream_t st);
+// A_0^{-1} of the same walkers: the lower triangle := the exact negative of the
+// upper, diagonal 0 (after the Pfaffian split-product flush)
+template <typename T>
+void launch_skew_project(int W, int n, int K, T* G, const int* tau, const uint8_t* force, cudaStream_t st);
 // hook(ctx, class, begin) brackets the panel (class 4) and update (class 5) launches
 bool launch_refresh_oz(int W, int n, const double* A, const OzWork& Z, const DevState<double>& S,
                        const uint8_t* mask, bool delayed, bool in_state, int* err, cudaStream_t st,

@@ -513,9 +513,11 @@ static void oz_prof_hook(void* p, int cls, int begin) {
     else prof_end(h, cls);
 }
 
+static int oz_cx(const lru_ctx* h) { return h->dtype == LRU_C128 ? 2 : 1; }
+
 static lru_status ensure_oz(lru_ctx* h) {
     if (h->ozw) return LRU_OK;
-    const size_t b = oz_work_layout(nullptr, nullptr, h->W, h->n_uni, 1, false);
+    const size_t b = oz_work_layout(nullptr, nullptr, h->W, oz_flush_rows(h->n_uni), oz_cx(h), false);
     if (cudaMalloc(&h->ozw, b) != cudaSuccess) {
         cudaGetLastError();
         h->ozw = nullptr;
@@ -523,6 +525,27 @@ static lru_status ensure_oz(lru_ctx* h) {
     }
     h->oz_bytes = b;
     return LRU_OK;
+}
+
+// nothing may be allocated while the stream is being captured
+static bool capturing(const lru_ctx* h) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool free = cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    if (!free) cudaGetLastError();
+    return !free;
+}
+
+// Whether a native flush of this handle runs as the split product (which has the
+// rounding of an FP64 update): where the FP64 flush would cost more per step than
+// the one launch that the split form adds (2^24 FMAs a step are 27 us of the FP64
+// pipe), and its workspace is to be had.  512 complex128 walkers, n = 512, K = 16:
+// 16.2 ms a flush in FP64 tiles, 1.5 ms split (0.6 ms of HBM traffic).
+static bool native_flush_split(lru_ctx* h) {
+    if ((h->dtype != LRU_F64 && h->dtype != LRU_C128) || h->n_uni < 128 || h->Kc * oz_cx(h) > OZ_B) return false;
+    const double madds = (double)h->W * h->n_uni * h->n_uni * h->kk * oz_cx(h) * oz_cx(h);   // FP64, per step
+    if (madds < (double)(1 << 24) || (long long)h->W * OZ_S * oz_flush_rows(h->n_uni) * oz_cx(h) >= (1ll << 31)) return false;
+    if (!h->ozw && capturing(h)) return false;
+    return ensure_oz(h) == LRU_OK;
 }
 
 // ---- the tensor-core elimination on padded copies ------------------------------
@@ -547,11 +570,7 @@ static int oz_chunk(int64_t W, int n, int cx) {
 // allocated).
 static bool ensure_ozg(lru_ctx* h, int cx) {
     if (h->ozg) return true;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return false;
-    }
+    if (capturing(h)) return false;
     const int chunk = oz_chunk(h->W, h->n_uni, cx);
     const size_t b = oz_work_layout(nullptr, nullptr, chunk, oz_rows(h->n_uni), cx, true) + (size_t)h->W;
     if (cudaMalloc(&h->ozg, b) != cudaSuccess) {
@@ -791,23 +810,29 @@ static lru_status do_flush(lru_handle h, const uint8_t* force) {
     DevLayout L = h->layout();
     prof_begin(h, LRU_PROF_FLUSH);
     h->launches += 2;
-    if (h->flush == LRU_FLUSH_SPLIT) {
+    if (h->flush == LRU_FLUSH_SPLIT || (h->flush == LRU_FLUSH_NATIVE && native_flush_split(h))) {
         lru_status s = ensure_oz(h);
         if (s != LRU_OK) { prof_end(h, LRU_PROF_FLUSH); return s; }
         OzWork Z{};
-        oz_work_layout(&Z, h->ozw, h->W, h->n_uni, 1, false);
+        oz_work_layout(&Z, h->ozw, h->W, oz_flush_rows(h->n_uni), oz_cx(h), false);
         Z.M = (double*)h->G;
-        h->launches += 4;   // flush flags, column balance, two slicings, GEMM (+ finish counted above)
+        h->launches += 1 + (h->pf ? 1 : 0);   // slices, GEMM (+ finish counted above)
         // determinant: A_0^{-1} -= P Q^T (Eq. delayed_Ainv); Pfaffian: A_0^{-1} += P Q^T
         // (Eq. pf_delayed_Ainv), then the lower triangle mirrored from the upper
-        if (!launch_flush_split(h->W, h->n_uni, h->K, h->Kc, h->kk, (const double*)h->P, (const double*)h->Q,
-                                h->pf ? 1.0 : -1.0, h->tau, force, Z, h->err, h->stream)) {
+        bool ok = false;
+        auto go = [&](auto tag) {
+            using T = decltype(tag);
+            ok = launch_flush_split<T>(h->W, h->n_uni, h->K, h->kk, (const T*)h->P, (const T*)h->Q, h->pf ? 1.0 : -1.0,
+                                       h->tau, force, Z, h->err, h->stream);
+            if (ok && h->pf) launch_skew_project<T>(h->W, h->n_uni, h->K, (T*)h->G, h->tau, force, h->stream);
+        };
+        if (h->dtype == LRU_C128) go(c128());
+        else go(double());
+        if (!ok && h->flush == LRU_FLUSH_NATIVE) {   // tensor maps unavailable
+            LRU_DISPATCH(h, { launch_flush_native<T>(h->pf, L, h->state<T>(), force, h->n_max, h->stream); });
+        } else if (!ok) {
             prof_end(h, LRU_PROF_FLUSH);
             return LRU_ERR_UNSUPPORTED;
-        }
-        if (h->pf) {
-            launch_skew_project(h->W, h->n_uni, (double*)h->G, Z.go, h->stream);
-            h->launches += 1;
         }
     } else if (h->flush == LRU_FLUSH_DF) {
         launch_flush_df(h->pf, L, h->state<double>(), force, h->stream);

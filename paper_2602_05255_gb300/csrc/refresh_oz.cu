@@ -230,7 +230,7 @@ __device__ __forceinline__ void oz_sum6(float a6, float tail, int& hi, uint32_t&
 }
 
 // F * 2^(e - 56) as a double, rounded to nearest (ties away), by integer operations
-// (normal results only: the scales stay far from the exponent limits).  The
+// (results below the normal range become zero; the callers keep away from the upper end).  The
 // mantissa with its leading one is added to the exponent field less one, so a
 // rounding that carries out of it needs no case of its own.
 __device__ __forceinline__ double oz_to_double(int hi, uint32_t lo, int e) {
@@ -243,7 +243,7 @@ __device__ __forceinline__ double oz_to_double(int hi, uint32_t lo, int e) {
     const unsigned long long v = a << (lz & 63);                 // leading one at bit 63
     const unsigned long long mant = (v >> 11) + ((v >> 10) & 1ull);
     const uint32_t rh = (uint32_t)(mant >> 32) + ((uint32_t)(1029 + e - lz) << 20);
-    const bool nz = a != 0;
+    const bool nz = a != 0 && 1029 + e - lz > 0;   // below the normal range: zero
     return __hiloint2double(nz ? (int)(rh | ((uint32_t)s & 0x80000000u)) : 0, nz ? (int)(uint32_t)mant : 0);
 }
 
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             if (mask && !mask[w]) continue;
             const int j0 = (cols.jt_lo + (int)(un % ntj)) * OZ_TJ;
             const int p0 = max(j0, cols.c_lo), p1 = min(j0 + OZ_TJ, cols.c_hi);   // multiples of 64
-            const double* Mp = Z.M + (long long)w * nr * nc + p0;
+            const double* Mp = Z.M + (long long)w * cols.rows * cols.ld + p0;
             // rows past the walker's last column (a 128-wide tile at nc % 128 == 64) are
             // the next slice's or zero, and their products are not kept
             const int ys = (int)((long long)w * OZ_S * nc) + j0;
@@ -388,10 +388,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                     }
                 }
                 ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (ok && p1 > p0)
-                    for (int r = lane; r < OZ_TI; r += 32)
-                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
-                                         Mp + (long long)(it * OZ_TI + r) * nc),
+                if (ok && p1 > p0 && ((cols.ld | p1) & 1) == 0)   // 16-byte rows
+                    for (int r = it * OZ_TI + lane; r < min(it * OZ_TI + OZ_TI, cols.rows); r += 32)
+                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Mp + (long long)r * cols.ld),
                                      "r"((uint32_t)(p1 - p0) * 8u)
                                      : "memory");
             }
@@ -448,12 +447,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             const int eSj = j < nc ? Z.eS[(long long)w * nc + j] : 0;
             for (int it = cols.it_lo; it < nti; ++it, ++T) {
                 const int i0 = it * OZ_TI + 16 * part;
-                double* Mj = Z.M + (long long)w * nr * nc + (long long)i0 * nc + j;
+                double* Mj = Z.M + ((long long)w * cols.rows + i0) * cols.ld + j;
+                const int nv = keep ? cols.rows - i0 : 0;   // rows c < nv are this thread's to write
                 const int* eP = Z.eP + (long long)w * nr + i0;
                 // this thread's 16 values of M: the loads overlap the MMAs
                 double m[16];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) m[c] = keep ? Mj[(long long)c * nc] : 0.0;
+                for (int c = 0; c < 16; ++c) m[c] = c < nv ? Mj[(long long)c * cols.ld] : 0.0;
                 ok = oz_wait(m_full, T & 1, &s_abort);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         const double d = oz_to_double(fh[c], fl[c], eP[c] + eSj);
-                        if (keep) Mj[(long long)c * nc] = m[c] + d;
+                        if (c < nv) Mj[(long long)c * cols.ld] = m[c] + d;
                     }
                 }
             }
@@ -504,77 +504,116 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
 // ---- the delayed flush as a split product ------------------------------------
 
-__global__ void k_oz_flush_go(int W, int K, const int* tau, const uint8_t* force, uint8_t* go) {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= W) return;
-    const int t = tau[w];
-    go[w] = (force ? (force[w] && t > 0) : (t >= K)) ? 1 : 0;
-}
+// Everything before the product, one CTA per walker that flushes (persistent
+// over walkers; on a step where none does every block leaves after reading tau):
+//   - the flush flag Z.go;
+//   - the column balance.  Every row is written as digits of one power-of-two
+//     scale (its largest entry), so a slot column much larger than the others (the
+//     step of a near-node update) would cost the other entries of the row their low
+//     bits.  Column c of P is scaled by 2^s_c and column c of Q by 2^-s_c, with s_c
+//     half the exponent gap of the two columns' maxima: P Q^T is unchanged exactly,
+//     and the entries of a row span a far smaller range;
+//   - the slices and exponents of the rows of P (complex: two rows each, see
+//     k_oz_slice_S) and of sgnQ Q, the cu filled slot columns, zeros after.
+// A walker with slots above 2^480, where a product of scales could leave the
+// exponent range, is folded here in FP64 instead and not flagged.
+// One launch in place of four (flags, balance, two slicings): a step without a
+// flush costs one launch less than the time of three.
+__device__ __forceinline__ double oz_pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
-// Column balance of the slot matrices before they are sliced.  Every row is
-// written as digits of one power-of-two scale (its largest entry), so a slot
-// column much larger than the others (the step of a near-node update) would
-// cost the other entries of the row their low bits.  Column c of P is scaled
-// by 2^s_c and column c of Q by 2^-s_c, with s_c half the exponent gap of the
-// two columns' maxima: P Q^T is unchanged exactly (powers of two), and the
-// entries of a row span a far smaller range.  Persistent over walkers.
-__global__ void __launch_bounds__(256) k_oz_col_balance(int W, int n, int ldx, int kk, const double* P,
-                                                        const double* Q, const int* tau, const uint8_t* go,
-                                                        int* cs) {
-    __shared__ int sp[4][OZ_B], sq[4][OZ_B];
+template <typename T>
+__global__ void __launch_bounds__(256) k_oz_flush_slices(int W, int n, int nr, int K, int kk, const T* P, const T* Q,
+                                                         double sgnQ, const int* tau, const uint8_t* force, OzWork Z) {
+    constexpr int CX = traits<T>::is_complex ? 2 : 1;
+    __shared__ int sp[4][OZ_B], sq[4][OZ_B], s_big;
+    __shared__ double s_fp[OZ_B], s_fq[OZ_B];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int c = threadIdx.x % OZ_B, g = threadIdx.x / OZ_B;   // 64 columns x 4 row groups
+    const int ldx = K * kk * CX, nc = nr * CX;
     for (int w = blockIdx.x; w < W; w += gridDim.x) {
-        if (!go[w]) continue;
-        const int cu = tau[w] * kk;
+        const int t = tau[w];
+        const bool due = force ? (force[w] && t > 0) : t >= K;
+        if (threadIdx.x == 0) {
+            Z.go[w] = due ? 1 : 0;
+            s_big = 0;
+        }
+        if (!due) continue;
+        const int cu = t * kk * CX;   // doubles
+        const double* Pw = reinterpret_cast<const double*>(P) + (long long)w * n * ldx;
+        const double* Qw = reinterpret_cast<const double*>(Q) + (long long)w * n * ldx;
         int ep = 0, eq = 0;
         if (c < cu)
+#pragma unroll 4
             for (int r = g; r < n; r += 4) {
-                ep = max(ep, oz_bexp(P[((long long)w * n + r) * ldx + c]));
-                eq = max(eq, oz_bexp(Q[((long long)w * n + r) * ldx + c]));
+                ep = max(ep, oz_bexp(Pw[(long long)r * ldx + c]));
+                eq = max(eq, oz_bexp(Qw[(long long)r * ldx + c]));
             }
+        __syncthreads();
         sp[g][c] = ep;
         sq[g][c] = eq;
         __syncthreads();
         if (g == 0) {
-            ep = max(max(sp[0][c], sp[1][c]), max(sp[2][c], sp[3][c]));
-            eq = max(max(sq[0][c], sq[1][c]), max(sq[2][c], sq[3][c]));
-            cs[(long long)w * OZ_B + c] = (ep > 0 && eq > 0) ? (eq - ep) / 2 : 0;
+            ep = eq = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int x = 0; x < CX; ++x) {   // both parts of a complex column share its scale
+                    ep = max(ep, sp[q][c ^ x]);
+                    eq = max(eq, sq[q][c ^ x]);
+                }
+            const int cs = (ep > 0 && eq > 0) ? (eq - ep) / 2 : 0;
+            s_fp[c] = c < cu ? oz_pow2(cs) : 0.0;
+            s_fq[c] = c < cu ? sgnQ * oz_pow2(-cs) : 0.0;
+            if (max(ep, eq) > 1023 + 480) s_big = 1;
         }
         __syncthreads();
-    }
-}
-
-// Rows of the walkers' slot matrices X (rows of ldx doubles): the cu =
-// tau * kk filled slot columns times sgn * 2^(cdir * cs[c]) (the column
-// balance, exact), zeros after; slices and exponent as for the panel rows.
-// Persistent over walkers: on steps where no walker flushes every block
-// leaves after reading the go flags.
-__device__ __forceinline__ double oz_pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
-__global__ void __launch_bounds__(256) k_oz_slice_rows(int W, int n, int ldx, int kk, const double* X, double sgn,
-                                                       const int* cs, int cdir, const int* tau, const uint8_t* go,
-                                                       uint16_t* dst, int* ex) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int w = blockIdx.x; w < W; w += gridDim.x) {
-        if (!go[w]) continue;
-        const int cu = tau[w] * kk;
-        const double fa = lane < cu ? sgn * oz_pow2(cdir * cs[(long long)w * OZ_B + lane]) : 0.0;
-        const double fb = lane + 32 < cu ? sgn * oz_pow2(cdir * cs[(long long)w * OZ_B + lane + 32]) : 0.0;
-        for (int r = wid; r < n; r += 8) {
-            const double* row = X + ((long long)w * n + r) * ldx;
-            const double a = lane < cu ? fa * row[lane] : 0.0;
-            const double b = lane + 32 < cu ? fb * row[lane + 32] : 0.0;
+        if (s_big) {
+            T* G = reinterpret_cast<T*>(Z.M) + (long long)w * n * n;
+            for (long long e = threadIdx.x; e < (long long)n * n; e += 256) {
+                const int l = (int)(e / n), j = (int)(e - (long long)l * n);
+                T d = s_zero(T());
+                for (int q = 0; q < t * kk; ++q)
+                    d = s_fma(P[((long long)w * n + j) * K * kk + q], Q[((long long)w * n + l) * K * kk + q], d);
+                G[e] = sgnQ < 0 ? G[e] - d : G[e] + d;
+            }
+            if (threadIdx.x == 0) Z.go[w] = 0;
+            __syncthreads();
+            continue;
+        }
+        const double pa = s_fp[lane], pb = s_fp[lane + 32], qa = s_fq[lane], qb = s_fq[lane + 32];
+        const bool second = ldx > 32;
+        for (int r = wid; r < 2 * n; r += 8) {
+            const bool isq = r >= n;
+            const int i = isq ? r - n : r;
+            const double* row = (isq ? Qw : Pw) + (long long)i * ldx;
+            double a = lane < cu ? (isq ? qa : pa) * row[lane] : 0.0;
+            double b = lane + 32 < cu ? (isq ? qb : pb) * row[lane + 32] : 0.0;
             const int mx = __reduce_max_sync(0xffffffffu, max(oz_bexp(a), oz_bexp(b)));
             const int E = mx > 0 ? mx - 1022 : 0;
-            uint16_t ha[OZ_S], hb[OZ_S];
-            oz_digits(oz_fixed(a, E), ha);
-            oz_digits(oz_fixed(b, E), hb);
+            const int outs = CX == 2 && !isq ? 2 : 1;
+            for (int o = 0; o < outs; ++o) {
+                if (CX == 2 && !isq) {
+                    if (o == 0) {
+                        if (lane & 1) { a = -a; b = -b; }            // (re, -im)
+                    } else {
+                        if (lane & 1) { a = -a; b = -b; }
+                        a = __shfl_xor_sync(0xffffffffu, a, 1);      // (im, re)
+                        b = __shfl_xor_sync(0xffffffffu, b, 1);
+                    }
+                }
+                const int ro = isq ? i : i * CX + o, rows = isq ? nr : nc;
+                uint16_t* plane = (isq ? Z.Pb : Z.Sb) + (long long)w * OZ_S * rows * OZ_B;
+                uint16_t ha[OZ_S], hb[OZ_S];
+                oz_digits(oz_fixed(a, E), ha);
+                if (second) oz_digits(oz_fixed(b, E), hb);
 #pragma unroll
-            for (int t = 0; t < OZ_S; ++t) {
-                uint16_t* d = dst + (((long long)w * OZ_S + t) * n + r) * OZ_B;
-                d[lane] = ha[t];
-                d[lane + 32] = hb[t];
+                for (int q = 0; q < OZ_S; ++q) {
+                    uint16_t* d = plane + ((long long)q * rows + ro) * OZ_B;
+                    d[lane] = ha[q];
+                    if (second) d[lane + 32] = hb[q];
+                }
+                if (lane == 0) (isq ? Z.eP : Z.eS)[(long long)w * rows + ro] = E;
             }
-            if (lane == 0) ex[(long long)w * n + r] = E;
         }
     }
 }
@@ -601,7 +640,6 @@ size_t oz_work_layout(OzWork* Z, void* base, int W, int nr, int cx, bool with_M)
     z.go = (uint8_t*)take((size_t)W);
     z.odd = (uint8_t*)take((size_t)W);
     z.piv = (double*)take(Wc * sizeof(double));
-    z.cs = (int*)take((size_t)W * OZ_B * sizeof(int));
     z.rmax = (int*)take(Wr * sizeof(int));
     if (with_M) z.M = (double*)take(Wr * nr * cx * sizeof(double));
     if (Z) *Z = z;
@@ -657,7 +695,7 @@ bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, 
             launch_oz_subpanel<T>(W, nr, k0, sp, lu, Z, mask, st);
             k_oz_slice_P16<<<dim3((nr - i0) / 16, W), 256, 0, st>>>(nr, nc, CX, i0, ks * CX, SW * CX, Z, mask);
             k_oz_slice_S<CX><<<dim3(1, W), 256, 0, st>>>(nr, nc, ks, SW, c0 / 64, Z, mask);
-            const OzCols inner{c0, c0 + OZ_B, ks * CX, (ks + SW) * CX, jt, jt + 1, it0};
+            const OzCols inner{c0, c0 + OZ_B, ks * CX, (ks + SW) * CX, jt, jt + 1, it0, nr, nc};
             k_oz_gemm<1><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, inner, Z, mask, err);
         }
         if (hook) { hook(hctx, 4, 0); hook(hctx, 5, 1); }
@@ -665,7 +703,7 @@ bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, 
         if (!lu || kn < nr) {
             k_oz_slice_P<<<dim3((nr - in) / 8, W), 256, 0, st>>>(nr, nc, CX, in, c0, OZ_B, Z, mask);
             k_oz_slice_S<CX><<<dim3((nc - cl) / 64, W), 256, 0, st>>>(nr, nc, k0, PB, cl / 64, Z, mask);
-            const OzCols outer{cl, nc, c0, c0 + OZ_B, cl / OZ_TJ, ntj, itn};
+            const OzCols outer{cl, nc, c0, c0 + OZ_B, cl / OZ_TJ, ntj, itn, nr, nc};
             k_oz_gemm<OZ_B / 16><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, outer, Z, mask, err);
         }
         if (hook) hook(hctx, 5, 0);
@@ -695,20 +733,27 @@ bool launch_refresh_oz(int W, int n, const double* A, const OzWork& Z, const Dev
 // A_0^{-1} -= P Q^T (Sec. 2.3, Eq. delayed_Ainv) for the walkers that flush:
 // with M = the stored A_0^{-1} (row l of storage = column l of A_0^{-1}),
 // M[l][j] += sum_c (-Q)[l][c] P[j][c]: the P rows take the place of the S
-// columns, the -Q rows that of the panel rows, no column is skipped.
-bool launch_flush_split(int W, int n, int K, int Kc, int kk, const double* P, const double* Q, double sgnQ,
-                        const int* tau, const uint8_t* force, const OzWork& Z, int* err, cudaStream_t st) {
-    if (Kc < 1 || Kc > OZ_B) return false;
-    const long long rows = (long long)W * OZ_S * n;
+// columns, the -Q rows that of the panel rows, no column is skipped.  The slices
+// are padded to a multiple of 64 rows, the state is not.
+template <typename T>
+bool launch_flush_split(int W, int n, int K, int kk, const T* P, const T* Q, double sgnQ, const int* tau,
+                        const uint8_t* force, const OzWork& Z, int* err, cudaStream_t st) {
+    constexpr int CX = traits<T>::is_complex ? 2 : 1;
+    const int kw = K * kk * CX, nr = oz_flush_rows(n), nc = nr * CX;
+    if (kw < 1 || kw > OZ_B) return false;
+    const long long rows = (long long)W * OZ_S * nc;
     if (rows >= (1ll << 31)) return false;
     static thread_local OzMaps maps;
     static thread_local const void* cached[2] = {nullptr, nullptr};
-    static thread_local long long cached_rows = -1;
-    if (cached[0] != Z.Sb || cached[1] != Z.Pb || cached_rows != rows) {
-        if (!oz_map(&maps.S, Z.Sb, rows, OZ_TJ) || !oz_map(&maps.P, Z.Pb, rows, OZ_TI)) return false;
+    static thread_local long long cached_rows[2] = {-1, -1};
+    const long long prow = (long long)W * OZ_S * nr;
+    if (cached[0] != Z.Sb || cached[1] != Z.Pb || cached_rows[0] != rows || cached_rows[1] != prow) {
+        cached[0] = nullptr;
+        if (!oz_map(&maps.S, Z.Sb, rows, OZ_TJ) || !oz_map(&maps.P, Z.Pb, prow, OZ_TI)) return false;
         cached[0] = Z.Sb;
         cached[1] = Z.Pb;
-        cached_rows = rows;
+        cached_rows[0] = rows;
+        cached_rows[1] = prow;
     }
     const size_t dyn = OZ_GEMM_SMEM;
     static thread_local bool attr = false;
@@ -725,22 +770,23 @@ bool launch_flush_split(int W, int n, int K, int Kc, int kk, const double* P, co
     int dev = 0, nsm = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    k_oz_flush_go<<<(W + 255) / 256, 256, 0, st>>>(W, K, tau, force, Z.go);
-    const int sgrid = std::min(W, 8 * nsm);
-    k_oz_col_balance<<<sgrid, 256, 0, st>>>(W, n, Kc, kk, P, Q, tau, Z.go, Z.cs);
-    k_oz_slice_rows<<<sgrid, 256, 0, st>>>(W, n, Kc, kk, P, 1.0, Z.cs, 1, tau, Z.go, Z.Sb, Z.eS);
-    k_oz_slice_rows<<<sgrid, 256, 0, st>>>(W, n, Kc, kk, Q, sgnQ, Z.cs, -1, tau, Z.go, Z.Pb, Z.eP);
+    k_oz_flush_slices<T><<<std::min(W, 8 * nsm), 256, 0, st>>>(W, n, nr, K, kk, P, Q, sgnQ, tau, force, Z);
     auto kern = k_oz_gemm<1>;
-    switch ((Kc + 15) / 16) {
+    switch ((kw + 15) / 16) {
         case 2: kern = k_oz_gemm<2>; break;
         case 3: kern = k_oz_gemm<3>; break;
         case 4: kern = k_oz_gemm<4>; break;
         default: break;
     }
-    const OzCols all{0, n, -1, -1, 0, n / OZ_TJ, 0};
-    kern<<<nsm, OZ_THREADS, dyn, st>>>(maps, W, n, n, all, Z, Z.go, err);
+    const OzCols all{0, n * CX, -1, -1, 0, (nc + OZ_TJ - 1) / OZ_TJ, 0, n, n * CX};
+    kern<<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, all, Z, Z.go, err);
     return true;
 }
+
+template bool launch_flush_split<double>(int, int, int, int, const double*, const double*, double, const int*,
+                                         const uint8_t*, const OzWork&, int*, cudaStream_t);
+template bool launch_flush_split<c128>(int, int, int, int, const c128*, const c128*, double, const int*,
+                                       const uint8_t*, const OzWork&, int*, cudaStream_t);
 
 // Exact skew symmetry of the flushed walkers' A_0^{-1}, after the Pfaffian
 // split-product flush A_0^{-1} += P Q^T: the product of the rounded slots
@@ -749,45 +795,48 @@ bool launch_flush_split(int W, int n, int K, int Kc, int kk, const double* P, co
 // lower triangle is written as its exact negative (a sign flip, no FP64
 // arithmetic), the diagonal as zero -- the same rule as the FP64 skew flush.
 // Reads the upper half, writes the lower half.  One CTA per (walker, 32 x 32
-// upper tile).
-__global__ void __launch_bounds__(256) k_skew_project(int n, double* G, const uint8_t* go) {
-    __shared__ double sU[32][33];
-    const int w = blockIdx.y;
-    if (!go[w]) return;
-    const int nt = n / 32;
+// upper tile).  A walker folded in FP64 (k_oz_flush_slices) is mirrored too:
+// the test is the slots', not the product's flag.
+template <typename T>
+__global__ void __launch_bounds__(256) k_skew_project(int n, int K, T* G, const int* tau, const uint8_t* force) {
+    __shared__ T sU[32][33];
+    const int w = blockIdx.y, t = tau[w];
+    if (!(force ? (force[w] && t > 0) : t >= K)) return;
+    const int nt = (n + 31) / 32;
     int r = 0, rem = (int)blockIdx.x;
     while (rem >= nt - r) { rem -= nt - r; ++r; }
     const int j0 = 32 * r, l0 = 32 * (r + rem);
-    double* Gw = G + (long long)w * n * n;
+    T* Gw = G + (long long)w * n * n;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     // sU[l][j] = G(j0 + j, l0 + l), stored at Gw[(l0 + l) * n + j0 + j]
     for (int q = 0; q < 4; ++q) {
         const int a = ty + 8 * q;
-        sU[a][tx] = Gw[(long long)(l0 + a) * n + j0 + tx];
+        if (l0 + a < n && j0 + tx < n) sU[a][tx] = Gw[(long long)(l0 + a) * n + j0 + tx];
     }
     __syncthreads();
-    const auto neg = [](double v) {
-        return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
-    };
     if (rem != 0) {
         // lower block: G(l0 + l, j0 + j) = -G(j0 + j, l0 + l), stored at Gw[(j0 + j) * n + l0 + l]
         for (int q = 0; q < 4; ++q) {
             const int a = ty + 8 * q;   // j within the tile, tx = l
-            Gw[(long long)(j0 + a) * n + l0 + tx] = neg(sU[tx][a]);
+            if (l0 + tx < n) Gw[(long long)(j0 + a) * n + l0 + tx] = s_neg(sU[tx][a]);
         }
     } else {
         // diagonal tile: entries below the diagonal from the ones above it
         for (int q = 0; q < 4; ++q) {
             const int a = ty + 8 * q;   // column l = j0 + a, row j = j0 + tx
-            if (tx > a) Gw[(long long)(j0 + a) * n + j0 + tx] = neg(sU[tx][a]);
-            else if (tx == a) Gw[(long long)(j0 + a) * n + j0 + tx] = 0.0;
+            if (j0 + a >= n || j0 + tx >= n) continue;
+            if (tx > a) Gw[(long long)(j0 + a) * n + j0 + tx] = s_neg(sU[tx][a]);
+            else if (tx == a) Gw[(long long)(j0 + a) * n + j0 + tx] = s_zero(T());
         }
     }
 }
 
-void launch_skew_project(int W, int n, double* G, const uint8_t* go, cudaStream_t st) {
-    const int nt = n / 32;
-    k_skew_project<<<dim3(nt * (nt + 1) / 2, W), 256, 0, st>>>(n, G, go);
+template <typename T>
+void launch_skew_project(int W, int n, int K, T* G, const int* tau, const uint8_t* force, cudaStream_t st) {
+    const int nt = (n + 31) / 32;
+    k_skew_project<T><<<dim3(nt * (nt + 1) / 2, W), 256, 0, st>>>(n, K, G, tau, force);
 }
+template void launch_skew_project<double>(int, int, int, double*, const int*, const uint8_t*, cudaStream_t);
+template void launch_skew_project<c128>(int, int, int, c128*, const int*, const uint8_t*, cudaStream_t);
 
 }  // namespace lru
