@@ -191,9 +191,15 @@ static void prof_end(lru_ctx* h, int cls) {
     if (h->prof_used[cls] < v.size()) cudaEventRecord(v[h->prof_used[cls]++].second, h->stream);
 }
 
+// matrices that the kernels with a CTA per matrix hold at once: two CTAs per SM, four
+// of the blocked Pfaffian where their copies stay below 5 GiB
+static int elimination_slots(int64_t W, int n, int n_sm) {
+    return (int)std::min<int64_t>(W, (n <= 1024 ? 4 : 2) * (int64_t)n_sm);
+}
+
 static lru_status ensure_ws(lru_ctx* h) {
     if (h->ws) return LRU_OK;
-    int nws = std::min(h->W, 2 * h->n_sm);
+    int nws = elimination_slots(h->W, h->n_max, h->n_sm);
     size_t b = (size_t)nws * h->n_max * h->n_max * dtype_size(h->dtype);
     if (cudaMalloc(&h->ws, b) != cudaSuccess) {
         cudaGetLastError();
@@ -1190,7 +1196,7 @@ static lru_status batched_dense(bool pf, int32_t dtype, int64_t W, int32_t n, co
     int dev = 0, nsm = 148;
     CK(cudaGetDevice(&dev));
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); nsm = 148; }
-    const int nws = (int)std::min<int64_t>(W, 2 * nsm);
+    const int nws = pf ? elimination_slots(W, n, nsm) : (int)std::min<int64_t>(W, 2 * nsm);
     void* ws = nullptr;
     CK(cudaMallocAsync(&ws, (size_t)nws * n * n * dtype_size(dtype), st));
     lru_ctx tmp;
