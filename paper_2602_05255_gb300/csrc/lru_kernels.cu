@@ -174,7 +174,11 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
         s_iu[tid] = iu;
         s_iv[tid] = iv;
     }
-    if (PF && tid == 0) {
+    // one row-and-column move with C = -J: the 2 x 2 core has closed forms (below)
+    const bool pf2 = PF && SKEWM && kk == 2 && C == nullptr;
+    if (pf2) {
+        if (tid < 4) s_cinv[(tid >> 1) * MAXKK + (tid & 1)] = make_real<T>(tid == 1 ? 1.0 : (tid == 2 ? -1.0 : 0.0));
+    } else if (PF && tid == 0) {
         // C^{-1} and pf(C^{-1}); C = NULL means C = -J, so C^{-1} = J (Sec. 3.1)
         const int k2 = kk;
         if (C == nullptr) {
@@ -327,6 +331,19 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
             for (int i = 0; i < kk; ++i)
                 for (int j = 0; j < kk; ++j) s_inv[i * MAXKK + j] = s_core[i * MAXKK + j];
             st = small_gj_inverse(s_inv, kk, MAXKK, &ratio);
+        } else if (pf2) {
+            // M = [[0, h], [-h, 0]] after the projection: pf M = h, pf C^{-1} = 1,
+            // M^{-1} = [[0, -1/h], [1/h, 0]]; the bits and the status of the loops
+            // below, without their dependent cycles in one thread (1024 walkers,
+            // n = 256, K = 8: a propose 57 -> 42 us)
+            const T h = s_half(s_core[1] - s_core[MAXKK]);
+            const T ih = s_recip(h);
+            s_inv[0] = s_inv[MAXKK + 1] = s_zero(T());
+            s_inv[1] = s_neg(ih);
+            s_inv[MAXKK] = ih;
+            ratio = h;
+            st = !((double)s_abs2(h) > 0.0) ? CORE_SINGULAR
+                                            : (s_isfinite(h * h) && s_isfinite(h) ? CORE_OK : CORE_NONFINITE);
         } else {
             // The skew-form updates (Eq. pf_delayed_Ainv, and the exactly skew
             // plain accept) need M and M^{-1} exactly skew; a generic Woodbury
@@ -1603,40 +1620,58 @@ __global__ void k_set_delay_zero(DevLayout L, DevState<T> S) {
     if (w < L.W) S.tau[w] = 0;
 }
 
-// current A^{-1} (row-major out) = A_0^{-1} -/+ P Q^T, 32 x 32 tiles
+// current A^{-1} (row-major out) = A_0^{-1} -/+ P Q^T: a transposing copy, bound by
+// HBM when no slots are pending.  TW x TW tiles (rows of 512 bytes), all loads of a thread in flight before the barrier: with 32 x 32 tiles of
+// four loads a thread, 1024 walkers of n = 1024 (17 GB) took 4.04 ms, now 2.36.
+template <typename T> constexpr int inv_tw() { return sizeof(T) == 16 ? 32 : 64; }
+
 template <typename T, bool PF, bool DELAYED>
 __global__ void __launch_bounds__(256) k_get_inverse(DevLayout L, DevState<T> S, T* out) {
-    __shared__ T sT[32][33];
+    constexpr int TW = inv_tw<T>(), TPR = TW / 32, NQ = 32 * TPR / 8;   // TW columns l x 32 * TPR rows j
+    __shared__ T sT[TW][32 * TPR + 1];
     const int w = blockIdx.z;
     const int n = L.nw(w), kk = L.kv(w);
-    const int nt = (n + 31) / 32;
-    if ((int)blockIdx.x >= nt || (int)blockIdx.y >= nt) return;
-    const int j0 = blockIdx.x * 32, l0 = blockIdx.y * 32;
+    const int j0 = blockIdx.x * 32 * TPR, l0 = blockIdx.y * TW;
+    if (j0 >= n || l0 >= n) return;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const T* Gw = S.G + L.mo(w);
     const long long vo = L.vo(w);
     const int cu = DELAYED ? S.tau[w] * kk : 0;
-    for (int q = 0; q < 4; ++q) {
-        const int j = j0 + tx, l = l0 + ty + 8 * q;
-        T v = s_zero(T());
-        if (j < n && l < n) {
-            v = Gw[(long long)l * n + j];
-            if (DELAYED) {
+    T v[NQ][TPR];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+        for (int h = 0; h < TPR; ++h) {
+            const int j = j0 + tx + 32 * h, l = l0 + ty + 8 * q;
+            v[q][h] = j < n && l < n ? Gw[(long long)l * n + j] : s_zero(T());
+        }
+    if (DELAYED && cu) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int h = 0; h < TPR; ++h) {
+                const int j = j0 + tx + 32 * h, l = l0 + ty + 8 * q;
+                if (j >= n || l >= n) continue;
                 const T* pr = S.P + (vo + j) * L.Kc;
                 const T* qr = S.Q + (vo + l) * L.Kc;
                 T s = s_zero(T());
                 for (int c = 0; c < cu; ++c) s = s_fma(pr[c], qr[c], s);
-                v = PF ? v + s : v - s;
+                v[q][h] = PF ? v[q][h] + s : v[q][h] - s;
             }
-        }
-        sT[ty + 8 * q][tx] = v;   // (j, l)
     }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+        for (int h = 0; h < TPR; ++h) sT[ty + 8 * q][tx + 32 * h] = v[q][h];   // (j, l)
     __syncthreads();
     T* ow = out + L.mo(w);
-    for (int q = 0; q < 4; ++q) {
-        const int i = j0 + ty + 8 * q, jj = l0 + tx;   // out[i][jj] = A^{-1}_{i, jj}
-        if (i < n && jj < n) ow[(long long)i * n + jj] = sT[tx][ty + 8 * q];
-    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+        for (int h = 0; h < TPR; ++h) {
+            const int i = j0 + ty + 8 * q, jj = l0 + tx + 32 * h;   // out[i][jj] = A^{-1}_{i, jj}
+            if (i < n && jj < n) ow[(long long)i * n + jj] = sT[tx + 32 * h][ty + 8 * q];
+        }
 }
 
 // ---- operand formation -----------------------------------------------------
@@ -1930,7 +1965,7 @@ void launch_set_delay_zero(const DevLayout& L, const DevState<T>& S, cudaStream_
 template <typename T>
 void launch_get_inverse(bool pf, bool delayed, const DevLayout& L, const DevState<T>& S, T* out,
                         cudaStream_t st) {
-    const int nt = (L.n_max + 31) / 32;
+    const int nt = (L.n_max + inv_tw<T>() - 1) / inv_tw<T>();   // square tiles
     dim3 grid(nt, nt, L.W);
     if (!pf && !delayed) k_get_inverse<T, false, false><<<grid, 256, 0, st>>>(L, S, out);
     if (!pf && delayed) k_get_inverse<T, false, true><<<grid, 256, 0, st>>>(L, S, out);

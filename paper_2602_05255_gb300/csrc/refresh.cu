@@ -1064,8 +1064,10 @@ template <typename T> int oz_subpanel_width(int nr) { return (nr <= 1024 ? 16 : 
 template <typename T>
 void launch_oz_subpanel(int W, int nr, int k0, int sp, bool lu, const OzWork& Z, const uint8_t* mask, cudaStream_t st) {
     constexpr int CX = traits<T>::is_complex ? 2 : 1;
-    if (nr <= 512) k_oz_subpanel_rows<T, 1, 16 / CX><<<W, nr, 0, st>>>(nr, k0, sp, lu, Z, mask);
-    else if (nr <= 1024) k_oz_subpanel_rows<T, 2, 16 / CX><<<W, nr / 2, 0, st>>>(nr, k0, sp, lu, Z, mask);
+    if (nr <= 1024) k_oz_subpanel_rows<T, 2, 16 / CX><<<W, nr / 2, 0, st>>>(nr, k0, sp, lu, Z, mask);
+    // (two rows per thread also below 512 rows: half as many threads, so two or more
+    // CTAs share an SM and one computes while another waits for its pivot; with one
+    // row the eliminations of 256 matrices, n = 500, took 10.0 ms instead of 6.1)
     // four rows of half as many sub-panel columns per thread keep the registers
     else k_oz_subpanel_rows<T, 4, 8 / CX><<<W, nr / 4, 0, st>>>(nr, k0, sp, lu, Z, mask);
 }
