@@ -129,6 +129,9 @@ def _check(code: int, where: str):
         raise LRUError(code, where)
 
 
+# Pointers and streams go to ctypes as plain integers (argtypes converts them):
+# a c_void_p per argument and a Stream object per call were a third of the 192 us that a
+# step of a single small walker (with its log-value and inverse) costs, now 124.
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
@@ -136,11 +139,11 @@ def _ptr(t: Optional[torch.Tensor]):
         raise ValueError("expected a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _mask_ptr(mask):
@@ -214,6 +217,8 @@ class LowRankState:
         _check(_lib.lru_create(C.byref(cfg), C.byref(h)), "lru_create")
         self._h = h
         self.kmax = self.k if self.kind == DET else 2 * self.k
+        self._uniform = len(set(self.n_list)) == 1
+        self._sum_n2 = sum(n * n for n in self.n_list)
 
     def close(self):
         if getattr(self, "_h", None):
@@ -294,12 +299,8 @@ class LowRankState:
     # ---- state access -----------------------------------------------------
     def inverse(self) -> torch.Tensor:
         self._bind()
-        total = sum(n * n for n in self.n_list)
-        out = torch.empty(total, dtype=self.dtype, device=self.device)
+        out = self._mats_like()
         _check(_lib.lru_get_inverse(self._h, _ptr(out)), "lru_get_inverse")
-        if len(set(self.n_list)) == 1:
-            n = self.n_list[0]
-            return out.view(self.W, n, n)
         return out
 
     def logvalue(self):
@@ -354,7 +355,7 @@ class LowRankState:
 
     @property
     def uniform(self) -> bool:
-        return len(set(self.n_list)) == 1
+        return self._uniform
 
     def _ops_like(self):
         """Zeros in the operand vector layout: (W, kmax, n), or flat sum(n) * kmax when n varies."""
@@ -367,7 +368,7 @@ class LowRankState:
         if self.uniform:
             n = self.n_list[0]
             return torch.empty(self.W, n, n, dtype=self.dtype, device=self.device)
-        return torch.empty(sum(x * x for x in self.n_list), dtype=self.dtype, device=self.device)
+        return torch.empty(self._sum_n2, dtype=self.dtype, device=self.device)
 
     def backward_det(self, g: torch.Tensor, want_U=True, want_V=True, want_A=True):
         """(gU, gV, gA): vector-Jacobian product of the pending proposal's log ratio."""
