@@ -718,6 +718,7 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
     __shared__ T s_rowk[SW], s_bufA[SW], s_bufB[SW];
     __shared__ unsigned long long s_wk[16];
     __shared__ int s_wi[16];
+    __shared__ int s_src[2048], s_row[2 * SW];   // composed exchanges (n <= 2048)
     __shared__ int s_sing;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
     const int w = blockIdx.x;
@@ -845,17 +846,54 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
         }
         __syncthreads();
         // ---- this sub-panel's exchanges on the other panel columns ----
-        for (int t = tid; t < PB - SW; t += nt) {
-            const int col = k0 + t + (t >= SW * sp ? SW : 0);
+        // The SW exchanges (k, perm[k]), applied in pivot order, move at most 2 SW
+        // rows: row r receives the old row s_src[r].  All their elements are loaded
+        // before any is stored (a loop of SW dependent swaps per column waits for
+        // global memory SW times: 36.7 -> 34.8 ms of eliminations a refresh at 512 walkers,
+        // n = 1024); a row listed twice is written twice alike.
+        if (tid < SW) {
+            const int k = ks + tid, p = perm[k];
+            s_src[k] = k;
+            s_src[p] = p;
+            s_row[tid] = k;
+            s_row[SW + tid] = p;
+        }
+        __syncthreads();
+        if (tid == 0)
             for (int kc = 0; kc < SW; ++kc) {
-                const int kk = ks + kc, p = perm[kk];
-                if (p != kk) {
-                    const T a = M[(long long)kk * n + col];
-                    M[(long long)kk * n + col] = M[(long long)p * n + col];
-                    M[(long long)p * n + col] = a;
-                }
+                const int k = ks + kc, p = s_row[SW + kc], a = s_src[k];
+                s_src[k] = s_src[p];
+                s_src[p] = a;
+            }
+        __syncthreads();
+        // elements in groups of four columns (a 32-byte sector of each row); a round of
+        // 4 nt elements holds whole groups, and columns do not depend on one another
+        constexpr int NB = PB - SW, NE = 2 * SW * NB;
+        static_assert(NB % 4 == 0 && 128 % (8 * SW) == 0, "rounds of whole column groups");
+        auto place = [&](int e, int& r, int& col) {
+            const int rem = e % (8 * SW), t = e / (8 * SW) * 4 + rem % 4;
+            r = rem / 4;
+            col = k0 + t + (t >= SW * sp ? SW : 0);
+        };
+        for (int e0 = 0; e0 < NE; e0 += 4 * nt) {
+            T x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int e = e0 + tid + u * nt;
+                int r, col;
+                place(e, r, col);
+                if (e < NE) x[u] = M[(long long)s_src[s_row[r]] * n + col];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int e = e0 + tid + u * nt;
+                int r, col;
+                place(e, r, col);
+                if (e < NE) M[(long long)s_row[r] * n + col] = x[u];
             }
         }
+        __syncthreads();
     }
     // ---- last sub-panel: the panel's exchanges on the columns outside it ----
     // The 64 exchanges (k, perm[k]), applied in pivot order, compose into one
@@ -864,7 +902,6 @@ __global__ void __launch_bounds__(512, 1) k_oz_subpanel_rows(int n, int k0, int 
     // is gathered into shared memory (independent, coalesced loads) and
     // written back permuted, instead of 64 dependent swaps per column.
     if (sp == PB / SW - 1) {
-        __shared__ int s_src[2048];            // n <= 2048 for this kernel
         __shared__ int s_from[2 * PB], s_to[2 * PB];
         __shared__ int s_cnt;
         __shared__ T s_xb[2 * PB][33];
