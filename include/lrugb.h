@@ -73,7 +73,9 @@ typedef enum { LRU_DET = 0, LRU_PF = 1 } lru_kind;
 /* Precision of the delayed flush A0^{-1} -/+= P Q^T (Sec. 2.3 Eq. delayed_Ainv,
  * Sec. 3.3 Eq. pf_delayed_Ainv).  Everything else stays in the handle dtype. */
 typedef enum {
-    LRU_FLUSH_NATIVE = 0,   /* dtype arithmetic on the CUDA cores (FP64 for F64/C128) */
+    LRU_FLUSH_NATIVE = 0,   /* the rounding of dtype arithmetic (FP64 for F64/C128): on the CUDA cores, and for
+                               large F64/C128 handles of uniform n >= 128 with at most 64 doubles of slots per
+                               row by the exact products of LRU_FLUSH_SPLIT */
     LRU_FLUSH_TF32X3 = 1,   /* tcgen05 TF32 tensor cores, 3-term split (about FP32 accuracy) */
     LRU_FLUSH_TF32 = 2,     /* tcgen05 TF32, one term */
     LRU_FLUSH_BF16 = 3,     /* tcgen05 BF16, one term */
@@ -98,18 +100,24 @@ typedef enum {
                                update, not exactly skew) refresh before such a propose */
 } lru_arith;
 
-/* How init and refresh compute the FP64 inverse (F64 determinant handles):
- * the update of each 64-column Gauss-Jordan panel on the other columns is an
- * n x n x 64 product; LRU_REFRESH_TENSOR runs it on the BF16 tensor cores as
- * an exact split product (7 slices of 8 bits per operand, FP64 recombination:
- * the accuracy of an FP64 update), the panels themselves in FP64.  It applies
- * to uniform n with n % 128 == 0, 128 <= n <= 2048 and W <= 65535; other
- * handles use LRU_REFRESH_FP64.  A refresh that asks for the drift allocates,
- * on first use, a second W x n x n workspace for the fresh inverses. */
+/* How init and refresh compute the FP64 inverse: the update of each 64-column
+ * Gauss-Jordan panel on the other columns is an n x n x 64 product, which the
+ * tensor-core form runs on the BF16 tensor cores as an exact split product (7
+ * slices of 8 bits per operand, FP64 recombination: the accuracy of an FP64
+ * update), the panels themselves in FP64.  For F64 determinants of uniform n
+ * with n % 128 == 0, 128 <= n <= 2048 and W <= 65535 it works in the state; a
+ * refresh that asks for the drift allocates, on first use, a second W x n x n
+ * workspace for the fresh inverses.  For other F64 and C128 handles of uniform
+ * n (56 .. 64 or >= 72; determinants and Pfaffians) it works on padded copies,
+ * a chunk of walkers at a time, in a workspace of at most about 3 GiB that is
+ * allocated on first use; matrices whose rows differ by more than 2^6 in size
+ * or that hold extreme or non-finite entries, and handles whose workspace
+ * cannot be allocated (memory, or a first use inside a stream capture), take
+ * the FP64 form, as do single precision, ragged and smaller handles. */
 typedef enum {
     LRU_REFRESH_AUTO = 0,     /* the tensor-core form where it applies */
     LRU_REFRESH_FP64 = 1,     /* blocked Gauss-Jordan entirely on the FP64 pipe */
-    LRU_REFRESH_TENSOR = 2    /* as AUTO; lru_create fails with LRU_ERR_UNSUPPORTED where it cannot apply */
+    LRU_REFRESH_TENSOR = 2    /* as AUTO; lru_create fails with LRU_ERR_UNSUPPORTED where it cannot work in the state */
 } lru_refresh;
 
 typedef struct {
@@ -309,7 +317,9 @@ lru_status lru_gather_pairs(lru_handle h, const void* F, int32_t m, const int32_
 
 /* ---- standalone batched dense operations (App. A.1) ---------------------- */
 
-/* slogdet of W matrices of size n (row-major), dtype as given. */
+/* slogdet of W matrices of size n (row-major), dtype as given.  F64 and C128 of
+ * n = 56 .. 64 or >= 72 are eliminated on the tensor cores (see lru_refresh), in
+ * a workspace of at most about 3 GiB allocated on the stream for the call. */
 lru_status lru_slogdet_batched(int32_t dtype, int64_t W, int32_t n, const void* A,
                                double* logabs, void* sign, void* stream);
 /* Same as lru_slogdet_batched, but allocates nothing (the paper has no

@@ -547,7 +547,8 @@ static bool capturing(const lru_ctx* h) {
 // pipe), and its workspace is to be had.  512 complex128 walkers, n = 512, K = 16:
 // 16.2 ms a flush in FP64 tiles, 1.5 ms split (0.6 ms of HBM traffic).
 static bool native_flush_split(lru_ctx* h) {
-    if ((h->dtype != LRU_F64 && h->dtype != LRU_C128) || h->n_uni < 128 || h->Kc * oz_cx(h) > OZ_B) return false;
+    if ((h->dtype != LRU_F64 && h->dtype != LRU_C128) || h->n_uni < 128 || h->Kc * oz_cx(h) > OZ_B || h->W > 65535)
+        return false;
     const double madds = (double)h->W * h->n_uni * h->n_uni * h->kk * oz_cx(h) * oz_cx(h);   // FP64, per step
     if (madds < (double)(1 << 24) || (long long)h->W * OZ_S * oz_flush_rows(h->n_uni) * oz_cx(h) >= (1ll << 31)) return false;
     if (!h->ozw && capturing(h)) return false;
@@ -661,6 +662,8 @@ static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, doub
         }
         cudaGetLastError();   // tensor maps unavailable: the FP64 form below
     }
+    // the workspace of the flushes to come, so that the first of them may be captured
+    if (h->delayed && h->flush == LRU_FLUSH_NATIVE) native_flush_split(h);
     prof_begin(h, LRU_PROF_REFRESH);
     bool done = false;
     if (!h->oz_ok && oz_padded(h->n_uni) && h->cfg.refresh != LRU_REFRESH_FP64) {
