@@ -635,6 +635,51 @@ __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> 
     __syncthreads();
 
     T* Gw = S.G + L.mo(w);
+    if constexpr (KKS == 1 && NPL * sizeof(T) <= 128) {
+        // rank 1: two columns at a time while they fit the registers.  The FP64 pipe
+        // bounds the pass, and five of its 38 instructions per column (n = 500) are the
+        // butterfly of the dot product: two columns share one, as they share the loads
+        // of V and X (384 walkers, n = 500: 455 -> 430 us an accept).
+        for (int l = it.y + wid; l < it.z; l += 2 * (PT / 32)) {
+            const bool two = l + PT / 32 < it.z;
+            T* c0 = Gw + (long long)l * n;
+            T* c1 = two ? c0 + (long long)(PT / 32) * n : c0;
+            T v[2][NPL];
+#pragma unroll
+            for (int m = 0; m < NPL; ++m) {
+                const int j = lane + 32 * m;
+                v[0][m] = j < n ? c0[j] : s_zero(T());
+                v[1][m] = j < n ? c1[j] : s_zero(T());
+            }
+            T y[2] = {s_zero(T()), s_zero(T())};
+            if (siv[0] >= 0) {
+                y[0] = lane < 16 ? c0[siv[0]] : c1[siv[0]];
+            } else {
+#pragma unroll
+                for (int m = 0; m < NPL; ++m) {
+                    const int j = lane + 32 * m;
+                    if (j < n) {
+                        const T vj = sV[j];
+                        y[0] = s_fma(vj, v[0][m], y[0]);
+                        y[1] = s_fma(vj, v[1][m], y[1]);
+                    }
+                }
+                warp_sum_spread<2>(y);   // lanes 0 .. 15: column l, the others: the second
+            }
+            const T z = s_fma(sR[0], y[0], s_zero(T()));
+            const T z0 = shfl(z, 0), z1 = shfl(z, 16);
+#pragma unroll
+            for (int m = 0; m < NPL; ++m) {
+                const int j = lane + 32 * m;
+                if (j < n) {
+                    const T xj = sX[j];
+                    c0[j] = s_fms(xj, z0, v[0][m]);
+                    if (two) c1[j] = s_fms(xj, z1, v[1][m]);
+                }
+            }
+        }
+        return;
+    }
     for (int l = it.y + wid; l < it.z; l += PT / 32) {
         T* col = Gw + (long long)l * n;
         T v[NPL];

@@ -104,3 +104,26 @@ def test_single_precision_ratio_bits_do_not_depend_on_the_path(dt):
         sts[0].accept()
         b, _, _ = sts[1].step_persistent(*ops)
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dt", list(DT))
+@pytest.mark.parametrize("n", [1, 9, 17, 33, 64, 250, 257, 513])
+@pytest.mark.parametrize("onehot", [False, True])
+def test_plain_rank_one_accept(dt, n, onehot):
+    """Pairs of columns per warp, a last column without a partner, one-hot V."""
+    L = lrugb()
+    tdt, tol, A, U, V = case(dt, n, 1)
+    W = A.shape[0]
+    st = L.LowRankState("det", W, n, k=1, dtype=tdt)
+    st.init(tdev(A, tdt))
+    cur = A.copy()
+    for t in range(2):
+        v, op = V[t].copy(), L.Operand(dense=tdev(V[t], tdt))
+        if onehot:
+            at = (np.arange(W) * 7 + t) % n
+            v = np.eye(n)[at][:, None, :]
+            op = L.Operand(idx=torch.tensor(at[:, None].astype(np.int32), device="cuda"), onehot_mask=1)
+        st.propose_det(L.Operand(dense=tdev(U[t], tdt)), op)
+        st.accept()
+        cur = cur + U[t].transpose(0, 2, 1) @ v
+    close(st.inverse().cpu().numpy(), np.linalg.inv(cur), tol)
