@@ -139,9 +139,10 @@ struct OzWork {
 };
 // columns a split-product update writes: [c_lo, c_hi) minus [s_lo, s_hi), in
 // the 128-column tiles jt_lo .. jt_hi - 1 (doubles), rows from tile it_lo on; a
-// walker's M is rows x ld (the padded sizes of the slices, or the state's own)
+// walker's M is rows x ld (the padded sizes of the slices, or the state's own);
+// the row tiles are cut into rsplit parts
 struct OzCols {
-    int c_lo, c_hi, s_lo, s_hi, jt_lo, jt_hi, it_lo, rows, ld;
+    int c_lo, c_hi, s_lo, s_hi, jt_lo, jt_hi, it_lo, rows, ld, rsplit;
 };
 // rows of the working matrix of an n x n inverse: n padded by the identity
 int oz_rows(int n);

@@ -344,7 +344,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const uint32_t tmem = s_tmem;
     const uint32_t bytes_a = (uint32_t)OZ_S * OZ_SLICE_A, bytes_b = STAGE;
     const int ntj = cols.jt_hi - cols.jt_lo, nti = nr / OZ_TI;
-    const long long units = (long long)W * ntj;
+    const int rs = cols.rsplit, ntr = nti - cols.it_lo;   // row tiles of a unit: an rs-th of the block's
+    const long long units = (long long)W * ntj * rs;
+    auto walker = [&](long long un) { return (int)(un / (ntj * rs)); };
+    auto block = [&](long long un) { return (cols.jt_lo + (int)(un % ntj)) * OZ_TJ; };
+    auto first = [&](long long un) { return cols.it_lo + (int)(un / ntj % rs) * ntr / rs; };
+    auto past = [&](long long un) { return cols.it_lo + ((int)(un / ntj % rs) + 1) * ntr / rs; };
     uint32_t T = 0, U = 0;   // tiles and units done; every role walks the same ones
     auto give_up = [&]() {
         set_dev_error(err, DEV_ERR_TIMEOUT);
@@ -356,9 +361,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         //      M values, and shared memory for one, are not to be had) ----
         bool ok = true;
         for (long long un = blockIdx.x; un < units && ok; un += gridDim.x) {
-            const int w = (int)(un / ntj);
+            const int w = walker(un);
             if (mask && !mask[w]) continue;
-            const int j0 = (cols.jt_lo + (int)(un % ntj)) * OZ_TJ;
+            const int j0 = block(un), end = past(un);
             const int p0 = max(j0, cols.c_lo), p1 = min(j0 + OZ_TJ, cols.c_hi);   // multiples of 64
             const double* Mp = Z.M + (long long)w * cols.rows * cols.ld + p0;
             // rows past the walker's last column (a 128-wide tile at nc % 128 == 64) are
@@ -375,7 +380,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 }
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
-            for (int it = cols.it_lo; it < nti && ok; ++it) {
+            for (int it = first(un); it < end && ok; ++it) {
                 if (lane == 0) {
                     const uint32_t st = T & 1;
                     if (T >= 2) ok = oz_wait(m_pfree + 8 * st, ((T - 2) >> 1) & 1, &s_abort);
@@ -409,10 +414,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const uint64_t a0 = desc_sw128(smem_u32(sA));
         bool ok = true;
         for (long long un = blockIdx.x; un < units && ok && lane == 0; un += gridDim.x) {
-            if (mask && !mask[(int)(un / ntj)]) continue;
+            if (mask && !mask[walker(un)]) continue;
             ok = oz_wait(m_sfull, U & 1, &s_abort);
             ++U;
-            for (int it = cols.it_lo; it < nti && ok; ++it, ++T) {
+            const int tiles = past(un) - first(un);
+            for (int it = 0; it < tiles && ok; ++it, ++T) {
                 const uint32_t st = T & 1;
                 ok = oz_wait(m_pfull + 8 * st, (T >> 1) & 1, &s_abort);
                 if (!ok) break;
@@ -439,13 +445,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const uint32_t lanes = (uint32_t)(32 * quad) << 16;
         bool ok = true;
         for (long long un = blockIdx.x; un < units && ok; un += gridDim.x) {
-            const int w = (int)(un / ntj);
+            const int w = walker(un), end = past(un);
             if (mask && !mask[w]) continue;
-            const int j = (cols.jt_lo + (int)(un % ntj)) * OZ_TJ + 32 * quad + lane;   // this thread's column
+            const int j = block(un) + 32 * quad + lane;   // this thread's column
             const bool keep = j >= cols.c_lo && j < cols.c_hi && !(j >= cols.s_lo && j < cols.s_hi);
             const bool wact = __any_sync(0xffffffffu, keep);   // a warp with no column to write only keeps step
             const int eSj = j < nc ? Z.eS[(long long)w * nc + j] : 0;
-            for (int it = cols.it_lo; it < nti; ++it, ++T) {
+            for (int it = first(un); it < end; ++it, ++T) {
                 const int i0 = it * OZ_TI + 16 * part;
                 double* Mj = Z.M + ((long long)w * cols.rows + i0) * cols.ld + j;
                 // this thread writes row c
@@ -660,6 +666,17 @@ static bool oz_map(CUtensorMap* m, const void* base, long long rows, int box_row
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Parts into which the row tiles of a column block are cut: few blocks (the
+// sub-panel products have one per walker) leave SMs idle or a last wave nearly
+// empty; a part loads the block's S slices again (about 2 us), so it keeps four
+// tiles (about 6 us each) or more.  Sub-panel products of a refresh of 512 walkers,
+// n = 1024: 20.5 -> 17.8 ms.
+static int oz_rsplit(int blocks, int tiles, int nsm) {
+    int rs = 1;
+    while (blocks * rs < 6 * nsm && tiles / (2 * rs) >= 4) rs *= 2;
+    return rs;
+}
+
 // Gauss-Jordan elimination of the W matrices Z.M (nr rows, nr % 64 == 0 up to
 // 1024, % 128 above) of the walkers with mask[w] (NULL: all): the row exchanges
 // stay in Z.perm, the pivots in Z.piv.  lu: rows above a panel and columns left
@@ -696,7 +713,7 @@ bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, 
             launch_oz_subpanel<T>(W, nr, k0, sp, lu, Z, mask, st);
             k_oz_slice_P16<<<dim3((nr - i0) / 16, W), 256, 0, st>>>(nr, nc, CX, i0, ks * CX, SW * CX, Z, mask);
             k_oz_slice_S<CX><<<dim3(1, W), 256, 0, st>>>(nr, nc, ks, SW, c0 / 64, Z, mask);
-            const OzCols inner{c0, c0 + OZ_B, ks * CX, (ks + SW) * CX, jt, jt + 1, it0, nr, nc};
+            const OzCols inner{c0, c0 + OZ_B, ks * CX, (ks + SW) * CX, jt, jt + 1, it0, nr, nc, oz_rsplit(W, nr / OZ_TI - it0, nsm)};
             k_oz_gemm<1, false><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, inner, Z, mask, err);
         }
         if (hook) { hook(hctx, 4, 0); hook(hctx, 5, 1); }
@@ -704,7 +721,8 @@ bool oz_eliminate(int W, int nr, const OzWork& Z, const uint8_t* mask, bool lu, 
         if (!lu || kn < nr) {
             k_oz_slice_P<<<dim3((nr - in) / 8, W), 256, 0, st>>>(nr, nc, CX, in, c0, OZ_B, Z, mask);
             k_oz_slice_S<CX><<<dim3((nc - cl) / 64, W), 256, 0, st>>>(nr, nc, k0, PB, cl / 64, Z, mask);
-            const OzCols outer{cl, nc, c0, c0 + OZ_B, cl / OZ_TJ, ntj, itn, nr, nc};
+            const OzCols outer{cl, nc, c0, c0 + OZ_B, cl / OZ_TJ, ntj, itn, nr, nc,
+                               oz_rsplit(W * (ntj - cl / OZ_TJ), nr / OZ_TI - itn, nsm)};
             k_oz_gemm<OZ_B / 16, false><<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, outer, Z, mask, err);
         }
         if (hook) hook(hctx, 5, 0);
@@ -781,7 +799,7 @@ bool launch_flush_split(int W, int n, int K, int kk, const T* P, const T* Q, dou
         case 4: kern = edge ? k_oz_gemm<4, true> : k_oz_gemm<4, false>; break;
         default: break;
     }
-    const OzCols all{0, n * CX, -1, -1, 0, (nc + OZ_TJ - 1) / OZ_TJ, 0, n, n * CX};
+    const OzCols all{0, n * CX, -1, -1, 0, (nc + OZ_TJ - 1) / OZ_TJ, 0, n, n * CX, 1};
     kern<<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, all, Z, Z.go, err);
     return true;
 }
