@@ -181,11 +181,12 @@ template <typename T>
 void launch_oz_store(int W, int w0, int n, int nr, const DevLayout& L, const DevState<T>& S, const OzWork& Z,
                      const uint8_t* mask, double* drift, bool delayed, bool pf, cudaStream_t st);
 // delayed flush A_0^{-1} += sgnQ * P Q^T (determinant: -1, Pfaffian: +1) as the
-// same exact split product (uniform n, K kk <= 64 doubles a row; Z of oz_flush_rows(n)
+// same exact split product (uniform n, K kk <= 64 doubles a row, kv: ranks of the
+// walkers, NULL: kk each; Z of oz_flush_rows(n)
 // rows, Z.M the state); walkers with tau >= K, or force && tau > 0
 constexpr int oz_flush_rows(int n) { return (n + 63) / 64 * 64; }
 template <typename T>
-bool launch_flush_split(int W, int n, int K, int kk, const T* P, const T* Q, double sgnQ, const int* tau,
+bool launch_flush_split(int W, int n, int K, int kk, const int* kv, const T* P, const T* Q, double sgnQ, const int* tau,
                         const uint8_t* force, const OzWork& Z, int* err, cudaStream_t st);
 // A_0^{-1} of the same walkers: the lower triangle := the exact negative of the
 // upper, diagonal 0 (after the Pfaffian split-product flush)

@@ -831,8 +831,8 @@ static lru_status do_flush(lru_handle h, const uint8_t* force) {
         bool ok = false;
         auto go = [&](auto tag) {
             using T = decltype(tag);
-            ok = launch_flush_split<T>(h->W, h->n_uni, h->K, h->kk, (const T*)h->P, (const T*)h->Q, h->pf ? 1.0 : -1.0,
-                                       h->tau, force, Z, h->err, h->stream);
+            ok = launch_flush_split<T>(h->W, h->n_uni, h->K, h->kk, h->d_kv, (const T*)h->P, (const T*)h->Q,
+                                       h->pf ? 1.0 : -1.0, h->tau, force, Z, h->err, h->stream);
             if (ok && h->pf) launch_skew_project<T>(h->W, h->n_uni, h->K, (T*)h->G, h->tau, force, h->stream);
         };
         if (h->dtype == LRU_C128) go(c128());

@@ -521,7 +521,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 //     half the exponent gap of the two columns' maxima: P Q^T is unchanged exactly,
 //     and the entries of a row span a far smaller range;
 //   - the slices and exponents of the rows of P (complex: two rows each, see
-//     k_oz_slice_S) and of sgnQ Q, the cu filled slot columns, zeros after.
+//     k_oz_slice_S) and of sgnQ Q, the cu columns of the tau filled slots (of the
+//     walker's own rank each, kv; the row stride is the handle's rank's), zeros after.
 // A walker with slots above 2^480, where a product of scales could leave the
 // exponent range, is folded here in FP64 instead and not flagged.
 // One launch in place of four (flags, balance, two slicings): a step without a
@@ -529,8 +530,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 __device__ __forceinline__ double oz_pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_oz_flush_slices(int W, int n, int nr, int K, int kk, const T* P, const T* Q,
-                                                         double sgnQ, const int* tau, const uint8_t* force, OzWork Z) {
+__global__ void __launch_bounds__(256) k_oz_flush_slices(int W, int n, int nr, int K, int kk, const int* kv, const T* P,
+                                                         const T* Q, double sgnQ, const int* tau, const uint8_t* force,
+                                                         OzWork Z) {
     constexpr int CX = traits<T>::is_complex ? 2 : 1;
     __shared__ int sp[4][OZ_B], sq[4][OZ_B], s_big;
     __shared__ double s_fp[OZ_B], s_fq[OZ_B];
@@ -545,7 +547,7 @@ __global__ void __launch_bounds__(256) k_oz_flush_slices(int W, int n, int nr, i
             s_big = 0;
         }
         if (!due) continue;
-        const int cu = t * kk * CX;   // doubles
+        const int slots = t * (kv ? kv[w] : kk), cu = slots * CX;   // filled columns, and their doubles
         const double* Pw = reinterpret_cast<const double*>(P) + (long long)w * n * ldx;
         const double* Qw = reinterpret_cast<const double*>(Q) + (long long)w * n * ldx;
         int ep = 0, eq = 0;
@@ -579,7 +581,7 @@ __global__ void __launch_bounds__(256) k_oz_flush_slices(int W, int n, int nr, i
             for (long long e = threadIdx.x; e < (long long)n * n; e += 256) {
                 const int l = (int)(e / n), j = (int)(e - (long long)l * n);
                 T d = s_zero(T());
-                for (int q = 0; q < t * kk; ++q)
+                for (int q = 0; q < slots; ++q)
                     d = s_fma(P[((long long)w * n + j) * K * kk + q], Q[((long long)w * n + l) * K * kk + q], d);
                 G[e] = sgnQ < 0 ? G[e] - d : G[e] + d;
             }
@@ -755,7 +757,7 @@ bool launch_refresh_oz(int W, int n, const double* A, const OzWork& Z, const Dev
 // columns, the -Q rows that of the panel rows, no column is skipped.  The slices
 // are padded to a multiple of 64 rows, the state is not.
 template <typename T>
-bool launch_flush_split(int W, int n, int K, int kk, const T* P, const T* Q, double sgnQ, const int* tau,
+bool launch_flush_split(int W, int n, int K, int kk, const int* kv, const T* P, const T* Q, double sgnQ, const int* tau,
                         const uint8_t* force, const OzWork& Z, int* err, cudaStream_t st) {
     constexpr int CX = traits<T>::is_complex ? 2 : 1;
     const int kw = K * kk * CX, nr = oz_flush_rows(n), nc = nr * CX;
@@ -790,7 +792,7 @@ bool launch_flush_split(int W, int n, int K, int kk, const T* P, const T* Q, dou
     int dev = 0, nsm = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    k_oz_flush_slices<T><<<std::min(W, 8 * nsm), 256, 0, st>>>(W, n, nr, K, kk, P, Q, sgnQ, tau, force, Z);
+    k_oz_flush_slices<T><<<std::min(W, 8 * nsm), 256, 0, st>>>(W, n, nr, K, kk, kv, P, Q, sgnQ, tau, force, Z);
     const bool edge = n != nr;
     auto kern = edge ? k_oz_gemm<1, true> : k_oz_gemm<1, false>;
     switch ((kw + 15) / 16) {
@@ -804,9 +806,9 @@ bool launch_flush_split(int W, int n, int K, int kk, const T* P, const T* Q, dou
     return true;
 }
 
-template bool launch_flush_split<double>(int, int, int, int, const double*, const double*, double, const int*,
+template bool launch_flush_split<double>(int, int, int, int, const int*, const double*, const double*, double, const int*,
                                          const uint8_t*, const OzWork&, int*, cudaStream_t);
-template bool launch_flush_split<c128>(int, int, int, int, const c128*, const c128*, double, const int*,
+template bool launch_flush_split<c128>(int, int, int, int, const int*, const c128*, const c128*, double, const int*,
                                        const uint8_t*, const OzWork&, int*, cudaStream_t);
 
 // Exact skew symmetry of the flushed walkers' A_0^{-1}, after the Pfaffian
