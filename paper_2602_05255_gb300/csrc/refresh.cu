@@ -1052,7 +1052,7 @@ __global__ void __launch_bounds__(ST) k_oz_store(int w0, int n, int nr, DevLayou
     T* G = S.G + (long long)w * n * n;
     const T* Mw = reinterpret_cast<const T*>(Z.M) + (long long)blockIdx.x * nr * nr;
     const long long vo = (long long)w * n;
-    const int cu = delayed ? S.tau[w] * L.kk : 0, lane = threadIdx.x & 31;
+    const int cu = delayed ? S.tau[w] * L.kv(w) : 0, lane = threadIdx.x & 31;
     double num = 0.0, den = 0.0;
     for (int l = threadIdx.x >> 5; l < n; l += ST / 32) {
         const T* mrow = Mw + (long long)l * nr;   // [l][j] = (A^{-1})_{jl}

@@ -1,5 +1,6 @@
 """Uniform n with a rank per walker below the handle's: a flush of partly filled
-slots reads the columns its walker has filled and no others.
+slots reads the columns its walker has filled and no others, and so does the
+drift of a refresh.
 
 The handle of W walkers takes the split-product flush (W n^2 kk cx^2 >= 2^24) and
 the padded elimination, the one of a few walkers FP64 tiles and the FP64
@@ -40,7 +41,7 @@ def build(kind, cplx, n, k, K):
             st.propose_pf(u) if kind == "pf" else st.propose_det(u, v)
             st.accept(None if accept is None else accept[:st.W].contiguous())
 
-    return sts, step, few, (64 * K * kk + 32 * n) * EPS
+    return sts, A, step, few, (64 * K * kk + 32 * n) * EPS
 
 
 def same(sts, few, tol):
@@ -55,7 +56,7 @@ CASES = [("det", False, 128, 2, 4), ("det", False, 130, 4, 8), ("det", True, 129
 
 @pytest.mark.parametrize("kind,cplx,n,k,K", CASES)
 def test_partial_flush(kind, cplx, n, k, K):
-    sts, step, few, tol = build(kind, cplx, n, k, K)
+    sts, _, step, few, tol = build(kind, cplx, n, k, K)
     for _ in range(K):
         step()
     same(sts, few, tol)
@@ -67,3 +68,13 @@ def test_partial_flush(kind, cplx, n, k, K):
     assert torch.equal(sts[0].tau()[:few], sts[1].tau())
     same(sts, few, tol)
     sts[0].check_device_error()
+
+
+@pytest.mark.parametrize("kind,cplx,n,k,K", CASES)
+def test_drift_of_pending_slots(kind, cplx, n, k, K):
+    sts, A, step, few, tol = build(kind, cplx, n, k, K)
+    for _ in range(K + K // 2):
+        step()
+    drift = [st.refresh(A[:st.W].contiguous())[:few] for st in sts]
+    assert (drift[0] - drift[1]).abs().max() <= tol * max(1.0, drift[1].abs().max().item()), drift
+    same(sts, few, tol)
