@@ -207,10 +207,11 @@ __device__ __forceinline__ void oz_mma(uint32_t dtmem, uint64_t a, uint64_t b, u
 
 // Levels 2 .. 6 of one element are integers N_l 2^(-8l), |N_l| < 2^23 (a float holds
 // them exactly), and the tail (levels 7 .. 10) is rounded to a multiple of 2^-56:
-// their sum F in units of 2^-56, |F| < 2^62, exactly, as two words.  N_2, N_3
-// (|N| <= 2^22) and the tail come out of the mantissa of x * scale + 1.5 * 2^23
-// (a tail above 2^22 is rounded to 2 units); the others can exceed 2^22 and take
-// the conversion unit.
+// their sum F in units of 2^-56, |F| < 2^62, exactly, as two words.  A level that
+// stays within 2^22 comes out of the mantissa of x * scale + 1.5 * 2^23, which
+// holds no more: N_2 and N_3 always, the tail of a single K-step (below 2^21 +
+// 2^14).  N_4 .. N_6 and the tail of more (up to 2^23 + 2^16 at 64) take the
+// conversion unit.
 __device__ __forceinline__ void oz_sum2(float a2, float a3, int& hi) {
     constexpr float magic = 12582912.0f;
     const int n2 = __float_as_int(__fmaf_rn(a2, 65536.0f, magic)), n3 = __float_as_int(__fmaf_rn(a3, 16777216.0f, magic));
@@ -221,9 +222,11 @@ __device__ __forceinline__ void oz_sum4(float a4, float a5, int& hi, uint32_t& l
     lo = (uint32_t)b << 16;
     hi += b >> 16;
 }
+template <bool ONE_STEP>
 __device__ __forceinline__ void oz_sum6(float a6, float tail, int& hi, uint32_t& lo) {
-    const int c = __float2int_rn(a6 * 281474976710656.0f) * 256 +
-                  (__float_as_int(__fmaf_rn(tail, 72057594037927936.0f, 12582912.0f)) - 0x4B400000);
+    constexpr float unit = 72057594037927936.0f;   // 2^56
+    const int t = ONE_STEP ? __float_as_int(__fmaf_rn(tail, unit, 12582912.0f)) - 0x4B400000 : __float2int_rn(tail * unit);
+    const int c = __float2int_rn(a6 * 281474976710656.0f) * 256 + t;
     const uint32_t l = lo + (uint32_t)c;
     hi += (c >> 31) + (l < lo ? 1 : 0);
     lo = l;
@@ -484,7 +487,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                         tmem_ld8(oz_acc(tmem, 4, T) + lanes + c0, x);
                         tmem_ld8(oz_acc(tmem, 5, T) + lanes + c0, y);
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) oz_sum6(x[c], y[c], fh[8 * ch + c], fl[8 * ch + c]);
+                        for (int c = 0; c < 8; ++c) oz_sum6<NKS == 1>(x[c], y[c], fh[8 * ch + c], fl[8 * ch + c]);
                     }
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
