@@ -232,7 +232,8 @@ __device__ __forceinline__ void oz_sum6(float a6, float tail, int& hi, uint32_t&
     lo = l;
 }
 
-// F * 2^(e - 56) as a double, rounded to nearest (ties away), by integer operations
+// F * 2^(e - 56) as a double, rounded to nearest even (products of 53-bit values have
+// many ties), by integer operations
 // (results below the normal range become zero; the callers keep away from the upper end).  The
 // mantissa with its leading one is added to the exponent field less one, so a
 // rounding that carries out of it needs no case of its own.
@@ -243,8 +244,8 @@ __device__ __forceinline__ double oz_to_double(int hi, uint32_t lo, int e) {
     const unsigned long long a = (F ^ sx) - sx;   // |F|
     const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a;
     const int lz = __clz((int)(ah ? ah : al)) + (ah ? 0 : 32);
-    const unsigned long long v = a << (lz & 63);                 // leading one at bit 63
-    const unsigned long long mant = (v >> 11) + ((v >> 10) & 1ull);
+    const unsigned long long v = a << ((lz - 1) & 63);           // leading one at bit 62 (|F| < 2^63)
+    const unsigned long long mant = (v + (0x1FFu + ((uint32_t)(v >> 10) & 1u))) >> 10;
     const uint32_t rh = (uint32_t)(mant >> 32) + ((uint32_t)(1029 + e - lz) << 20);
     const bool nz = a != 0 && 1029 + e - lz > 0;   // below the normal range: zero
     return __hiloint2double(nz ? (int)(rh | ((uint32_t)s & 0x80000000u)) : 0, nz ? (int)(uint32_t)mant : 0);

@@ -85,3 +85,18 @@ def test_level_sums_are_added_exactly(lib, products):
         lib.recombine(a.ctypes.data_as(ctypes.c_void_p), products == 16, 0, ctypes.byref(F), ctypes.byref(d))
         want = sum(x << (56 + s) for x, s in zip(N, SCALE))
         assert F.value == want, (N, F.value - want)
+
+
+def test_conversion_rounds_to_nearest_even(lib):
+    g = np.random.Generator(np.random.PCG64(3))
+    for trial in range(6000):
+        F = int(g.integers(-2 ** 62, 2 ** 62)) >> int(g.integers(0, 62))
+        if trial % 3 == 0:              # a tie, or one beside it
+            m = int(g.integers(2 ** 52, 2 ** 53))
+            sh = int(g.integers(1, 9))
+            F = (m << sh) + (1 << (sh - 1)) + int(g.integers(-1, 2))
+            F = -F if trial % 2 else F
+        e = int(g.integers(-400, 400))
+        assert lib.to_double(F, e) == np.ldexp(float(F), e - 56), (F, e)   # int to float rounds to even
+    assert lib.to_double(2 ** 62 - 1, 0) == 64.0
+    assert lib.to_double(0, 5) == 0.0
