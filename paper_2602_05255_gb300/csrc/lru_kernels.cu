@@ -334,16 +334,17 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
         } else if (pf2) {
             // M = [[0, h], [-h, 0]] after the projection: pf M = h, pf C^{-1} = 1,
             // M^{-1} = [[0, -1/h], [1/h, 0]]; the bits and the status of the loops
-            // below, without their dependent cycles in one thread (1024 walkers,
-            // n = 256, K = 8: a propose 57 -> 42 us)
+            // below (ratio 0 where the core is singular or NaN), without their
+            // dependent cycles in one thread (1024 walkers, n = 256, K = 8: a propose
+            // 57 -> 42 us)
             const T h = s_half(s_core[1] - s_core[MAXKK]);
             const T ih = s_recip(h);
             s_inv[0] = s_inv[MAXKK + 1] = s_zero(T());
             s_inv[1] = s_neg(ih);
             s_inv[MAXKK] = ih;
-            ratio = h;
-            st = !((double)s_abs2(h) > 0.0) ? CORE_SINGULAR
-                                            : (s_isfinite(h * h) && s_isfinite(h) ? CORE_OK : CORE_NONFINITE);
+            const bool regular = (double)s_abs2(h) > 0.0;
+            ratio = regular ? h : s_zero(T());
+            st = !regular ? CORE_SINGULAR : (s_isfinite(h * h) && s_isfinite(h) ? CORE_OK : CORE_NONFINITE);
         } else {
             // The skew-form updates (Eq. pf_delayed_Ainv, and the exactly skew
             // plain accept) need M and M^{-1} exactly skew; a generic Woodbury
