@@ -780,23 +780,6 @@ bool launch_flush_split(int W, int n, int K, int kk, const int* kv, const T* P, 
         cached_rows[0] = rows;
         cached_rows[1] = prow;
     }
-    const size_t dyn = OZ_GEMM_SMEM;
-    static thread_local bool attr = false;
-    if (!attr) {
-        bool ok = true;
-        for (auto kern : {k_oz_gemm<1, false>, k_oz_gemm<2, false>, k_oz_gemm<3, false>, k_oz_gemm<4, false>,
-                          k_oz_gemm<1, true>, k_oz_gemm<2, true>, k_oz_gemm<3, true>, k_oz_gemm<4, true>})
-            ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) == cudaSuccess;
-        if (!ok) {
-            cudaGetLastError();
-            return false;
-        }
-        attr = true;
-    }
-    int dev = 0, nsm = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    k_oz_flush_slices<T><<<std::min(W, 8 * nsm), 256, 0, st>>>(W, n, nr, K, kk, kv, P, Q, sgnQ, tau, force, Z);
     const bool edge = n != nr;
     auto kern = edge ? k_oz_gemm<1, true> : k_oz_gemm<1, false>;
     switch ((kw + 15) / 16) {
@@ -805,6 +788,16 @@ bool launch_flush_split(int W, int n, int K, int kk, const int* kv, const T* P, 
         case 4: kern = edge ? k_oz_gemm<4, true> : k_oz_gemm<4, false>; break;
         default: break;
     }
+    // on every call: the limit belongs to the current device, not to the thread
+    const size_t dyn = OZ_GEMM_SMEM;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    int dev = 0, nsm = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    k_oz_flush_slices<T><<<std::min(W, 8 * nsm), 256, 0, st>>>(W, n, nr, K, kk, kv, P, Q, sgnQ, tau, force, Z);
     const OzCols all{0, n * CX, -1, -1, 0, (nc + OZ_TJ - 1) / OZ_TJ, 0, n, n * CX, 1};
     kern<<<nsm, OZ_THREADS, dyn, st>>>(maps, W, nr, nc, all, Z, Z.go, err);
     return true;

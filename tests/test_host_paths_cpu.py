@@ -1,0 +1,90 @@
+"""Host side of the library on a fake CUDA runtime (fake_cudart.c): what is
+allocated, which launches are made and with which arguments, and what a call answers
+when the runtime refuses one.  Each scenario runs in a child process.
+"""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+HERE = os.path.dirname(os.path.abspath(__file__))
+LIB = os.path.join(ROOT, "paper_2602_05255_gb300", "liblrugb.so")
+
+PRELUDE = r"""
+import ctypes as C
+fake = C.CDLL(None)
+lib = C.CDLL(LIB)
+for f, r, a in (("fake_alloc_limit", None, [C.c_size_t]), ("fake_refuse_launch", None, [C.c_char_p]),
+                ("fake_watch", None, [C.c_char_p, C.c_int]), ("fake_launch_name", C.c_char_p, [C.c_int]),
+                ("fake_launch_arg", C.c_void_p, [C.c_int]), ("fake_alloc_bytes", C.c_size_t, [C.c_int])):
+    getattr(fake, f).restype, getattr(fake, f).argtypes = r, a
+DET, PF, F64, C128, F32, C64, OK = 0, 1, 0, 1, 2, 3, 0
+SIZE = {F64: 8, C128: 16, F32: 4, C64: 8}
+
+class Cfg(C.Structure):
+    _fields_ = [("kind", C.c_int32), ("dtype", C.c_int32), ("walkers", C.c_int64), ("n", C.c_int32),
+                ("n_per_walker", C.c_void_p), ("k", C.c_int32), ("k_per_walker", C.c_void_p),
+                ("delay", C.c_int32), ("flush", C.c_int32), ("device", C.c_int32), ("arith", C.c_int32),
+                ("tile_chunks", C.c_int32), ("refresh", C.c_int32)]
+
+class Operand(C.Structure):
+    _fields_ = [("dense", C.c_void_p), ("idx", C.c_void_p), ("onehot_mask", C.c_uint32)]
+
+PTR = C.c_void_p(4096)    # a device pointer: nothing reads through it
+
+def create(kind=DET, dtype=F64, W=1024, n=128, k=1, delay=4, device=0, refresh=0, flush=0):
+    cfg = Cfg(kind=kind, dtype=dtype, walkers=W, n=n, k=k, delay=delay, device=device, refresh=refresh, flush=flush)
+    h = C.c_void_p()
+    assert lib.lru_create(C.byref(cfg), C.byref(h)) == OK
+    return h
+
+def init(h, kind=DET):
+    return (lib.lru_init_pf if kind == PF else lib.lru_init_det)(h, PTR, PTR, PTR)
+
+def propose(h):
+    o = Operand(4096, None, 0)
+    return lib.lru_propose_det(h, C.byref(o), C.byref(o), PTR, PTR)
+
+def accept(h):
+    return lib.lru_accept(h, None)
+
+def names():
+    return [fake.fake_launch_name(i).decode() for i in range(fake.fake_launches())]
+
+def refused():
+    return [n for i, n in enumerate(names()) if not fake.fake_launch_ok(i)]
+
+def sizes(ok=None):
+    return [fake.fake_alloc_bytes(i) for i in range(fake.fake_allocs()) if ok is None or fake.fake_alloc_ok(i) == ok]
+"""
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    if not os.path.exists(LIB):
+        import __graft_entry__
+        __graft_entry__.build()
+    so = str(tmp_path_factory.mktemp("fake") / "libfakecudart.so")
+    subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-o", so, os.path.join(HERE, "fake_cudart.c")], check=True)
+
+    def go(body):
+        r = subprocess.run([sys.executable, "-c", f"LIB = {LIB!r}\n" + PRELUDE + textwrap.dedent(body)],
+                           env={**os.environ, "LD_PRELOAD": so}, capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stdout + r.stderr
+
+    return go
+
+
+def test_flush_of_handles_on_two_devices(run):
+    """The shared-memory limit of a kernel belongs to the device: the second one is not left with the first's."""
+    run("""
+        hs = [create(n=130, device=d) for d in (0, 1)]     # the kernel of ragged rows, which no elimination uses
+        for h in hs:
+            assert init(h) == OK
+            for _ in range(5):
+                assert propose(h) == OK and accept(h) == OK, (refused())
+        assert any("k_oz_gemm" in x for x in names()) and not refused()
+    """)
