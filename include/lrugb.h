@@ -201,7 +201,10 @@ lru_status lru_propose_pf(lru_handle h, const lru_operand* B, const void* C,
  * whose proposal status is OK: updates A^{-1} (plain: Eq. det_inv / Woodbury)
  * or stores the new delay slot (Sec. 2.3 / 3.3), adds log|ratio| to log|value|
  * and multiplies the sign/phase.  A walker whose delay slots are full is
- * folded into A_0^{-1} at once (the flush of Eq. delayed_Ainv). */
+ * folded into A_0^{-1} at once (the flush of Eq. delayed_Ainv).  If that fold
+ * cannot be launched the error is returned and the slots are kept; proposals and
+ * flushes then answer LRU_ERR_STATE until an init, a refresh of all walkers or
+ * lru_load_state. */
 lru_status lru_accept(lru_handle h, const uint8_t* mask);
 /* One persistent fused step for all walkers, including walkers of uneven n
  * and k: a single kernel launch of a fixed grid takes the proposals of every

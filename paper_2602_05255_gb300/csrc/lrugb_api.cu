@@ -100,6 +100,7 @@ struct lru_ctx {
     size_t prof_used[LRU_PROF_CLASSES] = {};
     long long launches = 0;
     // last proposal
+    bool flush_failed = false;   // a flush was not launched: its slots may be full, their fold half done
     bool has_prop = false;
     DevOperand lastV{};
     const void* lastC = nullptr;
@@ -658,6 +659,7 @@ static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, doub
                 CK(cudaMemcpyAsync(logabs_out, h->logabs, h->W * sizeof(double), cudaMemcpyDefault, h->stream));
             if (sign_out) CK(cudaMemcpyAsync(sign_out, h->sgn, h->W * sizeof(double), cudaMemcpyDefault, h->stream));
             h->has_prop = false;
+            if (!mask) h->flush_failed = false;
             return LRU_OK;
         }
         cudaGetLastError();   // tensor maps unavailable: the FP64 form below
@@ -690,6 +692,7 @@ static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, doub
     if (logabs_out) CK(cudaMemcpyAsync(logabs_out, h->logabs, h->W * sizeof(double), cudaMemcpyDefault, h->stream));
     if (sign_out) CK(cudaMemcpyAsync(sign_out, h->sgn, h->W * sz, cudaMemcpyDefault, h->stream));
     h->has_prop = false;
+    if (!mask) h->flush_failed = false;
     return LRU_OK;
 }
 
@@ -725,7 +728,7 @@ static bool operand_ok(const lru_operand* o, int kk) {
 lru_status lru_propose_det(lru_handle h, const lru_operand* U, const lru_operand* V, void* ratio, int32_t* st) {
     LRU_RANGE();
     if (!h || !ratio) return LRU_ERR_ARG;
-    if (h->pf) return LRU_ERR_STATE;
+    if (h->pf || h->flush_failed) return LRU_ERR_STATE;
     if (!operand_ok(U, h->kk) || !operand_ok(V, h->kk)) return LRU_ERR_ARG;
     CK(cudaSetDevice(h->device));
     DevOperand dU{U->dense, U->idx, U->onehot_mask, h->kk};
@@ -748,7 +751,7 @@ lru_status lru_propose_det(lru_handle h, const lru_operand* U, const lru_operand
 lru_status lru_propose_pf(lru_handle h, const lru_operand* B, const void* C, void* ratio, int32_t* st) {
     LRU_RANGE();
     if (!h || !ratio) return LRU_ERR_ARG;
-    if (!h->pf) return LRU_ERR_STATE;
+    if (!h->pf || h->flush_failed) return LRU_ERR_STATE;
     if (!operand_ok(B, h->kk)) return LRU_ERR_ARG;
     CK(cudaSetDevice(h->device));
     DevOperand dB{B->dense, B->idx, B->onehot_mask, h->kk};
@@ -773,6 +776,7 @@ lru_status lru_step_persistent(lru_handle h, const lru_operand* U, const lru_ope
                                uint8_t* acc_out) {
     LRU_RANGE();
     if (!h || !ratio) return LRU_ERR_ARG;
+    if (h->flush_failed) return LRU_ERR_STATE;
     if (!operand_ok(U, h->kk)) return LRU_ERR_ARG;
     if (!h->pf && !operand_ok(V, h->kk)) return LRU_ERR_ARG;
     CK(cudaSetDevice(h->device));
@@ -816,6 +820,8 @@ lru_status lru_step_persistent(lru_handle h, const lru_operand* U, const lru_ope
 }
 
 static lru_status do_flush(lru_handle h, const uint8_t* force) {
+    if (h->flush_failed) return LRU_ERR_STATE;
+    h->flush_failed = true;   // until the last launch is made
     DevLayout L = h->layout();
     prof_begin(h, LRU_PROF_FLUSH);
     h->launches += 2;
@@ -854,8 +860,14 @@ static lru_status do_flush(lru_handle h, const uint8_t* force) {
         LRU_DISPATCH(h, { launch_flush_native<T>(h->pf, L, h->state<T>(), force, h->n_max, h->stream); });
     }
     prof_end(h, LRU_PROF_FLUSH);
+    // slots whose product was not launched are not dropped (tau stays); the handle
+    // takes no update on top of them until an init, a full refresh or a load
+    lru_status s = cuda_check();
+    if (s != LRU_OK) return s;
     LRU_DISPATCH(h, { launch_flush_finish<T>(L, h->state<T>(), force, h->stream); });
-    return cuda_check();
+    s = cuda_check();
+    h->flush_failed = s != LRU_OK;
+    return s;
 }
 
 lru_status lru_accept(lru_handle h, const uint8_t* mask) {
@@ -943,6 +955,7 @@ lru_status lru_load_state(lru_handle h, const void* buf) {
     CK(cudaSetDevice(h->device));
     CK(cudaMemcpyAsync(h->base, buf, h->persist_bytes, cudaMemcpyDefault, h->stream));
     h->has_prop = false;
+    h->flush_failed = false;
     return LRU_OK;
 }
 

@@ -88,3 +88,22 @@ def test_flush_of_handles_on_two_devices(run):
                 assert propose(h) == OK and accept(h) == OK, (refused())
         assert any("k_oz_gemm" in x for x in names()) and not refused()
     """)
+
+
+@pytest.mark.parametrize("flush", [0, 6])
+def test_flush_that_is_not_launched_keeps_its_slots(run, flush):
+    """No launch that resets tau after a refused product, and no update on top of it before an init."""
+    run(f"""
+        h = create(flush={flush})
+        assert init(h) == OK
+        assert propose(h) == OK and accept(h) == OK
+        n = sum("k_flush_finish" in x for x in names())
+        assert n == 1
+        fake.fake_refuse_launch(b"k_oz_gemm")
+        assert propose(h) == OK and accept(h) == 2
+        assert sum("k_flush_finish" in x for x in names()) == n
+        fake.fake_refuse_launch(b"")
+        assert propose(h) == 4 and lib.lru_flush_delayed(h, None) == 4
+        assert init(h) == OK and propose(h) == OK and accept(h) == OK
+        assert sum("k_flush_finish" in x for x in names()) == n + 1
+    """)
