@@ -359,8 +359,9 @@ void launch_scatter_rows(const DevLayout& L, const T* gA, const int* rows, int m
 // inverses, Ginv[w][l n + j] = (A_w^{-1})_{jl}, so (A^{-H})_{ij} is
 // conj(Ginv[w][i n + j]).
 template <typename T>
-__global__ void k_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_t* compact, const double* g_l, const T* g_s, const T* sign,
-                            T* gA) {
+__global__ void k_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_t* compact, const int* fail,
+                            const double* g_l, const T* g_s, const T* sign, T* gA) {
+    const bool failed = fail && *fail;
     const long long nn = (long long)n * n, total = nn * W;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
@@ -368,7 +369,8 @@ __global__ void k_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const 
         const long long r = e - (long long)w * nn;
         const int i = (int)(r / n), j = (int)(r - (long long)i * n);
         const T* G = Ginv + (long long)w * nr * nr;
-        const int ld = compact && compact[w] ? n : nr;
+        const bool own = compact && compact[w];   // inverted by the FP64 form
+        const int ld = own ? n : nr;
         T c = make_real<T>(g_l ? g_l[w] : 0.0);
         if constexpr (traits<T>::is_complex) {
             if (g_s) {
@@ -378,21 +380,21 @@ __global__ void k_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const 
         }
         T v = G[(long long)i * ld + j];
         if (pf) v = s_half(s_half(v - G[(long long)j * ld + i]));   // (1/2) of the skew part
-        gA[e] = c * s_conj(v);
+        gA[e] = failed && !own ? make_real<T>(NAN) : c * s_conj(v);
     }
 }
 
 template <typename T>
-void launch_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_t* compact, const double* g_l, const T* g_s, const T* sign, T* gA,
-                      cudaStream_t st) {
+void launch_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_t* compact, const int* fail,
+                      const double* g_l, const T* g_s, const T* sign, T* gA, cudaStream_t st) {
     const long long total = (long long)n * n * W;
     const int grid = (int)std::min<long long>((total + 255) / 256, 152 * 16);
-    k_slog_grad<T><<<grid, 256, 0, st>>>(W, n, nr, pf, Ginv, compact, g_l, g_s, sign, gA);
+    k_slog_grad<T><<<grid, 256, 0, st>>>(W, n, nr, pf, Ginv, compact, fail, g_l, g_s, sign, gA);
 }
 
 #define LRU_INST_A(T)                                                                                        \
-    template void launch_slog_grad<T>(int, int, int, bool, const T*, const uint8_t*, const double*, const T*, const T*, T*,        \
-                                      cudaStream_t);                                                          \
+    template void launch_slog_grad<T>(int, int, int, bool, const T*, const uint8_t*, const int*, const double*, const T*,     \
+                                      const T*, T*, cudaStream_t);                                            \
     template void launch_backward<T>(bool, bool, const DevLayout&, const DevState<T>&, const DevOperand&,     \
                                      const T*, const T*, T*, T*, T*, T*, const int*, int, cudaStream_t);       \
     template void launch_backward_logvalue<T>(bool, bool, const DevLayout&, const DevState<T>&, const T*, T*, \

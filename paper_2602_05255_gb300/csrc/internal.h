@@ -136,6 +136,7 @@ struct OzWork {
     uint8_t* odd;     // W      walkers whose matrix is left to the FP64 form (see k_oz_sort)
     double* piv;      // W x nr scalars: pivots (log|det| and sign at the end)
     int* rmax;        // W x nr largest biased exponent of each row of M
+    int* fail;        // the error word of a call without a handle (its results become NaN), or NULL
 };
 // columns a split-product update writes: [c_lo, c_hi) minus [s_lo, s_hi), in
 // the 128-column tiles jt_lo .. jt_hi - 1 (doubles), rows from tile it_lo on; a
@@ -232,10 +233,11 @@ void launch_backward_logvalue(bool pf, bool delayed, const DevLayout& L, const D
 template <typename T>
 void launch_log_ratio(int W, const T* ratio, T* out, cudaStream_t st);
 // gradient of (sign, log|det|) or (phase, log|pf|) from the column-major inverses
-// (slots of nr^2 scalars, rows of nr; of n where compact[w])
+// (slots of nr^2 scalars, rows of nr; of n where compact[w]); NaN, except where
+// compact[w], if the word fail (NULL: none) is set
 template <typename T>
-void launch_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_t* compact, const double* g_l, const T* g_s, const T* sign, T* gA,
-                      cudaStream_t st);
+void launch_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_t* compact, const int* fail,
+                      const double* g_l, const T* g_s, const T* sign, T* gA, cudaStream_t st);
 template <typename T>
 void launch_scatter_rows(const DevLayout& L, const T* gA, const int* rows, int m, T* gPhi, int* err, cudaStream_t st);
 

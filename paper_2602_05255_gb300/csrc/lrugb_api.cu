@@ -1148,19 +1148,21 @@ static bool slogdet_padded(int W, int n, const T* A, double* logabs, T* sign, cu
     constexpr int cx = traits<T>::is_complex ? 2 : 1;
     const int nr = oz_rows(n), chunk = oz_chunk(W, n, cx);
     void* ws = nullptr;
-    if (cudaMallocAsync(&ws, oz_work_layout(nullptr, nullptr, chunk, nr, cx, true), st) != cudaSuccess) {
+    const size_t b = oz_work_layout(nullptr, nullptr, chunk, nr, cx, true);
+    if (cudaMallocAsync(&ws, b + sizeof(int), st) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     OzWork Z;
     oz_work_layout(&Z, ws, chunk, nr, cx, true);
-    bool ok = true;
+    Z.fail = (int*)((unsigned char*)ws + b);   // a wait that gives up sets it: NaN instead of a wrong result
+    bool ok = cudaMemsetAsync(Z.fail, 0, sizeof(int), st) == cudaSuccess;
     for (int w0 = 0; ok && w0 < W; w0 += chunk) {
         const int Wc = std::min(chunk, W - w0);
         const T* Aw = A + (size_t)w0 * n * n;
         launch_oz_load<T>(Wc, n, nr, Aw, false, true, Z, nullptr, st);
         launch_oz_sort(Wc, n, nr, Z, nullptr, st);
-        ok = oz_eliminate<T>(Wc, nr, Z, Z.go, true, nullptr, st, nullptr, nullptr);
+        ok = oz_eliminate<T>(Wc, nr, Z, Z.go, true, Z.fail, st, nullptr, nullptr);
         if (!ok) break;
         launch_oz_finish<T>(Wc, n, nr, false, Z, Z.go, logabs + w0, sign + w0, nullptr, nullptr, st);
         launch_slogdet<T>(Wc, n, Aw, (T*)Z.M, Wc, logabs + w0, sign + w0, Z.odd, st);
@@ -1176,23 +1178,25 @@ static bool slog_backward_padded(bool pf, int W, int n, const T* A, const double
     constexpr int cx = traits<T>::is_complex ? 2 : 1;
     const int nr = oz_rows(n), chunk = oz_chunk(W, n, cx);
     void* ws = nullptr;
-    if (cudaMallocAsync(&ws, oz_work_layout(nullptr, nullptr, chunk, nr, cx, true), st) != cudaSuccess) {
+    const size_t b = oz_work_layout(nullptr, nullptr, chunk, nr, cx, true);
+    if (cudaMallocAsync(&ws, b + sizeof(int), st) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     OzWork Z;
     oz_work_layout(&Z, ws, chunk, nr, cx, true);
-    bool ok = true;
+    Z.fail = (int*)((unsigned char*)ws + b);   // a wait that gives up sets it: NaN instead of a wrong result
+    bool ok = cudaMemsetAsync(Z.fail, 0, sizeof(int), st) == cudaSuccess;
     for (int w0 = 0; ok && w0 < W; w0 += chunk) {
         const int Wc = std::min(chunk, W - w0);
         const T* Aw = A + (size_t)w0 * n * n;
         launch_oz_load<T>(Wc, n, nr, Aw, true, true, Z, nullptr, st);
         launch_oz_sort(Wc, n, nr, Z, nullptr, st);
-        ok = oz_eliminate<T>(Wc, nr, Z, Z.go, false, nullptr, st, nullptr, nullptr);
+        ok = oz_eliminate<T>(Wc, nr, Z, Z.go, false, Z.fail, st, nullptr, nullptr);
         if (!ok) break;
         launch_oz_finish<T>(Wc, n, nr, true, Z, Z.go, nullptr, (T*)nullptr, nullptr, nullptr, st);
         launch_gj_compact<T>(Wc, n, nr, Aw, (T*)Z.M, Z.odd, st);
-        launch_slog_grad<T>(Wc, n, nr, pf, (const T*)Z.M, Z.odd, g_l ? g_l + w0 : nullptr, g_s ? g_s + w0 : nullptr,
+        launch_slog_grad<T>(Wc, n, nr, pf, (const T*)Z.M, Z.odd, Z.fail, g_l ? g_l + w0 : nullptr, g_s ? g_s + w0 : nullptr,
                             sign ? sign + w0 : nullptr, gA + (size_t)w0 * n * n, st);
     }
     cudaFreeAsync(ws, st);
@@ -1275,7 +1279,7 @@ static lru_status slog_backward(bool pf, int32_t dtype, int64_t W, int32_t n, co
         S.G = (T*)Ginv;
         S.pst = pst;
         launch_refresh<T>(false, false, L, S, (const T*)A, nullptr, (T*)ws, nws, nullptr, false, st);
-        launch_slog_grad<T>((int)W, n, n, pf, (const T*)Ginv, nullptr, g_logabs, (const T*)g_sign, (const T*)sign, (T*)gA, st);
+        launch_slog_grad<T>((int)W, n, n, pf, (const T*)Ginv, nullptr, nullptr, g_logabs, (const T*)g_sign, (const T*)sign, (T*)gA, st);
     });
     lru_status s = cuda_check();
     cudaFreeAsync(buf, st);

@@ -1006,6 +1006,10 @@ __global__ void __launch_bounds__(RT) k_oz_finish(int n, int nr, bool permute, O
         const int sing = Z.sing[w];
         if (logabs) logabs[w] = sing ? -INFINITY : la;
         if (sgn) sgn[w] = sing ? s_zero(T()) : s_renorm(s_unit_part[0]);
+        if (Z.fail && *Z.fail) {   // a wait of the products gave up, and there is no handle to say so
+            if (logabs) logabs[w] = NAN;
+            if (sgn) sgn[w] = make_real<T>(NAN);
+        }
         if (tau) tau[w] = 0;
         if (pst) pst[w] = sing ? 1 : 5;
     }

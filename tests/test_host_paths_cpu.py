@@ -107,3 +107,21 @@ def test_flush_that_is_not_launched_keeps_its_slots(run, flush):
         assert init(h) == OK and propose(h) == OK and accept(h) == OK
         assert sum("k_flush_finish" in x for x in names()) == n + 1
     """)
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_standalone_calls_see_a_wait_that_gives_up(run, dtype):
+    """The products of the calls without a handle get an error word, inside the call's own workspace."""
+    run(f"""
+        slogdet, grad = lib.lru_slogdet_batched, lib.lru_slogdet_backward
+        slogdet.argtypes = [C.c_int32, C.c_int64, C.c_int32] + [C.c_void_p] * 4
+        grad.argtypes = [C.c_int32, C.c_int64, C.c_int32] + [C.c_void_p] * 6
+        for watch, at, call in ((b"k_oz_gemm", 7, lambda: slogdet({dtype}, 4, 130, PTR, PTR, PTR, None)),
+                                (b"k_oz_gemm", 7, lambda: grad({dtype}, 4, 130, PTR, PTR, None, None, PTR, None)),
+                                (b"k_slog_grad", 6, lambda: grad({dtype}, 4, 130, PTR, PTR, None, None, PTR, None))):
+            fake.fake_reset()
+            fake.fake_watch(watch, at)
+            assert call() == OK
+            got = {{fake.fake_launch_arg(i) for i, x in enumerate(names()) if watch.decode() in x}}
+            assert len(got) == 1 and None not in got and len(sizes()) == 1, (watch, got)
+    """)
