@@ -404,14 +404,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                                      : "memory");
             }
         }
-        if (!ok) {
-            if (lane == 0) {
-                give_up();
-                // let copies in flight land before leaving
-                if (U > 0) mbar_wait(m_sfull, (U - 1) & 1);
-                if (T >= 1) mbar_wait(m_pfull + 8 * ((T - 1) & 1), ((T - 1) >> 1) & 1);
-                if (T >= 2) mbar_wait(m_pfull + 8 * (T & 1), ((T - 2) >> 1) & 1);
-            }
+        if (lane == 0) {
+            if (!ok) give_up();
+            // let copies in flight land before leaving, also when it is another role
+            // that has given up and does not wait for them
+            if (U > 0) mbar_wait(m_sfull, (U - 1) & 1);
+            if (T >= 1) mbar_wait(m_pfull + 8 * ((T - 1) & 1), ((T - 1) >> 1) & 1);
+            if (T >= 2) mbar_wait(m_pfull + 8 * (T & 1), ((T - 2) >> 1) & 1);
         }
     } else if (warp == OZ_EPI_WARPS + 1) {
         // ---- MMAs ----
@@ -437,10 +436,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 mma_commit(m_full);
             }
         }
-        if (!ok && lane == 0) {
-            give_up();
-            mma_commit(m_drain);
-            mbar_wait(m_drain, 0);
+        // MMAs in flight end before the TMEM goes back, whichever role gave up
+        if (lane == 0) {
+            if (!ok) {
+                give_up();
+                mma_commit(m_drain);
+                mbar_wait(m_drain, 0);
+            } else if (T > 0) {
+                mbar_wait(m_full, (T - 1) & 1);
+            }
         }
     } else {
         // ---- epilogue: warp q reads TMEM lanes 32 (q % 4) .. +31 (columns j) and
@@ -465,7 +469,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 double m[16];
 #pragma unroll
                 for (int c = 0; c < 16; ++c) m[c] = mine(c) ? Mj[(long long)c * cols.ld] : 0.0;
-                ok = oz_wait(m_full, T & 1, &s_abort);
+                // the lanes leave together: the TMEM loads below take the whole warp
+                ok = __all_sync(0xffffffffu, oz_wait(m_full, T & 1, &s_abort));
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 // the six accumulators into one exact sum per element, then the
