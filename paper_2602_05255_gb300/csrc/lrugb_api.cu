@@ -192,23 +192,25 @@ static void prof_end(lru_ctx* h, int cls) {
     if (h->prof_used[cls] < v.size()) cudaEventRecord(v[h->prof_used[cls]++].second, h->stream);
 }
 
-// matrices that the kernels with a CTA per matrix hold at once: two CTAs per SM, four
-// of the blocked Pfaffian where their copies stay below 5 GiB
-static int elimination_slots(int64_t W, int n, int n_sm) {
-    return (int)std::min<int64_t>(W, (n <= 1024 ? 4 : 2) * (int64_t)n_sm);
+// matrices that the kernels with a CTA per matrix hold at once: two CTAs per SM; four
+// of the real double Pfaffian, whose kernel alone is built for them (refresh.cu,
+// k_slogpf), while their copies stay below 5 GiB (n <= 1024)
+static int elimination_slots(bool pf, int32_t dtype, int64_t W, int n, int n_sm) {
+    return (int)std::min<int64_t>(W, (pf && dtype == LRU_F64 && n <= 1024 ? 4 : 2) * (int64_t)n_sm);
 }
 
 static lru_status ensure_ws(lru_ctx* h) {
     if (h->ws) return LRU_OK;
-    int nws = elimination_slots(h->W, h->n_max, h->n_sm);
-    size_t b = (size_t)nws * h->n_max * h->n_max * dtype_size(h->dtype);
-    if (cudaMalloc(&h->ws, b) != cudaSuccess) {
+    const int two = elimination_slots(false, h->dtype, h->W, h->n_max, h->n_sm);
+    for (int nws = elimination_slots(h->pf, h->dtype, h->W, h->n_max, h->n_sm); nws >= two; nws = nws > two ? two : 0) {
+        if (cudaMalloc(&h->ws, (size_t)nws * h->n_max * h->n_max * dtype_size(h->dtype)) == cudaSuccess) {
+            h->nws = nws;
+            return LRU_OK;
+        }
         cudaGetLastError();
         h->ws = nullptr;
-        return LRU_ERR_NOMEM;
     }
-    h->nws = nws;
-    return LRU_OK;
+    return LRU_ERR_NOMEM;
 }
 
 extern "C" {
@@ -1216,9 +1218,15 @@ static lru_status batched_dense(bool pf, int32_t dtype, int64_t W, int32_t n, co
     int dev = 0, nsm = 148;
     CK(cudaGetDevice(&dev));
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); nsm = 148; }
-    const int nws = pf ? elimination_slots(W, n, nsm) : (int)std::min<int64_t>(W, 2 * nsm);
+    const int two = elimination_slots(false, dtype, W, n, nsm);
+    int nws = elimination_slots(pf, dtype, W, n, nsm);
     void* ws = nullptr;
-    CK(cudaMallocAsync(&ws, (size_t)nws * n * n * dtype_size(dtype), st));
+    if (nws > two && cudaMallocAsync(&ws, (size_t)nws * n * n * dtype_size(dtype), st) != cudaSuccess) {
+        cudaGetLastError();
+        ws = nullptr;
+        nws = two;
+    }
+    if (!ws) CK(cudaMallocAsync(&ws, (size_t)nws * n * n * dtype_size(dtype), st));
     lru_ctx tmp;
     tmp.dtype = dtype;
     DevLayout L{};

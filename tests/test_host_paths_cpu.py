@@ -125,3 +125,25 @@ def test_standalone_calls_see_a_wait_that_gives_up(run, dtype):
             got = {{fake.fake_launch_arg(i) for i, x in enumerate(names()) if watch.decode() in x}}
             assert len(got) == 1 and None not in got and len(sizes()) == 1, (watch, got)
     """)
+
+
+@pytest.mark.parametrize("kind,dtype,n,per_sm", [("DET", "F64", 100, 2), ("DET", "C64", 100, 2), ("DET", "F32", 600, 2),
+                                                 ("PF", "F64", 64, 4), ("PF", "F64", 1024, 4), ("PF", "F64", 1026, 2),
+                                                 ("PF", "C128", 64, 2), ("PF", "C128", 1024, 2), ("PF", "F32", 64, 2)])
+def test_elimination_slots_are_those_the_kernel_fills(run, kind, dtype, n, per_sm):
+    """Copies of the kernels with a CTA per matrix: what a handle and the standalone Pfaffian allocate."""
+    run(f"""
+        slots = {per_sm} * 152 * {n} * {n} * SIZE[{dtype}]
+        h = create(kind={kind}, dtype={dtype}, W=1000, n={n}, delay=0, refresh=1)
+        fake.fake_reset()
+        assert lib.lru_refresh_from_scratch(h, PTR, None, PTR) == OK and sizes() == [slots], (sizes(), slots)
+        if {kind} == PF:
+            f = lib.lru_slogpf_batched
+            f.argtypes = [C.c_int32, C.c_int64, C.c_int32] + [C.c_void_p] * 4
+            fake.fake_reset()
+            assert f({dtype}, 1000, {n}, PTR, PTR, PTR, None) == OK and sizes() == [slots]
+            # where four copies per SM are not to be had, two still serve
+            fake.fake_reset()
+            fake.fake_alloc_limit(2 * 152 * {n} * {n} * SIZE[{dtype}])
+            assert f({dtype}, 1000, {n}, PTR, PTR, PTR, None) == OK
+    """)
