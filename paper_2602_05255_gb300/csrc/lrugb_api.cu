@@ -107,6 +107,7 @@ struct lru_ctx {
     // workspace of the tensor-core refresh (allocated on first use)
     void* ozw = nullptr;
     size_t oz_bytes = 0;
+    bool oz_refused = false;     // its allocation failed: a native flush does not ask again before the next init
     void* ozM = nullptr;         // fresh inverses when the drift is asked for
     size_t ozM_bytes = 0;
     bool oz_ok = false;          // the tensor-core refresh applies to this handle, in place
@@ -530,8 +531,10 @@ static lru_status ensure_oz(lru_ctx* h) {
     if (cudaMalloc(&h->ozw, b) != cudaSuccess) {
         cudaGetLastError();
         h->ozw = nullptr;
+        h->oz_refused = true;
         return LRU_ERR_NOMEM;
     }
+    h->oz_refused = false;
     h->oz_bytes = b;
     return LRU_OK;
 }
@@ -554,7 +557,7 @@ static bool native_flush_split(lru_ctx* h) {
         return false;
     const double madds = (double)h->W * h->n_uni * h->n_uni * h->kk * oz_cx(h) * oz_cx(h);   // FP64, per step
     if (madds < (double)(1 << 24) || (long long)h->W * OZ_S * oz_flush_rows(h->n_uni) * oz_cx(h) >= (1ll << 31)) return false;
-    if (!h->ozw && capturing(h)) return false;
+    if (!h->ozw && (h->oz_refused || capturing(h))) return false;
     return ensure_oz(h) == LRU_OK;
 }
 
@@ -667,6 +670,7 @@ static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, doub
         cudaGetLastError();   // tensor maps unavailable: the FP64 form below
     }
     // the workspace of the flushes to come, so that the first of them may be captured
+    h->oz_refused = false;
     if (h->delayed && h->flush == LRU_FLUSH_NATIVE) native_flush_split(h);
     prof_begin(h, LRU_PROF_REFRESH);
     bool done = false;

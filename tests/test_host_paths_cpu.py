@@ -147,3 +147,22 @@ def test_elimination_slots_are_those_the_kernel_fills(run, kind, dtype, n, per_s
             fake.fake_alloc_limit(2 * 152 * {n} * {n} * SIZE[{dtype}])
             assert f({dtype}, 1000, {n}, PTR, PTR, PTR, None) == OK
     """)
+
+
+def test_refused_flush_workspace_is_asked_for_once(run):
+    """A native flush whose workspace is not to be had runs in FP64 tiles and asks again at the next init only."""
+    run("""
+        h = create(n=130)
+        fake.fake_alloc_limit(1 << 20)
+        for _ in range(2):
+            fake.fake_reset()
+            assert init(h) == OK
+            for _ in range(9):
+                assert propose(h) == OK and accept(h) == OK
+            assert sum("k_flush_native" in x for x in names()) == 9 and not any("k_oz_gemm" in x for x in names())
+            # the flush's workspace, and the padded elimination's (which runs in its FP64 form)
+            assert len(sizes(ok=False)) == 2, sizes(ok=False)
+        fake.fake_alloc_limit(1 << 40)
+        assert init(h) == OK and propose(h) == OK and accept(h) == OK
+        assert "k_flush_native" not in names()[-2] and any("k_oz_gemm" in x for x in names())
+    """)
