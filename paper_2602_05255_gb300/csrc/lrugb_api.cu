@@ -669,16 +669,18 @@ static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, doub
         }
         cudaGetLastError();   // tensor maps unavailable: the FP64 form below
     }
-    // the workspace of the flushes to come, so that the first of them may be captured
-    h->oz_refused = false;
-    if (h->delayed && h->flush == LRU_FLUSH_NATIVE) native_flush_split(h);
+    // what the call cannot do without comes before what only makes it (or a flush) faster
+    if (h->pf) {
+        lru_status s = ensure_ws(h);
+        if (s != LRU_OK) return s;
+    }
     prof_begin(h, LRU_PROF_REFRESH);
     bool done = false;
     if (!h->oz_ok && oz_padded(h->n_uni) && h->cfg.refresh != LRU_REFRESH_FP64) {
         if (h->dtype == LRU_F64) done = refresh_padded<double>(h, (const double*)A, mask, drift);
         else if (h->dtype == LRU_C128) done = refresh_padded<c128>(h, (const c128*)A, mask, drift);
     }
-    if ((with_ws && !done) || h->pf) {
+    if (with_ws && !done) {
         lru_status s = ensure_ws(h);
         if (s != LRU_OK) { prof_end(h, LRU_PROF_REFRESH); return s; }
     }
@@ -692,6 +694,9 @@ static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, doub
         if (h->pf) launch_slogpf<T>(L, (const T*)A, mask, (T*)h->ws, h->nws, S.logabs, S.sgn, h->stream);
     });
     prof_end(h, LRU_PROF_REFRESH);
+    // the workspace of the flushes to come, so that the first of them may be captured
+    h->oz_refused = false;
+    if (h->delayed && h->flush == LRU_FLUSH_NATIVE) native_flush_split(h);
     lru_status s = cuda_check();
     if (s != LRU_OK) return s;
     const size_t sz = dtype_size(h->dtype);

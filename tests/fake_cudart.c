@@ -16,27 +16,28 @@ static struct { const void* fn; const char* name; int smem[DEVICES]; } funcs[MAX
 static int nfuncs, device, last;
 static struct { int func, device, ok; unsigned grid_x; void* arg; } launches[MAXL];
 static int nlaunches;
-static size_t alloc_limit = (size_t)-1;
+static size_t alloc_limit = (size_t)-1, total_limit = (size_t)-1, total;
 static char refuse[64], watch[64];
 static int watch_arg;
-static struct { size_t bytes; int ok; } allocs[MAXL];
-static int nallocs;
+static struct { size_t bytes; int ok; void* p; } allocs[MAXL];
+static int nallocs, first;
 
 static int fail(int e) { last = e; return e; }
 
 /* ---- what the test reads and sets ---- */
-void fake_alloc_limit(size_t b) { alloc_limit = b; }
+void fake_alloc_limit(size_t b) { alloc_limit = b; }      /* of one allocation */
+void fake_total_limit(size_t b) { total_limit = b; }      /* of all together */
 void fake_refuse_launch(const char* s) { strncpy(refuse, s, sizeof refuse - 1); }
 void fake_watch(const char* s, int arg) { strncpy(watch, s, sizeof watch - 1); watch_arg = arg; }
-void fake_reset(void) { nlaunches = nallocs = 0; }
+void fake_reset(void) { nlaunches = 0; first = nallocs; }
 int fake_launches(void) { return nlaunches; }
 const char* fake_launch_name(int i) { return funcs[launches[i].func].name; }
 int fake_launch_ok(int i) { return launches[i].ok; }
 unsigned fake_launch_grid(int i) { return launches[i].grid_x; }
 void* fake_launch_arg(int i) { return launches[i].arg; }
-int fake_allocs(void) { return nallocs; }
-size_t fake_alloc_bytes(int i) { return allocs[i].bytes; }
-int fake_alloc_ok(int i) { return allocs[i].ok; }
+int fake_allocs(void) { return nallocs - first; }
+size_t fake_alloc_bytes(int i) { return allocs[first + i].bytes; }
+int fake_alloc_ok(int i) { return allocs[first + i].ok; }
 
 /* ---- registration and launches ---- */
 void** __cudaRegisterFatBinary(void* f) { (void)f; return (void**)malloc(8); }
@@ -90,16 +91,23 @@ int cudaFuncSetAttribute(const void* fn, int attr, int value) {
 
 /* ---- memory ---- */
 static int alloc(void** p, size_t n) {
-    const int ok = n <= alloc_limit;
-    if (nallocs < MAXL) { allocs[nallocs].bytes = n; allocs[nallocs].ok = ok; ++nallocs; }
-    if (!ok) return fail(NOMEM);
-    *p = aligned_alloc(256, (n + 255) / 256 * 256);   /* untouched pages cost nothing */
-    return *p ? OK : fail(NOMEM);
+    int ok = n <= alloc_limit && total + n <= total_limit;
+    *p = ok ? aligned_alloc(256, (n + 255) / 256 * 256) : NULL;   /* untouched pages cost nothing */
+    ok = *p != NULL;
+    if (ok) total += n;
+    if (nallocs < MAXL) { allocs[nallocs].bytes = n; allocs[nallocs].ok = ok; allocs[nallocs].p = *p; ++nallocs; }
+    return ok ? OK : fail(NOMEM);
+}
+static int release(void* p) {
+    for (int i = 0; p && i < nallocs; ++i)
+        if (allocs[i].p == p) { total -= allocs[i].bytes; allocs[i].p = NULL; }
+    free(p);
+    return OK;
 }
 int cudaMalloc(void** p, size_t n) { return alloc(p, n); }
 int cudaMallocAsync(void** p, size_t n, void* s) { (void)s; return alloc(p, n); }
-int cudaFree(void* p) { free(p); return OK; }
-int cudaFreeAsync(void* p, void* s) { (void)s; free(p); return OK; }
+int cudaFree(void* p) { return release(p); }
+int cudaFreeAsync(void* p, void* s) { (void)s; return release(p); }
 int cudaMemcpy(void* d, const void* s, size_t n, int k) { (void)k; memcpy(d, s, n); return OK; }
 int cudaMemcpyAsync(void* d, const void* s, size_t n, int k, void* st) { (void)d; (void)s; (void)n; (void)k; (void)st; return OK; }
 int cudaMemset(void* d, int v, size_t n) { (void)d; (void)v; (void)n; return OK; }

@@ -17,9 +17,10 @@ PRELUDE = r"""
 import ctypes as C
 fake = C.CDLL(None)
 lib = C.CDLL(LIB)
-for f, r, a in (("fake_alloc_limit", None, [C.c_size_t]), ("fake_refuse_launch", None, [C.c_char_p]),
-                ("fake_watch", None, [C.c_char_p, C.c_int]), ("fake_launch_name", C.c_char_p, [C.c_int]),
-                ("fake_launch_arg", C.c_void_p, [C.c_int]), ("fake_alloc_bytes", C.c_size_t, [C.c_int])):
+for f, r, a in (("fake_alloc_limit", None, [C.c_size_t]), ("fake_total_limit", None, [C.c_size_t]),
+                ("fake_refuse_launch", None, [C.c_char_p]), ("fake_watch", None, [C.c_char_p, C.c_int]),
+                ("fake_launch_name", C.c_char_p, [C.c_int]), ("fake_launch_arg", C.c_void_p, [C.c_int]),
+                ("fake_alloc_bytes", C.c_size_t, [C.c_int])):
     getattr(fake, f).restype, getattr(fake, f).argtypes = r, a
 DET, PF, F64, C128, F32, C64, OK = 0, 1, 0, 1, 2, 3, 0
 SIZE = {F64: 8, C128: 16, F32: 4, C64: 8}
@@ -165,4 +166,15 @@ def test_refused_flush_workspace_is_asked_for_once(run):
         fake.fake_alloc_limit(1 << 40)
         assert init(h) == OK and propose(h) == OK and accept(h) == OK
         assert "k_flush_native" not in names()[-2] and any("k_oz_gemm" in x for x in names())
+    """)
+
+
+def test_optional_workspaces_come_after_the_required_one(run):
+    """A Pfaffian handle that fits beside its elimination slots is initialised, whatever else there is no room for."""
+    run("""
+        h = create(kind=PF, n=512, W=304)
+        slots = 304 * 512 * 512 * 8
+        fake.fake_total_limit(sum(sizes()) + slots + (1 << 20))
+        assert init(h, PF) == OK
+        assert sizes(ok=True)[1:] == [slots]
     """)
