@@ -194,7 +194,7 @@ static void prof_end(lru_ctx* h, int cls) {
 }
 
 // matrices that the kernels with a CTA per matrix hold at once: two CTAs per SM; four
-// of the real double Pfaffian, whose kernel alone is built for them (refresh.cu,
+// of the real double Pfaffian, whose kernels alone are built for them (refresh.cu,
 // k_slogpf), while their copies stay below 5 GiB (n <= 1024)
 static int elimination_slots(bool pf, int32_t dtype, int64_t W, int n, int n_sm) {
     return (int)std::min<int64_t>(W, (pf && dtype == LRU_F64 && n <= 1024 ? 4 : 2) * (int64_t)n_sm);

@@ -7,6 +7,7 @@
 #include "internal.h"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace lru {
 
@@ -378,16 +379,17 @@ __device__ void pr_pfaffian(T* M, int n, double* logabs, T* sgn, T* s_tau, T* s_
     __syncthreads();
 }
 
-// The same elimination for the double types, blocked: only the upper triangle is
-// kept (a row right of the diagonal is minus the column below it), and the
+// The same elimination for large matrices of the double types, blocked: only the
+// upper triangle is kept (a row right of the diagonal is minus the column below it), and the
 // congruences of PFB / 2 pairs are collected before they meet the trailing block,
 // as one rank-PFB update of its upper tiles in 64 x 64 register tiles.  Inside a
 // block of pairs the two rows that a pair needs are brought up to date one by one.
 // The collected vectors tau_t and r_t lie in the rows k and k + 1 that their pair
 // has used up.  The unblocked form reads and writes the whole trailing block for
 // every pair (n^3 / 6 scalars each way, twice the FMAs): 1024 matrices of n = 256
-// took 27.9 ms, of which the FP64 pipe accounts for 9; this form 12.0 ms, 4.6 of the
-// FP64 pipe, the rest the row-by-row phase and its barriers.
+// took 27.9 ms at two CTAs per SM and 18.9 at four, of which the FP64 pipe accounts
+// for 9; this form 12.0 ms (four), 4.6 of the FP64 pipe, the rest the row-by-row
+// phase and its barriers.
 constexpr int PFB = 16;   // rows (two per pair) collected per update
 
 template <typename T>
@@ -533,13 +535,8 @@ __device__ void pr_pfaffian_blocked(T* M, int n, double* logabs, T* sgn, PfSmem<
     __syncthreads();
 }
 
-// Single precision keeps the unblocked order of its sums: the log-value it
-// accumulates in double shows every bit of them.
-template <typename T> constexpr bool pf_blocked() { return sizeof(typename traits<T>::real) == 8; }
-template <typename T> constexpr size_t pf_smem() { return pf_blocked<T>() ? sizeof(PfSmem<T>) : 2 * 2048 * sizeof(T); }
-
-template <typename T>
-__global__ void __launch_bounds__(RT, pf_blocked<T>() && sizeof(T) == 8 ? 4 : 2)
+template <typename T, bool BLOCKED>
+__global__ void __launch_bounds__(RT, std::is_same<T, double>::value ? 4 : 2)
     k_slogpf(DevLayout L, const T* A, const uint8_t* mask, T* ws, double* logabs, T* sgn) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ double s_l;
@@ -551,11 +548,11 @@ __global__ void __launch_bounds__(RT, pf_blocked<T>() && sizeof(T) == 8 ? 4 : 2)
         const T* Aw = A + L.mo(w);
         for (long long e = threadIdx.x; e < (long long)n * n; e += RT) M[e] = Aw[e];
         __syncthreads();
-        if constexpr (pf_blocked<T>()) {
+        if constexpr (BLOCKED) {
             pr_pfaffian_blocked(M, n, &s_l, &s_s, *reinterpret_cast<PfSmem<T>*>(dsm));
         } else {
             T* s_tau = reinterpret_cast<T*>(dsm);
-            pr_pfaffian(M, n, &s_l, &s_s, s_tau, s_tau + 2048);
+            pr_pfaffian(M, n, &s_l, &s_s, s_tau, s_tau + L.n_max);
         }
         if (threadIdx.x == 0) {
             logabs[w] = s_l;
@@ -602,9 +599,30 @@ void launch_refresh(bool pf, bool delayed, const DevLayout& L, const DevState<T>
 template <typename T>
 void launch_slogpf(const DevLayout& L, const T* A, const uint8_t* mask, T* ws, int nws, double* logabs, T* sgn,
                    cudaStream_t st) {
-    const int dyn = (int)pf_smem<T>();
-    cudaFuncSetAttribute(k_slogpf<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-    k_slogpf<T><<<nws, RT, dyn, st>>>(L, A, mask, ws, logabs, sgn);
+    auto go = [&](auto kern, size_t dyn) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        kern<<<nws, RT, dyn, st>>>(L, A, mask, ws, logabs, sgn);
+    };
+    // The blocked form for the double types where it is the faster one (its row phase
+    // costs seven barriers a pair, whatever n).  Per call of 1 / 152 / 304 / 1024
+    // matrices on 152 SMs, blocked against unblocked, ms: F64 n = 112 0.55 / 0.55 / 0.77
+    // / 2.46 against 0.56 / 0.59 / 0.67 / 1.90, n = 144 0.73 / 0.75 / 1.11 / 3.68
+    // against 0.87 / 0.89 / 1.25 / 3.40, n = 256 2.0 / 2.1 / 3.5 / 12.3 against 4.6 /
+    // 5.1 / 7.7 / 18.9; C128 n = 130 1.78 / 1.81 / 3.20 / 10.4 against 1.43 / 1.51 / 2.35
+    // / 7.96, n = 192 3.28 / 3.41 / 6.16 / 20.5 against 3.61 / 4.17 / 6.27 / 21.8.
+    // Single precision keeps the unblocked order of its sums everywhere: the
+    // log-value it accumulates in double shows every bit of them.
+    if constexpr (sizeof(typename traits<T>::real) == 8) {
+        int dev = 0, nsm = 148;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        const bool blocked = traits<T>::is_complex ? L.n_max >= 192 : L.n_max >= (L.W <= nsm ? 112 : 140);
+        if (blocked) {
+            go(k_slogpf<T, true>, sizeof(PfSmem<T>));
+            return;
+        }
+    }
+    go(k_slogpf<T, false>, 2 * (size_t)L.n_max * sizeof(T));
 }
 
 template <typename T>
