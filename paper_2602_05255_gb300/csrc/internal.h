@@ -147,12 +147,20 @@ struct OzCols {
 };
 // rows of the working matrix of an n x n inverse: n padded by the identity
 int oz_rows(int n);
-// The sizes eliminated on padded copies.  Against the FP64 form (one CTA per
-// walker), refresh of 1 / 1024 F64 walkers on GB300: n = 64 0.35 / 1.1 ms against
-// 0.52 / 2.5, n = 72 (padded to 128) 0.72 / 3.1 against 0.73 / 4.0; between 64 and
-// 72 the padding costs a single walker more than the products gain, and below 56
-// a padded panel does.
+// The sizes eliminated on padded copies (rows in steps of 64): below 56 a padded
+// panel, and between 64 and 72 the padding, costs more than the products gain.
 constexpr bool oz_padded(int n) { return n >= 72 || (n >= 56 && n <= 64); }
+// For the determinant alone (LU form) and complex scalars that is the whole rule:
+// 1 / 1024 matrices, FP64 form (one CTA per matrix) against padded, ms: F64 LU n = 60
+// 0.54 / 2.3 against 0.45 / 1.2, n = 72 0.85 / 4.0 against 0.78 / 2.7; C128 inverse n = 56
+// 0.81 / 4.4 against 0.68 / 2.1, n = 72 2.0 / 11.9 against 1.4 / 6.1.  The inverse of F64
+// matrices is as fast in the FP64 form while its CTAs still fill one wave: n = 56 ..
+// 62 up to one per SM (n = 60, 1 / 152 / 228 walkers: 0.38 / 0.39 / 0.51 against 0.39 /
+// 0.41 / 0.46), n = 72 .. 79, padded to 128, up to two (n = 76, 1 / 304 / 456: 0.73 / 1.16
+// / 2.27 against 0.80 / 1.26 / 1.53; n = 80 0.89 / 1.33 / 2.64 against 0.79 / 1.26 / 1.54).
+inline bool oz_padded_inverse(int n, int cx, long long W, int n_sm) {
+    return oz_padded(n) && (cx == 2 || n >= 80 || n == 63 || n == 64 || W > (n < 64 ? 1 : 2) * (long long)n_sm);
+}
 // bytes of the workspace of W walkers of nr rows (cx = 2: complex), and its parts when Z is given
 size_t oz_work_layout(OzWork* Z, void* base, int W, int nr, int cx, bool with_M);
 // M[w] = A[w]^T (or A[w]) with an identity in rows and columns n .. nr - 1

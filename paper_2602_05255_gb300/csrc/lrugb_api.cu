@@ -676,7 +676,7 @@ static lru_status do_init(lru_handle h, const void* A, const uint8_t* mask, doub
     }
     prof_begin(h, LRU_PROF_REFRESH);
     bool done = false;
-    if (!h->oz_ok && oz_padded(h->n_uni) && h->cfg.refresh != LRU_REFRESH_FP64) {
+    if (!h->oz_ok && oz_padded_inverse(h->n_uni, oz_cx(h), h->W, h->n_sm) && h->cfg.refresh != LRU_REFRESH_FP64) {
         if (h->dtype == LRU_F64) done = refresh_padded<double>(h, (const double*)A, mask, drift);
         else if (h->dtype == LRU_C128) done = refresh_padded<c128>(h, (const c128*)A, mask, drift);
     }
@@ -1264,15 +1264,15 @@ static lru_status slog_backward(bool pf, int32_t dtype, int64_t W, int32_t n, co
     if (pf && (n & 1)) return LRU_ERR_ARG;
     if (g_sign && !sign) return LRU_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    if (oz_padded(n) &&
+    int dev = 0, nsm = 148;
+    CK(cudaGetDevice(&dev));
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); nsm = 148; }
+    if (oz_padded_inverse(n, dtype == LRU_C128 ? 2 : 1, W, nsm) &&
         ((dtype == LRU_F64 && slog_backward_padded<double>(pf, (int)W, n, (const double*)A, g_logabs,
                                                            (const double*)g_sign, (const double*)sign, (double*)gA, st)) ||
          (dtype == LRU_C128 && slog_backward_padded<c128>(pf, (int)W, n, (const c128*)A, g_logabs, (const c128*)g_sign,
                                                           (const c128*)sign, (c128*)gA, st))))
         return cuda_check();
-    int dev = 0, nsm = 148;
-    CK(cudaGetDevice(&dev));
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); nsm = 148; }
     const int nws = (int)std::min<int64_t>(W, 2 * nsm);
     const size_t sz = dtype_size(dtype), nn = (size_t)n * n;
     // the inverses (W n^2), the Gauss-Jordan slots (nws n^2) and the per-walker status

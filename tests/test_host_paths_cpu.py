@@ -178,3 +178,21 @@ def test_optional_workspaces_come_after_the_required_one(run):
         assert init(h, PF) == OK
         assert sizes(ok=True)[1:] == [slots]
     """)
+
+
+@pytest.mark.parametrize("dtype,n,W,padded", [
+    ("F64", 55, 1000, False), ("F64", 56, 152, False), ("F64", 56, 153, True), ("F64", 62, 1, False), ("F64", 62, 200, True),
+    ("F64", 63, 1, True), ("F64", 64, 1, True), ("F64", 65, 1000, False), ("F64", 72, 304, False), ("F64", 72, 305, True),
+    ("F64", 79, 1, False), ("F64", 80, 1, True), ("C128", 56, 1, True), ("C128", 65, 1000, False), ("C128", 72, 1, True)])
+def test_inverse_takes_the_faster_form(run, dtype, n, W, padded):
+    """Inverses of few small F64 matrices stay with the FP64 form (152 SMs here), those of complex ones do not."""
+    run(f"""
+        used = lambda: any("k_oz_gemm" in x for x in names())
+        h = create(dtype={dtype}, W={W}, n={n}, delay=0)
+        fake.fake_reset()
+        assert init(h) == OK and used() is {padded}
+        grad = lib.lru_slogdet_backward
+        grad.argtypes = [C.c_int32, C.c_int64, C.c_int32] + [C.c_void_p] * 6
+        fake.fake_reset()
+        assert grad({dtype}, {W}, {n}, PTR, PTR, None, None, PTR, None) == OK and used() is {padded}
+    """)
