@@ -100,15 +100,35 @@ __device__ void backward_core(const T* Cw, int m, const T* sR, T gw, T* gCw) {
         }
 }
 
-// |g| |x| between 2^-900 and 2^900, by the exponents of the larger parts, or x = 0
-__device__ __forceinline__ int part_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-__device__ __forceinline__ int part_exponent(c128 x) { return max(part_exponent(x.re), part_exponent(x.im)); }
-__device__ __forceinline__ bool is_zero(double x) { return x == 0.0; }
-__device__ __forceinline__ bool is_zero(c128 x) { return x.re == 0.0 && x.im == 0.0; }
+// gC of every walker, a thread each: where there are more walkers than SMs, beside
+// k_backward, whose CTAs would wait for one thread of theirs (1024 walkers, n = 34, F64
+// two-particle moves: 160 us with the core inside, 67 beside; 64 walkers 38 and 43)
+template <typename T>
+__global__ void __launch_bounds__(32) k_backward_core(DevLayout L, DevState<T> S, const T* C, const T* g, T* gC) {
+    const int w = blockIdx.x * 32 + threadIdx.x;
+    if (w >= L.W) return;
+    const int kk = L.kv(w);
+    T* gCw = gC + (long long)w * L.kk * L.kk;
+    if (S.pst[w] != 0) {
+        for (int e = 0; e < kk * kk; ++e) gCw[e] = s_zero(T());
+        return;
+    }
+    backward_core<T>(C ? C + (long long)w * L.kk * L.kk : nullptr, kk, S.Rinv + (long long)w * AMAXKK * AMAXKK, g[w], gCw);
+}
+
+// |g| |x| far inside the range (2^-900 .. 2^900, single precision 2^-100 .. 2^100), by
+// the exponents of the larger parts, or x = 0
+__device__ __forceinline__ int part_exponent(double x) { return (__double2hiint(x) >> 20 & 0x7ff) - 1023; }
+__device__ __forceinline__ int part_exponent(float x) { return (__float_as_int(x) >> 23 & 0xff) - 127; }
+template <typename R>
+__device__ __forceinline__ int part_exponent(cplx<R> x) { return max(part_exponent(x.re), part_exponent(x.im)); }
+template <typename R> __device__ __forceinline__ bool is_zero(R x) { return x == R(0); }
+template <typename R> __device__ __forceinline__ bool is_zero(cplx<R> x) { return x.re == R(0) && x.im == R(0); }
 template <typename T>
 __device__ __forceinline__ bool product_in_range(T g, T x) {
-    const int e = part_exponent(g) + part_exponent(x) - 2046;
-    return (e >= -900 && e <= 900) || is_zero(x);
+    constexpr int lim = sizeof(typename traits<T>::real) == 8 ? 900 : 100;
+    const int e = part_exponent(g) + part_exponent(x);
+    return (e >= -lim && e <= lim) || is_zero(x);
 }
 
 template <typename T>
@@ -154,7 +174,8 @@ __global__ void __launch_bounds__(AT, 2) k_backward(DevLayout L, DevState<T> S, 
         }
         if (gAw)
             for (long long e = threadIdx.x; e < (long long)rows * n; e += AT) gAw[(long long)it.y * n + e] = s_zero(T());
-        if (gC && it.y == 0 && threadIdx.x < kk * kk) gC[(long long)w * L.kk * L.kk + threadIdx.x] = s_zero(T());
+        if (PF && gC && it.y == 0 && threadIdx.x < kk * kk)
+            gC[(long long)w * L.kk * L.kk + threadIdx.x] = s_zero(T());
         return;
     }
     const T gw = g[w];
@@ -205,21 +226,24 @@ __global__ void __launch_bounds__(AT, 2) k_backward(DevLayout L, DevState<T> S, 
         __syncthreads();
         if (gAw) {
             const T gs = PF ? s_half(s_neg(gw)) : s_neg(gw);
-            for (int j = threadIdx.x; j < n; j += AT) {
+            // fewer columns than threads: the rows go to several groups of n threads
+            const int stride = min(n, AT), groups = AT / stride, grp = (int)threadIdx.x / stride;
+            auto column = [&](int j, auto one_group) {
                 T x[KBM];
-                // Where g X stays far inside the range (double types), g goes into the
-                // n kk factors and not the n^2 outputs: 551 against 611 us for the
-                // orbital gradient of 512 walkers, n = 256, which the FP64 pipe bounds.
-                // Otherwise, and in single precision, it multiplies the finished sum.
-                bool late = ordered<T>() || kk > KBM;
+                // Where g X stays far inside the range, g goes into the n kk factors and
+                // not the n^2 outputs: 551 against 611 us for the orbital gradient of 512
+                // walkers, n = 256, which the FP64 pipe bounds.  Otherwise it multiplies
+                // the finished sum.
+                bool late = kk > KBM;
 #pragma unroll
                 for (int b = 0; b < KBM; ++b) {
                     x[b] = b < kk ? s_conj(X[(long long)b * n + j]) : s_zero(T());
-                    if constexpr (!ordered<T>()) late = late || !product_in_range(gs, x[b]);
+                    late = late || !product_in_range(gs, x[b]);
                 }
+                constexpr bool one = decltype(one_group)::value;
                 auto rows = [&](auto after) {
 #pragma unroll 4
-                    for (int c = 0; c < nc; ++c) {
+                    for (int c = one ? 0 : grp; c < nc; c += one ? 1 : groups) {
                         T s = s_zero(T());
 #pragma unroll
                         for (int b = 0; b < KBM; ++b)
@@ -238,7 +262,11 @@ __global__ void __launch_bounds__(AT, 2) k_backward(DevLayout L, DevState<T> S, 
                     for (int b = 0; b < KBM; ++b) x[b] = gs * x[b];
                     rows(std::false_type());
                 }
-            }
+            };
+            if (groups == 1)
+                for (int j = threadIdx.x; j < n; j += AT) column(j, std::true_type());
+            else if (grp < groups)
+                column((int)threadIdx.x - grp * stride, std::false_type());
         }
         __syncthreads();
     }
@@ -320,8 +348,12 @@ static void launch_backward_k(bool pf, bool delayed, const DevLayout& L, const D
 template <typename T>
 void launch_backward(bool pf, bool delayed, const DevLayout& L, const DevState<T>& S, const DevOperand& V,
                      const T* C, const T* g, T* gU, T* gV, T* gA, T* gC, const int* items, int nitems,
-                     cudaStream_t st) {
+                     bool core_beside, cudaStream_t st) {
     const int4* it = reinterpret_cast<const int4*>(items);
+    if (pf && gC && core_beside) {
+        k_backward_core<T><<<(L.W + 31) / 32, 32, 0, st>>>(L, S, C, g, gC);
+        gC = nullptr;
+    }
     if (L.kk == 1) launch_backward_k<T, 1>(pf, delayed, L, S, V, C, g, gU, gV, gA, gC, it, nitems, st);
     else if (L.kk == 2) launch_backward_k<T, 2>(pf, delayed, L, S, V, C, g, gU, gV, gA, gC, it, nitems, st);
     else if (L.kk <= 4) launch_backward_k<T, 4>(pf, delayed, L, S, V, C, g, gU, gV, gA, gC, it, nitems, st);
@@ -396,7 +428,7 @@ void launch_slog_grad(int W, int n, int nr, bool pf, const T* Ginv, const uint8_
     template void launch_slog_grad<T>(int, int, int, bool, const T*, const uint8_t*, const int*, const double*, const T*,     \
                                       const T*, T*, cudaStream_t);                                            \
     template void launch_backward<T>(bool, bool, const DevLayout&, const DevState<T>&, const DevOperand&,     \
-                                     const T*, const T*, T*, T*, T*, T*, const int*, int, cudaStream_t);       \
+                                     const T*, const T*, T*, T*, T*, T*, const int*, int, bool, cudaStream_t); \
     template void launch_backward_logvalue<T>(bool, bool, const DevLayout&, const DevState<T>&, const T*, T*, \
                                               cudaStream_t);                                                  \
     template void launch_log_ratio<T>(int, const T*, T*, cudaStream_t);                                       \

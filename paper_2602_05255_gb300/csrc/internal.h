@@ -234,7 +234,7 @@ void launch_gj_compact(int W, int n, int nr, const T* A, T* M, const uint8_t* ma
 template <typename T>
 void launch_backward(bool pf, bool delayed, const DevLayout& L, const DevState<T>& S, const DevOperand& V,
                      const T* C, const T* g, T* gU, T* gV, T* gA, T* gC, const int* items, int nitems,
-                     cudaStream_t st);
+                     bool core_beside, cudaStream_t st);
 template <typename T>
 void launch_backward_logvalue(bool pf, bool delayed, const DevLayout& L, const DevState<T>& S, const T* g, T* gA,
                               cudaStream_t st);

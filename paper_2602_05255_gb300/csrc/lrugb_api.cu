@@ -70,6 +70,8 @@ struct lru_ctx {
     int* d_kv = nullptr;
     int* d_items = nullptr;
     int nitems = 0;
+    int* d_bitems = nullptr;     // the adjoint's work items
+    int nbitems = 0;
     // persistent step: propose order, accept items (largest walkers first), control block
     int* d_order = nullptr;
     int* d_sitems = nullptr;
@@ -338,6 +340,21 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
         }
     }
     h->nitems = (int)items.size() / 4;
+    // the adjoint's items: the same, but 64 columns or more each once there are eight
+    // for every SM (it works in blocks of 32 columns, and a CTA costs it more to start:
+    // 1024 walkers of n = 34 in items of 8 columns against one CTA a walker, complex128
+    // determinants of rank 1 128 against 92 us)
+    std::vector<int> bitems;
+    if (h->nitems > 8 * h->n_sm)
+        for (size_t q = 0; q < items.size(); q += 4) {
+            const bool more = !bitems.empty() && bitems[bitems.size() - 4] == items[q] &&
+                              items[q + 1] - bitems[bitems.size() - 3] < 64;
+            if (more) bitems[bitems.size() - 2] = items[q + 2];
+            else bitems.insert(bitems.end(), items.begin() + q, items.begin() + q + 4);
+        }
+    else
+        bitems = items;
+    h->nbitems = (int)bitems.size() / 4;
     // persistent-step queue: walkers by decreasing n^2 k (longest first)
     std::vector<int> order(h->W), nacc_w(h->W, 0), sitems;
     for (int w = 0; w < h->W; ++w) order[w] = w;
@@ -408,6 +425,7 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
     const size_t oVoff = take((size_t)h->W * sizeof(long long));
     const size_t oKv = take((size_t)h->W * sizeof(int));
     const size_t oItems = take(items.size() * sizeof(int));
+    const size_t oBItems = take(bitems.size() * sizeof(int));
     const size_t oOrder = take((size_t)h->W * sizeof(int));
     const size_t oSItems = take(sitems.size() * sizeof(int));
     const size_t oNacc = take((size_t)h->W * sizeof(int));
@@ -447,6 +465,7 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
     h->d_voff = (long long*)(b + oVoff);
     h->d_kv = kuni ? nullptr : (int*)(b + oKv);
     h->d_items = (int*)(b + oItems);
+    h->d_bitems = (int*)(b + oBItems);
     h->d_order = (int*)(b + oOrder);
     h->d_sitems = (int*)(b + oSItems);
     h->d_nacc_w = (int*)(b + oNacc);
@@ -463,6 +482,7 @@ lru_status lru_create(const lru_config* cfg, lru_handle* out) {
         cudaMemcpy(h->d_voff, h->voff_h.data(), h->W * sizeof(long long), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b + oKv, h->kv_h.data(), h->W * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_items, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(h->d_bitems, bitems.data(), bitems.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_order, order.data(), h->W * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_sitems, sitems.data(), sitems.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(h->d_xitems, xitems.data(), xitems.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -1080,10 +1100,11 @@ static lru_status do_backward(lru_handle h, bool pf, const void* g, void* gU, vo
     if (!h->has_prop) return LRU_ERR_STATE;
     CK(cudaSetDevice(h->device));
     DevLayout L = h->layout();
-    h->launches += 1;
+    const bool core_beside = pf && gC && h->W > h->n_sm;
+    h->launches += core_beside ? 2 : 1;
     LRU_DISPATCH(h, {
         launch_backward<T>(pf, h->delayed, L, h->state<T>(), h->lastV, (const T*)h->lastC, (const T*)g, (T*)gU,
-                           (T*)gV, (T*)gA, (T*)gC, h->d_items, h->nitems, h->stream);
+                           (T*)gV, (T*)gA, (T*)gC, h->d_bitems, h->nbitems, core_beside, h->stream);
     });
     return cuda_check();
 }
