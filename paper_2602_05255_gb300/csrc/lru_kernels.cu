@@ -277,39 +277,45 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
         }
     }
 
-    // ---- core: R = I + V X (det) or M = C^{-1} + B^T X (pf); a warp takes one
-    //      row of V against up to four columns of X ----
-    const int na4 = (kk + 3) / 4;
-    for (int p = wid; p < kk * na4; p += PT / 32) {
-        const int b = p / na4, a0 = (p - b * na4) * 4, na = min(4, kk - a0);
-        const T* Xa = X + (long long)a0 * n;
-        T s[4];
+    // ---- core: R = I + V X (det) or M = C^{-1} + B^T X (pf); a warp takes one row
+    //      of V against NA columns of X, as many as leave a task for every warp
+    //      (one walker of n = 2000, k = 2, complex128: a propose 56 us with four
+    //      columns a task, 23 with one) ----
+    auto core = [&](auto na_tag) {
+        constexpr int NA = decltype(na_tag)::value;
+        const int groups = (kk + NA - 1) / NA;
+        for (int p = wid; p < kk * groups; p += PT / 32) {
+            const int b = p / groups, a0 = (p - b * groups) * NA, na = min(NA, kk - a0);
+            const T* Xa = X + (long long)a0 * n;
+            T s[NA];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) s[q] = s_zero(T());
-        const int q = spread_index<4>();   // the column this lane holds after the sum
-        if (s_iv[b] >= 0) {
-            if (q < na) s[0] = Xa[(long long)q * n + s_iv[b]];
-        } else {
-            const T* vb = vec_ptr<T>(Vop, L, w, b, n);
-            if (na == 1) {
-                for (int j = lane; j < n; j += 32) s[0] = s_fma(vb[j], Xa[j], s[0]);
-                s[0] = warp_sum(s[0]);
+            for (int q = 0; q < NA; ++q) s[q] = s_zero(T());
+            const int q = spread_index<NA>();   // the column this lane holds after the sum
+            if (s_iv[b] >= 0) {
+                if (q < na) s[0] = Xa[(long long)q * n + s_iv[b]];
             } else {
+                const T* vb = vec_ptr<T>(Vop, L, w, b, n);
+                const T* xa[NA];
+#pragma unroll
+                for (int a = 0; a < NA; ++a) xa[a] = Xa + (long long)min(a, na - 1) * n;
+#pragma unroll (sizeof(T) == 16 && NA > 1 ? 1 : 4)
                 for (int j = lane; j < n; j += 32) {
                     const T v = vb[j];
 #pragma unroll
-                    for (int a = 0; a < 4; ++a)
-                        if (a < na) s[a] = s_fma(v, Xa[(long long)a * n + j], s[a]);
+                    for (int a = 0; a < NA; ++a) s[a] = s_fma(v, xa[a][j], s[a]);
                 }
-                warp_sum_spread<4>(s);
+                warp_sum_spread<NA>(s);
+            }
+            if (spread_owner<NA>() && q < na) {
+                const int a = a0 + q;
+                T base = PF ? s_cinv[b * MAXKK + a] : make_real<T>(b == a ? 1.0 : 0.0);
+                s_core[b * MAXKK + a] = base + s[0];
             }
         }
-        if (spread_owner<4>() && q < na) {
-            const int a = a0 + q;
-            T base = PF ? s_cinv[b * MAXKK + a] : make_real<T>(b == a ? 1.0 : 0.0);
-            s_core[b * MAXKK + a] = base + s[0];
-        }
-    }
+    };
+    if (kk <= 2) core(std::integral_constant<int, 1>());
+    else if (kk <= 4) core(std::integral_constant<int, 2>());
+    else core(std::integral_constant<int, 4>());
     // ---- det delayed: V P (kk x cu) for the accept's correction ----
     if constexpr (DELAYED && !PF) {
         T* VP = S.VP + (long long)w * MAXKK * Kc;
