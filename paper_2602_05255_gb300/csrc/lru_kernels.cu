@@ -230,7 +230,7 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
         for (int a = 0; a < kk; ++a)
             if (s_iu[a] >= 0)
                 for (int c = tid; c < cu; c += PT) s_qtu[c * MAXKK + a] = S.Q[(vo + s_iu[a]) * Kc + c];
-        if (ndu > 0)
+        if (ndu > 0 && cu > 0)
             slot_dot<T, false>(S.Q + vo * Kc, Kc, cu, n, vec_ptr<T>(U, L, w, 0, n), dlu, ndu, s_slot,
                                [&](int c, int a, T v) { s_qtu[c * MAXKK + a] = v; });
         __syncthreads();
@@ -249,7 +249,7 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
 
     if constexpr (DELAYED) {
         // X -= P (Q^T U) (det)   or   X += P (Q^T B) (pf)
-        for (int a = 0; a < kk; a += 4) {
+        for (int a = 0; cu > 0 && a < kk; a += 4) {
             T* Xa = X + (long long)a * n;
             const T *P = S.P + vo * Kc, *q = s_qtu + a;
             if (kk - a > 2) {
@@ -323,7 +323,7 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
             const int b = e / cu, c = e - b * cu;
             if (s_iv[b] >= 0) VP[b * Kc + c] = S.P[(vo + s_iv[b]) * Kc + c];
         }
-        if (ndv > 0)
+        if (ndv > 0 && cu > 0)
             slot_dot<T, true>(S.P + vo * Kc, Kc, cu, n, vec_ptr<T>(Vop, L, w, 0, n), dlv, ndv, s_slot,
                               [&](int c, int b, T v) { VP[b * Kc + c] = v; });
     }
@@ -590,8 +590,14 @@ __global__ void __launch_bounds__(PT, 2) k_dense_column_skew_df(DevLayout L, Dev
 
 // the standalone propose: the Pfaffian accept that follows is in skew form
 // (plain: k_accept_pf_skew; delayed: the slots), so M is projected
+//
+// CTAs per SM that the registers have to leave room for (0: as the compiler has it):
+// the products with dense slots hold 32 sums a thread in F32, for which it takes 80
+// registers (three CTAs; 1024 walkers of n = 64, K = 4, one-hot U: 14.6 us a propose,
+// 12.1 at four).
+template <typename T, bool DELAYED> constexpr int propose_ctas() { return sizeof(T) == 4 && DELAYED ? 4 : 0; }
 template <typename T, bool PF, bool DELAYED>
-__global__ void __launch_bounds__(PT) k_propose(DevLayout L, DevState<T> S, DevOperand U, DevOperand V,
+__global__ void __launch_bounds__(PT, propose_ctas<T, DELAYED>()) k_propose(DevLayout L, DevState<T> S, DevOperand U, DevOperand V,
                                                  const T* C, T* ratio_out, int* st_out) {
     propose_walker<T, PF, DELAYED, PF>(blockIdx.x, L, S, U, V, C, ratio_out, st_out);
 }
