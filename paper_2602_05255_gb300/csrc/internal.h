@@ -65,12 +65,26 @@ struct DevOperand {
 // rows of X per work item of the persistent step (XT in passes.cuh)
 constexpr int STEP_X_ROWS = 64;
 
+// Dense columns of U for small matrices: the propose's own CTA sums X = A^{-1} U, a
+// thread per row, instead of a pass that spreads it over the chip.  Up to
+// x_inline_rows for every proposal (that pass is a launch of its own: one F32 walker,
+// n = 4, k = 4, 14.7 us a propose with it, 11.4 without; complex128 pays for a longer
+// chain per row: 1024 walkers of n = 16 42 and 48 us).
+constexpr int x_inline_rows(size_t scalar) { return scalar == 16 ? 8 : 32; }
+// In the persistent step also, in single precision, for one dense column of up to a
+// row per thread while every walker's CTA has an SM to itself: handing the tiles
+// around costs more than it spreads (64 walkers, delayed, rank 1, complex64: n = 64
+// 37 / 32 us a step with tiles / in the CTA, n = 256 63 / 54).
+inline bool step_x_inline(int n_max, size_t scalar, int dense, int W, int n_sm, bool single) {
+    return n_max <= x_inline_rows(scalar) || (single && dense == 1 && W <= n_sm && n_max <= 256);
+}
+
 // Control block of the persistent fused step (see k_step).
 struct StepCtl {
     int* counter;             // work-queue head, zeroed before each launch
     int* x_done;              // W counters of finished X tiles (zeroed)
     const int2* x_items;      // X tiles (walker, row block), largest walkers first
-    int n_x_items;            // 0: every column of U is one-hot
+    int n_x_items;            // 0: every column of U is one-hot, or the propose sums them itself
     int* prop_done;           // W flags, zeroed before each launch
     int* items_done;          // W counters, zeroed before each launch
     int* fin;                 // W flags: the walker's propose, accept and commit are done (zeroed)

@@ -138,7 +138,7 @@ size_t propose_smem(int Kc, bool delayed) {
 // needs the inverse of M as computed (SKEWM = false there).
 template <typename T, bool PF, bool DELAYED, bool SKEWM = DELAYED>
 __device__ void propose_walker(const int w, const DevLayout L, const DevState<T> S, const DevOperand U,
-                               const DevOperand V, const T* C, T* ratio_out, int* st_out) {
+                               const DevOperand V, const T* C, T* ratio_out, int* st_out, const bool x_inline) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     // delayed only: the scratch of the slot products, then Q^T U (Kc x MAXKK)
     SlotSmem<T>& s_slot = *reinterpret_cast<SlotSmem<T>*>(dyn_smem);
@@ -237,7 +237,8 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
     }
 
     // ---- X = A^{-1} U: one-hot columns are a contiguous chunk copy; the dense
-    //      ones are there already (dense_x_rows, or a double-float pass) ----
+    //      ones are there already (dense_x_rows, or a double-float pass), or (see
+    //      x_inline_rows) a thread sums one of their rows here ----
     for (int a = 0; a < kk; ++a) {
         T* Xa = X + (long long)a * n;
         if (s_iu[a] >= 0) {
@@ -245,6 +246,15 @@ __device__ void propose_walker(const int w, const DevLayout L, const DevState<T>
             for (int j = tid; j < n; j += PT) Xa[j] = col[j];
         }
     }
+    if (x_inline)
+        for (int e = tid; e < ndu * n; e += PT) {
+            const int d = e / n, j = e - d * n;
+            const T* u = vec_ptr<T>(U, L, w, dlu[d], n);
+            T acc = s_zero(T());
+#pragma unroll 8
+            for (int l = 0; l < n; ++l) acc = s_fma(G[(long long)l * n + j], u[l], acc);
+            X[(long long)dlu[d] * n + j] = acc;
+        }
     __syncthreads();
 
     if constexpr (DELAYED) {
@@ -598,8 +608,8 @@ __global__ void __launch_bounds__(PT, 2) k_dense_column_skew_df(DevLayout L, Dev
 template <typename T, bool DELAYED> constexpr int propose_ctas() { return sizeof(T) == 4 && DELAYED ? 4 : 0; }
 template <typename T, bool PF, bool DELAYED>
 __global__ void __launch_bounds__(PT, propose_ctas<T, DELAYED>()) k_propose(DevLayout L, DevState<T> S, DevOperand U, DevOperand V,
-                                                 const T* C, T* ratio_out, int* st_out) {
-    propose_walker<T, PF, DELAYED, PF>(blockIdx.x, L, S, U, V, C, ratio_out, st_out);
+                                                 const T* C, T* ratio_out, int* st_out, bool x_inline) {
+    propose_walker<T, PF, DELAYED, PF>(blockIdx.x, L, S, U, V, C, ratio_out, st_out, x_inline);
 }
 
 // ---------------------------------------------------------------------------
@@ -1583,7 +1593,7 @@ __global__ void __launch_bounds__(PT, 2) k_step(DevLayout L, DevState<T> S, DevO
                                                             S.err)) ? 1 : 0;
                 __syncthreads();
                 if (s_ok) {
-                    propose_walker<T, PF, DEL, DEL>(w, L, S, U, V, C, ratio_out, st_out);
+                    propose_walker<T, PF, DEL, DEL>(w, L, S, U, V, C, ratio_out, st_out, nx == 0);
                     __syncthreads();
                     if (threadIdx.x == 0) {
                         bool acc = ctl.do_accept && S.pst[w] == 0;
@@ -1947,7 +1957,8 @@ void launch_propose(bool pf, bool delayed, bool df, const DevLayout& L, const De
             launched = true;
         }
     }
-    if (!launched) {
+    const bool x_inline = !launched && L.n_max <= x_inline_rows(sizeof(T));
+    if (!launched && !x_inline) {
         const int nt = (L.n_max + XT - 1) / XT;
         const int nd = __builtin_popcount(dense), tpc = nd == 1 ? PT / 64 : PT / 32;
         const dim3 grid = ordered<T>() ? dim3((unsigned)(((long long)L.W * nt + tpc - 1) / tpc)) : dim3(L.W, nt);
@@ -1956,15 +1967,15 @@ void launch_propose(bool pf, bool delayed, bool df, const DevLayout& L, const De
         else if (nd <= 4) k_dense_x<T, 4><<<grid, PT, 0, st>>>(L, S, U);
         else k_dense_x<T, kb_max<T>()><<<grid, PT, 0, st>>>(L, S, U);
     }
-    if (!pf && !delayed) k_propose<T, false, false><<<L.W, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out);
+    if (!pf && !delayed) k_propose<T, false, false><<<L.W, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out, x_inline);
     if (!pf && delayed) {
         cudaFuncSetAttribute(k_propose<T, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        k_propose<T, false, true><<<L.W, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out);
+        k_propose<T, false, true><<<L.W, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out, x_inline);
     }
-    if (pf && !delayed) k_propose<T, true, false><<<L.W, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out);
+    if (pf && !delayed) k_propose<T, true, false><<<L.W, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out, x_inline);
     if (pf && delayed) {
         cudaFuncSetAttribute(k_propose<T, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        k_propose<T, true, true><<<L.W, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out);
+        k_propose<T, true, true><<<L.W, PT, dyn, st>>>(L, S, U, V, C, ratio_out, st_out, x_inline);
     }
 }
 

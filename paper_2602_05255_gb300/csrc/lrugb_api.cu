@@ -756,6 +756,13 @@ static bool operand_ok(const lru_operand* o, int kk) {
     return true;
 }
 
+// launches of a propose besides its own kernel: the dense columns' pass
+static int dense_launches(const lru_ctx* h, unsigned dense) {
+    if (!dense) return 0;
+    const bool df = h->df && (dense & (dense - 1)) == 0;
+    return df || h->n_max > x_inline_rows(dtype_size(h->dtype)) ? 1 : 0;
+}
+
 lru_status lru_propose_det(lru_handle h, const lru_operand* U, const lru_operand* V, void* ratio, int32_t* st) {
     LRU_RANGE();
     if (!h || !ratio) return LRU_ERR_ARG;
@@ -766,7 +773,7 @@ lru_status lru_propose_det(lru_handle h, const lru_operand* U, const lru_operand
     DevOperand dV{V->dense, V->idx, V->onehot_mask, h->kk};
     DevLayout L = h->layout();
     const unsigned all = (1u << h->kk) - 1u;
-    h->launches += 1 + ((dU.mask & all) != all ? 1 : 0);
+    h->launches += 1 + dense_launches(h, ~dU.mask & all);
     prof_begin(h, LRU_PROF_PROPOSE);
     LRU_DISPATCH(h, {
         launch_propose<T>(false, h->delayed, h->df, L, h->state<T>(), dU, dV, nullptr, (T*)ratio, st, h->stream);
@@ -788,7 +795,7 @@ lru_status lru_propose_pf(lru_handle h, const lru_operand* B, const void* C, voi
     DevOperand dB{B->dense, B->idx, B->onehot_mask, h->kk};
     DevLayout L = h->layout();
     const unsigned all = (1u << h->kk) - 1u;
-    h->launches += 1 + ((dB.mask & all) != all ? 1 : 0);
+    h->launches += 1 + dense_launches(h, ~dB.mask & all);
     prof_begin(h, LRU_PROF_PROPOSE);
     LRU_DISPATCH(h, {
         launch_propose<T>(true, h->delayed, h->df, L, h->state<T>(), dB, dB, (const T*)C, (T*)ratio, st, h->stream);
@@ -821,7 +828,9 @@ lru_status lru_step_persistent(lru_handle h, const lru_operand* U, const lru_ope
     ctl.flush_done = h->d_ctl + 1 + 3 * h->W;
     ctl.x_done = h->d_ctl + 1 + 4 * h->W;
     ctl.x_items = reinterpret_cast<const int2*>(h->d_xitems);
-    ctl.n_x_items = (~dU.mask & ((1u << h->kk) - 1u)) != 0 ? h->nx : 0;
+    const int dense = __builtin_popcount(~dU.mask & ((1u << h->kk) - 1u));
+    const bool single = h->dtype == LRU_F32 || h->dtype == LRU_C64;
+    ctl.n_x_items = dense == 0 || step_x_inline(h->n_max, dtype_size(h->dtype), dense, h->W, h->n_sm, single) ? 0 : h->nx;
     ctl.acc = acc_out ? acc_out : h->d_acc;
     ctl.order = h->d_order;
     ctl.acc_items = reinterpret_cast<const int4*>(h->d_sitems);
