@@ -1751,11 +1751,13 @@ __global__ void k_set_delay_zero(DevLayout L, DevState<T> S) {
 }
 
 // current A^{-1} (row-major out) = A_0^{-1} -/+ P Q^T: a transposing copy, bound by
-// HBM when no slots are pending.  TW x TW tiles (rows of 512 bytes), all loads of a thread in flight before the barrier: with 32 x 32 tiles of
-// four loads a thread, 1024 walkers of n = 1024 (17 GB) took 4.04 ms, now 2.36.
+// HBM when no slots are pending.  TW x TW tiles (rows of 512 bytes), all loads of a
+// thread in flight before the barrier: with 32 x 32 tiles of four loads a thread, 1024
+// walkers of n = 1024 (17 GB) took 4.04 ms, now 2.36.  The plain form moves complex64 as
+// doubles: as pairs of floats 64 walkers of n = 1024 took 175 us, against 155.
 template <typename T> constexpr int inv_tw() { return sizeof(T) == 16 ? 32 : 64; }
 
-template <typename T, bool PF, bool DELAYED>
+template <typename T, bool PF, bool DELAYED, bool ROWS4>
 __global__ void __launch_bounds__(256) k_get_inverse(DevLayout L, DevState<T> S, T* out) {
     constexpr int TW = inv_tw<T>(), TPR = TW / 32, NQ = 32 * TPR / 8;   // TW columns l x 32 * TPR rows j
     __shared__ T sT[TW][32 * TPR + 1];
@@ -1775,7 +1777,7 @@ __global__ void __launch_bounds__(256) k_get_inverse(DevLayout L, DevState<T> S,
             const int j = j0 + tx + 32 * h, l = l0 + ty + 8 * q;
             v[q][h] = j < n && l < n ? Gw[(long long)l * n + j] : s_zero(T());
         }
-    if (DELAYED && cu) {
+    if (DELAYED && cu && !ROWS4) {   // a sum per element
 #pragma unroll
         for (int q = 0; q < NQ; ++q)
 #pragma unroll
@@ -1788,6 +1790,41 @@ __global__ void __launch_bounds__(256) k_get_inverse(DevLayout L, DevState<T> S,
                 for (int c = 0; c < cu; ++c) s = s_fma(pr[c], qr[c], s);
                 v[q][h] = PF ? v[q][h] + s : v[q][h] - s;
             }
+    } else if (DELAYED && cu) {
+        // four rows of Q against TPR of P at a time, so a load serves several products
+        // (see launch_get_inverse)
+        const T* pr[TPR];
+#pragma unroll
+        for (int h = 0; h < TPR; ++h) pr[h] = S.P + (vo + min(j0 + tx + 32 * h, n - 1)) * L.Kc;
+#pragma unroll
+        for (int q0 = 0; q0 < NQ; q0 += 4) {
+            if (l0 + ty + 8 * q0 >= n) break;   // a warp's rows past the walker's
+            const T* qr[4];
+            T s[4][TPR];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                qr[q] = S.Q + (vo + min(l0 + ty + 8 * (q0 + q), n - 1)) * L.Kc;
+#pragma unroll
+                for (int h = 0; h < TPR; ++h) s[q][h] = s_zero(T());
+            }
+            for (int c = 0; c < cu; ++c) {
+                T p[TPR];
+#pragma unroll
+                for (int h = 0; h < TPR; ++h) p[h] = pr[h][c];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (l0 + ty + 8 * (q0 + q) >= n) continue;
+                    const T y = qr[q][c];
+#pragma unroll
+                    for (int h = 0; h < TPR; ++h)
+                        if (j0 + 32 * h < n) s[q][h] = s_fma(p[h], y, s[q][h]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int h = 0; h < TPR; ++h) v[q0 + q][h] = PF ? v[q0 + q][h] + s[q][h] : v[q0 + q][h] - s[q][h];
+        }
     }
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
@@ -2098,10 +2135,28 @@ void launch_get_inverse(bool pf, bool delayed, const DevLayout& L, const DevStat
                         cudaStream_t st) {
     const int nt = (L.n_max + inv_tw<T>() - 1) / inv_tw<T>();   // square tiles
     dim3 grid(nt, nt, L.W);
-    if (!pf && !delayed) k_get_inverse<T, false, false><<<grid, 256, 0, st>>>(L, S, out);
-    if (!pf && delayed) k_get_inverse<T, false, true><<<grid, 256, 0, st>>>(L, S, out);
-    if (pf && !delayed) k_get_inverse<T, true, false><<<grid, 256, 0, st>>>(L, S, out);
-    if (pf && delayed) k_get_inverse<T, true, true><<<grid, 256, 0, st>>>(L, S, out);
+    if constexpr (std::is_same<T, c64>::value) {
+        if (!delayed) {   // a copy: as doubles
+            DevState<double> D{};
+            D.G = reinterpret_cast<double*>(S.G);
+            k_get_inverse<double, false, false, false><<<grid, 256, 0, st>>>(L, D, reinterpret_cast<double*>(out));
+            return;
+        }
+    }
+    if (!delayed) {
+        k_get_inverse<T, false, false, false><<<grid, 256, 0, st>>>(L, S, out);
+        return;
+    }
+    // Pending slots: sums of four rows at once save loads and cost registers.  1024
+    // Pfaffian walkers with full slots, rows / elements: F32 n = 100, 8 slot columns 33 / 65
+    // us, n = 256 154 / 311; F64 n = 16, 16 columns 42 / 18, n = 100 253 / 332, n = 256 1071 /
+    // 1922; with 8 columns n = 200 551 / 458, n = 256 615 / 676.  complex128, which the FP64
+    // pipe bounds: n = 100 855 / 741.
+    bool rows4 = sizeof(T) != 16 && L.n_max > 48;
+    if (std::is_same<T, double>::value) rows4 = rows4 && (L.Kc > 8 || L.n_max >= 256);
+    auto go = [&](auto kern) { kern<<<grid, 256, 0, st>>>(L, S, out); };
+    if (pf) rows4 ? go(k_get_inverse<T, true, true, sizeof(T) != 16>) : go(k_get_inverse<T, true, true, false>);
+    else rows4 ? go(k_get_inverse<T, false, true, sizeof(T) != 16>) : go(k_get_inverse<T, false, true, false>);
 }
 
 template <typename T>
