@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(PT, propose_ctas<T, DELAYED>()) k_propose(DevL
 //            generic Woodbury A^{-1} - X M^{-1} (B^T A^{-1}))
 //   delayed: y -= (V P) Q[l,:]^T ; Q[l, tau] = (R^{-1} y)^T     (b_tau equation)
 // ---------------------------------------------------------------------------
-template <typename T, int NPL, int KKS>
+template <typename T, int NPL, int KKS, bool PAIR>
 __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> S, const DevOperand V,
                             const uint8_t* mask) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
@@ -658,15 +658,18 @@ __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> 
     __syncthreads();
 
     T* Gw = S.G + L.mo(w);
-    if constexpr (KKS == 1 && NPL * sizeof(T) <= 128) {
-        // rank 1: two columns at a time while they fit the registers.  The FP64 pipe
-        // bounds the pass, and five of its 38 instructions per column (n = 500) are the
-        // butterfly of the dot product: two columns share one, as they share the loads
-        // of V and X (384 walkers, n = 500: 455 -> 430 us an accept).
-        for (int l = it.y + wid; l < it.z; l += 2 * (PT / 32)) {
-            const bool two = l + PT / 32 < it.z;
+    int l = it.y + wid;
+    if constexpr (PAIR) {
+        // rank 1, dense V: two columns at a time (accept_pairs).  The FP64 pipe bounds the
+        // pass, and five of its 38 instructions per column (n = 500) are the butterfly of
+        // the dot product: two columns share one, as they share the loads of V and X (384
+        // walkers, n = 500: 455 -> 430 us an accept).  A column without a partner goes to
+        // the loop below.  A one-hot V has no dot product, and its kernel no pairs, whose
+        // registers would cost it CTAs (1024 F64 walkers, n = 256: a propose and accept
+        // 342 us in pairs, 355 one by one beside them, 314 without).
+        for (; siv[0] < 0 && l + PT / 32 < it.z; l += 2 * (PT / 32)) {
             T* c0 = Gw + (long long)l * n;
-            T* c1 = two ? c0 + (long long)(PT / 32) * n : c0;
+            T* c1 = c0 + (long long)(PT / 32) * n;
             T v[2][NPL];
 #pragma unroll
             for (int m = 0; m < NPL; ++m) {
@@ -675,20 +678,16 @@ __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> 
                 v[1][m] = j < n ? c1[j] : s_zero(T());
             }
             T y[2] = {s_zero(T()), s_zero(T())};
-            if (siv[0] >= 0) {
-                y[0] = lane < 16 ? c0[siv[0]] : c1[siv[0]];
-            } else {
 #pragma unroll
-                for (int m = 0; m < NPL; ++m) {
-                    const int j = lane + 32 * m;
-                    if (j < n) {
-                        const T vj = sV[j];
-                        y[0] = s_fma(vj, v[0][m], y[0]);
-                        y[1] = s_fma(vj, v[1][m], y[1]);
-                    }
+            for (int m = 0; m < NPL; ++m) {
+                const int j = lane + 32 * m;
+                if (j < n) {
+                    const T vj = sV[j];
+                    y[0] = s_fma(vj, v[0][m], y[0]);
+                    y[1] = s_fma(vj, v[1][m], y[1]);
                 }
-                warp_sum_spread<2>(y);   // lanes 0 .. 15: column l, the others: the second
             }
+            warp_sum_spread<2>(y);   // lanes 0 .. 15: column l, the others: the second
             const T z = s_fma(sR[0], y[0], s_zero(T()));
             const T z0 = shfl(z, 0), z1 = shfl(z, 16);
 #pragma unroll
@@ -697,13 +696,12 @@ __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> 
                 if (j < n) {
                     const T xj = sX[j];
                     c0[j] = s_fms(xj, z0, v[0][m]);
-                    if (two) c1[j] = s_fms(xj, z1, v[1][m]);
+                    c1[j] = s_fms(xj, z1, v[1][m]);
                 }
             }
         }
-        return;
     }
-    for (int l = it.y + wid; l < it.z; l += PT / 32) {
+    for (; l < it.z; l += PT / 32) {
         T* col = Gw + (long long)l * n;
         T v[NPL];
 #pragma unroll
@@ -748,10 +746,10 @@ __device__ void accept_item(const int4 it, const DevLayout L, const DevState<T> 
     }
 }
 
-template <typename T, int NPL, int KKS>
+template <typename T, int NPL, int KKS, bool PAIR>
 __global__ void __launch_bounds__(PT, 2) k_accept(DevLayout L, DevState<T> S, DevOperand V, const uint8_t* mask,
                                                    const int4* items) {
-    accept_item<T, NPL, KKS>(items[blockIdx.x], L, S, V, mask);
+    accept_item<T, NPL, KKS, PAIR>(items[blockIdx.x], L, S, V, mask);
 }
 
 // The delayed accept of rank k for the columns of one work item: y = V A_0^{-1}
@@ -1618,7 +1616,7 @@ __global__ void __launch_bounds__(PT, 2) k_step(DevLayout L, DevState<T> S, DevO
             __syncthreads();
             if (s_ok && ctl.acc[w]) {
                 if constexpr (DEL) accept_delayed_item<T, KBM>(it, L, S, V, nullptr);
-                else accept_item<T, NPL, KKS>(it, L, S, V, nullptr);
+                else accept_item<T, NPL, KKS, KKS == 1 && NPL * sizeof(T) <= 128>(it, L, S, V, nullptr);
             }
             __syncthreads();
             if (threadIdx.x == 0 && s_ok) {
@@ -2016,13 +2014,32 @@ void launch_propose(bool pf, bool delayed, bool df, const DevLayout& L, const De
     }
 }
 
+// Whether a rank-1 accept with dense V takes two columns per warp: while they fit the
+// registers.  With 8-byte scalars and n = 129 .. 256 the pair leaves two CTAs per SM
+// in place of four, which pays while the items are one wave of them (64 walkers, n =
+// 256, a propose and accept: F64 35 against 40 us) and not where HBM bounds the pass
+// (1024 walkers: F64 n = 200 302 against 283, complex64 170 against 150).  Other sizes,
+// 1024 walkers: F64 n = 64 54 / 66, n = 128 116 / 142, n = 500 1121 / 1205; complex128
+// n = 100 300 / 373, n = 256 1047 / 1162; F32 n = 256 108 / 114.
+template <typename T, int NPL>
+static bool accept_pairs(int nitems) {
+    if (NPL * sizeof(T) > 128) return false;
+    if (sizeof(T) != 8 || NPL != 8) return true;
+    int dev = 0, nsm = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return nitems <= 2 * nsm;
+}
+
 template <typename T>
 static void accept_plain(int npl, const DevLayout& L, const DevState<T>& S, const DevOperand& V, const uint8_t* mask,
                          const int4* it, int nitems, size_t dyn, cudaStream_t st) {
     const bool rank1 = L.kk == 1 && L.kvec == nullptr;
 #define LRU_ACC(N)                                                                                          \
     case N: {                                                                                               \
-        auto k = rank1 ? k_accept<T, N, 1> : k_accept<T, N, 0>;                                             \
+        constexpr bool P = N * sizeof(T) <= 128;   /* built for */                                          \
+        auto k = rank1 ? k_accept<T, N, 1, false> : k_accept<T, N, 0, false>;                               \
+        if (rank1 && !(V.mask & 1u) && accept_pairs<T, N>(nitems)) k = k_accept<T, N, 1, P>;                \
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);                     \
         k<<<nitems, PT, dyn, st>>>(L, S, V, mask, it);                                                      \
     } break;
