@@ -1545,16 +1545,19 @@ __global__ void __launch_bounds__(PT, 2) k_step(DevLayout L, DevState<T> S, DevO
     const int nacc = (ctl.do_accept && !(PF && DEL)) ? ctl.nacc : 0;
     const int nfl = (ctl.do_accept && DEL) ? ctl.nflush : 0;
     const int total = nx + L.W + nacc + nfl;
+    const bool ahead = total > 8 * (int)gridDim.x;
     if (threadIdx.x == 0) s_item = atomicAdd(ctl.counter, 1);
     for (;;) {
         __syncthreads();
         int item = s_item;
         __syncthreads();
         if (item >= total) break;
-        // the next item is drawn while this one is worked on; a CTA works its
-        // items in the order drawn, so the waits below still end
+        // Where there are many items a CTA, the next one is drawn while this one is
+        // worked on; a CTA works its items in the order drawn, so the waits below
+        // still end.  With few, an item would wait for its CTA while others idle (64
+        // walkers, n = 34 .. 256: 2 to 10 us a step).
         int next = 0;
-        if (threadIdx.x == 0) next = atomicAdd(ctl.counter, 1);
+        if (ahead && threadIdx.x == 0) next = atomicAdd(ctl.counter, 1);
         if (item < nx) {
             if constexpr (ordered<T>()) {
                 // a warp per X tile
@@ -1657,7 +1660,7 @@ __global__ void __launch_bounds__(PT, 2) k_step(DevLayout L, DevState<T> S, DevO
                 }
             }
         }
-        if (threadIdx.x == 0) s_item = next;
+        if (threadIdx.x == 0) s_item = ahead ? next : atomicAdd(ctl.counter, 1);
     }
 }
 
