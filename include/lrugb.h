@@ -73,9 +73,11 @@ typedef enum { LRU_DET = 0, LRU_PF = 1 } lru_kind;
 /* Precision of the delayed flush A0^{-1} -/+= P Q^T (Sec. 2.3 Eq. delayed_Ainv,
  * Sec. 3.3 Eq. pf_delayed_Ainv).  Everything else stays in the handle dtype. */
 typedef enum {
-    LRU_FLUSH_NATIVE = 0,   /* the rounding of dtype arithmetic (FP64 for F64/C128): on the CUDA cores, and for
-                               large F64/C128 handles of uniform n >= 128 with at most 64 doubles of slots per
-                               row by the exact products of LRU_FLUSH_SPLIT */
+    LRU_FLUSH_NATIVE = 0,   /* dtype arithmetic (FP64 for F64/C128) on the CUDA cores; large F64/C128 handles of
+                               uniform n >= 128 with at most 64 doubles of slots per row take the products of
+                               LRU_FLUSH_SPLIT: each row of P and Q held to 2^-57 of its largest entry (slot
+                               columns balanced first), summed exactly, one FP64 rounding per entry.  The
+                               persistent step folds in FP64 tiles on every handle */
     LRU_FLUSH_TF32X3 = 1,   /* tcgen05 TF32 tensor cores, 3-term split (about FP32 accuracy) */
     LRU_FLUSH_TF32 = 2,     /* tcgen05 TF32, one term */
     LRU_FLUSH_BF16 = 3,     /* tcgen05 BF16, one term */
@@ -331,7 +333,9 @@ lru_status lru_slogdet_batched(int32_t dtype, int64_t W, int32_t n, const void* 
  * their own memory pool, code that must avoid the device-wide synchronisation
  * of cudaFree, and code recorded once and replayed later.  The Gauss-Jordan
  * workspace is a fixed 64 MiB array in the library's device memory, which
- * every GPU that loads the library holds until the process exits.  Limit:
+ * every GPU that loads the library holds until the process exits.  It runs the
+ * FP64 form at every size, so it agrees with lru_slogdet_batched to rounding
+ * only (F64 / C128 of n = 56 .. 64 and n >= 72 take split products there).  Limit:
  * one n x n matrix must fit it (n * n * sizeof(scalar) <= 64 MiB, so every
  * n <= 2048 of every dtype); other sizes return LRU_ERR_ARG.  The first call on a
  * device looks up the workspace's address for that device (a runtime query,

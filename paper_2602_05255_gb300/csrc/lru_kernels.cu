@@ -19,7 +19,6 @@
 namespace lru {
 
 constexpr int PT = 256;    // threads of the per-walker kernels
-constexpr int JPT = 8;     // vector elements per thread: n <= PT * JPT = 2048
 constexpr int MAXKK = 16;  // vector slots per update (det k <= 16, pf 2k <= 16)
 
 __device__ __forceinline__ float tf32_round(float x) {

@@ -75,8 +75,7 @@ struct GJSmem {
 // applying each panel's row exchanges and rank-GB transform to the other
 // columns of [j_lo, j_hi) only.  Pivot rows go to perm[k]; log|pivot| and the
 // sign/phase accumulate into the shared s_log / s_sgn, a zero pivot sets
-// s_sing.  The full inverse is c = j = [0, n); the tensor-core refresh runs it
-// on one 64-column panel at a time and updates the other columns itself.
+// s_sing.  The full inverse is c = j = [0, n).
 template <typename T>
 __device__ void gj_columns(T* M, int n, int c_lo, int c_hi, int j_lo, int j_hi, int* perm, double& s_log, T& s_sgn,
                            int& s_sing, GJSmem<T>& sm) {
@@ -1191,9 +1190,10 @@ LRU_INST_R(c64)
 // Some callers cannot let a library allocate device memory: runtimes that
 // preallocate most of the GPU for their own pool (so a cudaMalloc can fail),
 // code that must not hit the device-wide synchronisation of cudaFree, and
-// callers that record work for later replay.  This entry point runs the same
-// Gauss-Jordan kernel as lru_slogdet_batched, with its per-CTA matrix
-// workspace taken from the fixed array below instead of cudaMallocAsync.
+// callers that record work for later replay.  This entry point runs the FP64
+// Gauss-Jordan kernel at every size (lru_slogdet_batched takes split products for
+// F64 / C128 of n = 56 .. 64 and n >= 72, so the two agree to rounding there), with
+// its per-CTA matrix workspace taken from the fixed array below.
 // ---------------------------------------------------------------------------
 
 #include <mutex>
